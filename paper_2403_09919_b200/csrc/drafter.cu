@@ -102,7 +102,7 @@ __global__ void __maxnreg__(88) act_kernel(GemmOut proj, const T* __restrict__ b
   const int m = blockIdx.y;
   const int n = (blockIdx.x * ACT_THREADS + threadIdx.x) * 4;
   const bool active = n < N;
-  const bool fast = proj.m_tiles_max == 1 && (proj.partial == nullptr || proj.all_work);
+  const bool fast = proj.m_tiles_max == 1;
   const size_t stride = gemm_slot_stride(proj);
   GemmSrc src;
   float4 bv = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -457,7 +457,7 @@ __global__ void __maxnreg__(88) draft_seg_kernel(GemmOut proj, int V, int BW, in
   __shared__ float shf[32];
   const int r = blockIdx.y, sgm = blockIdx.x, S = gridDim.x;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const bool fast = proj.m_tiles_max == 1 && (proj.partial == nullptr || proj.all_work);
+  const bool fast = proj.m_tiles_max == 1;
   const size_t stride = gemm_slot_stride(proj);
   GemmSrc src[SEG_ITEMS];
   int col[SEG_ITEMS];

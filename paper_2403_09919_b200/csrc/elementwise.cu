@@ -113,14 +113,14 @@ __global__ void __maxnreg__(88)
   }
   float4* xr = reinterpret_cast<float4*>(x + (size_t)m * d);
   const bool add = proj.raw != nullptr;   // x += the projection that ends the previous block (O or down)
-  // Decode-time launches (one row tile, no idle CTA in the projection): every address is worked out while
+  // Decode-time launches (one row tile): every address is worked out while
   // waiting, and the row's loads do not wait for the row count (rows past it exist in memory and are
   // simply not written back).
   // (A launch laid out for several row tiles whose rows fit one after all is a single-tile launch; inside a
   // chain the row count is known up front.)
   int M = early ? *m_total : 0;
   const bool single = proj.m_tiles_max == 1 || (early && M <= proj.mt);
-  const bool fast = add && single && (proj.partial == nullptr || proj.all_work);
+  const bool fast = add && single;
   const size_t stride = add ? gemm_slot_stride(proj) : 0;
   GemmSrc src[NORM_MAXV];
   if (fast) {
@@ -373,10 +373,10 @@ __global__ void __maxnreg__(88) rope_kv_kernel(float* __restrict__ qkv, GemmOut 
   const int h = idx / (half >> 1), i = (idx - h * (half >> 1)) * 2;
   const int o = h * hd + i;
   float* row = qkv + (size_t)m * 3 * d;
-  // decode-time launches (one row tile, no idle CTA in the projection): every address is known before the
+  // decode-time launches (one row tile): every address is known before the
   // projection has produced anything
   const bool single = proj.m_tiles_max == 1 || (early && *rt.m_total <= proj.mt);   // rows that fit one row tile after all
-  const bool fast = single && (proj.partial == nullptr || proj.all_work);
+  const bool fast = single;
   GemmSrc sq, sk, sv;
   const size_t stride = gemm_slot_stride(proj);
   const float2* tab = table + (size_t)m * half + i;
@@ -417,7 +417,7 @@ __global__ void __maxnreg__(88) rope_kv_kernel(float* __restrict__ qkv, GemmOut 
       }
     }
   } else {
-    // prompt-sized launches (several row tiles) and projections shorter than the grid
+    // prompt-sized launches (several row tiles)
     M = *rt.m_total;
     if (m < M && active) {
       const GemmRows m_tiles = gemm_m_tiles(proj, M);
@@ -534,12 +534,11 @@ __global__ void __launch_bounds__(ROPW_THREADS, 4)
         const size_t doff = (size_t)(m - cur_tile * m_tiles.rows) * 128;
 #pragma unroll
         for (int part = 0; part < 3; ++part)
-          for (int c = f3[part].c_next; c <= f3[part].c_last; ++c)
-            if (gemm_has_work(proj, m_tiles, c)) {
-              const float* pp = proj.partial + (size_t)c * slot_stride + f3[part].off + doff;
-              const float2 t1 = __ldcg(reinterpret_cast<const float2*>(pp)), t2 = __ldcg(reinterpret_cast<const float2*>(pp + half));
-              v1[part].x += t1.x; v1[part].y += t1.y; v2[part].x += t2.x; v2[part].y += t2.y;
-            }
+          for (int c = f3[part].c_next; c <= f3[part].c_last; ++c) {
+            const float* pp = proj.partial + (size_t)c * slot_stride + f3[part].off + doff;
+            const float2 t1 = __ldcg(reinterpret_cast<const float2*>(pp)), t2 = __ldcg(reinterpret_cast<const float2*>(pp + half));
+            v1[part].x += t1.x; v1[part].y += t1.y; v2[part].x += t2.x; v2[part].y += t2.y;
+          }
       }
       const bool slot_ok = slot >= 0 && slot < dm.max_ctx;
       if (!slot_ok && i == 0 && h == 0) atomicOr(status, DEV_ERR_CAPACITY);
@@ -606,7 +605,7 @@ __global__ void __maxnreg__(88) swiglu_kernel(GemmOut proj, T* __restrict__ out,
   const size_t stride = gemm_slot_stride(proj);
   const int M = *m_total;
   const bool single = proj.m_tiles_max == 1 || M <= proj.mt;   // rows that fit one row tile after all
-  const bool fast = single && (proj.partial == nullptr || proj.all_work);
+  const bool fast = single;
   GemmSrc sg[SWIGLU_ITEMS], su[SWIGLU_ITEMS];
   T* dst[SWIGLU_ITEMS];
   bool act[SWIGLU_ITEMS];
@@ -727,16 +726,14 @@ __global__ void __launch_bounds__(SWS_THREADS, 3)
         float4 g = *reinterpret_cast<const float4*>(sg + j), u = *reinterpret_cast<const float4*>(su + j);
         if (cut[k]) {   // add the other contributors' sums in CTA order
           const size_t doff = (size_t)(m - cur_tile * m_tiles.rows) * 128;
-          for (int c = fg[k].c_next; c <= fg[k].c_last; ++c)
-            if (gemm_has_work(proj, m_tiles, c)) {
-              const float4 t = __ldcg(reinterpret_cast<const float4*>(proj.partial + (size_t)c * slot + fg[k].off + doff));
-              g.x += t.x; g.y += t.y; g.z += t.z; g.w += t.w;
-            }
-          for (int c = fu[k].c_next; c <= fu[k].c_last; ++c)
-            if (gemm_has_work(proj, m_tiles, c)) {
-              const float4 t = __ldcg(reinterpret_cast<const float4*>(proj.partial + (size_t)c * slot + fu[k].off + doff));
-              u.x += t.x; u.y += t.y; u.z += t.z; u.w += t.w;
-            }
+          for (int c = fg[k].c_next; c <= fg[k].c_last; ++c) {
+            const float4 t = __ldcg(reinterpret_cast<const float4*>(proj.partial + (size_t)c * slot + fg[k].off + doff));
+            g.x += t.x; g.y += t.y; g.z += t.z; g.w += t.w;
+          }
+          for (int c = fu[k].c_next; c <= fu[k].c_last; ++c) {
+            const float4 t = __ldcg(reinterpret_cast<const float4*>(proj.partial + (size_t)c * slot + fu[k].off + doff));
+            u.x += t.x; u.y += t.y; u.z += t.z; u.w += t.w;
+          }
         }
         store4(out + (size_t)m * F + c0 + j, silu_f(g.x) * u.x, silu_f(g.y) * u.y, silu_f(g.z) * u.z, silu_f(g.w) * u.w);
       }

@@ -19,7 +19,6 @@ struct GemmOut {
   const float* partial;  // [grid][mt * 128 (x 2 in pair mode)], nullptr when nothing is cut (CUDA-core path)
   int ld;
   int nkb, n_tiles, mt, grid, m_tiles_max;   // mt: most rows of a row tile; m_tiles_max: most row tiles of the launch
-  int all_work;          // every CTA has a non-empty range for any row count (units >= CTAs)
   int pair;              // 1: a unit is (pair of adjacent tiles, k-block); a slot holds two tiles, even one first
   int small32;           // (units + 1) * CTAs stays below 2^31 for any row count of the launch: 32-bit index arithmetic
 };
@@ -27,7 +26,21 @@ struct GemmOut {
 // Floats per partial slot (one slot per CTA).
 __host__ __device__ __forceinline__ size_t gemm_slot_stride(const GemmOut& g) { return (size_t)g.mt * 128 * (g.pair ? 2 : 1); }
 
-// Unit range of CTA c: [c*U/G, (c+1)*U/G).
+// CTAs that share U units on a launch of `grid` CTAs: all of them, or, where that would leave a CTA fewer than
+// GEMM_MIN_UNITS units, as many as get that many; the rest have nothing to do and write no slot.  A model of a few
+// hundred columns has fewer units than the part has SMs: spread over all of them, a tile of eight k-blocks lay between
+// 25 CTAs, eight of which held a unit, and the consumers searched the 25 with a 64-bit division each (d = 512, 4 layers,
+// batch 2: rotary 56 us per launch, norm 30; now 2.5 and 2).  Four such steps: 4.60 ms before, 1.72 / 1.63 / 1.65 ms with
+// a minimum of 1 / 2 / 4 units: fewer contributors are cheaper to fold, fewer weight bytes at once are slower to fetch.
+// From twice as many units as CTAs on nothing changes.
+constexpr int GEMM_MIN_UNITS = 2;
+template <typename I>
+__host__ __device__ __forceinline__ I gemm_working(I U, I grid) {
+  const I most = U / GEMM_MIN_UNITS;
+  return most >= grid ? grid : most > 1 ? most : 1;
+}
+
+// Unit range of CTA c of the G that work: [c*U/G, (c+1)*U/G); none for c >= G.
 __host__ __device__ __forceinline__ long long gemm_range_begin(long long c, long long U, long long G) { return c * U / G; }
 // The CTA whose range holds unit u (the largest c with range_begin(c) <= u).
 __host__ __device__ __forceinline__ int gemm_cta_of_unit(long long u, long long U, long long G) {
@@ -66,7 +79,7 @@ __device__ __forceinline__ GemmFold gemm_fold(const GemmOut& g, GemmRows m_tiles
     // (in pair mode the units run over pairs of tiles, and the odd tile sits in the second half of a slot)
     const uint32_t group = g.pair ? (uint32_t)(n_tile >> 1) : (uint32_t)n_tile;
     const uint32_t n_groups = g.pair ? (uint32_t)((g.n_tiles + 1) >> 1) : (uint32_t)g.n_tiles;
-    const uint32_t U = n_groups * g.nkb, G = g.grid, tu0 = group * g.nkb;
+    const uint32_t U = n_groups * g.nkb, G = gemm_working<uint32_t>(U, g.grid), tu0 = group * g.nkb;
     const uint32_t cf = ((tu0 + 1) * G - 1) / U, cl = ((tu0 + g.nkb) * G - 1) / U;
     f.c_next = (int)(cf > G - 1 ? G - 1 : cf) + 1;
     f.c_last = (int)(cl > G - 1 ? G - 1 : cl);
@@ -78,26 +91,19 @@ __device__ __forceinline__ GemmFold gemm_fold(const GemmOut& g, GemmRows m_tiles
   const int group = g.pair ? (n_tile >> 1) : n_tile, n_groups = g.pair ? ((g.n_tiles + 1) >> 1) : g.n_tiles;
   f.off = (size_t)col * 128 + row + ((g.pair && (n_tile & 1)) ? (size_t)g.mt * 128 : 0);
   if (g.small32) {   // the usual case; 64-bit divisions cost the consuming kernels more than their loads
-    const uint32_t U = (uint32_t)n_groups * m_tiles.n * g.nkb, G = g.grid, tu0 = ((uint32_t)m_tile * n_groups + group) * g.nkb;
+    const uint32_t U = (uint32_t)n_groups * m_tiles.n * g.nkb, G = gemm_working<uint32_t>(U, g.grid), tu0 = ((uint32_t)m_tile * n_groups + group) * g.nkb;
     const uint32_t cf = ((tu0 + 1) * G - 1) / U, cl = ((tu0 + g.nkb) * G - 1) / U;
     f.c_next = (int)(cf > G - 1 ? G - 1 : cf) + 1;
     f.c_last = (int)(cl > G - 1 ? G - 1 : cl);
     return f;
   }
   const long long t = (long long)m_tile * n_groups + group;
-  const long long U = (long long)n_groups * m_tiles.n * g.nkb, G = g.grid;
+  const long long U = (long long)n_groups * m_tiles.n * g.nkb, G = gemm_working<long long>(U, g.grid);
   const long long tu0 = t * g.nkb;
   f.c_next = gemm_cta_of_unit(tu0, U, G) + 1;
   f.c_last = gemm_cta_of_unit(tu0 + g.nkb - 1, U, G);
   return f;
 }
-// True when CTA c has work (with fewer units than CTAs some ranges are empty).
-__device__ __forceinline__ bool gemm_has_work(const GemmOut& g, GemmRows m_tiles, int c) {
-  if (g.all_work) return true;
-  const long long U = (long long)(g.pair ? ((g.n_tiles + 1) >> 1) : g.n_tiles) * m_tiles.n * g.nkb, G = g.grid;
-  return gemm_range_begin(c, U, G) < gemm_range_begin(c + 1, U, G);
-}
-
 constexpr int GEMM_FOLD_UNROLL = 8;  // slots loaded together (a tile rarely has more contributors)
 
 // Two-phase read of a projection value: gemm_issue starts every load (output element and up to U
@@ -127,7 +133,7 @@ __device__ __forceinline__ GemmPending<U> gemm_issue(const GemmOut& g, GemmRows 
 #pragma unroll
   for (int j = 0; j < U; ++j) {
     const int c = p.f.c_next + j;
-    p.q[j] = (c <= p.f.c_last && gemm_has_work(g, m_tiles, c)) ? __ldcg(g.partial + (size_t)c * slot + p.f.off) : 0.f;
+    p.q[j] = c <= p.f.c_last ? __ldcg(g.partial + (size_t)c * slot + p.f.off) : 0.f;
   }
   return p;
 }
@@ -138,7 +144,7 @@ __device__ __forceinline__ float gemm_finish(const GemmOut& g, GemmRows m_tiles,
   for (int j = 0; j < U; ++j) v += p.q[j];
   const size_t slot = gemm_slot_stride(g);
   for (int c = p.f.c_next + U; c <= p.f.c_last; ++c)
-    if (gemm_has_work(g, m_tiles, c)) v += __ldcg(g.partial + (size_t)c * slot + p.f.off);
+    v += __ldcg(g.partial + (size_t)c * slot + p.f.off);
   return v;
 }
 // Four consecutive columns n .. n+3 (n a multiple of 4: they share a tile and the slots' alignment).
@@ -152,7 +158,7 @@ __device__ __forceinline__ GemmPending4<U> gemm_issue4(const GemmOut& g, GemmRow
 #pragma unroll
   for (int j = 0; j < U; ++j) {
     const int c = p.f.c_next + j;
-    p.q[j] = (c <= p.f.c_last && gemm_has_work(g, m_tiles, c))
+    p.q[j] = (c <= p.f.c_last)
                  ? __ldcg(reinterpret_cast<const float4*>(g.partial + (size_t)c * slot + p.f.off))
                  : make_float4(0.f, 0.f, 0.f, 0.f);
   }
@@ -165,7 +171,6 @@ __device__ __forceinline__ float4 gemm_finish4(const GemmOut& g, GemmRows m_tile
   for (int j = 0; j < U; ++j) { v.x += p.q[j].x; v.y += p.q[j].y; v.z += p.q[j].z; v.w += p.q[j].w; }
   const size_t slot = gemm_slot_stride(g);
   for (int c = p.f.c_next + U; c <= p.f.c_last; ++c) {
-    if (!gemm_has_work(g, m_tiles, c)) continue;
     const float4 t = __ldcg(reinterpret_cast<const float4*>(g.partial + (size_t)c * slot + p.f.off));
     v.x += t.x; v.y += t.y; v.z += t.z; v.w += t.w;
   }
@@ -194,7 +199,7 @@ __device__ __forceinline__ GemmPending2<U> gemm_issue2(const GemmOut& g, GemmRow
 #pragma unroll
   for (int j = 0; j < U; ++j) {
     const int c = f.c_next + j;
-    p.q[j] = (c <= f.c_last && gemm_has_work(g, m_tiles, c))
+    p.q[j] = (c <= f.c_last)
                  ? __ldcg(reinterpret_cast<const float2*>(g.partial + (size_t)c * slot + f.off + doff))
                  : make_float2(0.f, 0.f);
   }
@@ -207,7 +212,6 @@ __device__ __forceinline__ float2 gemm_finish2(const GemmOut& g, GemmRows m_tile
   for (int j = 0; j < U; ++j) { v.x += p.q[j].x; v.y += p.q[j].y; }
   const size_t slot = gemm_slot_stride(g);
   for (int c = f.c_next + U; c <= f.c_last; ++c) {
-    if (!gemm_has_work(g, m_tiles, c)) continue;
     const float2 t = __ldcg(reinterpret_cast<const float2*>(g.partial + (size_t)c * slot + f.off + doff));
     v.x += t.x; v.y += t.y;
   }
@@ -224,8 +228,6 @@ struct GemmSrc {
   const float* part;   // the value's place in the first extra contributor's slot; slot j is at part + j * stride
   int n_extra;         // contributors other than the first (0 when the tile is not cut or on the CUDA-core path)
 };
-// Valid for launches where every CTA has work (all_work), which is every launch whose stream is at
-// least as long as the grid; callers fall back to gemm_value* otherwise.
 __device__ __forceinline__ GemmSrc gemm_src(const GemmOut& g, GemmRows m_tiles, int m, int n) {
   GemmSrc s;
   s.raw = g.raw + (size_t)m * g.ld + n;
@@ -323,7 +325,7 @@ __device__ __forceinline__ GemmPending4f<U> gemm_issue4f(const GemmOut& g, GemmR
 #pragma unroll
   for (int j = 0; j < U; ++j) {
     const int c = f.c_next + j;
-    p.q[j] = (c <= f.c_last && gemm_has_work(g, m_tiles, c))
+    p.q[j] = (c <= f.c_last)
                  ? __ldcg(reinterpret_cast<const float4*>(g.partial + (size_t)c * slot + f.off + doff))
                  : make_float4(0.f, 0.f, 0.f, 0.f);
   }
@@ -336,7 +338,6 @@ __device__ __forceinline__ float4 gemm_finish4f(const GemmOut& g, GemmRows m_til
   for (int j = 0; j < U; ++j) { v.x += p.q[j].x; v.y += p.q[j].y; v.z += p.q[j].z; v.w += p.q[j].w; }
   const size_t slot = gemm_slot_stride(g);
   for (int c = f.c_next + U; c <= f.c_last; ++c) {
-    if (!gemm_has_work(g, m_tiles, c)) continue;
     const float4 t = __ldcg(reinterpret_cast<const float4*>(g.partial + (size_t)c * slot + f.off + doff));
     v.x += t.x; v.y += t.y; v.z += t.z; v.w += t.w;
   }

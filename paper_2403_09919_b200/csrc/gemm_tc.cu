@@ -206,13 +206,13 @@ __global__ void __launch_bounds__(tc_threads(EW), EW == 4 ? 4 : 2) gemm_tc_kerne
   if (p.m_tiles_max > 1) rows = gemm_row_tiles(p.mt, p.m_tiles_max, *p.m_total);
   else if (chained) rows.rows = min(p.mt, max(16, (*p.m_total + 15) & ~15));
   const int m_tiles = rows.n;
-  const long long G = gridDim.x;
   // unit = (row tile, weight tile or tile pair, k-block), row tile slowest: the CTAs of each row tile then walk the
   // weight tiles abreast of the other row tiles' CTAs, and a weight tile leaves device memory once for all of them
   const int n_wt = PAIR ? (p.n_tiles + 1) / 2 : p.n_tiles;
   const int n_groups = n_wt * m_tiles;
-  const long long U = (long long)n_groups * p.nkb;
-  const long long u0 = gemm_range_begin(blockIdx.x, U, G), u1 = gemm_range_begin(blockIdx.x + 1, U, G);
+  const long long U = (long long)n_groups * p.nkb, G = gemm_working<long long>(U, gridDim.x);
+  const bool works = blockIdx.x < G;
+  const long long u0 = works ? gemm_range_begin(blockIdx.x, U, G) : U, u1 = works ? gemm_range_begin(blockIdx.x + 1, U, G) : U;
   const int mt_eff = rows.rows;   // several row tiles are equal: the fewest that hold the rows, each a multiple of 16 rows
   const CUtensorMap* map_a = &maps_a.m[(mt_eff >> 4) - 1];
 
@@ -536,11 +536,11 @@ __global__ void __launch_bounds__(tc_threads(EW), EW == 4 ? 4 : 2) gemm_tc2_kern
   if (p.m_tiles_max > 1) rows = gemm_row_tiles(p.mt, p.m_tiles_max, *p.m_total);
   else if (chained) rows.rows = min(p.mt, max(16, (*p.m_total + 15) & ~15));
   const int m_tiles = rows.n;
-  const long long C = gridDim.x >> 1;             // clusters
   const int n_wt = (p.n_tiles + 1) / 2;           // pairs of weight tiles
   const int n_groups = n_wt * m_tiles;
-  const long long U = (long long)n_groups * p.nkb;
-  const long long u0 = gemm_range_begin(cluster, U, C), u1 = gemm_range_begin(cluster + 1, U, C);
+  const long long U = (long long)n_groups * p.nkb, C = gemm_working<long long>(U, gridDim.x >> 1);   // clusters that work
+  const bool works = cluster < C;
+  const long long u0 = works ? gemm_range_begin(cluster, U, C) : U, u1 = works ? gemm_range_begin(cluster + 1, U, C) : U;
   const int mt_eff = rows.rows, half = mt_eff >> 1;   // rows of a row tile; rows of it this CTA loads
   const CUtensorMap* map_a = &maps_a.m[(half >> 3) - 1];
 
@@ -897,11 +897,11 @@ static cudaError_t launch_gemm_tc2(const void* map_w, const void* const map_a[16
   p.m_tiles_max = (m_max + p.mt - 1) / p.mt;
   p.pair = 1;
   const long long n_units = (long long)((p.n_tiles + 1) / 2) * p.nkb;
+  pairs = (int)gemm_working<long long>(n_units * p.m_tiles_max, pairs);
   if (out_desc) {
     // for the consumers a cluster is what a CTA is in pair mode: units over pairs of tiles, a slot holds both tiles
     out_desc->raw = raw; out_desc->partial = partial; out_desc->ld = ld_raw; out_desc->nkb = p.nkb;
     out_desc->n_tiles = p.n_tiles; out_desc->mt = p.mt; out_desc->grid = pairs; out_desc->m_tiles_max = p.m_tiles_max;
-    out_desc->all_work = (n_units >= pairs) ? 1 : 0;
     out_desc->pair = 1;
     out_desc->small32 = ((n_units * p.m_tiles_max + 1) * pairs < (1ll << 31)) ? 1 : 0;
   }
@@ -941,10 +941,10 @@ cudaError_t launch_gemm_tc(const void* map_w, const void* const map_a[16], int N
   static const int pair_ok = getenv("RD_TC_PAIR") ? atoi(getenv("RD_TC_PAIR")) : 1;   // tuning toggle
   p.pair = (pair && pair_ok && p.m_tiles_max == 1 && p.mt <= 128 && p.n_tiles >= 2) ? 1 : 0;
   const long long n_units = (long long)(p.pair ? (p.n_tiles + 1) / 2 : p.n_tiles) * p.nkb;
+  grid = (int)gemm_working<long long>(n_units * p.m_tiles_max, grid);
   if (out_desc) {
     out_desc->raw = raw; out_desc->partial = partial; out_desc->ld = ld_raw; out_desc->nkb = p.nkb;
     out_desc->n_tiles = p.n_tiles; out_desc->mt = p.mt; out_desc->grid = grid; out_desc->m_tiles_max = p.m_tiles_max;
-    out_desc->all_work = (n_units >= grid) ? 1 : 0;
     out_desc->pair = p.pair ? 1 : 0;
     out_desc->small32 = ((n_units * p.m_tiles_max + 1) * grid < (1ll << 31)) ? 1 : 0;
   }

@@ -77,6 +77,13 @@ def test_verify_7b_shapes_two_layers():
     check_verify(Rig(cfg=synth.with_layers(dict(synth.CONFIGS["7b"], max_ctx=256), 2), oracle_dtype=np.float32))
 
 
+@pytest.mark.parametrize("d,heads,d_ffn,vocab,bw", [(64, 1, 64, 100, 8), (128, 1, 192, 132, 8), (256, 2, 448, 260, 64), (512, 8, 1376, 1000, 64)])
+def test_verify_with_fewer_projection_units_than_sms(d, heads, d_ffn, vocab, bw):
+    """Projections of one k-block of one tile up to about twice as many units as the part has SMs: only some of a
+    launch's CTAs work, and the consumers have to find the same ones (one row tile, and a bound of several)."""
+    check_verify(Rig(cfg=dict(RAGGED, d_model=d, n_heads=heads, d_rnn=d, d_ffn=d_ffn, vocab=vocab, beam_width=bw, max_ctx=500)))
+
+
 @pytest.mark.parametrize("vocab,d_ffn", [(1000, 1376), (1100, 1440)])
 def test_tensor_core_path_matches_cuda_core_path(vocab, d_ffn):
     """The second shape gives the LM head 9 and the gate+up projection 23 weight tiles: odd counts, so the last
