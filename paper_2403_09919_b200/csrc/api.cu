@@ -42,7 +42,7 @@ struct Workspace {
   // step-internal packed beam, beams, verify outputs, accept scratch
   rd_packed pk;
   int32_t *beams, *argmax_p, *n_accept, *best, *ctx_prev, *acc_tokens;
-  float *scores, *hidden_p;
+  float* scores;
   // drafter
   void *xc_t, *x0_t, *x1_t, *x2_t, *se_t, *uw;   // se_t: [R][d_rnn + d] = [s ; e]; uw: [d_rnn][d_rnn + d] = [U W]
   float *xc_f, *x0_f, *x1_f, *x2_f, *sraw, *hraw, *dlogits, *lse, *cand_val, *score_a, *score_b;
@@ -215,7 +215,7 @@ void carve(Bump& bp, const Dims& dm, int m_cap, Workspace* w) {
   w->beams = bp.take<int32_t>((size_t)R * dm.L); w->argmax_p = bp.take<int32_t>((size_t)B * dm.NMAX);
   w->n_accept = bp.take<int32_t>(B); w->best = bp.take<int32_t>(B); w->ctx_prev = bp.take<int32_t>(B);
   w->acc_tokens = bp.take<int32_t>((size_t)B * C);
-  w->scores = bp.take<float>(R); w->hidden_p = bp.take<float>((size_t)B * dm.NMAX * dm.d);
+  w->scores = bp.take<float>(R);
   w->xc_t = bp.take<char>((size_t)B * dm.dh * es); w->x0_t = bp.take<char>((size_t)R * dm.dh * es);
   w->x1_t = bp.take<char>((size_t)R * dm.dh * es); w->x2_t = bp.take<char>((size_t)R * dm.dh * es);
   w->se_t = bp.take<char>((size_t)R * (dm.dr + dm.d) * es); w->uw = bp.take<char>((size_t)dm.dr * (dm.dr + dm.d) * es);
@@ -385,8 +385,8 @@ int forward_layers(rd_handle* h, const uint32_t* mask, int m_max, int n_seq, int
   Workspace& w = h->ws;
   const Dims& dm = h->dm;
   RowTables rt{w.row_tok, w.row_seq, w.row_pos, w.row_slot, w.row_ncache, w.row_local, mask, w.m_total};
-  CKP(h, PROF_MISC, launch_embed(dm.dtype, h->w.tok_emb, w.row_tok, w.x, dm.d, dm.V, w.m_total, m_max, w.status, st));
-  CKP(h, PROF_MISC, launch_rope_table(w.row_pos, w.rope_tab, dm.hd, dm.theta, w.m_total, m_max, st));
+  CKP(h, PROF_MISC, launch_embed_rope(dm.dtype, h->w.tok_emb, w.row_tok, w.row_pos, w.x, w.rope_tab, dm.d, dm.V, dm.hd, dm.theta,
+                                      w.m_total, m_max, w.status, st));
   // attention launch geometry (tensor-core path): tiles of 16 rows per sequence; keys split over CTAs only
   // for long contexts with few tiles
   int row_blocks = 1, n_splits = 1;
@@ -483,8 +483,7 @@ int do_draft(rd_handle* h, cudaStream_t st, int32_t* beams, float* scores) {
   Workspace& w = h->ws;
   const Dims& dm = h->dm;
   const int B = h->batch, R = B * dm.BW;
-  CKP(h, PROF_DRAFT_SMALL, launch_draft_init(dm.dtype, h->w.tok_emb, w.root, w.h, w.xc_t, w.xc_f, w.se_t, dm, B, w.status, st));
-  if (dm.L > 1) CKP(h, PROF_DRAFT_SMALL, launch_fill_h(dm.dtype, w.h, w.x0_t, w.x0_f, dm, B, st));
+  CKP(h, PROF_DRAFT_SMALL, launch_draft_init(dm.dtype, h->w.tok_emb, w.root, w.h, w.xc_t, w.xc_f, w.x0_t, w.x0_f, w.se_t, dm, B, w.status, st));
   float *sc_in = w.score_a, *sc_out = w.score_b;
   int32_t *hi_in = w.hist_a, *hi_out = w.hist_b;
   GemmOut g;
@@ -529,7 +528,7 @@ int do_verify(rd_handle* h, const rd_packed& pk, cudaStream_t st, int32_t* argma
   const Dims& dm = h->dm;
   const int B = h->batch, m_max = B * dm.NMAX;
   CKP(h, PROF_MISC, launch_build_rows_tree(pk, w.ctx, w.row_tok, w.row_seq, w.row_pos, w.row_slot, w.row_ncache, w.row_local,
-                               w.row_out_index, w.seq_off, w.seq_order, w.m_total, dm, B, w.status, st));
+                               w.row_out_index, w.seq_off, w.seq_order, argmax, w.m_total, dm, B, w.status, st));
   h->att_seq_order = B <= 1024 ? w.seq_order : nullptr;   // the row tables of this pass carry the sequences' order
   int rc = forward_layers(h, pk.mask, m_max, B, dm.NMAX, h->w.lm_head, st);
   h->att_seq_order = nullptr;
@@ -537,7 +536,6 @@ int do_verify(rd_handle* h, const rd_packed& pk, cudaStream_t st, int32_t* argma
   GemmOut g;
   rc = gemm(h, w.hidden_t, dm.d, h->w.lm_head, dm.V, dm.d, w.m_total, m_max, w.logits, dm.V, &g, nullptr, st, /*pair=*/1);
   if (rc) return rc;
-  CKP(h, PROF_MISC, launch_fill_i32(argmax, -1, B * dm.NMAX, st));
   CKP(h, PROF_MISC, launch_argmax_rows(w.logits, g, dm.V, argmax, w.row_out_index, w.m_total, m_max, h->sampling, w.row_seq, w.row_pos, 1, st));
   if (hidden) CKP(h, PROF_MISC, launch_scatter_rows(w.hidden_f, dm.d, hidden, w.row_out_index, w.m_total, m_max, st));
   if (logits) CK(h, launch_scatter_rows(w.logits, dm.V, logits, w.row_out_index, w.m_total, m_max, st));
@@ -846,7 +844,7 @@ int redrafter_accept(rd_handle* h, const int32_t* beams, const rd_packed* packed
   Workspace& w = h->ws;
   rd_accept_out o{};
   if (out) o = *out;
-  CK(h, launch_accept(h->dm.dtype, beams, *packed, argmax, hidden, h->kv, w.ctx, w.root, w.h, o, w.n_accept, w.best,
+  CK(h, launch_accept(h->dm.dtype, beams, *packed, argmax, hidden, nullptr, h->kv, w.ctx, w.root, w.h, o, w.n_accept, w.best,
                       w.ctx_prev, h->dm, h->batch, w.status, (cudaStream_t)stream));
   h->launches++;  // accept + compaction
   fb_advance(h, 1 + h->dm.L, (cudaStream_t)stream);
@@ -870,7 +868,7 @@ int redrafter_accept_static(rd_handle* h, const int32_t* beams, const rd_packed*
   Workspace& w = h->ws;
   rd_accept_out o{};
   if (out) o = *out;
-  CK(h, launch_accept(h->dm.dtype, beams, *packed, argmax, hidden, h->kv, w.ctx, w.root, w.h, o, n_accept, best, ctx_prev,
+  CK(h, launch_accept(h->dm.dtype, beams, *packed, argmax, hidden, nullptr, h->kv, w.ctx, w.root, w.h, o, n_accept, best, ctx_prev,
                       h->dm, h->batch, w.status, (cudaStream_t)stream));
   h->launches++;  // accept + compaction
   fb_advance(h, 1 + h->dm.L, (cudaStream_t)stream);
@@ -886,11 +884,11 @@ int redrafter_step(rd_handle* h, const int32_t* planted_beams, void* stream, con
   if (rc) return rc;
   const int32_t* beams = planted_beams ? planted_beams : w.beams;
   CKP(h, PROF_PACK_ACCEPT, launch_pack(beams, w.root, w.ctx, w.pk, h->dm, h->batch, (h->cfg.flags & RD_FLAG_NO_TREE) ? 1 : 0, st));
-  rc = do_verify(h, w.pk, st, w.argmax_p, w.hidden_p, nullptr);
+  rc = do_verify(h, w.pk, st, w.argmax_p, nullptr, nullptr);   // the hidden rows stay compact
   if (rc) return rc;
   rd_accept_out o{};
   if (out) o = *out;
-  CKP(h, PROF_PACK_ACCEPT, launch_accept(h->dm.dtype, beams, w.pk, w.argmax_p, w.hidden_p, h->kv, w.ctx, w.root, w.h, o, w.n_accept,
+  CKP(h, PROF_PACK_ACCEPT, launch_accept(h->dm.dtype, beams, w.pk, w.argmax_p, w.hidden_f, w.seq_off, h->kv, w.ctx, w.root, w.h, o, w.n_accept,
                       w.best, w.ctx_prev, h->dm, h->batch, w.status, st));
   h->launches++;
   fb_advance(h, 1 + h->dm.L, st);

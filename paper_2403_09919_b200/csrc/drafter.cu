@@ -18,52 +18,42 @@ namespace rd {
   if ((dtype) == RD_DTYPE_FP32) { using T = float; __VA_ARGS__; } \
   else { using T = __nv_bfloat16; __VA_ARGS__; }
 
-// ---------------------------------------------------------------- call-1 input and s_1
-// x[b] = [E[g_b], h_b] for the first call; the state half of se[r] = [s ; e] is E[g_b] = s_1 for
-// every beam row r of b.
+// ---------------------------------------------------------------- call-1 input, s_1, and h for the later calls
+// One CTA per beam row r of sequence b: the state half of se[r] = [s ; e] is E[g_b] = s_1, and the h half of
+// x0[r] = [s_t, h] is h_b (constant over the calls of a step).  A sequence's first CTA also writes the first call's
+// input xc[b] = [E[g_b], h_b].
 template <typename T>
-__global__ void draft_init_kernel(const T* __restrict__ emb, const int32_t* __restrict__ root, const float* __restrict__ h,
-                                  T* __restrict__ x_t, float* __restrict__ x_f, T* __restrict__ se_t, Dims dm,
-                                  int* status) {
+__global__ void __launch_bounds__(256) draft_init_kernel(const T* __restrict__ emb, const int32_t* __restrict__ root, const float* __restrict__ h,
+                                  T* __restrict__ xc_t, float* __restrict__ xc_f, T* __restrict__ x0_t, float* __restrict__ x0_f,
+                                  T* __restrict__ se_t, Dims dm, int* status) {
   pdl_enter();
-  const int b = blockIdx.x;
+  const int r = blockIdx.x, b = r / dm.BW, d = dm.d;
+  const bool first = r == b * dm.BW;
   int g = root[b];
   if (g < 0 || g >= dm.V) {
-    if (threadIdx.x == 0) atomicOr(status, DEV_ERR_TOKEN_RANGE);
+    if (threadIdx.x == 0 && first) atomicOr(status, DEV_ERR_TOKEN_RANGE);
     g = min(max(g, 0), dm.V - 1);
   }
-  const int d = dm.d;
+#pragma unroll 4
   for (int i = threadIdx.x; i < d; i += blockDim.x) {
     const T e = emb[(size_t)g * d + i];
-    x_t[(size_t)b * dm.dh + i] = e;
-    x_f[(size_t)b * dm.dh + i] = to_f<T>(e);
     const float hv = h[(size_t)b * d + i];
-    x_t[(size_t)b * dm.dh + dm.dr + i] = from_f<T>(hv);
-    x_f[(size_t)b * dm.dh + dm.dr + i] = hv;
-    for (int k = 0; k < dm.BW; ++k) se_t[((size_t)b * dm.BW + k) * (dm.dr + dm.d) + i] = e;
+    se_t[(size_t)r * (dm.dr + d) + i] = e;
+    x0_t[(size_t)r * dm.dh + dm.dr + i] = from_f<T>(hv);
+    x0_f[(size_t)r * dm.dh + dm.dr + i] = hv;
+    if (first) {
+      xc_t[(size_t)b * dm.dh + i] = e;
+      xc_f[(size_t)b * dm.dh + i] = to_f<T>(e);
+      xc_t[(size_t)b * dm.dh + dm.dr + i] = from_f<T>(hv);
+      xc_f[(size_t)b * dm.dh + dm.dr + i] = hv;
+    }
   }
 }
 
-cudaError_t launch_draft_init(int dtype, const void* emb, const int32_t* root, const float* h, void* x_t, float* x_f,
-                              void* se_t, const Dims& dm, int B, int* status, cudaStream_t st) {
-  RD_DISPATCH(dtype, launch_pdl(draft_init_kernel<T>, B, 256, 0, st, (const T*)emb, root, h, (T*)x_t, x_f, (T*)se_t, dm, status));
-  return cudaGetLastError();
-}
-
-// h part of g_t = [s_t, h] for every beam row (constant over the calls of one step).
-template <typename T>
-__global__ void fill_h_kernel(const float* __restrict__ h, T* __restrict__ x_t, float* __restrict__ x_f, Dims dm) {
-  pdl_enter();
-  const int r = blockIdx.x, b = r / dm.BW;
-  for (int i = threadIdx.x; i < dm.d; i += blockDim.x) {
-    const float hv = h[(size_t)b * dm.d + i];
-    x_t[(size_t)r * dm.dh + dm.dr + i] = from_f<T>(hv);
-    x_f[(size_t)r * dm.dh + dm.dr + i] = hv;
-  }
-}
-
-cudaError_t launch_fill_h(int dtype, const float* h, void* x_t, float* x_f, const Dims& dm, int B, cudaStream_t st) {
-  RD_DISPATCH(dtype, launch_pdl(fill_h_kernel<T>, B * dm.BW, 256, 0, st, h, (T*)x_t, x_f, dm));
+cudaError_t launch_draft_init(int dtype, const void* emb, const int32_t* root, const float* h, void* xc_t, float* xc_f, void* x0_t,
+                              float* x0_f, void* se_t, const Dims& dm, int B, int* status, cudaStream_t st) {
+  RD_DISPATCH(dtype, launch_pdl(draft_init_kernel<T>, B * dm.BW, 256, 0, st, (const T*)emb, root, h, (T*)xc_t, xc_f, (T*)x0_t, x0_f,
+                                (T*)se_t, dm, status));
   return cudaGetLastError();
 }
 

@@ -31,28 +31,6 @@ __device__ __forceinline__ float block_sum(float v, float* sh) {
   return t;
 }
 
-// ---------------------------------------------------------------- embedding gather
-template <typename T>
-__global__ void embed_kernel(const T* __restrict__ emb, const int32_t* __restrict__ tok, float* __restrict__ x, int d,
-                             int V, const int32_t* __restrict__ m_total, int* status) {
-  pdl_enter();
-  const int m = blockIdx.x;
-  if (m >= *m_total) return;
-  int t = tok[m];
-  if (t < 0 || t >= V) {
-    if (threadIdx.x == 0) atomicOr(status, DEV_ERR_TOKEN_RANGE);
-    t = min(max(t, 0), V - 1);
-  }
-  const T* src = emb + (size_t)t * d;
-  for (int i = threadIdx.x; i < d; i += blockDim.x) x[(size_t)m * d + i] = to_f<T>(src[i]);
-}
-
-cudaError_t launch_embed(int dtype, const void* emb, const int32_t* tok, float* x, int d, int V, const int32_t* m_total,
-                         int m_max, int* status, cudaStream_t st) {
-  RD_DISPATCH(dtype, launch_pdl(embed_kernel<T>, m_max, 256, 0, st, (const T*)emb, tok, x, d, V, m_total, status));
-  return cudaGetLastError();
-}
-
 // Four consecutive outputs in the activation type (16- or 8-byte store; the address is that much aligned).
 __device__ __forceinline__ void store4(float* p, float a, float b, float c, float d) { *reinterpret_cast<float4*>(p) = make_float4(a, b, c, d); }
 __device__ __forceinline__ void store4(__nv_bfloat16* p, float a, float b, float c, float d) {
@@ -311,15 +289,33 @@ cudaError_t launch_rmsnorm(int dtype, float* x, const GemmOut* proj, const void*
   return cudaGetLastError();
 }
 
-// ---------------------------------------------------------------- rotary table
-// cos/sin of pos * theta^(-2i/hd) for every row of the pass, computed once per forward (all layers
-// share it).  The angle is formed in double: positions reach several thousand and its rounding
+// ---------------------------------------------------------------- a pass's rows: embedding and rotary table
+// x[m] = E[tok[m]] and the cos/sin of pos * theta^(-2i/hd) of every row of the pass, computed once per forward (all
+// layers share them).  The angle is formed in double: positions reach several thousand and its rounding
 // error in single precision would scale with them.
-__global__ void rope_table_kernel(const int32_t* __restrict__ pos, float2* __restrict__ table, int half, float theta,
-                                  const int32_t* __restrict__ m_total) {
+template <typename T>
+__global__ void __launch_bounds__(256) embed_rope_kernel(const T* __restrict__ emb, const int32_t* __restrict__ tok, const int32_t* __restrict__ pos,
+                                  float* __restrict__ x, float2* __restrict__ table, int d, int V, int half, float theta,
+                                  const int32_t* __restrict__ m_total, int* status) {
   pdl_enter();
   const int m = blockIdx.x;
   if (m >= *m_total) return;
+  int t = tok[m];
+  if (t < 0 || t >= V) {
+    if (threadIdx.x == 0) atomicOr(status, DEV_ERR_TOKEN_RANGE);
+    t = min(max(t, 0), V - 1);
+  }
+  const T* src = emb + (size_t)t * d;
+  if (((uintptr_t)emb & (4 * sizeof(T) - 1)) == 0) {   // the caller's table starts on a vector boundary; d is a multiple of 4
+#pragma unroll 4
+    for (int i = threadIdx.x * 4; i < d; i += blockDim.x * 4) {
+      Gain4<T> e;
+      e.load(src + i);
+      *reinterpret_cast<float4*>(x + (size_t)m * d + i) = e.get();
+    }
+  } else {
+    for (int i = threadIdx.x; i < d; i += blockDim.x) x[(size_t)m * d + i] = to_f<T>(src[i]);
+  }
   const double l2t = log2((double)theta);
   for (int i = threadIdx.x; i < half; i += blockDim.x) {
     const double ang = (double)pos[m] * exp2(-((double)i / half) * l2t);
@@ -329,9 +325,10 @@ __global__ void rope_table_kernel(const int32_t* __restrict__ pos, float2* __res
   }
 }
 
-cudaError_t launch_rope_table(const int32_t* pos, float* table, int hd, float theta, const int32_t* m_total, int m_max,
-                              cudaStream_t st) {
-  launch_pdl(rope_table_kernel, m_max, 64, 0, st, pos, reinterpret_cast<float2*>(table), hd / 2, theta, m_total);
+cudaError_t launch_embed_rope(int dtype, const void* emb, const int32_t* tok, const int32_t* pos, float* x, float* table, int d, int V,
+                              int hd, float theta, const int32_t* m_total, int m_max, int* status, cudaStream_t st) {
+  RD_DISPATCH(dtype, launch_pdl(embed_rope_kernel<T>, m_max, 256, 0, st, (const T*)emb, tok, pos, x, reinterpret_cast<float2*>(table),
+                                d, V, hd / 2, theta, m_total, status));
   return cudaGetLastError();
 }
 
@@ -922,23 +919,39 @@ cudaError_t launch_fill_i32(int32_t* p, int32_t v, int n, cudaStream_t st) {
 // ---------------------------------------------------------------- row tables
 // Verification: the packed rows of all sequences are laid out back to back (compact), so the
 // projections see M = sum_b n[b] rows.  Row (b, n): token = packed token, position = ctx_b + depth,
-// provisional cache slot ctx_b + n, attends cache [0, ctx_b) plus its mask row.
-__global__ void build_rows_tree_kernel(rd_packed pk, const int32_t* __restrict__ ctx, int32_t* row_tok, int32_t* row_seq,
+// provisional cache slot ctx_b + n, attends cache [0, ctx_b) plus its mask row.  The LLM's tokens of the padding
+// rows (argmax, [B][NMAX]) become -1 here; those of the rows are written at the end of the pass.
+constexpr int ROWS_CTX = 1024;
+__global__ void __launch_bounds__(1024) build_rows_tree_kernel(rd_packed pk, const int32_t* __restrict__ ctx, int32_t* row_tok, int32_t* row_seq,
                                        int32_t* row_pos, int32_t* row_slot, int32_t* row_ncache, int32_t* row_local,
-                                       int32_t* row_out_index, int32_t* seq_off, int32_t* seq_order, int32_t* m_total, Dims dm,
-                                       int B, int* status) {
+                                       int32_t* row_out_index, int32_t* seq_off, int32_t* seq_order, int32_t* argmax, int32_t* m_total,
+                                       Dims dm, int B, int* status) {
   pdl_enter();
-  extern __shared__ int32_t off[];  // [B+1]
-  if (threadIdx.x == 0) {
-    int acc = 0;
-    for (int b = 0; b < B; ++b) {
-      off[b] = acc;
-      int n = pk.n[b];
-      if (n < 0 || n > dm.NMAX) { atomicOr(status, DEV_ERR_INDEX_RANGE); n = min(max(n, 0), dm.NMAX); }
-      acc += n;
+  extern __shared__ int32_t off[];  // [B+1], then the context lengths of a batch of up to ROWS_CTX sequences
+  __shared__ int32_t warp_tot[32];
+  int32_t* s_ctx = off + B + 1;
+  auto ctx_of = [&](int b) { return B <= ROWS_CTX ? s_ctx[b] : ctx[b]; };
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  // exclusive scan of the row counts, a block's worth of sequences at a time
+  for (int b0 = 0, acc = 0; b0 < B; b0 += blockDim.x) {
+    const int b = b0 + threadIdx.x;
+    int n = b < B ? pk.n[b] : 0;
+    if (b < B && B <= ROWS_CTX) s_ctx[b] = ctx[b];
+    if (n < 0 || n > dm.NMAX) { atomicOr(status, DEV_ERR_INDEX_RANGE); n = min(max(n, 0), dm.NMAX); }
+    int incl = n;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += v;
     }
-    off[B] = acc;
-    *m_total = acc;
+    __syncthreads();
+    if (lane == 31) warp_tot[w] = incl;
+    __syncthreads();
+    int before = acc;
+    for (int k = 0; k < w; ++k) before += warp_tot[k];
+    if (b < B) off[b] = before + incl - n;
+    for (int k = 0; k < 32; ++k) acc += warp_tot[k];
+    if (threadIdx.x == 0 && b0 + (int)blockDim.x >= B) { off[B] = acc; *m_total = acc; }
   }
   __syncthreads();
   for (int b = threadIdx.x; b <= B; b += blockDim.x) seq_off[b] = off[b];
@@ -946,25 +959,25 @@ __global__ void build_rows_tree_kernel(rd_packed pk, const int32_t* __restrict__
   // hand the long sequences out first, so that the last CTAs to start are short ones.  Ranked by counting.
   if (seq_order)
     for (int b = threadIdx.x; b < B; b += blockDim.x) {
-      const int kb = ctx[b] + (off[b + 1] - off[b]);
+      const int kb = ctx_of(b) + (off[b + 1] - off[b]);
       int rank = 0;
       for (int o = 0; o < B; ++o) {
-        const int ko = ctx[o] + (off[o + 1] - off[o]);
+        const int ko = ctx_of(o) + (off[o + 1] - off[o]);
         rank += (ko > kb || (ko == kb && o < b)) ? 1 : 0;
       }
       seq_order[rank] = b;
     }
   for (int idx = threadIdx.x; idx < B * dm.NMAX; idx += blockDim.x) {
     const int b = idx / dm.NMAX, n = idx - b * dm.NMAX;
-    if (n >= off[b + 1] - off[b]) continue;
+    if (n >= off[b + 1] - off[b]) { argmax[idx] = -1; continue; }
     const int m = off[b] + n;
     int t = pk.tokens[idx];
     if (t < 0 || t >= dm.V) { atomicOr(status, DEV_ERR_TOKEN_RANGE); t = min(max(t, 0), dm.V - 1); }
     row_tok[m] = t;
     row_seq[m] = b;
     row_pos[m] = pk.pos[idx];
-    row_slot[m] = ctx[b] + n;
-    row_ncache[m] = ctx[b];
+    row_slot[m] = ctx_of(b) + n;
+    row_ncache[m] = ctx_of(b);
     row_local[m] = n;
     row_out_index[m] = idx;
   }
@@ -972,11 +985,11 @@ __global__ void build_rows_tree_kernel(rd_packed pk, const int32_t* __restrict__
 
 cudaError_t launch_build_rows_tree(const rd_packed& pk, const int32_t* ctx, int32_t* row_tok, int32_t* row_seq,
                                    int32_t* row_pos, int32_t* row_slot, int32_t* row_ncache, int32_t* row_local,
-                                   int32_t* row_out_index, int32_t* seq_off, int32_t* seq_order, int32_t* m_total,
+                                   int32_t* row_out_index, int32_t* seq_off, int32_t* seq_order, int32_t* argmax, int32_t* m_total,
                                    const Dims& dm, int B, int* status, cudaStream_t st) {
-  launch_pdl(build_rows_tree_kernel, 1, 1024, (B + 1) * sizeof(int32_t), st, pk, ctx, row_tok, row_seq, row_pos, row_slot,
+  launch_pdl(build_rows_tree_kernel, 1, 1024, ((size_t)B + 1 + (B <= ROWS_CTX ? B : 0)) * sizeof(int32_t), st, pk, ctx, row_tok, row_seq, row_pos, row_slot,
                                                                     row_ncache, row_local, row_out_index, seq_off,
-                                                                    B <= 1024 ? seq_order : nullptr, m_total, dm, B, status);
+                                                                    B <= ROWS_CTX ? seq_order : nullptr, argmax, m_total, dm, B, status);
   return cudaGetLastError();
 }
 

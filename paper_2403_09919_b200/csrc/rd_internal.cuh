@@ -66,12 +66,10 @@ cudaError_t launch_gemm_tc(const void* map_w, const void* const map_a[16], int N
                            float* raw, int ld_raw, float* partial, int32_t* status, int grid, int pairs, int smem_limit,
                            unsigned long long* trace, GemmOut* out_desc, Chain* chain, int pair, cudaStream_t st);
 
-cudaError_t launch_embed(int dtype, const void* emb, const int32_t* tok, float* x, int d, int V, const int32_t* m_total,
-                         int m_max, int* status, cudaStream_t st);
+cudaError_t launch_embed_rope(int dtype, const void* emb, const int32_t* tok, const int32_t* pos, float* x, float* table, int d, int V,
+                              int hd, float theta, const int32_t* m_total, int m_max, int* status, cudaStream_t st);
 cudaError_t launch_rmsnorm(int dtype, float* x, const GemmOut* proj, const void* gain, void* out_t, float* out_f32, int d,
                            float eps, const int32_t* m_total, int m_max, Chain* chain, cudaStream_t st);
-cudaError_t launch_rope_table(const int32_t* pos, float* table, int hd, float theta, const int32_t* m_total, int m_max,
-                              cudaStream_t st);
 cudaError_t launch_rope_kv(int dtype, float* qkv, const GemmOut& proj, void* kcache, void* vcache, const float* table,
                            const RowTables& rt, const Dims& dm, int m_max, int* status, Chain* chain, cudaStream_t st);
 cudaError_t launch_attention(int dtype, const float* qkv, const void* kcache, const void* vcache, void* out_t,
@@ -109,8 +107,8 @@ cudaError_t launch_argmax_rows(float* logits, const GemmOut& proj, int V, int32_
                                const int32_t* row_pos, int pos_add, cudaStream_t st);
 
 // drafter
-cudaError_t launch_draft_init(int dtype, const void* emb, const int32_t* root, const float* h, void* x_t, float* x_f,
-                              void* se_t, const Dims& dm, int B, int* status, cudaStream_t st);
+cudaError_t launch_draft_init(int dtype, const void* emb, const int32_t* root, const float* h, void* xc_t, float* xc_f, void* x0_t,
+                              float* x0_f, void* se_t, const Dims& dm, int B, int* status, cudaStream_t st);
 cudaError_t launch_act(int dtype, const GemmOut& proj, const void* bias, const float* resid, int ld_resid, float* out_f,
                        void* out_t, int ld_out, int N, const int32_t* m_total, int m_max, Chain* chain, cudaStream_t st);
 // Scratch of the two-kernel selection (seg_max == nullptr: single-kernel selection only).
@@ -126,15 +124,14 @@ cudaError_t launch_draft_select(int dtype, const GemmOut& proj, int call, float*
                                 const void* emb, const float* s_new_f, int ld_s, void* se_t, const Dims& dm, int B,
                                 int32_t* beams_out, float* scores_out, int32_t* counters, const int32_t* m_total,
                                 unsigned long long* dbg, const SelectScratch& sc, Chain* chain, cudaStream_t st);
-cudaError_t launch_fill_h(int dtype, const float* h, void* x_t, float* x_f, const Dims& dm, int B, cudaStream_t st);
 
 // pack / accept
 cudaError_t launch_pack(const int32_t* beams, const int32_t* root, const int32_t* ctx, const rd_packed& out,
                         const Dims& dm, int B, int no_tree, cudaStream_t st);
 cudaError_t launch_build_rows_tree(const rd_packed& pk, const int32_t* ctx, int32_t* row_tok, int32_t* row_seq,
                                    int32_t* row_pos, int32_t* row_slot, int32_t* row_ncache, int32_t* row_local,
-                                   int32_t* row_out_index, int32_t* seq_off, int32_t* seq_order, int32_t* m_total, const Dims& dm, int B,
-                                   int* status, cudaStream_t st);
+                                   int32_t* row_out_index, int32_t* seq_off, int32_t* seq_order, int32_t* argmax, int32_t* m_total,
+                                   const Dims& dm, int B, int* status, cudaStream_t st);
 cudaError_t launch_build_rows_ar(const int32_t* root, const int32_t* ctx, int32_t* row_tok, int32_t* row_seq,
                                  int32_t* row_pos, int32_t* row_slot, int32_t* row_ncache, int32_t* row_local,
                                  int32_t* row_out_index, int32_t* seq_off, int32_t* m_total, const Dims& dm, int B,
@@ -144,7 +141,7 @@ cudaError_t launch_scatter_rows(const float* src, int width, float* dst, const i
 cudaError_t launch_cast_rows(int dtype, const float* src, void* dst, int n, cudaStream_t st);
 cudaError_t launch_fill_i32(int32_t* p, int32_t v, int n, cudaStream_t st);
 cudaError_t launch_accept(int dtype, const int32_t* beams, const rd_packed& pk, const int32_t* argmax,
-                          const float* hidden, void* kcache, int32_t* ctx, int32_t* root, float* h,
+                          const float* hidden, const int32_t* seq_off, void* kcache, int32_t* ctx, int32_t* root, float* h,
                           const rd_accept_out& out, int32_t* n_accept_ws, int32_t* best_ws, int32_t* ctx_prev,
                           const Dims& dm, int B, int* status, cudaStream_t st);
 int accept_static_max_batch();

@@ -9,6 +9,7 @@ import torch
 
 from oracle import redrafter_oracle as ora
 from paper_2403_09919_b200 import synth
+from paper_2403_09919_b200.binding import ReDrafter
 
 pytestmark = pytest.mark.gpu
 
@@ -301,6 +302,44 @@ def test_batched_ragged_step():
             assert np.abs(c_h[b].cpu().numpy() - ref["h"]).max() < TOL_FP32
             kvg = r.eng.kv_view()[:, 0, b, :, :ref["ctx"]].cpu().numpy().transpose(0, 2, 1, 3)
             assert np.abs(kvg - kv.k[:, :ref["ctx"]]).max() < TOL_FP32
+
+
+@pytest.mark.parametrize("dtype,L,a", [("fp32", 5, 3), ("fp32", 7, 7), ("fp32", 9, 8), ("fp32", 17, 17), ("bf16", 8, 8), ("bf16", 9, 9),
+                                       ("bf16", 16, 0), ("bf16", 20, 11)])
+def test_accept_and_compaction_along_long_paths(dtype, L, a):
+    """Paths up to, at and beyond the eight nodes that acceptance and compaction handle at a time: lengths, tokens, the
+    handed-over hidden row and every slot of the cache, bit for bit."""
+    BW, B = 3, 2
+    cfg = dict(synth.CONFIGS["tiny"], dtype=dtype, n_heads=4 if dtype == "fp32" else 2, max_batch=B, beam_width=BW, beam_length=L, max_ctx=120)
+    eng = ReDrafter(cfg, synth.make_weights(cfg, "cuda:0"))
+    ctx = [5, 40]
+    eng.set_state(dev(ctx), dev([1, 2]), torch.zeros(B, cfg["d_model"], device="cuda"), ctx_bound=40)
+    rng = np.random.default_rng(L * 100 + a)
+    beams = rng.permutation(900)[:B * BW * L].reshape(B, BW, L) + 10     # no shared prefixes: candidate 2's nodes lie far out
+    pk = eng.pack(dev(beams))
+    unpack = pk.unpack.cpu().numpy()
+    argmax = np.full((B, eng.nmax), 3)
+    for b in range(B):
+        argmax[b, unpack[b, 2, :a]] = beams[b, 2, :a]
+        argmax[b, unpack[b, 2, a]] = 4 + b
+    hidden = torch.randn(B, eng.nmax, cfg["d_model"], device="cuda")
+    kv = eng.kv_view()
+    kv.copy_(torch.randn(kv.shape, device="cuda"))
+    want = kv.clone()
+    for b in range(B):
+        for j in range(1, a + 1):
+            want[:, :, b, :, ctx[b] + j] = kv[:, :, b, :, ctx[b] + int(unpack[b, 2, j])]
+    out = eng.accept(dev(beams), pk, dev(argmax), hidden)
+    eng.poll()
+    assert out.n_accept.tolist() == [a] * B and out.best.tolist() == [2 if a else 0] * B
+    node = [int(unpack[b, 2 if a else 0, a]) for b in range(B)]
+    for b in range(B):
+        assert out.tokens[b].tolist() == beams[b, 2, :a].tolist() + [int(argmax[b, node[b]])] + [-1] * (L - a)
+    c, r, h = eng.get_state()
+    assert c.tolist() == [x + 1 + a for x in ctx] and r.tolist() == [int(argmax[b, node[b]]) for b in range(B)]
+    assert torch.equal(h, torch.stack([hidden[b, node[b]] for b in range(B)]))
+    assert torch.equal(kv, want)
+    eng.close()
 
 
 def test_context_bound_follows_the_real_context():
