@@ -322,9 +322,19 @@ int gemm(rd_handle* h, const void* A, int lda, const void* W, int N, int K, cons
     h->route[pairs ? RD_ROUTE_GEMM_PAIRS : RD_ROUTE_GEMM_ONE_CTA]++;
     return RD_OK;
   }
-  if (chain) chain->cut();
+  SimtEpilogue e{};
+  e.out_f = raw; e.ld = ld_raw;
   h->route[RD_ROUTE_GEMM_SIMT]++;
-  CK(h, launch_gemm_simt(h->dm.dtype, A, lda, W, N, K, m_total, m_max, raw, ld_raw, out, st));
+  CK(h, launch_gemm_simt(h->dm.dtype, SIMT_RAW, SimtOperands{A, lda, nullptr, 0.f, W, K, N, m_total}, e, h->dm, m_max, chain, st));
+  *out = simt_out(raw, ld_raw);
+  return RD_OK;
+}
+
+// CUDA-core projection with the function behind it.
+int gemm_simt(rd_handle* h, int epi, const SimtOperands& p, const SimtEpilogue& e, int n_weight_rows, int m_max, Chain* chain, cudaStream_t st) {
+  ProfScope ps(h, 0, (double)n_weight_rows * p.K * esize(h->dm.dtype), st);
+  h->route[RD_ROUTE_GEMM_SIMT]++;
+  CK(h, launch_gemm_simt(h->dm.dtype, epi, p, e, h->dm, m_max, chain, st));
   return RD_OK;
 }
 
@@ -378,6 +388,46 @@ char* kv_plane_ptr(rd_handle* h, int layer, int which) {
   return h->kv + ((size_t)(layer * 2 + which)) * h->kv_plane * esize(h->dm.dtype);
 }
 
+// The layers on the CUDA-core path: a projection takes the norm in front of it (where a row fits its staging) and the
+// residual, rotary or SwiGLU behind it along.  Leaves the complete residual stream in ws.x.
+int layers_simt(rd_handle* h, const RowTables& rt, int m_max, Chain* ch, cudaStream_t st) {
+  Workspace& w = h->ws;
+  const Dims& dm = h->dm;
+  const bool fuse_norm = dm.d <= simt_norm_max_k();
+  auto normed = [&](const void* gain, const void* W, int items) {   // the operands of a projection of the normalised rows
+    return fuse_norm ? SimtOperands{w.x, dm.d, gain, dm.eps, W, dm.d, items, w.m_total}
+                     : SimtOperands{w.a_t, dm.d, nullptr, 0.f, W, dm.d, items, w.m_total};
+  };
+  for (int l = 0; l < dm.n_layers; ++l) {
+    if (!fuse_norm)
+      CKP(h, PROF_NORM, launch_rmsnorm(dm.dtype, w.x, nullptr, h->attn_norm[l], w.a_t, nullptr, dm.d, dm.eps, w.m_total, m_max, ch, st));
+    SimtEpilogue e{};
+    e.out_f = w.qkv; e.ld = 3 * dm.d;
+    e.kcache = kv_plane_ptr(h, l, 0); e.vcache = kv_plane_ptr(h, l, 1);
+    e.table = reinterpret_cast<const float2*>(w.rope_tab); e.seq = rt.seq; e.slot = rt.slot; e.status = w.status;
+    int rc = gemm_simt(h, SIMT_ROPE, normed(h->attn_norm[l], h->wqkv[l], 3 * dm.H * (dm.hd / 2)), e, 3 * dm.d, m_max, ch, st);
+    if (rc) return rc;
+    {
+      ProfScope ps(h, 1, 0.0, st);
+      h->route[RD_ROUTE_ATT_FP32]++;
+      CK(h, launch_attention(dm.dtype, w.qkv, kv_plane_ptr(h, l, 0), kv_plane_ptr(h, l, 1), w.attn_t, rt, dm, m_max, ch, st));
+    }
+    e = SimtEpilogue{};
+    e.out_f = w.x; e.ld = dm.d;
+    rc = gemm_simt(h, SIMT_RESIDUAL, SimtOperands{w.attn_t, dm.d, nullptr, 0.f, h->wo[l], dm.d, dm.d, w.m_total}, e, dm.d, m_max, ch, st);
+    if (rc) return rc;
+    if (!fuse_norm)
+      CKP(h, PROF_NORM, launch_rmsnorm(dm.dtype, w.x, nullptr, h->ffn_norm[l], w.a_t, nullptr, dm.d, dm.eps, w.m_total, m_max, ch, st));
+    SimtEpilogue sw{};
+    sw.out_t = w.act_t; sw.F = dm.F;
+    rc = gemm_simt(h, SIMT_SWIGLU, normed(h->ffn_norm[l], h->w_gate_up[l], dm.F), sw, 2 * dm.F, m_max, ch, st);
+    if (rc) return rc;
+    rc = gemm_simt(h, SIMT_RESIDUAL, SimtOperands{w.act_t, dm.F, nullptr, 0.f, h->w_down[l], dm.F, dm.d, w.m_total}, e, dm.d, m_max, ch, st);
+    if (rc) return rc;
+  }
+  return RD_OK;
+}
+
 // Embedding -> n_layers x {attention block, FFN block} -> final norm.  Rows and masks come from the
 // row tables in the workspace; results: ws.hidden_f / ws.hidden_t (compact rows).
 int forward_layers(rd_handle* h, const uint32_t* mask, int m_max, int n_seq, int rows_per_seq_max, const void* after_w,
@@ -424,34 +474,38 @@ int forward_layers(rd_handle* h, const uint32_t* mask, int m_max, int n_seq, int
   GemmOut g_qkv, g_o, g_gu, g_dn;
   // inside the layer loop every launch hands over to the next through a counter; the launches before
   // and after it use the grid dependency
-  Chain* ch = h->use_tc ? &h->chain : nullptr;
+  Chain* ch = &h->chain;
   if (int rc0 = chain_start(h, st)) return rc0;
+  if (!h->use_tc) {
+    if (int rc = layers_simt(h, rt, m_max, ch, st)) return rc;
+    CKP(h, PROF_NORM, launch_rmsnorm(dm.dtype, w.x, nullptr, h->w.final_norm, w.hidden_t, w.hidden_f, dm.d, dm.eps, w.m_total, m_max, ch, st));
+    h->chain.cut();
+    return RD_OK;
+  }
   for (int l = 0; l < dm.n_layers; ++l) {
     // attention block: (x += down of the previous layer) -> norm -> QKV -> rotary + KV write -> attention -> O
     CKP(h, PROF_NORM, launch_rmsnorm(dm.dtype, w.x, l ? &g_dn : nullptr, h->attn_norm[l], w.a_t, nullptr, dm.d, dm.eps,
                                      w.m_total, m_max, ch, st));
     int rc = gemm(h, w.a_t, dm.d, h->wqkv[l], 3 * dm.d, dm.d, w.m_total, m_max, w.qkv, 3 * dm.d, &g_qkv, ch, st, /*pair=*/1);
     if (rc) return rc;
-    CKP(h, PROF_ROPE, launch_rope_kv(dm.dtype, w.qkv, g_qkv, kv_plane_ptr(h, l, 0), kv_plane_ptr(h, l, 1), w.rope_tab, rt, dm,
+    CKP(h, PROF_ROPE, launch_rope_kv(w.qkv, g_qkv, kv_plane_ptr(h, l, 0), kv_plane_ptr(h, l, 1), w.rope_tab, rt, dm,
                                      m_max, w.status, ch, st));
     {
       ProfScope ps(h, 1, 0.0, st);
-      h->route[!h->use_tc ? RD_ROUTE_ATT_FP32 : att_t5 ? RD_ROUTE_ATT_ROWS128_TC5 : att_wide ? RD_ROUTE_ATT_ROWS64
+      h->route[att_t5 ? RD_ROUTE_ATT_ROWS128_TC5 : att_wide ? RD_ROUTE_ATT_ROWS64
                : att_shallow ? RD_ROUTE_ATT_ROWS16_SHALLOW : RD_ROUTE_ATT_ROWS16]++;
-      if (h->use_tc && !att_t5 && !att_wide && n_splits > 1) h->route[RD_ROUTE_ATT_KEY_SPLIT]++;
-      if (h->use_tc && att_t5)
+      if (!att_t5 && !att_wide && n_splits > 1) h->route[RD_ROUTE_ATT_KEY_SPLIT]++;
+      if (att_t5)
         CK(h, launch_attention_t5(h->kv_maps[(size_t)l * 2].bytes, h->kv_maps[(size_t)l * 2 + 1].bytes, w.qkv, w.attn_t, rt, w.seq_off, h->att_seq_order, dm, n_seq,
                                   row_blocks, w.status, ch, st));
-      else if (h->use_tc && att_wide)
+      else if (att_wide)
         CK(h, launch_attention_wide(w.qkv, kv_plane_ptr(h, l, 0), kv_plane_ptr(h, l, 1), w.attn_t, rt, w.seq_off, dm, n_seq,
                                     row_blocks, ch, st));
-      else if (h->use_tc)
+      else
         CK(h, launch_attention_tc(w.qkv, kv_plane_ptr(h, l, 0), kv_plane_ptr(h, l, 1), w.attn_t, rt, w.seq_off, dm, n_seq,
                                   row_blocks, n_splits, w.att_scratch, w.att_counters,
                                   (h->trace_next >= 0 && h->trace_next < TRACE_SLOTS) ? w.trace + (size_t)8 * h->trace_next++ : nullptr, ch,
                                   att_shallow ? 1 : 0, st));
-      else
-        CK(h, launch_attention(dm.dtype, w.qkv, kv_plane_ptr(h, l, 0), kv_plane_ptr(h, l, 1), w.attn_t, rt, dm, m_max, st));
     }
     rc = gemm(h, w.attn_t, dm.d, h->wo[l], dm.d, dm.d, w.m_total, m_max, w.proj_d, dm.d, &g_o, ch, st, /*pair=*/1);
     if (rc) return rc;
@@ -459,7 +513,7 @@ int forward_layers(rd_handle* h, const uint32_t* mask, int m_max, int n_seq, int
     CKP(h, PROF_NORM, launch_rmsnorm(dm.dtype, w.x, &g_o, h->ffn_norm[l], w.a_t, nullptr, dm.d, dm.eps, w.m_total, m_max, ch, st));
     rc = gemm(h, w.a_t, dm.d, h->w_gate_up[l], 2 * dm.F, dm.d, w.m_total, m_max, w.gu, 2 * dm.F, &g_gu, ch, st, /*pair=*/1);
     if (rc) return rc;
-    CKP(h, PROF_SWIGLU, launch_swiglu(dm.dtype, g_gu, w.act_t, dm.F, w.m_total, m_max, w.status, ch, st));
+    CKP(h, PROF_SWIGLU, launch_swiglu(g_gu, w.act_t, dm.F, w.m_total, m_max, w.status, ch, st));
     rc = gemm(h, w.act_t, dm.F, h->w_down[l], dm.d, dm.F, w.m_total, m_max, w.proj_d, dm.d, &g_dn, ch, st, /*pair=*/1);
     if (rc) return rc;
   }
@@ -487,9 +541,26 @@ int do_draft(rd_handle* h, cudaStream_t st, int32_t* beams, float* scores) {
   float *sc_in = w.score_a, *sc_out = w.score_b;
   int32_t *hi_in = w.hist_a, *hi_out = w.hist_b;
   GemmOut g;
-  // the calls' launches hand over to each other through counters (tensor-core path)
-  Chain* ch = h->use_tc ? &h->chain : nullptr;
+  // the calls' launches hand over to each other through counters
+  Chain* ch = &h->chain;
   if (int rc0 = chain_start(h, st)) return rc0;
+  // out = (resid) + SiLU(W x + bias), rows of out and resid d_rnn + d_model wide
+  auto cell = [&](const void* x, int K, const void* W, const void* bias, int N, const float* resid, float* of, void* ot, float* raw,
+                  const int32_t* mt, int rows) -> int {
+    if (!h->use_tc) {
+      SimtEpilogue e{};
+      e.out_f = of; e.out_t = ot; e.ld = dm.dh; e.bias = bias; e.resid = resid; e.ld_resid = dm.dh;
+      return gemm_simt(h, SIMT_ACT, SimtOperands{x, K, nullptr, 0.f, W, K, N, mt}, e, N, rows, ch, st);
+    }
+    int rc = gemm(h, x, K, W, N, K, mt, rows, raw, N, &g, ch, st, /*pair=*/1);
+    if (rc) return rc;
+    CKP(h, PROF_DRAFT_SMALL, launch_act(g, bias, resid, resid ? dm.dh : 0, of, ot, dm.dh, N, mt, rows, ch, st));
+    return RD_OK;
+  };
+  // On the CUDA-core path (small models) the one-kernel selection is ahead for narrow beams: it takes a round per beam
+  // where the three kernels count (V = 1024, batch 1, four calls: 92 against 101 us at beam width 4, 126 / 125 at 8,
+  // 184 / 132 at 16, 1609 / 229 at 64).
+  const bool three = h->use_tc || dm.BW >= 8;
   for (int call = 1; call <= dm.L; ++call) {
     const int rows = call == 1 ? B : R;
     const int32_t* mt = call == 1 ? w.one_b : w.one_r;
@@ -497,16 +568,14 @@ int do_draft(rd_handle* h, cudaStream_t st, int32_t* beams, float* scores) {
     const float* xin_f = call == 1 ? w.xc_f : w.x0_f;
     if (call > 1) {
       // s_t = SiLU([U W][s_{t-1}; e_t] + b), written into the first d_rnn columns of x0 = [s_t, h]
-      int rc = gemm(h, w.se_t, dm.dr + dm.d, w.uw, dm.dr, dm.dr + dm.d, mt, rows, w.sraw, dm.dr, &g, ch, st, /*pair=*/1);
+      int rc = cell(w.se_t, dm.dr + dm.d, w.uw, h->w.rnn_b, dm.dr, nullptr, w.x0_f, w.x0_t, w.sraw, mt, rows);
       if (rc) return rc;
-      CKP(h, PROF_DRAFT_SMALL, launch_act(dm.dtype, g, h->w.rnn_b, nullptr, 0, w.x0_f, w.x0_t, dm.dh, dm.dr, mt, rows, ch, st));
     }
     for (int l = 0; l < dm.n_head_layers; ++l) {
       float* of = (l & 1) ? w.x2_f : w.x1_f;
       void* ot = (l & 1) ? w.x2_t : w.x1_t;
-      int rc = gemm(h, xin_t, dm.dh, h->head_w[l], dm.dh, dm.dh, mt, rows, w.hraw, dm.dh, &g, ch, st, /*pair=*/1);
+      int rc = cell(xin_t, dm.dh, h->head_w[l], h->head_b[l], dm.dh, xin_f, of, ot, w.hraw, mt, rows);
       if (rc) return rc;
-      CKP(h, PROF_DRAFT_SMALL, launch_act(dm.dtype, g, h->head_b[l], xin_f, dm.dh, of, ot, dm.dh, dm.dh, mt, rows, ch, st));
       xin_t = ot; xin_f = of;
     }
     int rc = gemm(h, xin_t, dm.dh, h->w.draft_out, dm.V, dm.dh, mt, rows, w.dlogits, dm.V, &g, ch, st, /*pair=*/1);
@@ -514,8 +583,8 @@ int do_draft(rd_handle* h, cudaStream_t st, int32_t* beams, float* scores) {
     CKP(h, PROF_DRAFT_SMALL, launch_draft_select(dm.dtype, g, call, w.lse, w.cand_val, w.cand_idx, sc_in, sc_out, hi_in, hi_out,
                                                  h->w.tok_emb, w.x0_f, dm.dh, w.se_t, dm, B, beams, scores, w.sel_counters, mt,
                                                  (h->trace_next >= 0 && h->trace_next < TRACE_SLOTS) ? w.trace + (size_t)8 * h->trace_next++ : nullptr,
-                                                 SelectScratch{h->use_tc ? w.seg_max : nullptr, w.seg_sum, w.seg_val, w.seg_idx, h->tc_grid, w.sel_top}, ch, st));
-    if (h->use_tc && draft_select_segments(dm, rows, h->tc_grid) > 0) h->launches += 2;   // that selection is three launches
+                                                 SelectScratch{three ? w.seg_max : nullptr, w.seg_sum, w.seg_val, w.seg_idx, h->tc_grid, w.sel_top}, ch, st));
+    if (three && draft_select_segments(dm, rows, h->tc_grid) > 0) h->launches += 2;   // that selection is three launches
     float* tf = sc_in; sc_in = sc_out; sc_out = tf;
     int32_t* ti = hi_in; hi_in = hi_out; hi_out = ti;
   }
@@ -601,22 +670,26 @@ int redrafter_init(const rd_config* cfg, const rd_weights* wt, void* kv_cache, s
   carve(bp, dm, h->m_cap, &h->ws);
   h->use_tc = dm.dtype == RD_DTYPE_BF16 && !(cfg->flags & RD_FLAG_FORCE_SIMT);
   {
-    cudaError_t ce = elementwise_prepare(dm.dtype);
+    cudaError_t ce = elementwise_prepare();
     if (ce == cudaSuccess) ce = drafter_prepare(dm.dtype);
     if (ce != cudaSuccess) return init_fail(h, RD_ERR_CUDA, "kernel set-up: %s", cudaGetErrorString(ce));
   }
   h->tc_pairs = 0; h->tc_pairs_avail = 0; h->tc_pairs_min_rows = 1024; h->tc_pairs_prefill = false;
-  if (h->use_tc) {
-    int dev = 0, sms = 0;
+  int sms = 0;
+  {
+    int dev = 0;
     cudaError_t ce = cudaGetDevice(&dev);
     if (ce == cudaSuccess) ce = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (ce == cudaSuccess) ce = tc_prepare(&h->tc_smem, &h->tc_pairs_avail);
+    if (ce != cudaSuccess || sms <= 0) return init_fail(h, RD_ERR_CUDA, "device query: %s", cudaGetErrorString(ce));
+    h->tc_grid = sms < TC_MAX_GRID ? sms : TC_MAX_GRID;
+  }
+  if (h->use_tc) {
+    cudaError_t ce = tc_prepare(&h->tc_smem, &h->tc_pairs_avail);
     if (ce == cudaSuccess) ce = attn_tc_prepare(dm.hd, dm.MW);
     if (ce == cudaSuccess) ce = attn_wide_prepare(dm.hd, dm.MW);
     if (ce == cudaSuccess) ce = attn_t5_prepare(dm.hd, dm.MW);
-    if (ce != cudaSuccess || sms <= 0)
+    if (ce != cudaSuccess)
       return init_fail(h, RD_ERR_CUDA, "tensor-core path set-up: %s", cudaGetErrorString(ce));
-    h->tc_grid = sms < TC_MAX_GRID ? sms : TC_MAX_GRID;
     // CTA-pair projections (tuning toggles, read when the handle is made): from a bound of 1024 rows in decode steps
     // (measured: 1-4 % of the step from about 650 packed rows; with bounds around 650 rows, 300-420 rows present, the
     // one-CTA kernel, which starts earlier and has shorter tails, is 3-5 % ahead); RD_TC_CTA2=0 never, RD_TC_CTA2_MIN the row bound, RD_TC_CTA2_PREFILL=1 also in prompt passes.

@@ -8,6 +8,8 @@
 //   beam_merge: per sequence, score_r + logit - lse_r over the BW*BW survivors, best BW in
 //               (score desc, flat index r*V + v asc) order; reorders histories and states and
 //               gathers the next call's input [s_t of the parent ; E[token]].
+#include <algorithm>
+
 #include "rd_internal.cuh"
 #include "gemm_out.cuh"
 #include "pdl.cuh"
@@ -129,12 +131,12 @@ __global__ void __maxnreg__(88) act_kernel(GemmOut proj, const T* __restrict__ b
 }
 
 // N, ld_resid, ld_out multiples of 4 (8 for bf16 outputs); bias 16-byte aligned.
-cudaError_t launch_act(int dtype, const GemmOut& proj, const void* bias, const float* resid, int ld_resid, float* out_f,
+cudaError_t launch_act(const GemmOut& proj, const void* bias, const float* resid, int ld_resid, float* out_f,
                        void* out_t, int ld_out, int N, const int32_t* m_total, int m_max, Chain* chain, cudaStream_t st) {
   dim3 grid((N / 4 + ACT_THREADS - 1) / ACT_THREADS, m_max);
   const ChainSync cs = chain ? chain->link(grid.x * grid.y, true) : ChainSync{nullptr, 0u, nullptr, nullptr, nullptr};
-  RD_DISPATCH(dtype, launch_pdl(act_kernel<T>, grid, ACT_THREADS, 0, st, proj, (const T*)bias, resid, ld_resid, out_f,
-                                (T*)out_t, ld_out, N, m_total, cs));
+  launch_pdl(act_kernel<__nv_bfloat16>, grid, ACT_THREADS, 0, st, proj, (const __nv_bfloat16*)bias, resid, ld_resid, out_f,
+             (__nv_bfloat16*)out_t, ld_out, N, m_total, cs);
   return cudaGetLastError();
 }
 
@@ -172,7 +174,7 @@ __device__ __forceinline__ float block_reduce_sum(float s, float* sh) {
   return s;
 }
 
-constexpr int SEL_THREADS = 1024;
+constexpr int SEL_THREADS_MAX = 1024;   // one per four vocabulary entries, up to this many (V = 1024: 8 us per call with 256, 10 with 1024)
 constexpr int SEL_MAX_BW = 128;
 constexpr int SEL_LIST_CAP = 1024;  // elements at or above the selection threshold
 
@@ -185,7 +187,7 @@ constexpr int SEL_LIST_CAP = 1024;  // elements at or above the selection thresh
 //     score_r + logit - lse_r to the BW best in (score desc, flat index r*V + v asc) order, writes the
 //     new scores and histories, and gathers the next call's input rows [s_t of the parent ; E[token]].
 template <typename T>
-__global__ void __launch_bounds__(SEL_THREADS) draft_select_kernel(
+__global__ void __launch_bounds__(SEL_THREADS_MAX) draft_select_kernel(
     GemmOut proj, int call, float* __restrict__ lse, float* __restrict__ val, int32_t* __restrict__ idx,
     const float* __restrict__ score_in, float* __restrict__ score_out, const int32_t* __restrict__ hist_in,
     int32_t* __restrict__ hist_out, const T* __restrict__ emb, const float* __restrict__ s_new_f, int ld_s,
@@ -196,7 +198,7 @@ __global__ void __launch_bounds__(SEL_THREADS) draft_select_kernel(
   chain_enter(cs);
   asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t_dbg[1]));
   extern __shared__ __align__(16) uint8_t sel_smem[];
-  Cand* wl = reinterpret_cast<Cand*>(sel_smem);            // [32 warps][BW] per-warp survivors; reused by the pruning
+  Cand* wl = reinterpret_cast<Cand*>(sel_smem);            // [warps][BW] per-warp survivors; reused by the pruning
   __shared__ float shf[32];
   __shared__ Cand sh_top[SEL_MAX_BW];
   __shared__ int sel_parent[SEL_MAX_BW], sel_tok[SEL_MAX_BW];
@@ -205,7 +207,7 @@ __global__ void __launch_bounds__(SEL_THREADS) draft_select_kernel(
   __shared__ float s_tau;
   const int BW = dm.BW, L = dm.L, V = dm.V;
   const int r = blockIdx.x;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
   const GemmRows m_tiles = gemm_m_tiles(proj, *m_total);
   Cand* cl = wl + 32 * BW;   // [SEL_LIST_CAP] values at or above the threshold
   // ---- 1. logits into shared memory (compact loops from here on: the kernel runs once per launch,
@@ -213,14 +215,14 @@ __global__ void __launch_bounds__(SEL_THREADS) draft_select_kernel(
   float* zrow = reinterpret_cast<float*>(cl + SEL_LIST_CAP);   // [V]
   float tmax = -INFINITY;
 #pragma unroll 4
-  for (int i = 4 * threadIdx.x; i < V; i += 4 * SEL_THREADS) {
+  for (int i = 4 * threadIdx.x; i < V; i += 4 * blockDim.x) {
     const float4 q = gemm_value4<2>(proj, m_tiles, r, i);   // V is a multiple of 4
     *reinterpret_cast<float4*>(zrow + i) = q;
     tmax = fmaxf(tmax, fmaxf(fmaxf(q.x, q.y), fmaxf(q.z, q.w)));
   }
   asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t_dbg[2]));
-  // ---- 2a. a threshold that at least BW elements reach: the BW-th largest of the 1024 per-thread maxima
-  // (per warp BW rounds over one value per lane, then warp 0 over the 32 x BW survivors)
+  // ---- 2a. a threshold that at least BW elements reach: the BW-th largest of the per-thread maxima
+  // (per warp BW rounds over one value per lane, then warp 0 over the warps' survivors)
   {
     Cand prev{INFINITY, -1};
     for (int p = 0; p < BW; ++p) {
@@ -239,12 +241,12 @@ __global__ void __launch_bounds__(SEL_THREADS) draft_select_kernel(
   if (lane == 0) shf[warp] = wmax;
   if (threadIdx.x == 0) s_count = 0;
   __syncthreads();
-  float rmax = shf[lane];
+  float rmax = lane < n_warps ? shf[lane] : -INFINITY;
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) rmax = fmaxf(rmax, __shfl_xor_sync(0xffffffffu, rmax, o));
   float s = 0.f;
 #pragma unroll 4
-  for (int i = 4 * threadIdx.x; i < V; i += 4 * SEL_THREADS) {
+  for (int i = 4 * threadIdx.x; i < V; i += 4 * blockDim.x) {
     const float4 q = *reinterpret_cast<const float4*>(zrow + i);
     s += __expf(q.x - rmax) + __expf(q.y - rmax) + __expf(q.z - rmax) + __expf(q.w - rmax);
   }
@@ -254,7 +256,7 @@ __global__ void __launch_bounds__(SEL_THREADS) draft_select_kernel(
     Cand pv{INFINITY, -1};
     for (int p = 0; p < BW; ++p) {
       Cand best{-INFINITY, 0x7fffffff};
-      for (int c = lane; c < 32 * BW; c += 32) {
+      for (int c = lane; c < n_warps * BW; c += 32) {
         const float x = wl[c].v;
         if (cand_before(pv.v, pv.i, x, c)) best = cand_best(best, Cand{x, c});
       }
@@ -268,7 +270,7 @@ __global__ void __launch_bounds__(SEL_THREADS) draft_select_kernel(
   // ---- 2c. every element that reaches the threshold goes to a short list; warp 0 ranks the list
   const float tau = s_tau;
 #pragma unroll 4
-  for (int i = 4 * threadIdx.x; i < V; i += 4 * SEL_THREADS) {
+  for (int i = 4 * threadIdx.x; i < V; i += 4 * blockDim.x) {
     const float4 q = *reinterpret_cast<const float4*>(zrow + i);
     const float e[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
@@ -303,13 +305,13 @@ __global__ void __launch_bounds__(SEL_THREADS) draft_select_kernel(
     Cand prev{INFINITY, -1};
     for (int p = 0; p < BW; ++p) {
       Cand best{-INFINITY, 0x7fffffff};
-      for (int i = threadIdx.x; i < V; i += SEL_THREADS)
+      for (int i = threadIdx.x; i < V; i += blockDim.x)
         if (cand_before(prev.v, prev.i, zrow[i], i)) best = cand_best(best, Cand{zrow[i], i});
       best = warp_best(best);
       __syncthreads();
       if (lane == 0) wl[warp] = best;
       __syncthreads();
-      best = warp_best(wl[lane]);
+      best = warp_best(lane < n_warps ? wl[lane] : Cand{-INFINITY, 0x7fffffff});
       if (threadIdx.x == 0) {
         val[(size_t)r * BW + p] = best.v;
         idx[(size_t)r * BW + p] = best.i == 0x7fffffff ? 0 : best.i;
@@ -342,7 +344,7 @@ __global__ void __launch_bounds__(SEL_THREADS) draft_select_kernel(
   for (int c = threadIdx.x; c < n_cand; c += blockDim.x) {
     const int rr = c / BW;
     const size_t o = (size_t)(row0 + rr) * BW + (c - rr * BW);
-    const float base = call == 1 ? 0.f : score_in[row0 + rr];
+    const float base = call == 1 ? 0.f : __ldcg(score_in + row0 + rr);
     wl[c] = Cand{base + (__ldcg(val + o) - __ldcg(lse + row0 + rr)), rr * V + __ldcg(idx + o)};
   }
   __syncthreads();
@@ -366,10 +368,10 @@ __global__ void __launch_bounds__(SEL_THREADS) draft_select_kernel(
     sel_parent[k] = parent; sel_tok[k] = tok; sel_score[k] = c.v;
     const int orow = b * BW + k, prow = b * BW + parent;
     score_out[orow] = c.v;
-    for (int t = 0; t < call - 1; ++t) hist_out[(size_t)orow * L + t] = hist_in[(size_t)prow * L + t];
+    for (int t = 0; t < call - 1; ++t) hist_out[(size_t)orow * L + t] = __ldcg(hist_in + (size_t)prow * L + t);
     hist_out[(size_t)orow * L + call - 1] = tok;
     if (call == L) {
-      for (int t = 0; t < L - 1; ++t) beams_out[(size_t)orow * L + t] = hist_in[(size_t)prow * L + t];
+      for (int t = 0; t < L - 1; ++t) beams_out[(size_t)orow * L + t] = __ldcg(hist_in + (size_t)prow * L + t);
       beams_out[(size_t)orow * L + L - 1] = tok;
       if (scores_out) scores_out[orow] = c.v;
     }
@@ -387,7 +389,7 @@ __global__ void __launch_bounds__(SEL_THREADS) draft_select_kernel(
     if (call > 1) {
       for (int item = threadIdx.x; item < BW * sv; item += blockDim.x) {
         const int k = item / sv, i = item - k * sv;
-        const float4 q = reinterpret_cast<const float4*>(s_new_f + (size_t)(b * BW + sel_parent[k]) * ld_s)[i];
+        const float4 q = __ldcg(reinterpret_cast<const float4*>(s_new_f + (size_t)(b * BW + sel_parent[k]) * ld_s) + i);
         T* so = se_t + (size_t)(b * BW + k) * (dm.dr + dm.d) + 4 * i;
         so[0] = from_f<T>(q.x); so[1] = from_f<T>(q.y); so[2] = from_f<T>(q.z); so[3] = from_f<T>(q.w);
       }
@@ -817,8 +819,9 @@ cudaError_t launch_draft_select(int dtype, const GemmOut& proj, int call, float*
   const size_t prune = (size_t)dm.BW * dm.BW * sizeof(Cand);
   const size_t smem = select > prune ? select : prune;
   if (smem > 200 * 1024) return cudaErrorInvalidValue;   // vocabulary too large for the shared-memory row
+  const int threads = std::min(SEL_THREADS_MAX, (std::max(dm.V / 4, dm.BW) + 31) & ~31);
   const ChainSync cs = chain ? chain->link((unsigned)rows) : ChainSync{nullptr, 0u, nullptr, nullptr, nullptr};
-  RD_DISPATCH(dtype, launch_pdl(draft_select_kernel<T>, rows, SEL_THREADS, smem, st, proj, call, lse, val, idx, score_in,
+  RD_DISPATCH(dtype, launch_pdl(draft_select_kernel<T>, rows, threads, smem, st, proj, call, lse, val, idx, score_in,
                                 score_out, hist_in, hist_out, (const T*)emb, s_new_f, ld_s, (T*)se_t, dm, beams_out,
                                 scores_out, counters, m_total, dbg, cs));
   return cudaGetLastError();

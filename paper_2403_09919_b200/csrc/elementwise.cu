@@ -557,7 +557,7 @@ __global__ void __launch_bounds__(ROPW_THREADS, 4)
   chain_exit(cs);
 }
 
-cudaError_t launch_rope_kv(int dtype, float* qkv, const GemmOut& proj, void* kcache, void* vcache, const float* table,
+cudaError_t launch_rope_kv(float* qkv, const GemmOut& proj, void* kcache, void* vcache, const float* table,
                            const RowTables& rt, const Dims& dm, int m_max, int* status, Chain* chain, cudaStream_t st) {
   const int n_items = dm.H * (dm.hd / 4);
   dim3 grid(m_max, (n_items + ROPE_THREADS - 1) / ROPE_THREADS);
@@ -568,13 +568,13 @@ cudaError_t launch_rope_kv(int dtype, float* qkv, const GemmOut& proj, void* kca
     const int gy = (4 * wide_sm_count() + (int)gw.x - 1) / (int)gw.x;
     gw.y = gy < m_max ? gy : m_max;
     const ChainSync cs = chain ? chain->link(gw.x * gw.y, true) : ChainSync{nullptr, 0u, nullptr, nullptr, nullptr};
-    RD_DISPATCH(dtype, launch_pdl(rope_kv_wide_kernel<T>, gw, ROPW_THREADS, 0, st, qkv, proj, (T*)kcache, (T*)vcache,
-                                  reinterpret_cast<const float2*>(table), rt, dm, status, cs));
+    launch_pdl(rope_kv_wide_kernel<__nv_bfloat16>, gw, ROPW_THREADS, 0, st, qkv, proj, (__nv_bfloat16*)kcache, (__nv_bfloat16*)vcache,
+               reinterpret_cast<const float2*>(table), rt, dm, status, cs);
     return cudaGetLastError();
   }
   const ChainSync cs = chain ? chain->link(grid.x * grid.y, true) : ChainSync{nullptr, 0u, nullptr, nullptr, nullptr};
-  RD_DISPATCH(dtype, launch_pdl(rope_kv_kernel<T>, grid, ROPE_THREADS, 0, st, qkv, proj, (T*)kcache, (T*)vcache,
-                                reinterpret_cast<const float2*>(table), rt, dm, status, cs));
+  launch_pdl(rope_kv_kernel<__nv_bfloat16>, grid, ROPE_THREADS, 0, st, qkv, proj, (__nv_bfloat16*)kcache, (__nv_bfloat16*)vcache,
+             reinterpret_cast<const float2*>(table), rt, dm, status, cs);
   return cudaGetLastError();
 }
 
@@ -742,15 +742,13 @@ __global__ void __launch_bounds__(SWS_THREADS, 3)
 }
 
 // Once per handle (and so per device): opt-in of the kernels that take more than 48 KB of dynamic shared memory.
-cudaError_t elementwise_prepare(int dtype) {
-  cudaError_t e = cudaErrorInvalidValue;
+cudaError_t elementwise_prepare() {
   const int smem = SWS_STAGES * 2 * SWS_COLS * (int)sizeof(float);
-  RD_DISPATCH(dtype, e = cudaFuncSetAttribute(swiglu_wide_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-  return e;
+  return cudaFuncSetAttribute(swiglu_wide_kernel<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
 }
 
 // proj: the gate|up projection [M][2F]; out: [M][F].  F must be a multiple of 4.
-cudaError_t launch_swiglu(int dtype, const GemmOut& proj, void* out_t, int F, const int32_t* m_total, int m_max,
+cudaError_t launch_swiglu(const GemmOut& proj, void* out_t, int F, const int32_t* m_total, int m_max,
                           int32_t* status, Chain* chain, cudaStream_t st) {
   const int per_cta = SWIGLU_THREADS * SWIGLU_ITEMS * 4;
   dim3 grid((F + per_cta - 1) / per_cta, m_max);
@@ -760,11 +758,11 @@ cudaError_t launch_swiglu(int dtype, const GemmOut& proj, void* out_t, int F, co
     const int gy = (3 * wide_sm_count() + (int)grid.x - 1) / (int)grid.x;
     grid.y = gy < m_max ? gy : m_max;
     const ChainSync cs = chain ? chain->link(grid.x * grid.y, true) : ChainSync{nullptr, 0u, nullptr, nullptr, nullptr};
-    RD_DISPATCH(dtype, launch_pdl(swiglu_wide_kernel<T>, grid, SWS_THREADS, smem, st, proj, (T*)out_t, F, m_total, status, cs));
+    launch_pdl(swiglu_wide_kernel<__nv_bfloat16>, grid, SWS_THREADS, smem, st, proj, (__nv_bfloat16*)out_t, F, m_total, status, cs);
     return cudaGetLastError();
   }
   const ChainSync cs = chain ? chain->link(grid.x * grid.y, true) : ChainSync{nullptr, 0u, nullptr, nullptr, nullptr};
-  RD_DISPATCH(dtype, launch_pdl(swiglu_kernel<T>, grid, SWIGLU_THREADS, 0, st, proj, (T*)out_t, F, m_total, cs));
+  launch_pdl(swiglu_kernel<__nv_bfloat16>, grid, SWIGLU_THREADS, 0, st, proj, (__nv_bfloat16*)out_t, F, m_total, cs);
   return cudaGetLastError();
 }
 

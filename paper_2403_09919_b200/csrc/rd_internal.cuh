@@ -50,9 +50,35 @@ struct Dims {
 };
 
 // ---- launchers (definitions in the .cu files; all enqueue on `st`, return cudaGetLastError) ----
-// Y[m][n] = sum_k A[m][k] W[n][k], M rows given by *m_total (<= m_max), on CUDA cores.  Fills *out_desc.
-cudaError_t launch_gemm_simt(int dtype, const void* A, int lda, const void* W, int N, int K, const int32_t* m_total,
-                             int m_max, float* raw, int ld_raw, GemmOut* out_desc, cudaStream_t st);
+// CUDA-core projection with the function behind it (gemm_simt.cu).  M rows are given by *m_total (<= m_max).
+struct SimtOperands {
+  const void* A;          // [M][lda] activations in the storage type; with norm_gain: the fp32 residual stream
+  int lda;
+  const void* norm_gain;  // RMSNorm in front of the projection (K <= simt_norm_max_k()), or nullptr
+  float eps;
+  const void* W;          // [N][K]
+  int K;
+  int items;              // weight rows, or pairs of them (SIMT_ROPE: half heads of Q, K and V; SIMT_SWIGLU: F)
+  const int32_t* m_total;
+};
+enum { SIMT_RAW = 0, SIMT_RESIDUAL = 1, SIMT_SWIGLU = 2, SIMT_ACT = 3, SIMT_ROPE = 4 };
+struct SimtEpilogue {
+  float* out_f;           // RAW, ACT: [M][ld]; RESIDUAL: [M][ld], added to; ROPE: [M][3d], Q written
+  int ld;
+  void* out_t;            // SWIGLU: [M][F]; ACT: [M][ld]
+  int F;
+  const void* bias;       // ACT
+  const float* resid;     // ACT: [M][ld_resid] or nullptr
+  int ld_resid;
+  void *kcache, *vcache;  // ROPE
+  const float2* table;
+  const int32_t *seq, *slot;
+  int32_t* status;
+};
+int simt_norm_max_k();
+GemmOut simt_out(float* raw, int ld);   // the description of a complete [M][ld] buffer
+cudaError_t launch_gemm_simt(int dtype, int epi, const SimtOperands& p, const SimtEpilogue& e, const Dims& dm, int m_max, Chain* chain,
+                             cudaStream_t st);
 
 // Tensor-core (tcgen05) projection, bf16 only.  Operands are passed as TMA descriptors.
 int tc_make_map(void* out_map, const void* ptr, uint64_t rows, uint64_t cols, uint32_t box_rows);
@@ -70,10 +96,10 @@ cudaError_t launch_embed_rope(int dtype, const void* emb, const int32_t* tok, co
                               int hd, float theta, const int32_t* m_total, int m_max, int* status, cudaStream_t st);
 cudaError_t launch_rmsnorm(int dtype, float* x, const GemmOut* proj, const void* gain, void* out_t, float* out_f32, int d,
                            float eps, const int32_t* m_total, int m_max, Chain* chain, cudaStream_t st);
-cudaError_t launch_rope_kv(int dtype, float* qkv, const GemmOut& proj, void* kcache, void* vcache, const float* table,
+cudaError_t launch_rope_kv(float* qkv, const GemmOut& proj, void* kcache, void* vcache, const float* table,
                            const RowTables& rt, const Dims& dm, int m_max, int* status, Chain* chain, cudaStream_t st);
 cudaError_t launch_attention(int dtype, const float* qkv, const void* kcache, const void* vcache, void* out_t,
-                             const RowTables& rt, const Dims& dm, int m_max, cudaStream_t st);
+                             const RowTables& rt, const Dims& dm, int m_max, Chain* chain, cudaStream_t st);
 // Tensor-core attention (bf16): KV tiles staged through shared memory, split over the keys.
 size_t attn_tc_scratch_floats(int blocks, int n_splits, int hd);
 // many rows per sequence (prompts, wide beams, large batches): tiles of 64 rows, a warp per 16 of them
@@ -93,9 +119,9 @@ cudaError_t attn_tc_prepare(int hd, int MW);
 cudaError_t launch_attention_tc(const float* qkv, const void* kcache, const void* vcache, void* out, const RowTables& rt,
                                 const int32_t* seq_off, const Dims& dm, int n_seq, int row_blocks, int n_splits,
                                 float* scratch, int32_t* counters, unsigned long long* dbg, Chain* chain, int shallow, cudaStream_t st);
-cudaError_t elementwise_prepare(int dtype);
+cudaError_t elementwise_prepare();
 cudaError_t drafter_prepare(int dtype);
-cudaError_t launch_swiglu(int dtype, const GemmOut& proj, void* out_t, int F, const int32_t* m_total, int m_max,
+cudaError_t launch_swiglu(const GemmOut& proj, void* out_t, int F, const int32_t* m_total, int m_max,
                           int32_t* status, Chain* chain, cudaStream_t st);
 // Token choice at temperature > 0: inv_t = 1 / temperature (0: greedy), (k0, k1) the seed's two halves.
 struct Sampling {
@@ -109,7 +135,7 @@ cudaError_t launch_argmax_rows(float* logits, const GemmOut& proj, int V, int32_
 // drafter
 cudaError_t launch_draft_init(int dtype, const void* emb, const int32_t* root, const float* h, void* xc_t, float* xc_f, void* x0_t,
                               float* x0_f, void* se_t, const Dims& dm, int B, int* status, cudaStream_t st);
-cudaError_t launch_act(int dtype, const GemmOut& proj, const void* bias, const float* resid, int ld_resid, float* out_f,
+cudaError_t launch_act(const GemmOut& proj, const void* bias, const float* resid, int ld_resid, float* out_f,
                        void* out_t, int ld_out, int N, const int32_t* m_total, int m_max, Chain* chain, cudaStream_t st);
 // Scratch of the two-kernel selection (seg_max == nullptr: single-kernel selection only).
 struct SelectScratch {

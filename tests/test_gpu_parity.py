@@ -131,6 +131,36 @@ def test_verify_logits_and_argmax(rig):
     assert np.abs(kvg - kv.k[:, ctx:ctx + n]).max() < TOL_FP32
 
 
+@pytest.mark.parametrize("d,heads,d_ffn,vocab,bw,L", [(64, 1, 4, 36, 1, 1), (192, 3, 172, 100, 2, 3), (512, 4, 516, 260, 3, 3), (576, 9, 1028, 132, 1, 2),
+                                                      (1152, 9, 1156, 200, 9, 2)])
+def test_cuda_core_projections_at_the_edges_of_their_chunks(d, heads, d_ffn, vocab, bw, L):
+    """Rows of one 512-column chunk and of several (with a remainder), the norm in front of a projection taken along (d up
+    to 512) or not, groups of 2, 4 and 8 rows with rows missing, both head dimensions: prompt, drafter and verification."""
+    cfg = dict(synth.CONFIGS["tiny"], d_model=d, n_heads=heads, d_rnn=d, d_ffn=d_ffn, vocab=vocab, beam_width=bw, beam_length=L, max_ctx=160)
+    r = Rig(cfg=cfg)
+    prompt = np.random.default_rng(3).integers(0, vocab, size=67)
+    r.eng.prefill([prompt])
+    kv = r.new_kv()
+    ctx, g, h = ora.prefill(r.W, cfg, prompt, kv)
+    c_ctx, c_root, c_h = r.eng.get_state()
+    assert int(c_ctx[0]) == ctx and np.abs(c_h[0].cpu().numpy() - h).max() < TOL_FP32
+    r.eng.set_state(None, dev([g]), dev(np.asarray(h, dtype=np.float32)[None], torch.float32))
+    beams, scores = r.eng.draft()
+    for b, s in zip(beams[0].cpu().numpy(), scores[0].cpu().numpy()):
+        assert abs(ora.sequence_logprob(r.D, r.W["tok_emb"], g, h, b) - s) < TOL_FP32
+    planted = np.random.default_rng(6).integers(0, 3, size=(1, bw, L))
+    pk = r.eng.pack(dev(planted))
+    argmax, hidden, logits = r.eng.verify(pk, want_logits=True)
+    r.eng.poll()
+    p = ora.pack_beam(np.concatenate([np.full((bw, 1), g), planted[0]], axis=1), ctx)
+    rh, rl = ora.llm_forward(r.W, cfg, p["tokens"], p["pos"], p["mask"], kv, ctx)
+    assert np.abs(logits[0, :p["n"]].cpu().numpy() - rl).max() < TOL_FP32
+    assert np.abs(hidden[0, :p["n"]].cpu().numpy() - rh).max() < TOL_FP32
+    kvg = r.eng.kv_view()[:, :, 0, :, :ctx + p["n"]].cpu().numpy().transpose(1, 0, 3, 2, 4)
+    assert np.abs(kvg[0] - kv.k[:, :ctx + p["n"]]).max() < TOL_FP32 and np.abs(kvg[1] - kv.v[:, :ctx + p["n"]]).max() < TOL_FP32
+    r.eng.close()
+
+
 def test_draft_beams_and_scores(rig):
     prompt, kv, ctx, g, h = prefilled(rig)
     beams, scores = rig.eng.draft()
