@@ -97,6 +97,7 @@ struct rd_handle {
   int tc_pairs;   // CTA pairs of the pair projection kernel that fit the device at once (0: not used)
   int tc_pairs_avail, tc_pairs_min_rows;   // the pairs the device offers; row bound from which launches use them
   bool tc_pairs_prefill;
+  int swiglu_min_rows;   // row bound from which gate|up takes SwiGLU along (0: use_fused_swiglu's own)
   std::vector<TensorMapBox> kv_maps;   // [layer][K | V]: cache planes as [sequences * heads * max_ctx][head dim] matrices
   Chain chain;  // counter hand-off between the launches of a forward pass
   bool chain_dirty;  // a launch failed after the chain had counted it: reset the counters before the next pass
@@ -111,6 +112,7 @@ struct rd_handle {
   int fb_next;
   unsigned fb_calls;         // a copy is enqueued on every eighth call: the bound lags by at most 8 (1 + L) tokens
   std::unordered_map<const void*, TensorMapBox> maps;               // weights
+  std::unordered_map<const void*, TensorMapBox> maps64;             // gate|up weights in boxes of half a tile (fused SwiGLU)
   std::unordered_map<const void*, std::pair<int, int>> act_shape;   // activation buffers: rows, cols
   std::map<std::pair<const void*, int>, TensorMapBox> act_maps;     // by (buffer, rows per box), made on first use
   // optional per-launch timing of the projections (class 0) and the attention kernel (class 1)
@@ -276,46 +278,56 @@ struct ProfScope {
     CK(h, expr);                       \
   } while (0)
 
+// Activation descriptors of buffer A: box heights step, 2 step, ..., one per 16 rows of a row tile of mt; made on first use.
+int act_maps_of(rd_handle* h, const void* A, int K, int mt, int step, const void* (&out)[16]) {
+  auto is = h->act_shape.find(A);
+  if (is == h->act_shape.end() || is->second.second != K) return fail(h, RD_ERR_STATE, "projection operand without a TMA descriptor");
+  for (int i = 0; i < 16; ++i) {
+    out[i] = nullptr;
+    if (i >= mt / 16) continue;
+    const int box_rows = step * (i + 1);
+    auto key = std::make_pair(A, box_rows);
+    auto ia = h->act_maps.find(key);
+    if (ia == h->act_maps.end()) {
+      TensorMapBox box;
+      box.rows = is->second.first; box.cols = K;
+      const int rc = tc_make_map(&box, A, (uint64_t)box.rows, (uint64_t)K, (uint32_t)box_rows);
+      if (rc) return fail(h, RD_ERR_CUDA, "cuTensorMapEncodeTiled failed with %d for an activation buffer", rc);
+      ia = h->act_maps.emplace(key, box).first;
+    }
+    out[i] = &ia->second;
+  }
+  return RD_OK;
+}
+
+// The next trace slot for a projection of that many weight bytes, or nullptr when tracing is off.
+unsigned long long* gemm_trace_slot(rd_handle* h, double bytes, int* slot) {
+  *slot = -1;
+  if (h->trace_next < 0 || h->trace_next >= TRACE_SLOTS) return nullptr;
+  if ((int)h->trace_bytes.size() < TRACE_SLOTS) h->trace_bytes.assign(TRACE_SLOTS, 0.0);
+  if ((int)h->trace_prefetch.size() < TRACE_SLOTS) h->trace_prefetch.assign(TRACE_SLOTS, 0.0);
+  h->trace_bytes[h->trace_next] = bytes;
+  *slot = h->trace_next;
+  return h->ws.trace + (size_t)8 * h->trace_next++;
+}
+
 // One projection Y = A W^T into the fp32 buffer `raw` (row stride ld_raw); fills `out` for the consumer.
 int gemm(rd_handle* h, const void* A, int lda, const void* W, int N, int K, const int32_t* m_total, int m_max, float* raw,
          int ld_raw, GemmOut* out, Chain* chain, cudaStream_t st, int pair = 0) {
   ProfScope ps(h, 0, (double)N * K * esize(h->dm.dtype), st);
   if (h->use_tc) {
     auto iw = h->maps.find(W);
-    auto is = h->act_shape.find(A);
-    if (iw == h->maps.end() || is == h->act_shape.end() || lda != K || is->second.second != K)
+    if (iw == h->maps.end() || lda != K)
       return fail(h, RD_ERR_STATE, "projection operand without a TMA descriptor");
     const int mt = tc_pick_mt(m_max > 0 ? m_max : 1);
     // activation descriptors: box heights 16..mt in steps of 16 (a launch that has a single row tile picks by the
     // actual row count); made on first use
-    const void* amaps[16] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr,
-                             nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
+    const void* amaps[16];
     // (on CTA pairs each CTA loads half a row tile: heights 8..mt/2 in steps of 8)
     const int pairs = tc_use_pairs(m_max, N, h->tc_grid, h->tc_pairs, h->tc_pairs_min_rows) ? h->tc_pairs : 0;
-    const int box_step = pairs ? 8 : 16;
-    const int n_maps = mt / 16;
-    for (int i = 0; i < n_maps; ++i) {
-      const int box_rows = box_step * (i + 1);
-      auto key = std::make_pair(A, box_rows);
-      auto ia = h->act_maps.find(key);
-      if (ia == h->act_maps.end()) {
-        TensorMapBox box;
-        box.rows = is->second.first; box.cols = K;
-        const int rc = tc_make_map(&box, A, (uint64_t)box.rows, (uint64_t)K, (uint32_t)box_rows);
-        if (rc) return fail(h, RD_ERR_CUDA, "cuTensorMapEncodeTiled failed with %d for an activation buffer", rc);
-        ia = h->act_maps.emplace(key, box).first;
-      }
-      amaps[i] = &ia->second;
-    }
-    unsigned long long* tr = nullptr;
+    if (int rc = act_maps_of(h, A, K, mt, pairs ? 8 : 16, amaps)) return rc;
     int tr_slot = -1;
-    if (h->trace_next >= 0 && h->trace_next < TRACE_SLOTS) {
-      if ((int)h->trace_bytes.size() < TRACE_SLOTS) h->trace_bytes.assign(TRACE_SLOTS, 0.0);
-      if ((int)h->trace_prefetch.size() < TRACE_SLOTS) h->trace_prefetch.assign(TRACE_SLOTS, 0.0);
-      h->trace_bytes[h->trace_next] = (double)N * K * esize(h->dm.dtype);
-      tr_slot = h->trace_next;
-      tr = h->ws.trace + (size_t)8 * h->trace_next++;
-    }
+    unsigned long long* tr = gemm_trace_slot(h, (double)N * K * esize(h->dm.dtype), &tr_slot);
     CK(h, launch_gemm_tc(&iw->second, amaps, N, K, m_total, m_max, raw, ld_raw, h->ws.tc_partial, h->ws.status,
                          h->tc_grid, pairs, h->tc_smem, tr, out, chain, pair, st));
     if (tr_slot >= 0) h->trace_prefetch[tr_slot] = tc_last_prefetch_bytes();
@@ -327,6 +339,34 @@ int gemm(rd_handle* h, const void* A, int lda, const void* W, int N, int K, cons
   h->route[RD_ROUTE_GEMM_SIMT]++;
   CK(h, launch_gemm_simt(h->dm.dtype, SIMT_RAW, SimtOperands{A, lda, nullptr, 0.f, W, K, N, m_total}, e, h->dm, m_max, chain, st));
   *out = simt_out(raw, ld_raw);
+  return RD_OK;
+}
+
+// Whether a pass bounded by m_max rows takes the gate|up projection with SwiGLU in its epilogue.  Measured against the
+// two kernels: prompt passes, whose bound is their row count, win from about 350 rows (8 layers of the 7B shape: 264 rows
+// 1548 -> 1584 us, 320 1581 -> 1596, 400 1824 -> 1721, 500 2110 -> 1944; 13B 300 rows 1660 -> 1553); a verification pass
+// brings about half of its bound (7B: bound 328 6.77 -> 7.04 ms, 644 2958 -> 2939 us at 312 rows, 656 4190 -> 3782 at
+// 529; 33B, 644: 17.1 -> 16.2 ms; 7B batch 16, 1296: 19.1 -> 17.6 ms).
+bool use_fused_swiglu(const rd_handle* h, int m_max, bool exact) {
+  const int min_rows = h->swiglu_min_rows > 0 ? h->swiglu_min_rows : exact ? 352 : 512;
+  return m_max >= min_rows && h->dm.F % 2 == 0 && tc_use_pairs(m_max, 2 * h->dm.F, h->tc_grid, h->tc_pairs_avail, 0);
+}
+
+// act = SwiGLU of the gate|up projection of A (tensor cores, CTA pairs).
+int gemm_swiglu(rd_handle* h, const void* A, const void* W, int m_max, void* act, Chain* chain, cudaStream_t st) {
+  const Dims& dm = h->dm;
+  const double bytes = 2.0 * dm.F * dm.d * esize(dm.dtype);
+  ProfScope ps(h, 0, bytes, st);
+  auto iw = h->maps64.find(W);
+  if (iw == h->maps64.end()) return fail(h, RD_ERR_STATE, "projection operand without a TMA descriptor");
+  const void* amaps[16];
+  if (int rc = act_maps_of(h, A, dm.d, tc_pick_mt(m_max), 8, amaps)) return rc;
+  int tr_slot = -1;
+  unsigned long long* tr = gemm_trace_slot(h, bytes, &tr_slot);
+  const int pairs = h->tc_pairs_avail < h->tc_grid / 2 ? h->tc_pairs_avail : h->tc_grid / 2;
+  CK(h, launch_gemm_swiglu(&iw->second, amaps, dm.F, dm.d, h->ws.m_total, m_max, act, h->ws.status, pairs, h->tc_smem, tr, chain, st));
+  if (tr_slot >= 0) h->trace_prefetch[tr_slot] = tc_last_prefetch_bytes();
+  h->route[RD_ROUTE_GEMM_PAIRS]++;
   return RD_OK;
 }
 
@@ -482,6 +522,7 @@ int forward_layers(rd_handle* h, const uint32_t* mask, int m_max, int n_seq, int
     h->chain.cut();
     return RD_OK;
   }
+  const bool fused_swiglu = use_fused_swiglu(h, m_max, mask == nullptr);
   for (int l = 0; l < dm.n_layers; ++l) {
     // attention block: (x += down of the previous layer) -> norm -> QKV -> rotary + KV write -> attention -> O
     CKP(h, PROF_NORM, launch_rmsnorm(dm.dtype, w.x, l ? &g_dn : nullptr, h->attn_norm[l], w.a_t, nullptr, dm.d, dm.eps,
@@ -511,9 +552,14 @@ int forward_layers(rd_handle* h, const uint32_t* mask, int m_max, int n_seq, int
     if (rc) return rc;
     // FFN block: (x += O) -> norm -> gate|up -> SwiGLU -> down
     CKP(h, PROF_NORM, launch_rmsnorm(dm.dtype, w.x, &g_o, h->ffn_norm[l], w.a_t, nullptr, dm.d, dm.eps, w.m_total, m_max, ch, st));
-    rc = gemm(h, w.a_t, dm.d, h->w_gate_up[l], 2 * dm.F, dm.d, w.m_total, m_max, w.gu, 2 * dm.F, &g_gu, ch, st, /*pair=*/1);
-    if (rc) return rc;
-    CKP(h, PROF_SWIGLU, launch_swiglu(g_gu, w.act_t, dm.F, w.m_total, m_max, w.status, ch, st));
+    if (fused_swiglu) {
+      rc = gemm_swiglu(h, w.a_t, h->w_gate_up[l], m_max, w.act_t, ch, st);
+      if (rc) return rc;
+    } else {
+      rc = gemm(h, w.a_t, dm.d, h->w_gate_up[l], 2 * dm.F, dm.d, w.m_total, m_max, w.gu, 2 * dm.F, &g_gu, ch, st, /*pair=*/1);
+      if (rc) return rc;
+      CKP(h, PROF_SWIGLU, launch_swiglu(g_gu, w.act_t, dm.F, w.m_total, m_max, w.status, ch, st));
+    }
     rc = gemm(h, w.act_t, dm.F, h->w_down[l], dm.d, dm.F, w.m_total, m_max, w.proj_d, dm.d, &g_dn, ch, st, /*pair=*/1);
     if (rc) return rc;
   }
@@ -674,7 +720,7 @@ int redrafter_init(const rd_config* cfg, const rd_weights* wt, void* kv_cache, s
     if (ce == cudaSuccess) ce = drafter_prepare(dm.dtype);
     if (ce != cudaSuccess) return init_fail(h, RD_ERR_CUDA, "kernel set-up: %s", cudaGetErrorString(ce));
   }
-  h->tc_pairs = 0; h->tc_pairs_avail = 0; h->tc_pairs_min_rows = 1024; h->tc_pairs_prefill = false;
+  h->tc_pairs = 0; h->tc_pairs_avail = 0; h->tc_pairs_min_rows = 512; h->tc_pairs_prefill = false;
   int sms = 0;
   {
     int dev = 0;
@@ -690,12 +736,13 @@ int redrafter_init(const rd_config* cfg, const rd_weights* wt, void* kv_cache, s
     if (ce == cudaSuccess) ce = attn_t5_prepare(dm.hd, dm.MW);
     if (ce != cudaSuccess)
       return init_fail(h, RD_ERR_CUDA, "tensor-core path set-up: %s", cudaGetErrorString(ce));
-    // CTA-pair projections (tuning toggles, read when the handle is made): from a bound of 1024 rows in decode steps
-    // (measured: 1-4 % of the step from about 650 packed rows; with bounds around 650 rows, 300-420 rows present, the
-    // one-CTA kernel, which starts earlier and has shorter tails, is 3-5 % ahead); RD_TC_CTA2=0 never, RD_TC_CTA2_MIN the row bound, RD_TC_CTA2_PREFILL=1 also in prompt passes.
+    // CTA-pair projections (tuning toggles, read when the handle is made): from a bound of 512 rows in decode steps
+    // (8 layers of the 7B shape, one-CTA kernel against pairs: 312 rows 2939 / 2967 us, 435 3157 / 3088, 529 3782 / 3764,
+    // 674 4631 / 4468; 33B with 287 rows 16.2 / 15.8 ms; smaller bounds bring too few rows for the pairs' later start); RD_TC_CTA2=0 never, RD_TC_CTA2_MIN the row bound, RD_TC_CTA2_PREFILL=1 also in prompt passes.
     if (getenv("RD_TC_CTA2") && atoi(getenv("RD_TC_CTA2")) == 0) h->tc_pairs_avail = 0;
-    h->tc_pairs_min_rows = getenv("RD_TC_CTA2_MIN") ? atoi(getenv("RD_TC_CTA2_MIN")) : 1024;
+    h->tc_pairs_min_rows = getenv("RD_TC_CTA2_MIN") ? atoi(getenv("RD_TC_CTA2_MIN")) : 512;
     h->tc_pairs_prefill = getenv("RD_TC_CTA2_PREFILL") && atoi(getenv("RD_TC_CTA2_PREFILL")) != 0;
+    h->swiglu_min_rows = getenv("RD_SWIGLU_MIN") ? atoi(getenv("RD_SWIGLU_MIN")) : 0;   // tuning toggle, as those above
     h->tc_pairs = h->tc_pairs_avail;
     if (attn_t5_supported(dm.hd)) {
       // The tensor-core attention multiplies masked-out V rows by exact zeros: the cache has to hold finite values.
@@ -711,17 +758,17 @@ int redrafter_init(const rd_config* cfg, const rd_weights* wt, void* kv_cache, s
     bool ok = true;
     int failed_rc = 0;
     const void* failed_ptr = nullptr;
-    auto add_w = [&](const void* p, int N, int K) {
+    auto add_w = [&](const void* p, int N, int K, bool half = false) {
       if (!ok) return;
-      TensorMapBox& box = h->maps[p];
+      TensorMapBox& box = half ? h->maps64[p] : h->maps[p];
       box.rows = N; box.cols = K;
-      failed_rc = tc_make_map(&box, p, (uint64_t)N, (uint64_t)K, (uint32_t)tc_weight_box_rows());
+      failed_rc = tc_make_map(&box, p, (uint64_t)N, (uint64_t)K, (uint32_t)(half ? tc_weight_box_rows() / 2 : tc_weight_box_rows()));
       if (failed_rc) { ok = false; failed_ptr = p; }
     };
     auto add_a = [&](const void* p, int rows, int K) { h->act_shape[p] = std::make_pair(rows, K); };
     for (int l = 0; l < dm.n_layers; ++l) {
       add_w(h->wqkv[l], 3 * dm.d, dm.d); add_w(h->wo[l], dm.d, dm.d);
-      add_w(h->w_gate_up[l], 2 * dm.F, dm.d); add_w(h->w_down[l], dm.d, dm.F);
+      add_w(h->w_gate_up[l], 2 * dm.F, dm.d); add_w(h->w_gate_up[l], 2 * dm.F, dm.d, /*half=*/true); add_w(h->w_down[l], dm.d, dm.F);
     }
     add_w(wt->lm_head, dm.V, dm.d); add_w(h->ws.uw, dm.dr, dm.dr + dm.d);
     for (int l = 0; l < dm.n_head_layers; ++l) add_w(h->head_w[l], dm.dh, dm.dh);
@@ -860,8 +907,8 @@ int redrafter_prefill(rd_handle* h, const int32_t* tokens, const int32_t* prompt
     CKRT(h, cudaMemcpyAsync(w.m_total, &m, sizeof(int32_t), cudaMemcpyHostToDevice, st));
     CKRT(h, cudaStreamSynchronize(st));  // the host staging vectors are reused by the next pass
     h->ctx_bound = longest;  // bound of the key extent for this pass
-    // Prompt passes keep the one-CTA projection: their rows fill 256-row tiles exactly, projection plus consumer
-    // take the same time with either kernel (the fp32 intermediate bounds the pair), and the CTA pairs start later.
+    // Prompt passes keep the one-CTA projection for QKV, O and down: projection plus consumer take the same time with
+    // either kernel (the fp32 intermediate bounds the pair), and the CTA pairs start later.
     if (!h->tc_pairs_prefill) h->tc_pairs = 0;
     rc = forward_layers(h, nullptr, m, batch, longest_run, nullptr, st);
     h->tc_pairs = h->tc_pairs_avail;

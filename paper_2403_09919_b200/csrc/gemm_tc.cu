@@ -73,6 +73,7 @@ struct TcParams {
   // 1: a unit is (pair of adjacent weight tiles, k-block): both tiles of a stage are multiplied by ONE activation
   // box, which halves what the activation operand costs an SM.  Single row tile only.
   int pair;
+  __nv_bfloat16* act;   // SwiGLU output [M][N] of the fused gate|up projection (N: features)
 };
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -515,7 +516,30 @@ __device__ __forceinline__ void umma_commit_pair(uint32_t cluster_bar) {
   asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(cluster_bar) : "memory");
 }
 
-template <int EW>
+constexpr uint32_t SWAP_BYTES = 2 * 2 * 2 * 8 * 64 * 4;
+// Row tiles of a SwiGLU launch: whole tiles run in waves of n_clusters, so the fewest waves times the cost of a tile win
+// (a tile's k-block costs its rows, and 64 rows' worth for its share of the weights).
+__device__ __forceinline__ GemmRows swiglu_row_tiles(int M, int mt, int n_wt, int n_clusters) {
+  GemmRows best;
+  int cost = 0x7fffffff;
+  const int n0 = max(1, (M + mt - 1) / mt);
+  for (int n = n0; n < n0 + 4; ++n) {
+    const int rows = min(mt, max(16, ((M + n - 1) / n + 15) & ~15));
+    const int c = (n_wt * n + n_clusters - 1) / n_clusters * (rows + 64);
+    if (c < cost) { cost = c; best = GemmRows(n, rows); }
+  }
+  return best;
+}
+
+// SWIGLU: the gate|up projection with SwiGLU in its epilogue, for launches of many rows.  A weight tile is 64 gate rows and
+// the 64 up rows that belong to them, so lanes i and i + 64 of an accumulator hold a feature's two sums; the epilogue warps
+// of the two halves swap eight columns each through shared memory and write SiLU(gate) * up as bf16.  Tiles are not cut:
+// cluster c takes tiles c, c + C, ... of the (weight tile, row tile) list, row tile fastest, so the row tiles of a weight
+// tile run side by side; what whole tiles leave idle in the last wave is kept small by the choice of row tile
+// (swiglu_row_tiles).  The two-kernel form writes the sums as fp32 and reads them back (90 MB at 1024 rows of the 7B
+// shape, more than the L2 keeps, and the kernel between them): 133 + 4 + 34 us per layer there, now 140; a 512-token prompt
+// 9.21 -> 8.54 ms, 8192 tokens 153 -> 141 ms, the batch-16 step 19.1 -> 17.6 ms.
+template <int EW, bool SWIGLU>
 __global__ void __launch_bounds__(tc_threads(EW), EW == 4 ? 4 : 2) gemm_tc2_kernel(const __grid_constant__ CUtensorMap map_w,
                                                                   const __grid_constant__ ActMaps maps_a,   // box heights 8, 16, ..., 128
                                                                   const TcParams p) {
@@ -527,20 +551,25 @@ __global__ void __launch_bounds__(tc_threads(EW), EW == 4 ? 4 : 2) gemm_tc2_kern
   const uint32_t rank = cluster_ctarank();        // 0: leader (issues the MMAs), 1: peer
   const uint32_t cluster = cluster_id_x();
   const bool chained = p.cs.signal_ptr != nullptr;
-  const bool early = (p.m_tiles_max == 1) || chained;
+  const bool early = (!SWIGLU && p.m_tiles_max == 1) || chained;   // (SWIGLU splits by the row count)
   if (!early) {
     if (threadIdx.x == 0) chain_wait_thread(p.cs);
     __syncthreads();
   }
   GemmRows rows(1, p.mt);
-  if (p.m_tiles_max > 1) rows = gemm_row_tiles(p.mt, p.m_tiles_max, *p.m_total);
+  if (SWIGLU) rows = swiglu_row_tiles(*p.m_total, p.mt, (p.n_tiles + 1) / 2, gridDim.x >> 1);
+  else if (p.m_tiles_max > 1) rows = gemm_row_tiles(p.mt, p.m_tiles_max, *p.m_total);
   else if (chained) rows.rows = min(p.mt, max(16, (*p.m_total + 15) & ~15));
   const int m_tiles = rows.n;
   const int n_wt = (p.n_tiles + 1) / 2;           // pairs of weight tiles
   const int n_groups = n_wt * m_tiles;
-  const long long U = (long long)n_groups * p.nkb, C = gemm_working<long long>(U, gridDim.x >> 1);   // clusters that work
+  const int n_clusters = gridDim.x >> 1;
+  const long long U = (long long)n_groups * p.nkb, C = SWIGLU ? n_clusters : gemm_working<long long>(U, n_clusters);   // clusters that work
   const bool works = cluster < C;
-  const long long u0 = works ? gemm_range_begin(cluster, U, C) : U, u1 = works ? gemm_range_begin(cluster + 1, U, C) : U;
+  // SWIGLU: units of this cluster's own list of whole tiles, cluster + i * C
+  const int my_tiles = (int)cluster < n_groups ? (n_groups - 1 - (int)cluster) / n_clusters + 1 : 0;
+  const long long u0 = SWIGLU ? 0 : works ? gemm_range_begin(cluster, U, C) : U;
+  const long long u1 = SWIGLU ? (long long)my_tiles * p.nkb : works ? gemm_range_begin(cluster + 1, U, C) : U;
   const int mt_eff = rows.rows, half = mt_eff >> 1;   // rows of a row tile; rows of it this CTA loads
   const CUtensorMap* map_a = &maps_a.m[(half >> 3) - 1];
 
@@ -549,7 +578,9 @@ __global__ void __launch_bounds__(tc_threads(EW), EW == 4 ? 4 : 2) gemm_tc2_kern
   const uint32_t a_stage_bytes = (uint32_t)(p.mt >> 1) * TILE_K * 2;   // reserved
   const uint32_t stage_bytes = (uint32_t)W_STAGE_BYTES + a_stage_bytes;
   const uint32_t tx_bytes = 2u * ((uint32_t)W_STAGE_BYTES + (uint32_t)half * TILE_K * 2);   // both CTAs' copies of a stage
-  const uint32_t bar_base = base + p.stages * stage_bytes;
+  const uint32_t swap_bytes = SWIGLU ? SWAP_BYTES : 0u;
+  const uint32_t bar_base = base + p.stages * stage_bytes + swap_bytes;
+  float* swap = reinterpret_cast<float*>(smem_raw + (bar_base - swap_bytes - raw));   // [column group][2][8 columns of gate | of up][64]
   auto full_bar = [&](int s) { return bar_base + 8u * s; };
   auto empty_bar = [&](int s) { return bar_base + 8u * (p.stages + s); };
   auto tfull_bar = [&](int a) { return bar_base + 8u * (2 * p.stages + a); };
@@ -563,28 +594,46 @@ __global__ void __launch_bounds__(tc_threads(EW), EW == 4 ? 4 : 2) gemm_tc2_kern
   const uint32_t pre = early ? min(n_it, (uint32_t)p.stages) : 0u;
   const uint64_t pol_w = l2_policy_evict_first();
   struct UnitPos {
-    int g, m_tile, kb;
+    int g, m_tile, kb, t;
     uint32_t s, ph;
+  };
+  // weight tile pair and row tile of the i-th tile (SWIGLU: of this cluster's list)
+  auto tile_at = [&](int i, int& g, int& m_tile) {
+    if (SWIGLU) {
+      const int t = (int)cluster + i * n_clusters;
+      g = t / m_tiles;
+      m_tile = t - g * m_tiles;
+    } else {
+      m_tile = i / n_wt;
+      g = i - m_tile * n_wt;
+    }
   };
   auto pos_at = [&](long long u) {
     UnitPos q;
-    const int t = (int)(u / p.nkb);
-    q.kb = (int)(u - (long long)t * p.nkb);
-    q.m_tile = t / n_wt;
-    q.g = t - q.m_tile * n_wt;
+    q.t = (int)(u / p.nkb);
+    q.kb = (int)(u - (long long)q.t * p.nkb);
+    tile_at(q.t, q.g, q.m_tile);
     q.s = 0; q.ph = 0;
     return q;
   };
   auto advance = [&](UnitPos& q) {
     if (++q.kb == p.nkb) {
       q.kb = 0;
-      if (++q.g == n_wt) { q.g = 0; ++q.m_tile; }
+      if (SWIGLU) tile_at(++q.t, q.g, q.m_tile);   // one division per tile
+      else if (++q.g == n_wt) { q.g = 0; ++q.m_tile; }
     }
     if (++q.s == (uint32_t)p.stages) { q.s = 0; q.ph ^= 1u; }
   };
   // the bytes of both CTAs are counted on the leader's barrier; the leader announces them
   auto issue_w = [&](const UnitPos& q) {
     if (rank == 0) mbar_expect_tx(full_bar(q.s), tx_bytes);
+    if (SWIGLU) {   // 64 gate rows and their 64 up rows (what lies past them belongs to features that are not stored)
+      const uint32_t dst = base + q.s * stage_bytes, bar = map_to_cta(full_bar(q.s), 0);
+      const int f = (2 * q.g + (int)rank) * (TILE_N / 2);
+      tma_load_2d_pair_hint(dst, &map_w, bar, q.kb * TILE_K, f, pol_w);
+      tma_load_2d_pair_hint(dst + W_STAGE_BYTES / 2, &map_w, bar, q.kb * TILE_K, p.N + f, pol_w);
+      return;
+    }
     // tile 2g + rank (the odd one may lie past the matrix: the copy then delivers zeros)
     tma_load_2d_pair_hint(base + q.s * stage_bytes, &map_w, map_to_cta(full_bar(q.s), 0), q.kb * TILE_K,
                           (2 * q.g + (int)rank) * TILE_N, pol_w);
@@ -714,12 +763,13 @@ __global__ void __launch_bounds__(tc_threads(EW), EW == 4 ? 4 : 2) gemm_tc2_kern
     const int chunk_par = ((warp - 2) >> 2) & 1;
     constexpr int chunk_step = two_per_quarter ? 32 : 16;
     const uint32_t tempty_leader0 = map_to_cta(tempty_bar(0), 0), tempty_leader1 = map_to_cta(tempty_bar(1), 0);
-    uint32_t seg = 0;
+    uint32_t seg = 0, turn = 0;
     bool ok = true;
     for (long long u = u0; u < u1 && ok; ++seg) {
       const int t = (int)(u / p.nkb), kb0 = (int)(u - (long long)t * p.nkb);
       const int kb1 = (int)min((long long)p.nkb, kb0 + (u1 - u));
-      const int m_tile = t / n_wt, grp = t - m_tile * n_wt;
+      int m_tile, grp;
+      tile_at(t, grp, m_tile);
       const int m_base = m_tile * mt_eff;
       const int c_end = min(mt_eff, ((M - m_base) + 15) & ~15);
       const uint32_t a = seg & 1u, aph = (seg >> 1) & 1u;
@@ -727,14 +777,40 @@ __global__ void __launch_bounds__(tc_threads(EW), EW == 4 ? 4 : 2) gemm_tc2_kern
       epi_bar_sync<EW>();
       if (!*epi_ok) { ok = false; break; }
       tc_fence_after();
-      const int n = (2 * grp + (int)rank) * TILE_N + row;
+      const int n = (2 * grp + (int)rank) * (SWIGLU ? TILE_N / 2 : TILE_N) + (SWIGLU ? row & 63 : row);
       const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + a * (uint32_t)p.mt;
       // slot of the cluster: [tile 2g | tile 2g + 1], each [mt][128]
       float* my_partial = p.partial + ((size_t)cluster * 2 + rank) * (size_t)p.mt * TILE_N;
       for (int c0 = two_per_quarter ? 16 * chunk_par : 0; c0 < c_end; c0 += chunk_step) {
         uint32_t r[16];
         tmem_ld16(taddr + c0, r);
-        if (kb0 == 0) {
+        if constexpr (SWIGLU) {
+          // gate lanes keep columns 0..7 and get their up sums; up lanes keep 8..15 and get their gate sums
+          const bool gate = row < 64;
+          float* mine = swap + (((chunk_par * 2 + (int)turn) * 2 + (gate ? 0 : 1)) * 8) * 64 + (row & 63);
+          const float* other = swap + (((chunk_par * 2 + (int)turn) * 2 + (gate ? 1 : 0)) * 8) * 64 + (row & 63);
+          turn ^= 1u;   // two buffers: the barrier of the next round covers the reads of this one
+#pragma unroll
+          for (int j = 0; j < 8; ++j) mine[j * 64] = __uint_as_float(gate ? r[8 + j] : r[j]);
+          asm volatile("bar.sync %0, 128;" ::"r"(2 + chunk_par) : "memory");
+          float y[8];
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            const float o = other[j * 64];
+            y[j] = gate ? silu_f(__uint_as_float(r[j])) * o : silu_f(o) * __uint_as_float(r[8 + j]);
+          }
+          // neighbouring lanes hold neighbouring features: the even lane writes both for one row, the odd lane for the next
+          const bool odd = lane & 1;
+          const int m0 = m_base + c0 + (gate ? 0 : 8) + (odd ? 1 : 0);
+#pragma unroll
+          for (int j = 0; j < 8; j += 2) {
+            const float give = odd ? y[j] : y[j + 1], got = __shfl_xor_sync(0xffffffffu, give, 1);
+            const float lo = odd ? got : y[j], hi = odd ? y[j + 1] : got;
+            const int m = m0 + j, f = n & ~1;
+            if (m < M && f < p.N)   // the number of features is even
+              *reinterpret_cast<__nv_bfloat162*>(p.act + (size_t)m * p.N + f) = __floats2bfloat162_rn(lo, hi);
+          }
+        } else if (kb0 == 0) {
           if (n < p.N) {
 #pragma unroll
             for (int j = 0; j < 16; ++j) {
@@ -855,7 +931,8 @@ cudaError_t tc_prepare(int* smem_limit_out, int* pairs_out) {
   if (e == cudaSuccess) e = cudaFuncSetAttribute(gemm_tc_kernel<false, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(gemm_tc_kernel<true, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(gemm_tc_kernel<true, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(gemm_tc2_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(gemm_tc2_kernel<8, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(gemm_tc2_kernel<8, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
   if (smem_limit_out) *smem_limit_out = lim;
   if (pairs_out) {
     *pairs_out = 0;
@@ -872,7 +949,7 @@ cudaError_t tc_prepare(int* smem_limit_out, int* pairs_out) {
       cfg.attrs = attr;
       cfg.numAttrs = 1;
       int n = 0;
-      const cudaError_t oe = cudaOccupancyMaxActiveClusters(&n, gemm_tc2_kernel<8>, &cfg);
+      const cudaError_t oe = cudaOccupancyMaxActiveClusters(&n, gemm_tc2_kernel<8, false>, &cfg);
       if (oe == cudaSuccess) *pairs_out = n;
       else cudaGetLastError();
     }
@@ -924,7 +1001,34 @@ static cudaError_t launch_gemm_tc2(const void* map_w, const void* const map_a[16
   }
   ActMaps am;
   for (int i = 0; i < ACT_MAPS; ++i) am.m[i] = *(const CUtensorMap*)(map_a[i] ? map_a[i] : map_a[0]);
-  launch_pairs(first, gemm_tc2_kernel<8>, 2 * pairs, tc_threads(8), smem, st, *(const CUtensorMap*)map_w, am, p);
+  launch_pairs(first, gemm_tc2_kernel<8, false>, 2 * pairs, tc_threads(8), smem, st, *(const CUtensorMap*)map_w, am, p);
+  return cudaGetLastError();
+}
+
+// The gate|up projection with SwiGLU behind it on CTA pairs: act[m][f], f < F.  map_w: box of tc_weight_box_rows() / 2 rows.
+cudaError_t launch_gemm_swiglu(const void* map_w, const void* const map_a[16], int F, int K, const int32_t* m_total, int m_max, void* act,
+                               int32_t* status, int pairs, int smem_limit, unsigned long long* trace, Chain* chain, cudaStream_t st) {
+  TcParams p{};
+  p.N = F; p.K = K; p.nkb = (K + TILE_K - 1) / TILE_K; p.n_tiles = (2 * F + TILE_N - 1) / TILE_N;
+  p.mt = tc_pick_mt(m_max);
+  p.m_tiles_max = (m_max + p.mt - 1) / p.mt;
+  p.pair = 1;
+  const int stage_bytes = W_STAGE_BYTES + (p.mt / 2) * TILE_K * 2;
+  const int overhead = 1024 + (int)SWAP_BYTES + 8 * (2 * 16 + 4) + 64;
+  int stages = (smem_limit - overhead) / stage_bytes;
+  if (stages > 16) stages = 16;
+  if (stages < 2) return cudaErrorInvalidConfiguration;
+  p.stages = stages;
+  int cols = 32;
+  while (cols < 2 * p.mt) cols <<= 1;
+  p.tmem_cols = cols;
+  p.m_total = m_total; p.act = (__nv_bfloat16*)act; p.status = status; p.trace = trace;
+  const bool first = chain && chain->enabled && chain->prev_ptr == nullptr;
+  p.cs = chain ? chain->link((unsigned)(2 * pairs)) : ChainSync{nullptr, 0u, nullptr, status, nullptr};
+  g_last_prefetch_bytes = chain ? 2.0 * pairs * stages * W_STAGE_BYTES : 0.0;
+  ActMaps am;
+  for (int i = 0; i < ACT_MAPS; ++i) am.m[i] = *(const CUtensorMap*)(map_a[i] ? map_a[i] : map_a[0]);
+  launch_pairs(first, gemm_tc2_kernel<8, true>, 2 * pairs, tc_threads(8), (size_t)stages * stage_bytes + overhead, st, *(const CUtensorMap*)map_w, am, p);
   return cudaGetLastError();
 }
 

@@ -92,6 +92,9 @@ cudaError_t launch_gemm_tc(const void* map_w, const void* const map_a[16], int N
                            float* raw, int ld_raw, float* partial, int32_t* status, int grid, int pairs, int smem_limit,
                            unsigned long long* trace, GemmOut* out_desc, Chain* chain, int pair, cudaStream_t st);
 
+cudaError_t launch_gemm_swiglu(const void* map_w, const void* const map_a[16], int F, int K, const int32_t* m_total, int m_max, void* act,
+                               int32_t* status, int pairs, int smem_limit, unsigned long long* trace, Chain* chain, cudaStream_t st);
+
 cudaError_t launch_embed_rope(int dtype, const void* emb, const int32_t* tok, const int32_t* pos, float* x, float* table, int d, int V,
                               int hd, float theta, const int32_t* m_total, int m_max, int* status, cudaStream_t st);
 cudaError_t launch_rmsnorm(int dtype, float* x, const GemmOut* proj, const void* gain, void* out_t, float* out_f32, int d,

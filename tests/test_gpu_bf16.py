@@ -398,6 +398,32 @@ def test_projection_on_cta_pairs_matches_the_one_cta_kernel(bw, batch, prompt):
     assert rel_err(outs[0][2], outs[1][2]) < 1e-2
 
 
+@pytest.mark.parametrize("bw,batch,prompt,d_ffn", [(4, 1, 17, 64), (8, 1, 129, 1376), (16, 3, 300, 1440), (32, 2, 700, 130 * 8), (8, 1, 1024, 9504)])
+def test_swiglu_in_the_projection_matches_the_separate_kernel(bw, batch, prompt, d_ffn):
+    """gate|up with SwiGLU in its epilogue against projection and kernel: one tile, half tiles at the end (d_ffn / 64 odd or
+    not whole), one row tile to several, more tiles than CTA pairs.  Sums differ in their grouping only (tolerance as
+    between the projection kernels)."""
+    cfg = dict(RAGGED, d_ffn=d_ffn, beam_width=bw, max_batch=batch, max_ctx=prompt + 200)
+    outs, roots = [], None
+    for env in (dict(RD_SWIGLU_MIN="17"), dict(RD_SWIGLU_MIN="1000000")):
+        r = _rig_with_env(env, cfg=cfg)
+        rng = np.random.default_rng(0)
+        r.eng.prefill([rng.integers(0, cfg["vocab"], size=prompt - 7 * b) for b in range(batch)])
+        if roots is None:
+            roots = r.eng.get_state()[1].clone()
+        r.eng.set_state(None, roots, None)
+        pk = r.eng.pack(dev(np.random.default_rng(1).integers(0, 3, size=(batch, bw, 5))))
+        am, hid, lg = r.eng.verify(pk, want_logits=True)
+        r.eng.poll()
+        outs.append((pk.n.cpu().numpy(), lg.cpu().numpy(), r.eng.get_state()[2].cpu().numpy()))
+        r.eng.close()
+    assert (outs[0][0] == outs[1][0]).all()
+    for b in range(batch):
+        n = int(outs[0][0][b])
+        assert rel_err(outs[0][1][b, :n], outs[1][1][b, :n]) < 1e-2
+    assert rel_err(outs[0][2], outs[1][2]) < 1e-2
+
+
 @pytest.mark.parametrize("bw", [33, 64])
 def test_draft_scores_wide_beams(bw):
     """Beam widths above 32 through the two-kernel selection (segments of the vocabulary, then one merging CTA per
