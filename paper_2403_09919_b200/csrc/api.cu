@@ -97,6 +97,7 @@ struct rd_handle {
   int tc_pairs;   // CTA pairs of the pair projection kernel that fit the device at once (0: not used)
   int tc_pairs_avail, tc_pairs_min_rows;   // the pairs the device offers; row bound from which launches use them
   bool tc_pairs_prefill;
+  int qkv_min_rows;      // likewise for QKV and the rotary embedding
   int swiglu_min_rows;   // row bound from which gate|up takes SwiGLU along (0: use_fused_swiglu's own)
   std::vector<TensorMapBox> kv_maps;   // [layer][K | V]: cache planes as [sequences * heads * max_ctx][head dim] matrices
   Chain chain;  // counter hand-off between the launches of a forward pass
@@ -278,6 +279,10 @@ struct ProfScope {
     CK(h, expr);                       \
   } while (0)
 
+char* kv_plane_ptr(rd_handle* h, int layer, int which) {
+  return h->kv + ((size_t)(layer * 2 + which)) * h->kv_plane * esize(h->dm.dtype);
+}
+
 // Activation descriptors of buffer A: box heights step, 2 step, ..., one per 16 rows of a row tile of mt; made on first use.
 int act_maps_of(rd_handle* h, const void* A, int K, int mt, int step, const void* (&out)[16]) {
   auto is = h->act_shape.find(A);
@@ -352,6 +357,41 @@ bool use_fused_swiglu(const rd_handle* h, int m_max, bool exact) {
   return m_max >= min_rows && h->dm.F % 2 == 0 && tc_use_pairs(m_max, 2 * h->dm.F, h->tc_grid, h->tc_pairs_avail, 0);
 }
 
+// Whether such a pass takes the QKV projection with rotary embedding and cache write in its epilogue.  It has few tiles, so
+// what counts is what its last wave leaves idle (1.25 ns per k-block and row of a tile, weights as 64 rows) against the
+// kernel it saves (8 us and 5.5 ns per 1000 elements).  A verification pass is taken to bring half of its bound.  Prompt
+// passes, whose two-kernel form runs on single CTAs, win throughout: 7B, 8 layers, 360 rows 1670 -> 1643 us, 500 1974 ->
+// 1870, 1000 3275 -> 3073; 33B, 4 layers, 512 rows 2065 -> 1991.  Verification: 7B batch 16 (bound 1296) 17.1 -> 16.6 ms,
+// 8 layers with bounds of 644 to 808 2929 -> 2905, 3701 -> 3487, 4298 -> 4125 us; 33B, bound 644, 15.1 -> 15.3 ms: not taken.
+bool use_fused_qkv(const rd_handle* h, int m_max, bool exact) {
+  const Dims& dm = h->dm;
+  if (dm.hd != 128 || !tc_use_pairs(m_max, 3 * dm.d, h->tc_grid, h->tc_pairs_avail, 0)) return false;
+  if (h->qkv_min_rows > 0) return m_max >= h->qkv_min_rows;
+  if (exact) return m_max >= 352;
+  if (m_max < 512) return false;
+  double idle_tiles, tile_rows;
+  tc_whole_idle(m_max / 2, m_max, (3 * dm.H + 1) / 2, h->tc_pairs_avail < h->tc_grid / 2 ? h->tc_pairs_avail : h->tc_grid / 2, &idle_tiles, &tile_rows);
+  return idle_tiles * (dm.d / 64) * (tile_rows + 64) * 1.25e-3 < 8.0 + (double)(m_max / 2) * dm.d * 5.5e-6;
+}
+
+int gemm_qkv(rd_handle* h, const void* A, int layer, const RowTables& rt, int m_max, Chain* chain, cudaStream_t st) {
+  const Dims& dm = h->dm;
+  const double bytes = 3.0 * dm.d * dm.d * esize(dm.dtype);
+  ProfScope ps(h, 0, bytes, st);
+  auto iw = h->maps.find(h->wqkv[layer]);
+  if (iw == h->maps.end()) return fail(h, RD_ERR_STATE, "projection operand without a TMA descriptor");
+  const void* amaps[16];
+  if (int rc = act_maps_of(h, A, dm.d, tc_pick_mt(m_max), 8, amaps)) return rc;
+  int tr_slot = -1;
+  unsigned long long* tr = gemm_trace_slot(h, bytes, &tr_slot);
+  const int pairs = h->tc_pairs_avail < h->tc_grid / 2 ? h->tc_pairs_avail : h->tc_grid / 2;
+  CK(h, launch_gemm_qkv(&iw->second, amaps, h->ws.qkv, kv_plane_ptr(h, layer, 0), kv_plane_ptr(h, layer, 1), h->ws.rope_tab, rt, dm, m_max,
+                        h->ws.status, pairs, h->tc_smem, tr, chain, st));
+  if (tr_slot >= 0) h->trace_prefetch[tr_slot] = tc_last_prefetch_bytes();
+  h->route[RD_ROUTE_GEMM_PAIRS]++;
+  return RD_OK;
+}
+
 // act = SwiGLU of the gate|up projection of A (tensor cores, CTA pairs).
 int gemm_swiglu(rd_handle* h, const void* A, const void* W, int m_max, void* act, Chain* chain, cudaStream_t st) {
   const Dims& dm = h->dm;
@@ -422,10 +462,6 @@ void fb_advance(rd_handle* h, int grow, cudaStream_t st) {
   h->fb_pending[s] = true;
   h->fb_growth_at[s] = h->fb_growth;
   h->fb_next = s ^ 1;
-}
-
-char* kv_plane_ptr(rd_handle* h, int layer, int which) {
-  return h->kv + ((size_t)(layer * 2 + which)) * h->kv_plane * esize(h->dm.dtype);
 }
 
 // The layers on the CUDA-core path: a projection takes the norm in front of it (where a row fits its staging) and the
@@ -522,15 +558,21 @@ int forward_layers(rd_handle* h, const uint32_t* mask, int m_max, int n_seq, int
     h->chain.cut();
     return RD_OK;
   }
-  const bool fused_swiglu = use_fused_swiglu(h, m_max, mask == nullptr);
+  const bool fused_swiglu = use_fused_swiglu(h, m_max, mask == nullptr), fused_qkv = use_fused_qkv(h, m_max, mask == nullptr);
   for (int l = 0; l < dm.n_layers; ++l) {
     // attention block: (x += down of the previous layer) -> norm -> QKV -> rotary + KV write -> attention -> O
     CKP(h, PROF_NORM, launch_rmsnorm(dm.dtype, w.x, l ? &g_dn : nullptr, h->attn_norm[l], w.a_t, nullptr, dm.d, dm.eps,
                                      w.m_total, m_max, ch, st));
-    int rc = gemm(h, w.a_t, dm.d, h->wqkv[l], 3 * dm.d, dm.d, w.m_total, m_max, w.qkv, 3 * dm.d, &g_qkv, ch, st, /*pair=*/1);
-    if (rc) return rc;
-    CKP(h, PROF_ROPE, launch_rope_kv(w.qkv, g_qkv, kv_plane_ptr(h, l, 0), kv_plane_ptr(h, l, 1), w.rope_tab, rt, dm,
-                                     m_max, w.status, ch, st));
+    int rc;
+    if (fused_qkv) {
+      rc = gemm_qkv(h, w.a_t, l, rt, m_max, ch, st);
+      if (rc) return rc;
+    } else {
+      rc = gemm(h, w.a_t, dm.d, h->wqkv[l], 3 * dm.d, dm.d, w.m_total, m_max, w.qkv, 3 * dm.d, &g_qkv, ch, st, /*pair=*/1);
+      if (rc) return rc;
+      CKP(h, PROF_ROPE, launch_rope_kv(w.qkv, g_qkv, kv_plane_ptr(h, l, 0), kv_plane_ptr(h, l, 1), w.rope_tab, rt, dm,
+                                       m_max, w.status, ch, st));
+    }
     {
       ProfScope ps(h, 1, 0.0, st);
       h->route[att_t5 ? RD_ROUTE_ATT_ROWS128_TC5 : att_wide ? RD_ROUTE_ATT_ROWS64
@@ -742,6 +784,7 @@ int redrafter_init(const rd_config* cfg, const rd_weights* wt, void* kv_cache, s
     if (getenv("RD_TC_CTA2") && atoi(getenv("RD_TC_CTA2")) == 0) h->tc_pairs_avail = 0;
     h->tc_pairs_min_rows = getenv("RD_TC_CTA2_MIN") ? atoi(getenv("RD_TC_CTA2_MIN")) : 512;
     h->tc_pairs_prefill = getenv("RD_TC_CTA2_PREFILL") && atoi(getenv("RD_TC_CTA2_PREFILL")) != 0;
+    h->qkv_min_rows = getenv("RD_QKV_MIN") ? atoi(getenv("RD_QKV_MIN")) : 0;
     h->swiglu_min_rows = getenv("RD_SWIGLU_MIN") ? atoi(getenv("RD_SWIGLU_MIN")) : 0;   // tuning toggle, as those above
     h->tc_pairs = h->tc_pairs_avail;
     if (attn_t5_supported(dm.hd)) {

@@ -73,7 +73,12 @@ struct TcParams {
   // 1: a unit is (pair of adjacent weight tiles, k-block): both tiles of a stage are multiplied by ONE activation
   // box, which halves what the activation operand costs an SM.  Single row tile only.
   int pair;
-  __nv_bfloat16* act;   // SwiGLU output [M][N] of the fused gate|up projection (N: features)
+  __nv_bfloat16* act;   // TC2_SWIGLU: output [M][N] (N: features)
+  // TC2_QKV: cache planes, rotary table [M][64], the rows' sequences and cache slots
+  __nv_bfloat16 *kc, *vc;
+  const float2* table;
+  const int32_t *seq, *slot;
+  int H, max_ctx;
 };
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -517,14 +522,16 @@ __device__ __forceinline__ void umma_commit_pair(uint32_t cluster_bar) {
 }
 
 constexpr uint32_t SWAP_BYTES = 2 * 2 * 2 * 8 * 64 * 4;
-// Row tiles of a SwiGLU launch: whole tiles run in waves of n_clusters, so the fewest waves times the cost of a tile win
+constexpr uint32_t ROW_INFO_BYTES = 2 * 256 * 8;
+// Row tiles of a launch of whole tiles: whole tiles run in waves of n_clusters, so the fewest waves times the cost of a tile win
 // (a tile's k-block costs its rows, and 64 rows' worth for its share of the weights).
-__device__ __forceinline__ GemmRows swiglu_row_tiles(int M, int mt, int n_wt, int n_clusters) {
+__host__ __device__ __forceinline__ GemmRows whole_row_tiles(int M, int mt, int n_wt, int n_clusters) {
   GemmRows best;
   int cost = 0x7fffffff;
-  const int n0 = max(1, (M + mt - 1) / mt);
+  const int n0 = M > mt ? (M + mt - 1) / mt : 1;
   for (int n = n0; n < n0 + 4; ++n) {
-    const int rows = min(mt, max(16, ((M + n - 1) / n + 15) & ~15));
+    int rows = ((M + n - 1) / n + 15) & ~15;
+    rows = rows < 16 ? 16 : rows > mt ? mt : rows;
     const int c = (n_wt * n + n_clusters - 1) / n_clusters * (rows + 64);
     if (c < cost) { cost = c; best = GemmRows(n, rows); }
   }
@@ -536,14 +543,20 @@ __device__ __forceinline__ GemmRows swiglu_row_tiles(int M, int mt, int n_wt, in
 // of the two halves swap eight columns each through shared memory and write SiLU(gate) * up as bf16.  Tiles are not cut:
 // cluster c takes tiles c, c + C, ... of the (weight tile, row tile) list, row tile fastest, so the row tiles of a weight
 // tile run side by side; what whole tiles leave idle in the last wave is kept small by the choice of row tile
-// (swiglu_row_tiles).  The two-kernel form writes the sums as fp32 and reads them back (90 MB at 1024 rows of the 7B
+// (whole_row_tiles).  The two-kernel form writes the sums as fp32 and reads them back (90 MB at 1024 rows of the 7B
 // shape, more than the L2 keeps, and the kernel between them): 133 + 4 + 34 us per layer there, now 140; a 512-token prompt
 // 9.21 -> 8.54 ms, 8192 tokens 153 -> 141 ms, the batch-16 step 19.1 -> 17.6 ms.
-template <int EW, bool SWIGLU>
+// QKV: likewise the QKV projection of a model with 128-dimensional heads, where a weight tile is one head of Q, K or V and lanes
+// i and i + 64 hold a rotary pair: rotated Q goes to the fp32 buffer that attention reads, rotated K and V to the cache.
+// QKV + rotary of a 1024-row prompt pass: 79 + 3 + 19 us per layer as two kernels; a 512-token prompt 8.32 -> 7.92 ms, 8192
+// tokens 137 -> 131 ms, the batch-16 step 17.1 -> 16.6 ms.
+enum { TC2_PLAIN = 0, TC2_SWIGLU = 1, TC2_QKV = 2 };
+template <int EW, int MODE>
 __global__ void __launch_bounds__(tc_threads(EW), EW == 4 ? 4 : 2) gemm_tc2_kernel(const __grid_constant__ CUtensorMap map_w,
                                                                   const __grid_constant__ ActMaps maps_a,   // box heights 8, 16, ..., 128
                                                                   const TcParams p) {
   extern __shared__ uint8_t smem_raw[];
+  constexpr bool SWIGLU = MODE == TC2_SWIGLU, QKV = MODE == TC2_QKV, WHOLE = SWIGLU || QKV;   // WHOLE: tiles are not cut
   pdl_launch_dependents();
   if (p.trace && threadIdx.x == 0) { atomicMin(p.trace + 0, globaltimer()); }
 
@@ -551,25 +564,25 @@ __global__ void __launch_bounds__(tc_threads(EW), EW == 4 ? 4 : 2) gemm_tc2_kern
   const uint32_t rank = cluster_ctarank();        // 0: leader (issues the MMAs), 1: peer
   const uint32_t cluster = cluster_id_x();
   const bool chained = p.cs.signal_ptr != nullptr;
-  const bool early = (!SWIGLU && p.m_tiles_max == 1) || chained;   // (SWIGLU splits by the row count)
+  const bool early = (!WHOLE && p.m_tiles_max == 1) || chained;   // (whole tiles are dealt out by the row count)
   if (!early) {
     if (threadIdx.x == 0) chain_wait_thread(p.cs);
     __syncthreads();
   }
   GemmRows rows(1, p.mt);
-  if (SWIGLU) rows = swiglu_row_tiles(*p.m_total, p.mt, (p.n_tiles + 1) / 2, gridDim.x >> 1);
+  if (WHOLE) rows = whole_row_tiles(*p.m_total, p.mt, (p.n_tiles + 1) / 2, gridDim.x >> 1);
   else if (p.m_tiles_max > 1) rows = gemm_row_tiles(p.mt, p.m_tiles_max, *p.m_total);
   else if (chained) rows.rows = min(p.mt, max(16, (*p.m_total + 15) & ~15));
   const int m_tiles = rows.n;
   const int n_wt = (p.n_tiles + 1) / 2;           // pairs of weight tiles
   const int n_groups = n_wt * m_tiles;
   const int n_clusters = gridDim.x >> 1;
-  const long long U = (long long)n_groups * p.nkb, C = SWIGLU ? n_clusters : gemm_working<long long>(U, n_clusters);   // clusters that work
+  const long long U = (long long)n_groups * p.nkb, C = WHOLE ? n_clusters : gemm_working<long long>(U, n_clusters);   // clusters that work
   const bool works = cluster < C;
-  // SWIGLU: units of this cluster's own list of whole tiles, cluster + i * C
+  // WHOLE: units of this cluster's own list of tiles, cluster + i * C
   const int my_tiles = (int)cluster < n_groups ? (n_groups - 1 - (int)cluster) / n_clusters + 1 : 0;
-  const long long u0 = SWIGLU ? 0 : works ? gemm_range_begin(cluster, U, C) : U;
-  const long long u1 = SWIGLU ? (long long)my_tiles * p.nkb : works ? gemm_range_begin(cluster + 1, U, C) : U;
+  const long long u0 = WHOLE ? 0 : works ? gemm_range_begin(cluster, U, C) : U;
+  const long long u1 = WHOLE ? (long long)my_tiles * p.nkb : works ? gemm_range_begin(cluster + 1, U, C) : U;
   const int mt_eff = rows.rows, half = mt_eff >> 1;   // rows of a row tile; rows of it this CTA loads
   const CUtensorMap* map_a = &maps_a.m[(half >> 3) - 1];
 
@@ -578,9 +591,10 @@ __global__ void __launch_bounds__(tc_threads(EW), EW == 4 ? 4 : 2) gemm_tc2_kern
   const uint32_t a_stage_bytes = (uint32_t)(p.mt >> 1) * TILE_K * 2;   // reserved
   const uint32_t stage_bytes = (uint32_t)W_STAGE_BYTES + a_stage_bytes;
   const uint32_t tx_bytes = 2u * ((uint32_t)W_STAGE_BYTES + (uint32_t)half * TILE_K * 2);   // both CTAs' copies of a stage
-  const uint32_t swap_bytes = SWIGLU ? SWAP_BYTES : 0u;
+  const uint32_t swap_bytes = WHOLE ? SWAP_BYTES + (QKV ? ROW_INFO_BYTES : 0u) : 0u;
   const uint32_t bar_base = base + p.stages * stage_bytes + swap_bytes;
   float* swap = reinterpret_cast<float*>(smem_raw + (bar_base - swap_bytes - raw));   // [column group][2][8 columns of gate | of up][64]
+  int2* row_info = reinterpret_cast<int2*>(swap + SWAP_BYTES / 4);   // QKV: [2][256] sequence and cache slot of a tile's rows
   auto full_bar = [&](int s) { return bar_base + 8u * s; };
   auto empty_bar = [&](int s) { return bar_base + 8u * (p.stages + s); };
   auto tfull_bar = [&](int a) { return bar_base + 8u * (2 * p.stages + a); };
@@ -597,9 +611,9 @@ __global__ void __launch_bounds__(tc_threads(EW), EW == 4 ? 4 : 2) gemm_tc2_kern
     int g, m_tile, kb, t;
     uint32_t s, ph;
   };
-  // weight tile pair and row tile of the i-th tile (SWIGLU: of this cluster's list)
+  // weight tile pair and row tile of the i-th tile (WHOLE: of this cluster's list)
   auto tile_at = [&](int i, int& g, int& m_tile) {
-    if (SWIGLU) {
+    if (WHOLE) {
       const int t = (int)cluster + i * n_clusters;
       g = t / m_tiles;
       m_tile = t - g * m_tiles;
@@ -619,7 +633,7 @@ __global__ void __launch_bounds__(tc_threads(EW), EW == 4 ? 4 : 2) gemm_tc2_kern
   auto advance = [&](UnitPos& q) {
     if (++q.kb == p.nkb) {
       q.kb = 0;
-      if (SWIGLU) tile_at(++q.t, q.g, q.m_tile);   // one division per tile
+      if (WHOLE) tile_at(++q.t, q.g, q.m_tile);   // one division per tile
       else if (++q.g == n_wt) { q.g = 0; ++q.m_tile; }
     }
     if (++q.s == (uint32_t)p.stages) { q.s = 0; q.ph ^= 1u; }
@@ -773,6 +787,9 @@ __global__ void __launch_bounds__(tc_threads(EW), EW == 4 ? 4 : 2) gemm_tc2_kern
       const int m_base = m_tile * mt_eff;
       const int c_end = min(mt_eff, ((M - m_base) + 15) & ~15);
       const uint32_t a = seg & 1u, aph = (seg >> 1) & 1u;
+      if constexpr (QKV) {   // the rows' tables, while the tile is being multiplied (read after the barrier below)
+        if (et < mt_eff) row_info[(seg & 1u) * 256 + et] = m_base + et < M ? make_int2(p.seq[m_base + et], p.slot[m_base + et]) : make_int2(0, -1);
+      }
       if (et == 0) *epi_ok = mbar_wait(tfull_bar(a), aph, abort_flag, p.status) ? 1 : 0;
       epi_bar_sync<EW>();
       if (!*epi_ok) { ok = false; break; }
@@ -809,6 +826,52 @@ __global__ void __launch_bounds__(tc_threads(EW), EW == 4 ? 4 : 2) gemm_tc2_kern
             const int m = m0 + j, f = n & ~1;
             if (m < M && f < p.N)   // the number of features is even
               *reinterpret_cast<__nv_bfloat162*>(p.act + (size_t)m * p.N + f) = __floats2bfloat162_rn(lo, hi);
+          }
+        } else if constexpr (QKV) {
+          // as above: lanes of the first half keep columns 0..7, those of the second 8..15, and get their partners' sums
+          const bool first = row < 64;
+          const int i = row & 63, ti = 2 * grp + (int)rank, part = ti / p.H, h = ti - part * p.H;   // part 3: past the matrix
+          const int mc = c0 + (first ? 0 : 8), m0 = m_base + mc;
+          float2 cs2[8];   // (cos, sin) of this thread's eight rows
+#pragma unroll
+          for (int j = 0; j < 8; ++j) cs2[j] = part < 2 && m0 + j < M ? __ldg(p.table + (size_t)(m0 + j) * 64 + i) : make_float2(1.f, 0.f);
+          float* mine = swap + (((chunk_par * 2 + (int)turn) * 2 + (first ? 0 : 1)) * 8) * 64 + i;
+          const float* other = swap + (((chunk_par * 2 + (int)turn) * 2 + (first ? 1 : 0)) * 8) * 64 + i;
+          turn ^= 1u;
+#pragma unroll
+          for (int j = 0; j < 8; ++j) mine[j * 64] = __uint_as_float(first ? r[8 + j] : r[j]);
+          asm volatile("bar.sync %0, 128;" ::"r"(2 + chunk_par) : "memory");
+          float ya[8], yb[8];   // dimensions i and i + 64
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            const float o = other[j * 64];
+            const float x1 = first ? __uint_as_float(r[j]) : o, x2 = first ? o : __uint_as_float(r[8 + j]);
+            ya[j] = x1 * cs2[j].x - x2 * cs2[j].y;
+            yb[j] = x2 * cs2[j].x + x1 * cs2[j].y;
+          }
+          if (part == 0) {
+            float* q = p.raw + (size_t)m0 * p.ld_raw + h * 128 + i;
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+              if (m0 + j < M) { q[(size_t)j * p.ld_raw] = ya[j]; q[(size_t)j * p.ld_raw + 64] = yb[j]; }
+          } else if (part < 3) {
+            __nv_bfloat16* cache = part == 1 ? p.kc : p.vc;
+            const bool odd = lane & 1;
+#pragma unroll
+            for (int j = 0; j < 8; j += 2) {   // the even lane writes both neighbours for one row, the odd lane for the next
+              const float ga = __shfl_xor_sync(0xffffffffu, odd ? ya[j] : ya[j + 1], 1), gb = __shfl_xor_sync(0xffffffffu, odd ? yb[j] : yb[j + 1], 1);
+              const int jj = j + (odd ? 1 : 0);
+              const int2 at = row_info[(seg & 1u) * 256 + mc + jj];
+              if (m0 + jj < M) {
+                if (at.y >= 0 && at.y < p.max_ctx) {
+                  __nv_bfloat16* dst = cache + (((size_t)at.x * p.H + h) * p.max_ctx + at.y) * 128 + (i & ~1);
+                  *reinterpret_cast<__nv_bfloat162*>(dst) = odd ? __floats2bfloat162_rn(ga, ya[j + 1]) : __floats2bfloat162_rn(ya[j], ga);
+                  *reinterpret_cast<__nv_bfloat162*>(dst + 64) = odd ? __floats2bfloat162_rn(gb, yb[j + 1]) : __floats2bfloat162_rn(yb[j], gb);
+                } else if (h == 0 && i < 2) {
+                  atomicOr(p.status, DEV_ERR_CAPACITY);
+                }
+              }
+            }
           }
         } else if (kb0 == 0) {
           if (n < p.N) {
@@ -931,8 +994,9 @@ cudaError_t tc_prepare(int* smem_limit_out, int* pairs_out) {
   if (e == cudaSuccess) e = cudaFuncSetAttribute(gemm_tc_kernel<false, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(gemm_tc_kernel<true, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(gemm_tc_kernel<true, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(gemm_tc2_kernel<8, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(gemm_tc2_kernel<8, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(gemm_tc2_kernel<8, TC2_PLAIN>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(gemm_tc2_kernel<8, TC2_SWIGLU>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(gemm_tc2_kernel<8, TC2_QKV>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
   if (smem_limit_out) *smem_limit_out = lim;
   if (pairs_out) {
     *pairs_out = 0;
@@ -949,7 +1013,7 @@ cudaError_t tc_prepare(int* smem_limit_out, int* pairs_out) {
       cfg.attrs = attr;
       cfg.numAttrs = 1;
       int n = 0;
-      const cudaError_t oe = cudaOccupancyMaxActiveClusters(&n, gemm_tc2_kernel<8, false>, &cfg);
+      const cudaError_t oe = cudaOccupancyMaxActiveClusters(&n, gemm_tc2_kernel<8, TC2_PLAIN>, &cfg);
       if (oe == cudaSuccess) *pairs_out = n;
       else cudaGetLastError();
     }
@@ -1001,20 +1065,28 @@ static cudaError_t launch_gemm_tc2(const void* map_w, const void* const map_a[16
   }
   ActMaps am;
   for (int i = 0; i < ACT_MAPS; ++i) am.m[i] = *(const CUtensorMap*)(map_a[i] ? map_a[i] : map_a[0]);
-  launch_pairs(first, gemm_tc2_kernel<8, false>, 2 * pairs, tc_threads(8), smem, st, *(const CUtensorMap*)map_w, am, p);
+  launch_pairs(first, gemm_tc2_kernel<8, TC2_PLAIN>, 2 * pairs, tc_threads(8), smem, st, *(const CUtensorMap*)map_w, am, p);
   return cudaGetLastError();
 }
 
-// The gate|up projection with SwiGLU behind it on CTA pairs: act[m][f], f < F.  map_w: box of tc_weight_box_rows() / 2 rows.
-cudaError_t launch_gemm_swiglu(const void* map_w, const void* const map_a[16], int F, int K, const int32_t* m_total, int m_max, void* act,
-                               int32_t* status, int pairs, int smem_limit, unsigned long long* trace, Chain* chain, cudaStream_t st) {
-  TcParams p{};
-  p.N = F; p.K = K; p.nkb = (K + TILE_K - 1) / TILE_K; p.n_tiles = (2 * F + TILE_N - 1) / TILE_N;
+// What a launch of whole tiles over M rows leaves idle: tiles per cluster missing in the last wave, and rows of a tile.
+void tc_whole_idle(int M, int m_max, int n_wt, int n_clusters, double* idle_tiles, double* tile_rows) {
+  const GemmRows g = whole_row_tiles(M, tc_pick_mt(m_max), n_wt, n_clusters);
+  const int tiles = n_wt * g.n, waves = (tiles + n_clusters - 1) / n_clusters;
+  *idle_tiles = waves - (double)tiles / n_clusters;
+  *tile_rows = g.rows;
+}
+
+// A projection of whole tiles on CTA pairs with the function behind it in the epilogue.
+template <int MODE>
+static cudaError_t launch_whole(TcParams p, const void* map_w, const void* const map_a[16], int m_max, int pairs, int smem_limit, Chain* chain,
+                                cudaStream_t st) {
+  p.nkb = (p.K + TILE_K - 1) / TILE_K;
   p.mt = tc_pick_mt(m_max);
   p.m_tiles_max = (m_max + p.mt - 1) / p.mt;
   p.pair = 1;
   const int stage_bytes = W_STAGE_BYTES + (p.mt / 2) * TILE_K * 2;
-  const int overhead = 1024 + (int)SWAP_BYTES + 8 * (2 * 16 + 4) + 64;
+  const int overhead = 1024 + (int)(SWAP_BYTES + (MODE == TC2_QKV ? ROW_INFO_BYTES : 0u)) + 8 * (2 * 16 + 4) + 64;
   int stages = (smem_limit - overhead) / stage_bytes;
   if (stages > 16) stages = 16;
   if (stages < 2) return cudaErrorInvalidConfiguration;
@@ -1022,14 +1094,35 @@ cudaError_t launch_gemm_swiglu(const void* map_w, const void* const map_a[16], i
   int cols = 32;
   while (cols < 2 * p.mt) cols <<= 1;
   p.tmem_cols = cols;
-  p.m_total = m_total; p.act = (__nv_bfloat16*)act; p.status = status; p.trace = trace;
   const bool first = chain && chain->enabled && chain->prev_ptr == nullptr;
-  p.cs = chain ? chain->link((unsigned)(2 * pairs)) : ChainSync{nullptr, 0u, nullptr, status, nullptr};
+  p.cs = chain ? chain->link((unsigned)(2 * pairs)) : ChainSync{nullptr, 0u, nullptr, p.status, nullptr};
   g_last_prefetch_bytes = chain ? 2.0 * pairs * stages * W_STAGE_BYTES : 0.0;
   ActMaps am;
   for (int i = 0; i < ACT_MAPS; ++i) am.m[i] = *(const CUtensorMap*)(map_a[i] ? map_a[i] : map_a[0]);
-  launch_pairs(first, gemm_tc2_kernel<8, true>, 2 * pairs, tc_threads(8), (size_t)stages * stage_bytes + overhead, st, *(const CUtensorMap*)map_w, am, p);
+  launch_pairs(first, gemm_tc2_kernel<8, MODE>, 2 * pairs, tc_threads(8), (size_t)stages * stage_bytes + overhead, st, *(const CUtensorMap*)map_w, am, p);
   return cudaGetLastError();
+}
+
+// The gate|up projection with SwiGLU behind it: act[m][f], f < F (even).  map_w: box of tc_weight_box_rows() / 2 rows.
+cudaError_t launch_gemm_swiglu(const void* map_w, const void* const map_a[16], int F, int K, const int32_t* m_total, int m_max, void* act,
+                               int32_t* status, int pairs, int smem_limit, unsigned long long* trace, Chain* chain, cudaStream_t st) {
+  TcParams p{};
+  p.N = F; p.K = K; p.n_tiles = (2 * F + TILE_N - 1) / TILE_N;
+  p.m_total = m_total; p.act = (__nv_bfloat16*)act; p.status = status; p.trace = trace;
+  return launch_whole<TC2_SWIGLU>(p, map_w, map_a, m_max, pairs, smem_limit, chain, st);
+}
+
+// The QKV projection with the rotary embedding and the cache write behind it (head dimension 128).
+cudaError_t launch_gemm_qkv(const void* map_w, const void* const map_a[16], float* qkv, void* kcache, void* vcache, const float* table,
+                            const RowTables& rt, const Dims& dm, int m_max, int32_t* status, int pairs, int smem_limit,
+                            unsigned long long* trace, Chain* chain, cudaStream_t st) {
+  if (dm.hd != TILE_N) return cudaErrorInvalidValue;
+  TcParams p{};
+  p.N = 3 * dm.d; p.K = dm.d; p.n_tiles = 3 * dm.H;
+  p.m_total = rt.m_total; p.raw = qkv; p.ld_raw = 3 * dm.d; p.status = status; p.trace = trace;
+  p.kc = (__nv_bfloat16*)kcache; p.vc = (__nv_bfloat16*)vcache; p.table = reinterpret_cast<const float2*>(table);
+  p.seq = rt.seq; p.slot = rt.slot; p.H = dm.H; p.max_ctx = dm.max_ctx;
+  return launch_whole<TC2_QKV>(p, map_w, map_a, m_max, pairs, smem_limit, chain, st);
 }
 
 cudaError_t launch_gemm_tc(const void* map_w, const void* const map_a[16], int N, int K, const int32_t* m_total, int m_max,

@@ -398,14 +398,16 @@ def test_projection_on_cta_pairs_matches_the_one_cta_kernel(bw, batch, prompt):
     assert rel_err(outs[0][2], outs[1][2]) < 1e-2
 
 
-@pytest.mark.parametrize("bw,batch,prompt,d_ffn", [(4, 1, 17, 64), (8, 1, 129, 1376), (16, 3, 300, 1440), (32, 2, 700, 130 * 8), (8, 1, 1024, 9504)])
-def test_swiglu_in_the_projection_matches_the_separate_kernel(bw, batch, prompt, d_ffn):
-    """gate|up with SwiGLU in its epilogue against projection and kernel: one tile, half tiles at the end (d_ffn / 64 odd or
-    not whole), one row tile to several, more tiles than CTA pairs.  Sums differ in their grouping only (tolerance as
-    between the projection kernels)."""
-    cfg = dict(RAGGED, d_ffn=d_ffn, beam_width=bw, max_batch=batch, max_ctx=prompt + 200)
+@pytest.mark.parametrize("bw,batch,prompt,d_ffn,heads", [(4, 1, 17, 64, 4), (8, 1, 129, 1376, 3), (16, 3, 300, 1440, 4), (32, 2, 700, 1040, 1),
+                                                         (8, 1, 1024, 9504, 5)])
+def test_projections_with_their_functions_match_the_separate_kernels(bw, batch, prompt, d_ffn, heads):
+    """gate|up with SwiGLU and QKV with rotary embedding and cache write in their epilogues against projection and kernel:
+    one tile, half tiles at the end (d_ffn / 64 odd or not whole; an odd number of heads), one row tile to several, more
+    tiles than CTA pairs.  Sums differ in their grouping only (tolerance as between the projection kernels)."""
+    d = 128 * heads
+    cfg = dict(RAGGED, d_model=d, d_rnn=d, n_heads=heads, d_ffn=d_ffn, beam_width=bw, max_batch=batch, max_ctx=prompt + 200)
     outs, roots = [], None
-    for env in (dict(RD_SWIGLU_MIN="17"), dict(RD_SWIGLU_MIN="1000000")):
+    for env in (dict(RD_SWIGLU_MIN="17", RD_QKV_MIN="17"), dict(RD_SWIGLU_MIN="1000000", RD_QKV_MIN="1000000")):
         r = _rig_with_env(env, cfg=cfg)
         rng = np.random.default_rng(0)
         r.eng.prefill([rng.integers(0, cfg["vocab"], size=prompt - 7 * b) for b in range(batch)])
@@ -415,12 +417,15 @@ def test_swiglu_in_the_projection_matches_the_separate_kernel(bw, batch, prompt,
         pk = r.eng.pack(dev(np.random.default_rng(1).integers(0, 3, size=(batch, bw, 5))))
         am, hid, lg = r.eng.verify(pk, want_logits=True)
         r.eng.poll()
-        outs.append((pk.n.cpu().numpy(), lg.cpu().numpy(), r.eng.get_state()[2].cpu().numpy()))
+        outs.append((pk.n.cpu().numpy(), lg.cpu().numpy(), r.eng.get_state()[2].cpu().numpy(), r.eng.kv_view().float().cpu().numpy()))
         r.eng.close()
     assert (outs[0][0] == outs[1][0]).all()
     for b in range(batch):
         n = int(outs[0][0][b])
         assert rel_err(outs[0][1][b, :n], outs[1][1][b, :n]) < 1e-2
+        kv = [o[3][:, :, b, :, :prompt - 7 * b + n] for o in outs]
+        assert rel_err(*kv) < 1e-2
+        assert (outs[0][3][:, :, b, :, prompt - 7 * b + n:] == outs[1][3][:, :, b, :, prompt - 7 * b + n:]).all()   # nothing written past the rows
     assert rel_err(outs[0][2], outs[1][2]) < 1e-2
 
 
