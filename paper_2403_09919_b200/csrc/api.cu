@@ -358,7 +358,7 @@ bool use_fused_swiglu(const rd_handle* h, int m_max, bool exact) {
 }
 
 // Whether such a pass takes the QKV projection with rotary embedding and cache write in its epilogue.  It has few tiles, so
-// what counts is what its last wave leaves idle (1.25 ns per k-block and row of a tile, weights as 64 rows) against the
+// what counts is what its last wave leaves idle (1.4 ns per k-block and row of a tile, weights as 64 rows) against the
 // kernel it saves (8 us and 5.5 ns per 1000 elements).  A verification pass is taken to bring half of its bound.  Prompt
 // passes, whose two-kernel form runs on single CTAs, win throughout: 7B, 8 layers, 360 rows 1670 -> 1643 us, 500 1974 ->
 // 1870, 1000 3275 -> 3073; 33B, 4 layers, 512 rows 2065 -> 1991.  Verification: 7B batch 16 (bound 1296) 17.1 -> 16.6 ms,
@@ -371,7 +371,7 @@ bool use_fused_qkv(const rd_handle* h, int m_max, bool exact) {
   if (m_max < 512) return false;
   double idle_tiles, tile_rows;
   tc_whole_idle(m_max / 2, m_max, (3 * dm.H + 1) / 2, h->tc_pairs_avail < h->tc_grid / 2 ? h->tc_pairs_avail : h->tc_grid / 2, &idle_tiles, &tile_rows);
-  return idle_tiles * (dm.d / 64) * (tile_rows + 64) * 1.25e-3 < 8.0 + (double)(m_max / 2) * dm.d * 5.5e-6;
+  return idle_tiles * (dm.d / 64) * (tile_rows + 64) * 1.4e-3 < 8.0 + (double)(m_max / 2) * dm.d * 5.5e-6;
 }
 
 int gemm_qkv(rd_handle* h, const void* A, int layer, const RowTables& rt, int m_max, Chain* chain, cudaStream_t st) {
@@ -422,6 +422,8 @@ int gemm_simt(rd_handle* h, int epi, const SimtOperands& p, const SimtEpilogue& 
 int chain_start(rd_handle* h, cudaStream_t st) {
   if (h->chain_dirty) {
     cudaError_t e = h->chain.reset(st);
+    // (attention's merge counters too: a launch that gave up may have left some behind)
+    if (e == cudaSuccess) e = cudaMemsetAsync(h->ws.att_counters, 0, ATT_MAX_SPLIT_BLOCKS * sizeof(int32_t), st);
     if (e != cudaSuccess) return fail(h, RD_ERR_CUDA, "resetting the hand-off counters: %s", cudaGetErrorString(e));
     h->chain_dirty = false;
   }
@@ -538,14 +540,23 @@ int forward_layers(rd_handle* h, const uint32_t* mask, int m_max, int n_seq, int
     else if (att_wide) row_blocks = (rows_per_seq_max + attn_wide_rows_per_block() - 1) / attn_wide_rows_per_block();
     // more 16-row CTAs than SMs (many sequences of a few rows): a two-chunk ring so that three CTAs share an SM
     static const int shallow_ok = getenv("RD_ATT_SHALLOW") ? atoi(getenv("RD_ATT_SHALLOW")) : 1;   // tuning toggle
-    att_shallow = shallow_ok && !att_wide && blocks > h->tc_grid;
-    n_splits = h->tc_grid / blocks;  // at most one CTA per SM: a second wave would double the time
-    // ... and only when a CTA would otherwise walk many chunks: the cross-CTA merge costs several microseconds
+    // Keys split over CTAs: with fewer tiles than half the SMs, one CTA per SM and at least three chunks each; with more, up
+    // to three CTAs per SM (short ring) of at least six chunks, which also evens out sequences of different lengths.  (8
+    // layers of the 7B shape, one split per SM and eight chunks before: autoregressive, 1 x 600 tokens 822 -> 807 us; 4 x
+    // 1100 940 -> 934; 2 x 800 tokens with 58 rows 1988 -> 1940.  Three per SM for few tiles too: 1 x 3000 877 -> 896; of
+    // three chunks: the 7B step at 512 tokens 8.35 -> 8.66 ms; two chunks each for few tiles: small steps 1.60 -> 1.64.)
     const int max_chunks = (h->ctx_bound + rows_per_seq_max + 63) / 64;
-    if (n_splits > (max_chunks + 7) / 8) n_splits = (max_chunks + 7) / 8;
+    if (2 * blocks <= h->tc_grid) {
+      n_splits = h->tc_grid / blocks;
+      if (n_splits > max_chunks / 3) n_splits = max_chunks / 3;
+    } else {
+      n_splits = 3 * h->tc_grid / blocks;
+      if (n_splits > max_chunks / 6) n_splits = max_chunks / 6;
+    }
     if (n_splits > 16) n_splits = 16;
     if (n_splits < 1) n_splits = 1;
     while (n_splits > 1 && (long long)blocks * n_splits > ATT_MAX_SPLIT_BLOCKS) --n_splits;
+    att_shallow = shallow_ok && !att_wide && blocks * n_splits > h->tc_grid;
   }
   GemmOut g_qkv, g_o, g_gu, g_dn;
   // inside the layer loop every launch hands over to the next through a counter; the launches before

@@ -363,10 +363,9 @@ __global__ void __launch_bounds__(128) attention_tc_kernel(const float* __restri
   }
 
   // ---- keys split over CTAs: publish the partial, the last arriver merges the splits in split order
-  __threadfence();
   __syncthreads();
   if (tid == 0) {
-    const int old = atomicAdd(counters + blk, 1);
+    const int old = chain_arrive_count(counters + blk);
     s_last = (old == n_splits - 1) ? 1 : 0;
     if (old == n_splits - 1) counters[blk] = 0;  // ready for the next launch
   }
@@ -376,7 +375,6 @@ __global__ void __launch_bounds__(128) attention_tc_kernel(const float* __restri
     chain_exit(cs);
     return;
   }
-  __threadfence();
   const float* all = scratch + (size_t)blk * n_splits * ROWS * PW;
   if (tid < nrows) {
     const int r = tid;

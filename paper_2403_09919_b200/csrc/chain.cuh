@@ -82,6 +82,14 @@ __device__ __forceinline__ unsigned int chain_load_acquire(const unsigned int* p
   return v;
 }
 
+// One thread, after a barrier that the CTA's stores lie before: count the CTA in and return how many came earlier.  Releases
+// those stores and, for what follows the next barrier, acquires those of the CTAs counted before.
+__device__ __forceinline__ int chain_arrive_count(int32_t* p) {
+  int old;
+  asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], 1;" : "=r"(old) : "l"(p) : "memory");
+  return old;
+}
+
 // One thread: wait until the predecessor has signalled completely (or fall back to the grid dependency).
 // Bounded; gives up at once when an earlier wait of the step already timed out.
 __device__ __forceinline__ void chain_wait_thread(const ChainSync& cs) {

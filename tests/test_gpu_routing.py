@@ -118,3 +118,11 @@ def test_long_context_few_heads_splits_the_keys():
     cfg = dict(BASE, d_model=512, n_heads=4, d_rnn=512, max_batch=2, beam_width=8, max_ctx=4096 + 41 + 16)
     route, n_max, n_sum = verify_on_long_contexts(cfg, [4096, 3000], follow=[0], rho=0.3, seed=23)
     assert route["att_rows16"] == cfg["n_layers"] and route["att_key_split"] == cfg["n_layers"]
+
+
+def test_many_tiles_split_the_keys_too():
+    """More 16-row tiles than half the SMs: the keys are split over up to three CTAs per SM (two-chunk ring), also for a
+    sequence of one chunk of keys, which leaves one of its splits empty."""
+    cfg = dict(BASE, d_model=1024, n_heads=8, d_rnn=1024, max_batch=4, beam_width=8, max_ctx=760 + 41 + 16)
+    route, n_max, n_sum = verify_on_long_contexts(cfg, [760, 12, 400, 90], follow=[0, 1, 3], rho=0.3, seed=24)
+    assert route["att_rows16_shallow"] == cfg["n_layers"] and route["att_key_split"] == cfg["n_layers"]
