@@ -101,6 +101,7 @@ struct rd_handle {
   int swiglu_min_rows;   // row bound from which gate|up takes SwiGLU along (0: use_fused_swiglu's own)
   std::vector<TensorMapBox> kv_maps;   // [layer][K | V]: cache planes as [sequences * heads * max_ctx][head dim] matrices
   Chain chain;  // counter hand-off between the launches of a forward pass
+  bool chain_allowed;   // RD_CHAIN=0: never hand over by counters
   bool chain_dirty;  // a launch failed after the chain had counted it: reset the counters before the next pass
   int device;        // ordinal of the device the handle was made on
   // Context-bound feedback: after a step the device-side context lengths are copied to pinned host memory without
@@ -427,6 +428,11 @@ int chain_start(rd_handle* h, cudaStream_t st) {
     if (e != cudaSuccess) return fail(h, RD_ERR_CUDA, "resetting the hand-off counters: %s", cudaGetErrorString(e));
     h->chain_dirty = false;
   }
+  // The counters only grow and a launch carries the value it waits for, so a captured launch that is replayed would find its
+  // wait already over: under capture every launch waits for the grid before it instead.
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) (void)cudaGetLastError();
+  h->chain.enabled = h->chain_allowed && cap == cudaStreamCaptureStatusNone;
   h->chain.cut();
   return RD_OK;
 }
@@ -844,7 +850,8 @@ int redrafter_init(const rd_config* cfg, const rd_weights* wt, void* kv_cache, s
   h->trace_next = -1;
   h->chain.ctr = h->ws.chain_ctr; h->chain.status = h->ws.status;
   h->chain.trace_base = h->ws.trace; h->chain.trace_next = &h->trace_next; h->chain.trace_cap = TRACE_SLOTS;
-  h->chain.enabled = !(getenv("RD_CHAIN") && atoi(getenv("RD_CHAIN")) == 0);
+  h->chain_allowed = !(getenv("RD_CHAIN") && atoi(getenv("RD_CHAIN")) == 0);
+  h->chain.enabled = h->chain_allowed;
   h->chain_dirty = false;
   h->device = 0;
   (void)cudaGetDevice(&h->device);

@@ -105,3 +105,40 @@ def test_a_wait_that_nothing_satisfies_gives_up_and_is_reported():
     r.eng.step(None, out)                                 # and the engine still decodes
     r.eng.poll()
     assert int(out.n_accept[0]) >= 0
+
+
+@pytest.mark.parametrize("dtype", ["fp32", "bf16"])
+def test_captured_calls_replay_with_new_state(dtype):
+    """A drafter call captured into a graph and replayed after the state has changed gives what an eager call gives: under
+    capture the launches do not hand over by counters, whose values a replay would find already reached."""
+    from paper_2403_09919_b200.binding import ReDrafter
+    cfg = dict(synth.CONFIGS["tiny"], dtype=dtype, d_model=256, n_heads=2, max_ctx=200)
+    eng = ReDrafter(cfg, synth.make_weights(cfg, "cuda:0"))
+    gen = torch.Generator(device="cuda").manual_seed(1)
+    states = [(torch.tensor([11 + 7 * i], dtype=torch.int32, device="cuda"), torch.randn(1, 256, device="cuda", generator=gen)) for i in range(4)]
+    ctx = torch.tensor([20], dtype=torch.int32, device="cuda")
+
+    def put(i):
+        eng.set_state(ctx, states[i][0], states[i][1], ctx_bound=20)
+
+    want = []
+    for i in range(4):
+        put(i)
+        want.append([x.clone() for x in eng.draft()])
+    beams, scores = [torch.zeros_like(x) for x in want[0]]
+    put(0)
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        eng.draft(beams, scores)
+    for i in (0, 1, 2, 3, 1):
+        put(i)
+        g.replay()
+        eng.poll()
+        assert torch.equal(beams, want[i][0]) and torch.equal(scores, want[i][1])
+    put(2)
+    again = eng.draft()                     # and eager calls go on as before
+    eng.poll()
+    assert torch.equal(again[0], want[2][0]) and torch.equal(again[1], want[2][1])
+    del g
+    eng.close()
