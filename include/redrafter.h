@@ -11,7 +11,7 @@
  *   - The library allocates NO device memory: all scratch lives in the caller's workspace
  *     given to redrafter_init (size from redrafter_workspace_bytes).
  *   - Calls enqueue work on the given stream and return without synchronising it (the
- *     two exceptions, redrafter_prefill and redrafter_poll, say so).  The calls on one handle
+ *     exception, redrafter_poll, says so).  The calls on one handle
  *     must be issued in stream order on one stream at a time: inside a call consecutive kernels
  *     hand over through counters in the workspace (each is resident before its predecessor has
  *     finished, and waits -- bounded, 1 s -> RD_ERR_TIMEOUT at the next poll -- for the
@@ -138,8 +138,8 @@ RD_API const char* redrafter_last_error(const rd_handle* h);
  * cache, sets ctx[b] = prompt_len[b], root g[b] = the LLM's greedy token after the prompt and
  * h[b] = its last hidden state (after the final norm).
  * tokens: HOST pointer [batch][max_prompt] (row stride max_prompt); prompt_len: HOST [batch].
- * Copies the inputs from pageable host memory, so it may block the host; the forward itself is
- * only enqueued.  Errors: INVALID_ARG, CAPACITY (prompt_len + NMAX > max_ctx). */
+ * The inputs are copied before the call returns (they travel as kernel arguments); the work is only
+ * enqueued.  Errors: INVALID_ARG, CAPACITY (prompt_len + NMAX > max_ctx). */
 RD_API int redrafter_prefill(rd_handle* h, const int32_t* tokens, const int32_t* prompt_len, int32_t max_prompt,
                       int32_t batch, void* stream);
 

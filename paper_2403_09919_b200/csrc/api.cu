@@ -938,37 +938,34 @@ int redrafter_prefill(rd_handle* h, const int32_t* tokens, const int32_t* prompt
   if (rc) return rc;
   // passes of up to m_cap rows; a sequence's rows may span passes (its earlier rows are in the cache by then)
   const int cap = h->m_cap;
-  std::vector<int32_t> tok(cap), seq(cap), pos(cap), ncache(cap), local(cap), last(batch), soff(batch + 1), count(batch);
   int b = 0, done = 0;  // next sequence, tokens of it already processed
   while (b < batch) {
-    int m = 0, longest_run = 0;
-    for (int i = 0; i < batch; ++i) { last[i] = -1; count[i] = 0; }
-    while (b < batch && m < cap) {
-      const int take = (prompt_len[b] - done) < (cap - m) ? (prompt_len[b] - done) : (cap - m);
-      for (int i = 0; i < take; ++i) {
-        tok[m] = tokens[(size_t)b * max_prompt + done + i];
-        seq[m] = b; pos[m] = done + i; ncache[m] = done + i + 1; local[m] = 0;
-        ++m;
-      }
-      count[b] = take;
+    // what the pass holds: its sequences are consecutive and their rows contiguous from row 0
+    int m = 0, longest_run = 0, b_last = b;
+    for (int q = b, d = done; q < batch && m < cap; ++q, d = 0) {
+      const int take = (prompt_len[q] - d) < (cap - m) ? (prompt_len[q] - d) : (cap - m);
+      m += take;
       if (take > longest_run) longest_run = take;
-      done += take;
-      if (done == prompt_len[b]) { last[b] = m - 1; ++b; done = 0; }
+      b_last = q;
     }
-    // the sequences of a pass are consecutive and their rows contiguous from row 0
-    soff[0] = 0;
-    for (int i = 0; i < batch; ++i) soff[i + 1] = soff[i] + count[i];
-    const size_t nb = (size_t)m * sizeof(int32_t);
-    CKRT(h, cudaMemcpyAsync(w.row_tok, tok.data(), nb, cudaMemcpyHostToDevice, st));
-    CKRT(h, cudaMemcpyAsync(w.row_seq, seq.data(), nb, cudaMemcpyHostToDevice, st));
-    CKRT(h, cudaMemcpyAsync(w.row_pos, pos.data(), nb, cudaMemcpyHostToDevice, st));
-    CKRT(h, cudaMemcpyAsync(w.row_slot, pos.data(), nb, cudaMemcpyHostToDevice, st));
-    CKRT(h, cudaMemcpyAsync(w.row_ncache, ncache.data(), nb, cudaMemcpyHostToDevice, st));
-    CKRT(h, cudaMemcpyAsync(w.row_local, local.data(), nb, cudaMemcpyHostToDevice, st));
-    CKRT(h, cudaMemcpyAsync(w.last_row, last.data(), batch * sizeof(int32_t), cudaMemcpyHostToDevice, st));
-    CKRT(h, cudaMemcpyAsync(w.seq_off, soff.data(), (batch + 1) * sizeof(int32_t), cudaMemcpyHostToDevice, st));
-    CKRT(h, cudaMemcpyAsync(w.m_total, &m, sizeof(int32_t), cudaMemcpyHostToDevice, st));
-    CKRT(h, cudaStreamSynchronize(st));  // the host staging vectors are reused by the next pass
+    PrefillRows rows;
+    rows.batch = batch; rows.b_first = b; rows.b_last = b_last; rows.m = m;
+    for (int at = 0; at < m;) {
+      rows.row0 = at; rows.n = 0; rows.n_runs = 0; rows.first = at == 0;
+      while (at < m && rows.n < PREFILL_TOKENS && rows.n_runs < PREFILL_RUNS) {
+        int take = prompt_len[b] - done;
+        if (take > m - at) take = m - at;
+        const bool whole = take <= PREFILL_TOKENS - rows.n;   // the run ends the sequence's part of this pass
+        if (!whole) take = PREFILL_TOKENS - rows.n;
+        const int r = rows.n_runs++;
+        rows.run_row[r] = at; rows.run_row[r + 1] = at + take; rows.run_b[r] = b; rows.run_pos[r] = done;
+        memcpy(rows.tok + rows.n, tokens + (size_t)b * max_prompt + done, (size_t)take * sizeof(int32_t));
+        rows.n += take; at += take; done += take;
+        rows.run_flags[r] = (whole ? PREFILL_PART_ENDS : 0) | (done == prompt_len[b] ? PREFILL_PROMPT_ENDS : 0);
+        if (done == prompt_len[b]) { ++b; done = 0; }
+      }
+      CK(h, launch_prefill_rows(rows, w.row_tok, w.row_seq, w.row_pos, w.row_slot, w.row_ncache, w.row_local, w.last_row, w.seq_off, w.m_total, st));
+    }
     h->ctx_bound = longest;  // bound of the key extent for this pass
     // Prompt passes keep the one-CTA projection for QKV, O and down: projection plus consumer take the same time with
     // either kernel (the fp32 intermediate bounds the pair), and the CTA pairs start later.
@@ -983,7 +980,8 @@ int redrafter_prefill(rd_handle* h, const int32_t* tokens, const int32_t* prompt
   GemmOut g;
   rc = gemm(h, w.h_t, dm.d, h->w.lm_head, dm.V, dm.d, w.one_b, batch, w.logits, dm.V, &g, nullptr, st);
   if (rc) return rc;
-  CKRT(h, cudaMemcpyAsync(w.ctx, prompt_len, batch * sizeof(int32_t), cudaMemcpyHostToDevice, st));
+  for (int i = 0; i < batch; i += PREFILL_TOKENS)
+    CK(h, launch_store_i32(w.ctx + i, prompt_len + i, batch - i < PREFILL_TOKENS ? batch - i : PREFILL_TOKENS, st));
   // row b is sequence b's last prompt row: the root is the token at position prompt_len[b]
   CK(h, launch_argmax_rows(w.logits, g, dm.V, w.root, nullptr, w.one_b, batch, h->sampling, nullptr, w.ctx, 0, st));
   h->prefilled = true;

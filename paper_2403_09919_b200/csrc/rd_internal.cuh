@@ -170,6 +170,19 @@ cudaError_t launch_build_rows_ar(const int32_t* root, const int32_t* ctx, int32_
                                  int32_t* row_pos, int32_t* row_slot, int32_t* row_ncache, int32_t* row_local,
                                  int32_t* row_out_index, int32_t* seq_off, int32_t* m_total, const Dims& dm, int B,
                                  int* status, cudaStream_t st);
+// Row tables of a prompt pass, up to PREFILL_TOKENS rows of it per launch, carried by the kernel's arguments.
+constexpr int PREFILL_TOKENS = 512, PREFILL_RUNS = 64;
+enum { PREFILL_PART_ENDS = 1, PREFILL_PROMPT_ENDS = 2 };
+struct PrefillRows {
+  int32_t row0, n, n_runs;                      // first row and rows of this launch; runs of one sequence among them
+  int32_t first, batch, b_first, b_last, m;     // first launch of the pass; the pass's sequences and rows
+  int32_t run_row[PREFILL_RUNS + 1];            // first row of every run (one more: the end)
+  int32_t run_b[PREFILL_RUNS], run_pos[PREFILL_RUNS], run_flags[PREFILL_RUNS];
+  int32_t tok[PREFILL_TOKENS];
+};
+cudaError_t launch_prefill_rows(const PrefillRows& p, int32_t* row_tok, int32_t* row_seq, int32_t* row_pos, int32_t* row_slot, int32_t* row_ncache,
+                                int32_t* row_local, int32_t* last_row, int32_t* seq_off, int32_t* m_total, cudaStream_t st);
+cudaError_t launch_store_i32(int32_t* dst, const int32_t* values, int n, cudaStream_t st);   // host values, n <= PREFILL_TOKENS
 cudaError_t launch_scatter_rows(const float* src, int width, float* dst, const int32_t* row_out_index,
                                 const int32_t* m_total, int m_max, cudaStream_t st);
 cudaError_t launch_cast_rows(int dtype, const float* src, void* dst, int n, cudaStream_t st);

@@ -110,6 +110,30 @@ def test_prefill_in_several_passes():
     assert int(c_ctx[0]) == 600 and np.abs(c_h[0].cpu().numpy() - h).max() < TOL_FP32
 
 
+def test_prefill_of_many_short_and_one_long_prompt():
+    """More sequences than one launch of the row tables takes, prompts of one token to several launches and passes: every
+    sequence's state and cache as from a call with that prompt alone (the fp32 path treats rows independently: bit for bit)."""
+    rng = np.random.default_rng(8)
+    lens = [int(x) for x in rng.integers(1, 10, size=100)]
+    lens[7], lens[50], lens[99] = 1300, 512, 1
+    cfg = dict(synth.CONFIGS["tiny"], max_batch=100, beam_width=2, beam_length=2, max_ctx=1320)
+    w = synth.make_weights(cfg, "cuda:0")
+    prompts = [rng.integers(0, cfg["vocab"], size=n) for n in lens]
+    many, one = ReDrafter(cfg, w), ReDrafter(dict(cfg, max_batch=1), w)
+    many.prefill(prompts)
+    many.poll()
+    c, r, h = many.get_state()
+    assert c.tolist() == lens
+    for b in (0, 6, 7, 8, 49, 50, 51, 63, 64, 65, 98, 99):
+        one.prefill([prompts[b]])
+        one.poll()
+        c1, r1, h1 = one.get_state()
+        assert int(c1[0]) == lens[b] and int(r1[0]) == int(r[b]) and torch.equal(h1[0], h[b])
+        assert torch.equal(one.kv_view()[:, :, 0, :, :lens[b]], many.kv_view()[:, :, b, :, :lens[b]])
+    many.close()
+    one.close()
+
+
 def test_verify_logits_and_argmax(rig):
     prompt, kv, ctx, g, h = prefilled(rig)
     rng = np.random.default_rng(6)
