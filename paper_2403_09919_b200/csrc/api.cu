@@ -419,9 +419,19 @@ int gemm_simt(rd_handle* h, int epi, const SimtOperands& p, const SimtEpilogue& 
   return RD_OK;
 }
 
+bool capturing(cudaStream_t st) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) (void)cudaGetLastError();
+  return cap != cudaStreamCaptureStatusNone;
+}
+
 // Start of a chained region: counters back in step with the host if an earlier launch was counted but never ran.
 int chain_start(rd_handle* h, cudaStream_t st) {
+  const bool cap = capturing(st);
   if (h->chain_dirty) {
+    // Not under capture: the graph would hold the reset, and until a replay the host's targets would start from zero
+    // with the device's counters still at their old values, so that eager calls would find every wait over.
+    if (cap) return fail(h, RD_ERR_STATE, "an earlier launch failed or a wait gave up: one call outside the capture has to reset the counters");
     cudaError_t e = h->chain.reset(st);
     // (attention's merge counters too: a launch that gave up may have left some behind)
     if (e == cudaSuccess) e = cudaMemsetAsync(h->ws.att_counters, 0, ATT_MAX_SPLIT_BLOCKS * sizeof(int32_t), st);
@@ -430,9 +440,7 @@ int chain_start(rd_handle* h, cudaStream_t st) {
   }
   // The counters only grow and a launch carries the value it waits for, so a captured launch that is replayed would find its
   // wait already over: under capture every launch waits for the grid before it instead.
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) (void)cudaGetLastError();
-  h->chain.enabled = h->chain_allowed && cap == cudaStreamCaptureStatusNone;
+  h->chain.enabled = h->chain_allowed && !cap;
   h->chain.cut();
   return RD_OK;
 }
@@ -644,13 +652,13 @@ int do_draft(rd_handle* h, cudaStream_t st, int32_t* beams, float* scores) {
   Workspace& w = h->ws;
   const Dims& dm = h->dm;
   const int B = h->batch, R = B * dm.BW;
+  if (int rc0 = chain_start(h, st)) return rc0;
   CKP(h, PROF_DRAFT_SMALL, launch_draft_init(dm.dtype, h->w.tok_emb, w.root, w.h, w.xc_t, w.xc_f, w.x0_t, w.x0_f, w.se_t, dm, B, w.status, st));
   float *sc_in = w.score_a, *sc_out = w.score_b;
   int32_t *hi_in = w.hist_a, *hi_out = w.hist_b;
   GemmOut g;
   // the calls' launches hand over to each other through counters
   Chain* ch = &h->chain;
-  if (int rc0 = chain_start(h, st)) return rc0;
   // out = (resid) + SiLU(W x + bias), rows of out and resid d_rnn + d_model wide
   auto cell = [&](const void* x, int K, const void* W, const void* bias, int N, const float* resid, float* of, void* ot, float* raw,
                   const int32_t* mt, int rows) -> int {

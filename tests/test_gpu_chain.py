@@ -142,3 +142,40 @@ def test_captured_calls_replay_with_new_state(dtype):
     assert torch.equal(again[0], want[2][0]) and torch.equal(again[1], want[2][1])
     del g
     eng.close()
+
+
+def test_a_capture_after_a_wait_that_gave_up_is_refused():
+    """After a wait that gave up the next call resets the hand-off counters.  A captured call cannot: its graph would hold the
+    reset, while the host already counts from zero.  It is refused until an eager call has been made; eager calls and, from
+    then on, captured ones give what they gave before."""
+    from paper_2403_09919_b200.binding import RdError, ReDrafter
+    cfg = dict(synth.CONFIGS["tiny"], dtype="bf16", d_model=256, n_heads=2, max_ctx=200)
+    eng = ReDrafter(cfg, synth.make_weights(cfg, "cuda:0"))
+    i32 = dict(dtype=torch.int32, device="cuda")
+    eng.set_state(torch.tensor([20], **i32), torch.tensor([11], **i32), torch.ones(1, 256, device="cuda"), ctx_bound=20)
+    want = eng.draft()
+    eng.poll()
+    eng.selftest_wait()
+    with pytest.raises(RdError) as e:
+        eng.poll()
+    assert e.value.code == 6
+    beams, scores = [torch.zeros_like(x) for x in want]
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        with pytest.raises(RdError) as e:
+            eng.draft(beams, scores)
+    assert e.value.code == 4
+    got = eng.draft()
+    eng.poll()
+    assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        eng.draft(beams, scores)
+    for _ in range(2):
+        g.replay()
+        got = eng.draft()
+        eng.poll()
+        for a, b, c in zip(want, got, (beams, scores)):
+            assert torch.equal(a, b) and torch.equal(a, c)
+    del g
+    eng.close()
