@@ -16,6 +16,11 @@
  *     hand over through counters in the workspace (each is resident before its predecessor has
  *     finished, and waits -- bounded, 1 s -> RD_ERR_TIMEOUT at the next poll -- for the
  *     predecessor's last store), and the bookkeeping of those counters follows the call order.
+ *   - Stream capture: redrafter_draft, pack, verify, accept, step and ar_step may be captured into a CUDA graph
+ *     (accept_static after its first call).  A captured launch waits for the one before it and not on a counter.
+ *     The host learns nothing of a replay: after replays of a call that advances the contexts, and before the
+ *     next call, pass the contexts' new bound to redrafter_set_ctx_bound.  RD_ERR_STATE is returned under
+ *     capture while a failed launch or a wait that gave up is still to be cleared by an eager call.
  *   - Every call returns an rd_status.  Nothing throws, traps or asserts on the device;
  *     problems detected by kernels are recorded in a device status word (redrafter_poll).
  *   - Sizes: B = batch, BW = beam_width, L = beam_length (drafted tokens per candidate =

@@ -449,9 +449,9 @@ int chain_start(rd_handle* h, cudaStream_t st) {
 void fb_invalidate(rd_handle* h) { h->fb_pending[0] = h->fb_pending[1] = false; }
 
 // A copy of the context lengths that has completed bounds every sequence's context by its largest value plus
-// whatever the calls enqueued since can have added.
-void fb_poll(rd_handle* h) {
-  if (!h->fb_host) return;
+// whatever the calls enqueued since can have added.  Not under capture: querying an event would end the capture.
+void fb_poll(rd_handle* h, cudaStream_t st) {
+  if (!h->fb_host || !(h->fb_pending[0] || h->fb_pending[1]) || capturing(st)) return;
   for (int s = 0; s < 2; ++s) {
     if (!h->fb_pending[s] || cudaEventQuery(h->fb_event[s]) != cudaSuccess) continue;
     h->fb_pending[s] = false;
@@ -463,11 +463,12 @@ void fb_poll(rd_handle* h) {
   (void)cudaGetLastError();   // cudaEventQuery's cudaErrorNotReady is not an error of this handle
 }
 
-// After a call that advanced the contexts by at most `grow` tokens each.
+// After a call that advanced the contexts by at most `grow` tokens each.  A captured call adds to the bound and copies
+// nothing: an event recorded in a capture could not be queried afterwards, and its slot would stay taken.
 void fb_advance(rd_handle* h, int grow, cudaStream_t st) {
   h->ctx_bound += grow;
   h->fb_growth += grow;
-  if (!h->fb_host || (h->fb_calls++ & 7u) != 0u) return;
+  if (!h->fb_host || capturing(st) || (h->fb_calls++ & 7u) != 0u) return;
   const int s = h->fb_next;
   if (h->fb_pending[s]) return;   // that slot's copy is still on its way: try again after the next call
   if (cudaMemcpyAsync(h->fb_host + (size_t)s * h->dm.B, h->ws.ctx, (size_t)h->batch * sizeof(int32_t), cudaMemcpyDeviceToHost, st) !=
@@ -638,10 +639,10 @@ int forward_layers(rd_handle* h, const uint32_t* mask, int m_max, int n_seq, int
   return RD_OK;
 }
 
-int check_stepable(rd_handle* h) {
+int check_stepable(rd_handle* h, cudaStream_t st) {
   if (!h) return RD_ERR_INVALID_ARG;
   if (!h->prefilled) return fail(h, RD_ERR_STATE, "no state: call redrafter_prefill or redrafter_set_state first");
-  fb_poll(h);
+  fb_poll(h, st);
   if (h->ctx_bound + h->dm.NMAX > h->dm.max_ctx)
     return fail(h, RD_ERR_CAPACITY, "context bound %d + %d packed rows exceeds max_ctx %d", h->ctx_bound, h->dm.NMAX,
                 h->dm.max_ctx);
@@ -999,7 +1000,7 @@ int redrafter_prefill(rd_handle* h, const int32_t* tokens, const int32_t* prompt
 }
 
 int redrafter_draft(rd_handle* h, void* stream, int32_t* beams, float* scores) {
-  int rc = check_stepable(h);
+  int rc = check_stepable(h, (cudaStream_t)stream);
   if (rc) return rc;
   if (!beams) return fail(h, RD_ERR_INVALID_ARG, "beams is null");
   return do_draft(h, (cudaStream_t)stream, beams, scores);
@@ -1010,7 +1011,7 @@ static bool packed_ok(const rd_packed* p) {
 }
 
 int redrafter_pack(rd_handle* h, const int32_t* beams, void* stream, const rd_packed* out) {
-  int rc = check_stepable(h);
+  int rc = check_stepable(h, (cudaStream_t)stream);
   if (rc) return rc;
   if (!beams || !packed_ok(out)) return fail(h, RD_ERR_INVALID_ARG, "null beams or packed member");
   cudaStream_t st = (cudaStream_t)stream;
@@ -1019,7 +1020,7 @@ int redrafter_pack(rd_handle* h, const int32_t* beams, void* stream, const rd_pa
 }
 
 int redrafter_verify(rd_handle* h, const rd_packed* packed, void* stream, int32_t* argmax, float* hidden, float* logits) {
-  int rc = check_stepable(h);
+  int rc = check_stepable(h, (cudaStream_t)stream);
   if (rc) return rc;
   if (!packed_ok(packed) || !argmax) return fail(h, RD_ERR_INVALID_ARG, "null packed member or argmax");
   return do_verify(h, *packed, (cudaStream_t)stream, argmax, hidden, logits);
@@ -1027,7 +1028,7 @@ int redrafter_verify(rd_handle* h, const rd_packed* packed, void* stream, int32_
 
 int redrafter_accept(rd_handle* h, const int32_t* beams, const rd_packed* packed, const int32_t* argmax,
                      const float* hidden, void* stream, const rd_accept_out* out) {
-  int rc = check_stepable(h);
+  int rc = check_stepable(h, (cudaStream_t)stream);
   if (rc) return rc;
   if (!beams || !packed_ok(packed) || !argmax || !hidden) return fail(h, RD_ERR_INVALID_ARG, "null argument");
   Workspace& w = h->ws;
@@ -1042,7 +1043,7 @@ int redrafter_accept(rd_handle* h, const int32_t* beams, const rd_packed* packed
 
 int redrafter_accept_static(rd_handle* h, const int32_t* beams, const rd_packed* packed, const int32_t* argmax,
                             const float* hidden, void* stream, const rd_accept_out* out) {
-  int rc = check_stepable(h);
+  int rc = check_stepable(h, (cudaStream_t)stream);
   if (rc) return rc;
   if (!beams || !packed_ok(packed) || !argmax || !hidden) return fail(h, RD_ERR_INVALID_ARG, "null argument");
   int dev_now = -1;
@@ -1065,7 +1066,7 @@ int redrafter_accept_static(rd_handle* h, const int32_t* beams, const rd_packed*
 }
 
 int redrafter_step(rd_handle* h, const int32_t* planted_beams, void* stream, const rd_accept_out* out) {
-  int rc = check_stepable(h);
+  int rc = check_stepable(h, (cudaStream_t)stream);
   if (rc) return rc;
   cudaStream_t st = (cudaStream_t)stream;
   Workspace& w = h->ws;
@@ -1087,7 +1088,7 @@ int redrafter_step(rd_handle* h, const int32_t* planted_beams, void* stream, con
 int redrafter_ar_step(rd_handle* h, void* stream, int32_t* token) {
   if (!h) return RD_ERR_INVALID_ARG;
   if (!h->prefilled) return fail(h, RD_ERR_STATE, "no state: call redrafter_prefill or redrafter_set_state first");
-  fb_poll(h);
+  fb_poll(h, (cudaStream_t)stream);
   if (h->ctx_bound + 1 > h->dm.max_ctx) return fail(h, RD_ERR_CAPACITY, "KV cache full");
   cudaStream_t st = (cudaStream_t)stream;
   Workspace& w = h->ws;

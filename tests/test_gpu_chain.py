@@ -179,3 +179,59 @@ def test_a_capture_after_a_wait_that_gave_up_is_refused():
             assert torch.equal(a, b) and torch.equal(a, c)
     del g
     eng.close()
+
+
+@pytest.mark.parametrize("call", ["step", "ar_step"])
+@pytest.mark.parametrize("pending", [True, False])
+def test_captured_steps_leave_the_context_feedback_working(call, pending):
+    """A step captured while a copy of the context lengths is on its way (after an eager step): its replays give what an
+    eager step gives.  A step captured as the call that would enqueue such a copy (the handle's first): the feedback goes
+    on -- 48 steps that accept about one token each fit a cache that the bound alone would have run out of."""
+    from paper_2403_09919_b200.binding import AcceptOut, ReDrafter
+    L = 4
+    cfg = dict(synth.CONFIGS["tiny"], beam_width=4, beam_length=L, max_ctx=20 + 48 * 2 + 17 + 10 * L)
+    eng = ReDrafter(cfg, synth.make_weights(cfg, "cuda:0"))
+    i32 = dict(dtype=torch.int32, device="cuda")
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    eng.kv_view().normal_(generator=gen)
+    kv0 = eng.kv_view().clone()
+    ctx, root = torch.tensor([20], **i32), torch.tensor([11], **i32)
+    h = torch.randn(1, cfg["d_model"], device="cuda", generator=gen)
+    rng = np.random.default_rng(15)
+    beams = lambda: torch.from_numpy(rng.integers(0, cfg["vocab"], size=(1, 4, L)).astype(np.int32)).cuda()
+    fixed, out, token = beams(), AcceptOut(1, L, "cuda:0"), torch.zeros(1, **i32)
+
+    def one(b=None):
+        return eng.step(fixed if b is None else b, out) if call == "step" else eng.ar_step(token)
+
+    def put():
+        eng.kv_view().copy_(kv0)
+        eng.set_state(ctx, root, h)
+
+    def seen():
+        got = [out.n_accept, out.best, out.tokens, token, *eng.get_state(), eng.kv_view()]
+        return [x.clone() for x in got]
+
+    eng.set_state(ctx, root, h, ctx_bound=20)
+    if pending:
+        one()                                # its copy of the context lengths stays pending: nothing polls before the capture
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        one()
+    if not pending:
+        for i in range(48):
+            one(beams())
+            if i % 8 == 7:
+                eng.poll()
+        eng.set_ctx_bound(20)
+    put()
+    one()
+    want = seen()
+    for _ in range(2):
+        put()
+        g.replay()
+        eng.poll()
+        for a, b in zip(seen(), want):
+            assert torch.equal(a, b)
+    del g
+    eng.close()
