@@ -144,7 +144,8 @@ RD_API const char* redrafter_last_error(const rd_handle* h);
  * h[b] = its last hidden state (after the final norm).
  * tokens: HOST pointer [batch][max_prompt] (row stride max_prompt); prompt_len: HOST [batch].
  * The inputs are copied before the call returns (they travel as kernel arguments); the work is only
- * enqueued.  Errors: INVALID_ARG, CAPACITY (prompt_len + NMAX > max_ctx). */
+ * enqueued.  Errors: INVALID_ARG, CAPACITY (prompt_len + NMAX > max_ctx), STATE (the stream is being captured;
+ * nothing is enqueued). */
 RD_API int redrafter_prefill(rd_handle* h, const int32_t* tokens, const int32_t* prompt_len, int32_t max_prompt,
                       int32_t batch, void* stream);
 

@@ -942,6 +942,8 @@ int redrafter_prefill(rd_handle* h, const int32_t* tokens, const int32_t* prompt
     if (prompt_len[b] + dm.NMAX > dm.max_ctx) return fail(h, RD_ERR_CAPACITY, "prompt %d of length %d leaves no room for a step", b, prompt_len[b]);
     longest = prompt_len[b] > longest ? prompt_len[b] : longest;
   }
+  // (the prompt would be baked into the graph, and a replay would leave the host's batch and bound as they are)
+  if (capturing(st)) return fail(h, RD_ERR_STATE, "prompts cannot be processed under stream capture");
   h->batch = batch;
   int rc = set_row_counts(h, st);
   if (rc) return rc;

@@ -235,3 +235,25 @@ def test_captured_steps_leave_the_context_feedback_working(call, pending):
             assert torch.equal(a, b)
     del g
     eng.close()
+
+
+def test_a_captured_prompt_is_refused_and_the_capture_goes_on():
+    from paper_2403_09919_b200.binding import RdError, ReDrafter
+    cfg = dict(synth.CONFIGS["tiny"], max_ctx=200)
+    eng = ReDrafter(cfg, synth.make_weights(cfg, "cuda:0"))
+    prompt = [np.arange(1, 40)]
+    eng.prefill(prompt)
+    want = [x.clone() for x in (*eng.get_state(), *eng.draft())]
+    beams, scores = [torch.zeros_like(x) for x in want[3:]]
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        with pytest.raises(RdError) as e:
+            eng.prefill(prompt)
+        eng.draft(beams, scores)
+    assert e.value.code == 4
+    g.replay()
+    eng.poll()
+    for a, b in zip(want, (*eng.get_state(), beams, scores)):
+        assert torch.equal(a, b)
+    del g
+    eng.close()
