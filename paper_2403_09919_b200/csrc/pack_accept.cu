@@ -119,10 +119,12 @@ __global__ void __launch_bounds__(256) accept_kernel(const int32_t* __restrict__
   const int b = blockIdx.x, BW = dm.BW, L = dm.L, C = L + 1;
   const size_t rb = (size_t)b * dm.NMAX;
   int a = -1, bi = 0x7fffffff, node = 0, bonus = 0;   // the best of this thread's candidates, where it ends and the token there
+  bool bad = false;
   for (int i = threadIdx.x; i < BW; i += blockDim.x) {
     const int32_t* up = pk.unpack + ((size_t)b * BW + i) * C;
     const int32_t* bm = beams + ((size_t)b * BW + i) * L;
     int ai = 0, an = 0, at = 0;
+    bool bad_end = false;
     for (bool go = true; go;) {
       int nd[ACCEPT_BATCH], tk[ACCEPT_BATCH], want[ACCEPT_BATCH];
       const int j0 = ai;
@@ -137,12 +139,15 @@ __global__ void __launch_bounds__(256) accept_kernel(const int32_t* __restrict__
       for (int k = 0; k < ACCEPT_BATCH; ++k) {
         if (!go) continue;
         an = nd[k]; at = tk[k];
-        if (an < 0 || an >= dm.NMAX) { atomicOr(status, DEV_ERR_INDEX_RANGE); an = 0; go = false; }   // tk is the token at node 0
-        else if (j0 + k == L || want[k] != at) go = false;
+        if (an < 0 || an >= dm.NMAX) {   // (tk is the token at node 0) behind the last token only the winner's node counts
+          if (j0 + k < L) atomicOr(status, DEV_ERR_INDEX_RANGE);
+          else bad_end = true;
+          an = 0; go = false;
+        } else if (j0 + k == L || want[k] != at) go = false;
         else ++ai;
       }
     }
-    if (ai > a || (ai == a && i < bi)) { a = ai; bi = i; node = an; bonus = at; }
+    if (ai > a || (ai == a && i < bi)) { a = ai; bi = i; node = an; bonus = at; bad = bad_end; }
   }
   const int mine = bi;
 #pragma unroll
@@ -156,7 +161,10 @@ __global__ void __launch_bounds__(256) accept_kernel(const int32_t* __restrict__
   a = sh_a[0]; bi = sh_i[0];
   for (int k = 1; k < (int)(blockDim.x >> 5); ++k)
     if (sh_a[k] > a || (sh_a[k] == a && sh_i[k] < bi)) { a = sh_a[k]; bi = sh_i[k]; }
-  if (mine == bi) { s_node = node; s_bonus = bonus; }   // one thread holds the winner
+  if (mine == bi) {   // one thread holds the winner
+    s_node = node; s_bonus = bonus;
+    if (bad) atomicOr(status, DEV_ERR_INDEX_RANGE);
+  }
   __syncthreads();
   if (out.tokens)
     for (int j = threadIdx.x; j < C; j += blockDim.x)

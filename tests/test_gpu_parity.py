@@ -9,7 +9,7 @@ import torch
 
 from oracle import redrafter_oracle as ora
 from paper_2403_09919_b200 import synth
-from paper_2403_09919_b200.binding import ReDrafter
+from paper_2403_09919_b200.binding import RdError, ReDrafter
 
 pytestmark = pytest.mark.gpu
 
@@ -393,6 +393,42 @@ def test_accept_and_compaction_along_long_paths(dtype, L, a):
     assert c.tolist() == [x + 1 + a for x in ctx] and r.tolist() == [int(argmax[b, node[b]]) for b in range(B)]
     assert torch.equal(h, torch.stack([hidden[b, node[b]] for b in range(B)]))
     assert torch.equal(kv, want)
+    eng.close()
+
+
+@pytest.mark.parametrize("L", [3, 7, 8])
+def test_accept_checks_the_last_node_of_the_winner_only(L):
+    """Two candidates accepted to their ends: an index out of range behind the last token of the second is never used and
+    is no error; behind the last token of the first, the winner, it is reported; in the middle of either it is too."""
+    cfg = dict(synth.CONFIGS["tiny"], beam_width=3, beam_length=L, max_ctx=120)
+    eng = ReDrafter(cfg, synth.make_weights(cfg, "cuda:0"))
+    beams = np.arange(3 * L).reshape(1, 3, L) + 10
+    hidden = torch.randn(1, eng.nmax, cfg["d_model"], device="cuda")
+    matched = beams.copy()
+    matched[0, 2, 0] = beams[0, 0, 0]                       # both leave the root by the one token that the LLM says there
+
+    def accept(cand, j):
+        eng.set_state(dev([5]), dev([1]), torch.zeros(1, cfg["d_model"], device="cuda"), ctx_bound=5)
+        pk = eng.pack(dev(beams))                           # no shared prefixes: every candidate has nodes of its own
+        unpack = pk.unpack.cpu().numpy()
+        argmax = np.full((1, eng.nmax), 3)
+        argmax[0, 0] = beams[0, 0, 0]
+        for c in (0, 2):
+            argmax[0, unpack[0, c, 1:L]] = beams[0, c, 1:]
+        if cand is not None:
+            pk.unpack[0, cand, j] = -1
+        return eng.accept(dev(matched), pk, dev(argmax), hidden)
+
+    for cand, j, ok in ((None, 0, True), (2, L, True), (0, L, False), (2, 1, False), (0, 1, False)):
+        out = accept(cand, j)
+        if ok:
+            eng.poll()
+            assert out.n_accept.tolist() == [L] and out.best.tolist() == [0]
+            assert out.tokens[0].tolist() == beams[0, 0].tolist() + [3]
+        else:
+            with pytest.raises(RdError) as e:
+                eng.poll()
+            assert e.value.code == 1
     eng.close()
 
 
