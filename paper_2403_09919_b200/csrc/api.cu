@@ -532,7 +532,7 @@ int forward_layers(rd_handle* h, const uint32_t* mask, int m_max, int n_seq, int
                                       w.m_total, m_max, w.status, st));
   // attention launch geometry (tensor-core path): tiles of 16 rows per sequence; keys split over CTAs only
   // for long contexts with few tiles
-  int row_blocks = 1, n_splits = 1;
+  int row_blocks = 1, n_splits = 1, split_chunks = 1;
   bool att_wide = false, att_shallow = false, att_t5 = false;
   if (h->use_tc) {
     const int rpb = attn_tc_rows_per_block();
@@ -562,14 +562,12 @@ int forward_layers(rd_handle* h, const uint32_t* mask, int m_max, int n_seq, int
     // layers of the 7B shape, one split per SM and eight chunks before: autoregressive, 1 x 600 tokens 822 -> 807 us; 4 x
     // 1100 940 -> 934; 2 x 800 tokens with 58 rows 1988 -> 1940.  Three per SM for few tiles too: 1 x 3000 877 -> 896; of
     // three chunks: the 7B step at 512 tokens 8.35 -> 8.66 ms; two chunks each for few tiles: small steps 1.60 -> 1.64.)
+    // The kernel takes the real lengths for it; the host's bound only limits the launch.
     const int max_chunks = (h->ctx_bound + rows_per_seq_max + 63) / 64;
-    if (2 * blocks <= h->tc_grid) {
-      n_splits = h->tc_grid / blocks;
-      if (n_splits > max_chunks / 3) n_splits = max_chunks / 3;
-    } else {
-      n_splits = 3 * h->tc_grid / blocks;
-      if (n_splits > max_chunks / 6) n_splits = max_chunks / 6;
-    }
+    const bool few = 2 * blocks <= h->tc_grid;
+    split_chunks = few ? 3 : 6;
+    n_splits = (few ? h->tc_grid : 3 * h->tc_grid) / blocks;
+    if (n_splits > max_chunks / split_chunks) n_splits = max_chunks / split_chunks;
     if (n_splits > 16) n_splits = 16;
     if (n_splits < 1) n_splits = 1;
     while (n_splits > 1 && (long long)blocks * n_splits > ATT_MAX_SPLIT_BLOCKS) --n_splits;
@@ -614,7 +612,7 @@ int forward_layers(rd_handle* h, const uint32_t* mask, int m_max, int n_seq, int
                                     row_blocks, ch, st));
       else
         CK(h, launch_attention_tc(w.qkv, kv_plane_ptr(h, l, 0), kv_plane_ptr(h, l, 1), w.attn_t, rt, w.seq_off, dm, n_seq,
-                                  row_blocks, n_splits, w.att_scratch, w.att_counters,
+                                  row_blocks, n_splits, split_chunks, w.att_scratch, w.att_counters,
                                   (h->trace_next >= 0 && h->trace_next < TRACE_SLOTS) ? w.trace + (size_t)8 * h->trace_next++ : nullptr, ch,
                                   att_shallow ? 1 : 0, st));
     }
@@ -952,15 +950,16 @@ int redrafter_prefill(rd_handle* h, const int32_t* tokens, const int32_t* prompt
   int b = 0, done = 0;  // next sequence, tokens of it already processed
   while (b < batch) {
     // what the pass holds: its sequences are consecutive and their rows contiguous from row 0
-    int m = 0, longest_run = 0, b_last = b;
+    int m = 0, longest_run = 0, keys = 0, b_last = b;
     for (int q = b, d = done; q < batch && m < cap; ++q, d = 0) {
       const int take = (prompt_len[q] - d) < (cap - m) ? (prompt_len[q] - d) : (cap - m);
       m += take;
       if (take > longest_run) longest_run = take;
+      if (d + take > keys) keys = d + take;
       b_last = q;
     }
     PrefillRows rows;
-    rows.batch = batch; rows.b_first = b; rows.b_last = b_last; rows.m = m;
+    rows.batch = batch; rows.b_first = b; rows.b_last = b_last; rows.m = m; rows.longest = keys;
     for (int at = 0; at < m;) {
       rows.row0 = at; rows.n = 0; rows.n_runs = 0; rows.first = at == 0;
       while (at < m && rows.n < PREFILL_TOKENS && rows.n_runs < PREFILL_RUNS) {

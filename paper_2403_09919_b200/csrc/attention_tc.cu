@@ -10,7 +10,10 @@
 // provisional slots n_cache + t whose bit t is set in its mask row.  For long contexts with few
 // CTAs the keys are also split over S CTAs (chunks [z*C/S, (z+1)*C/S)); then every CTA writes its
 // unnormalised (m, l, O) to scratch and the last one to arrive for that (head, row tile) -- found
-// with an atomic counter, never by waiting -- merges the splits in split order.
+// with an atomic counter, never by waiting -- merges the splits in split order.  S follows from the
+// longest key extent among the pass's sequences, left beside the row tables, and not from the host's
+// bound of it: that bound is lowered whenever a copy of the real lengths happens to have arrived, and
+// results must not depend on when.  The launch has as many CTAs as the bound allows; the rest leave.
 #include "pdl.cuh"
 #include "rd_internal.cuh"
 
@@ -54,7 +57,7 @@ __global__ void __launch_bounds__(128) attention_tc_kernel(const float* __restri
                                                            const __nv_bfloat16* __restrict__ vc,
                                                            __nv_bfloat16* __restrict__ out, RowTables rt,
                                                            const int32_t* __restrict__ seq_off, Dims dm, int row_tiles,
-                                                           int n_splits, float* __restrict__ scratch,
+                                                           int split_chunks, float* __restrict__ scratch,
                                                            int32_t* __restrict__ counters, unsigned long long* dbg, ChainSync cs) {
   unsigned long long t_dbg[6] = {0, 0, 0, 0, 0, 0};
   RD_STAMP(0);
@@ -82,17 +85,19 @@ __global__ void __launch_bounds__(128) attention_tc_kernel(const float* __restri
   const int h = blockIdx.x;
   const int b = blockIdx.y / row_tiles, rb = blockIdx.y - b * row_tiles;
   const int z = blockIdx.z;
+  const bool tree = rt.mask != nullptr;
+  // as many splits as leave each split_chunks chunks of the longest sequence
+  const int n_splits = gridDim.z == 1 ? 1 : min(max((min(rt.m_total[1], dm.max_ctx) + KEYS - 1) / KEYS / split_chunks, 1), (int)gridDim.z);
   const int seq_row0 = seq_off[b], seq_rows = seq_off[b + 1] - seq_row0;
   const int row0 = seq_row0 + rb * ROWS;
   const int nrows = min(ROWS, seq_rows - rb * ROWS);
-  if (nrows <= 0) {  // the same for every split and head of this row tile
+  if (nrows <= 0 || z >= n_splits) {  // the former is the same for every split and head of this row tile
     if (early) chain_wait_cta(cs);
     chain_exit(cs);
     return;
   }
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t4 = lane & 3;
   const int MW = dm.MW;
-  const bool tree = rt.mask != nullptr;
   const int r_lo = g, r_hi = g + 8;
 
   // ---- row tables and mask
@@ -329,7 +334,7 @@ __global__ void __launch_bounds__(128) attention_tc_kernel(const float* __restri
   }
   __syncthreads();
   const int blk = blockIdx.y * gridDim.x + h;  // (sequence, row tile, head)
-  float* part = scratch + ((size_t)blk * n_splits + z) * ROWS * PW;   // only touched when n_splits > 1
+  float* part = scratch + ((size_t)blk * n_splits + z) * ROWS * PW;   // only touched when n_splits > 1 (never more than the launch's)
   for (int idx = tid; idx < ROWS * (HD / 4); idx += 128) {
     const int r = idx / (HD / 4), c = (idx - r * (HD / 4)) * 4;
     float mw[4], gm = -INFINITY;
@@ -447,15 +452,16 @@ cudaError_t attn_tc_prepare(int hd, int MW) {
   return e;
 }
 
-// grid (H, sequences * row_tiles, n_splits); `shallow`: more CTAs than SMs, so several should share an SM
+// grid (H, sequences * row_tiles, n_splits); n_splits: the most that the keys may be split, split_chunks: the fewest chunks of
+// the longest sequence that a split is worth; `shallow`: more CTAs than SMs, so several should share an SM
 cudaError_t launch_attention_tc(const float* qkv, const void* kcache, const void* vcache, void* out, const RowTables& rt,
                                 const int32_t* seq_off, const Dims& dm, int n_seq, int row_tiles, int n_splits,
-                                float* scratch, int32_t* counters, unsigned long long* dbg, Chain* chain, int shallow, cudaStream_t st) {
+                                int split_chunks, float* scratch, int32_t* counters, unsigned long long* dbg, Chain* chain, int shallow, cudaStream_t st) {
   dim3 grid(dm.H, n_seq * row_tiles, n_splits);
   const ChainSync cs = chain ? chain->link(grid.x * grid.y * grid.z) : ChainSync{nullptr, 0u, nullptr, nullptr, nullptr};
 #define RD_ATT_LAUNCH(HD, NST)                                                                                              \
   launch_pdl(attention_tc_kernel<HD, NST>, grid, 128, smem_bytes<HD, NST>(dm.MW), st, qkv, (const __nv_bfloat16*)kcache,    \
-             (const __nv_bfloat16*)vcache, (__nv_bfloat16*)out, rt, seq_off, dm, row_tiles, n_splits, scratch, counters, dbg, cs)
+             (const __nv_bfloat16*)vcache, (__nv_bfloat16*)out, rt, seq_off, dm, row_tiles, split_chunks, scratch, counters, dbg, cs)
   if (dm.hd == 128) {
     if (shallow) RD_ATT_LAUNCH(128, NSTAGE_SHALLOW); else RD_ATT_LAUNCH(128, NSTAGE_DEEP);
   } else if (dm.hd == 64) {

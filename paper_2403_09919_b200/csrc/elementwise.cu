@@ -964,7 +964,9 @@ __global__ void __launch_bounds__(1024) build_rows_tree_kernel(rd_packed pk, con
         rank += (ko > kb || (ko == kb && o < b)) ? 1 : 0;
       }
       seq_order[rank] = b;
+      if (rank == 0) m_total[1] = kb;
     }
+  else if (threadIdx.x == 0) m_total[1] = 0;   // so many sequences that no kernel splits their keys
   for (int idx = threadIdx.x; idx < B * dm.NMAX; idx += blockDim.x) {
     const int b = idx / dm.NMAX, n = idx - b * dm.NMAX;
     if (n >= off[b + 1] - off[b]) { argmax[idx] = -1; continue; }
@@ -991,32 +993,38 @@ cudaError_t launch_build_rows_tree(const rd_packed& pk, const int32_t* ctx, int3
   return cudaGetLastError();
 }
 
-// Autoregressive step: one row per sequence, the root token at position ctx_b.
-__global__ void build_rows_ar_kernel(const int32_t* __restrict__ root, const int32_t* __restrict__ ctx, int32_t* row_tok,
+// Autoregressive step: one row per sequence, the root token at position ctx_b.  One block.
+__global__ void __launch_bounds__(256) build_rows_ar_kernel(const int32_t* __restrict__ root, const int32_t* __restrict__ ctx, int32_t* row_tok,
                                      int32_t* row_seq, int32_t* row_pos, int32_t* row_slot, int32_t* row_ncache,
                                      int32_t* row_local, int32_t* row_out_index, int32_t* seq_off, int32_t* m_total,
                                      Dims dm, int B, int* status) {
   pdl_enter();
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b == 0) { *m_total = B; seq_off[B] = B; }
-  if (b >= B) return;
-  seq_off[b] = b;
-  int t = root[b];
-  if (t < 0 || t >= dm.V) { atomicOr(status, DEV_ERR_TOKEN_RANGE); t = min(max(t, 0), dm.V - 1); }
-  row_tok[b] = t;
-  row_seq[b] = b;
-  row_pos[b] = ctx[b];
-  row_slot[b] = ctx[b];
-  row_ncache[b] = ctx[b] + 1;
-  row_local[b] = 0;
-  row_out_index[b] = b;
+  __shared__ int s_longest;
+  if (threadIdx.x == 0) { *m_total = B; seq_off[B] = B; s_longest = 0; }
+  __syncthreads();
+  for (int b = threadIdx.x; b < B; b += blockDim.x) {
+    seq_off[b] = b;
+    int t = root[b];
+    if (t < 0 || t >= dm.V) { atomicOr(status, DEV_ERR_TOKEN_RANGE); t = min(max(t, 0), dm.V - 1); }
+    const int c = ctx[b];
+    row_tok[b] = t;
+    row_seq[b] = b;
+    row_pos[b] = c;
+    row_slot[b] = c;
+    row_ncache[b] = c + 1;
+    row_local[b] = 0;
+    row_out_index[b] = b;
+    atomicMax(&s_longest, c + 1);
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) m_total[1] = s_longest;
 }
 
 cudaError_t launch_build_rows_ar(const int32_t* root, const int32_t* ctx, int32_t* row_tok, int32_t* row_seq,
                                  int32_t* row_pos, int32_t* row_slot, int32_t* row_ncache, int32_t* row_local,
                                  int32_t* row_out_index, int32_t* seq_off, int32_t* m_total, const Dims& dm, int B,
                                  int* status, cudaStream_t st) {
-  launch_pdl(build_rows_ar_kernel, (B + 127) / 128, 128, 0, st, root, ctx, row_tok, row_seq, row_pos, row_slot, row_ncache,
+  launch_pdl(build_rows_ar_kernel, 1, B > 128 ? 256 : 128, 0, st, root, ctx, row_tok, row_seq, row_pos, row_slot, row_ncache,
                                                         row_local, row_out_index, seq_off, m_total, dm, B, status);
   return cudaGetLastError();
 }
@@ -1071,7 +1079,7 @@ __global__ void __launch_bounds__(256) prefill_rows_kernel(const __grid_constant
         seq_off[b + 1] = b < p.b_first ? 0 : p.m;
         last_row[b] = -1;
       }
-    if (i0 == 0) { seq_off[0] = 0; *m_total = p.m; }
+    if (i0 == 0) { seq_off[0] = 0; m_total[0] = p.m; m_total[1] = p.longest; }
   }
 }
 

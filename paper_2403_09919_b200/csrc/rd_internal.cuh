@@ -39,7 +39,7 @@ struct RowTables {
   const int32_t* n_cache;     // [M] number of leading cache slots the row attends
   const int32_t* local;       // [M] index of the row inside its sequence's group of rows (its mask row)
   const uint32_t* mask;       // [B][NMAX][MW] tree mask or nullptr (causal: n_cache covers everything)
-  const int32_t* m_total;     // [1] number of valid rows (device)
+  const int32_t* m_total;     // [2] number of valid rows, and the most keys that any of them attends (device)
 };
 
 struct Dims {
@@ -126,7 +126,7 @@ int attn_tc_rows_per_block();
 cudaError_t attn_tc_prepare(int hd, int MW);
 cudaError_t launch_attention_tc(const float* qkv, const void* kcache, const void* vcache, void* out, const RowTables& rt,
                                 const int32_t* seq_off, const Dims& dm, int n_seq, int row_blocks, int n_splits,
-                                float* scratch, int32_t* counters, unsigned long long* dbg, Chain* chain, int shallow, cudaStream_t st);
+                                int split_chunks, float* scratch, int32_t* counters, unsigned long long* dbg, Chain* chain, int shallow, cudaStream_t st);
 cudaError_t elementwise_prepare();
 cudaError_t drafter_prepare(int dtype);
 cudaError_t launch_swiglu(const GemmOut& proj, void* out_t, int F, const int32_t* m_total, int m_max,
@@ -176,6 +176,7 @@ enum { PREFILL_PART_ENDS = 1, PREFILL_PROMPT_ENDS = 2 };
 struct PrefillRows {
   int32_t row0, n, n_runs;                      // first row and rows of this launch; runs of one sequence among them
   int32_t first, batch, b_first, b_last, m;     // first launch of the pass; the pass's sequences and rows
+  int32_t longest;                              // the most keys that a row of the pass attends
   int32_t run_row[PREFILL_RUNS + 1];            // first row of every run (one more: the end)
   int32_t run_b[PREFILL_RUNS], run_pos[PREFILL_RUNS], run_flags[PREFILL_RUNS];
   int32_t tok[PREFILL_TOKENS];

@@ -16,6 +16,7 @@ import torch
 from helpers import Rig, check_against_storage_noise, dev, top2_gap
 from oracle import redrafter_oracle as ora
 from paper_2403_09919_b200 import synth
+from paper_2403_09919_b200.binding import ReDrafter
 
 pytestmark = pytest.mark.gpu
 
@@ -126,3 +127,36 @@ def test_many_tiles_split_the_keys_too():
     cfg = dict(BASE, d_model=1024, n_heads=8, d_rnn=1024, max_batch=4, beam_width=8, max_ctx=760 + 41 + 16)
     route, n_max, n_sum = verify_on_long_contexts(cfg, [760, 12, 400, 90], follow=[0, 1, 3], rho=0.3, seed=24)
     assert route["att_rows16_shallow"] == cfg["n_layers"] and route["att_key_split"] == cfg["n_layers"]
+
+
+@pytest.mark.parametrize("heads,head_dim,batch", [(4, 128, 2), (8, 128, 4), (12, 64, 3)])
+def test_key_splits_do_not_depend_on_the_hosts_bound(heads, head_dim, batch):
+    """The host's bound of the contexts is lowered whenever a copy of the real lengths has arrived, so what a step computes
+    must not follow it: the same verification pass and autoregressive step under a tight and a loose bound, bit for bit, with
+    the keys split over several CTAs (few tiles, and more than half the SMs)."""
+    d = heads * head_dim
+    cfg = dict(BASE, d_model=d, n_heads=heads, d_rnn=d, max_batch=batch, beam_width=8, max_ctx=2000)
+    eng = ReDrafter(cfg, synth.make_weights(cfg, "cuda:0"))
+    gen = torch.Generator(device="cuda").manual_seed(4)
+    eng.kv_view().normal_(generator=gen)
+    kv0 = eng.kv_view().clone()
+    rng = np.random.default_rng(25)
+    lens = [900] + [int(x) for x in rng.integers(1, 900, size=batch - 1)]
+    roots, h = dev(rng.integers(0, cfg["vocab"], size=batch)), torch.randn(batch, d, device="cuda", generator=gen)
+    beams = dev(rng.integers(0, 3, size=(batch, 8, cfg["beam_length"])))
+    seen = []
+    for bound in (900, 1100, 1900):
+        eng.kv_view().copy_(kv0)
+        eng.set_state(dev(lens), roots, h, ctx_bound=bound)
+        before = eng.route_counts()["att_key_split"]
+        pk = eng.pack(beams)
+        am, hid, lg = eng.verify(pk, want_logits=True)
+        assert eng.route_counts()["att_key_split"] == before + cfg["n_layers"]
+        eng.ar_step()
+        eng.poll()
+        assert eng.route_counts()["att_key_split"] == before + 2 * cfg["n_layers"]
+        seen.append([am, hid, lg, eng.last_logits(batch), *eng.get_state()])
+    for other in seen[1:]:
+        for a, b in zip(seen[0], other):
+            assert torch.equal(a, b)
+    eng.close()
