@@ -84,6 +84,7 @@ struct rd_handle {
   bool prefilled;
   int batch;      // active sequences
   int ctx_bound;  // host-side upper bound of every sequence's context length
+  int route_bound;  // the same without the feedback below: kernels are chosen by it, so that results follow from the calls alone
   Sampling sampling;  // how the LLM's tokens are chosen (inv_t = 0: greedy)
   int64_t launches;
   int64_t route[RD_ROUTE_COUNT];  // launches per kernel variant (redrafter_route_counts)
@@ -467,6 +468,7 @@ void fb_poll(rd_handle* h, cudaStream_t st) {
 // nothing: an event recorded in a capture could not be queried afterwards, and its slot would stay taken.
 void fb_advance(rd_handle* h, int grow, cudaStream_t st) {
   h->ctx_bound += grow;
+  h->route_bound += grow;
   h->fb_growth += grow;
   if (!h->fb_host || capturing(st) || (h->fb_calls++ & 7u) != 0u) return;
   const int s = h->fb_next;
@@ -551,7 +553,7 @@ int forward_layers(rd_handle* h, const uint32_t* mask, int m_max, int n_seq, int
     // 64-row kernel would run.)
     static const int t5_rows = getenv("RD_ATT_T5_ROWS") ? atoi(getenv("RD_ATT_T5_ROWS")) : 64;   // tuning toggle
     const bool t5_pays = rows_per_seq_max >= 512 ||
-                         (rows_per_seq_max >= t5_rows && h->ctx_bound + rows_per_seq_max >= (mask ? 320 : 1024));
+                         (rows_per_seq_max >= t5_rows && h->route_bound + rows_per_seq_max >= (mask ? 320 : 1024));
     att_t5 = att_wide && !h->kv_maps.empty() && ((t5_ok == 1 && t5_pays) || t5_ok >= 2);
     if (att_t5) row_blocks = (rows_per_seq_max + attn_t5_rows_per_block() - 1) / attn_t5_rows_per_block();
     else if (att_wide) row_blocks = (rows_per_seq_max + attn_wide_rows_per_block() - 1) / attn_wide_rows_per_block();
@@ -850,7 +852,7 @@ int redrafter_init(const rd_config* cfg, const rd_weights* wt, void* kv_cache, s
     add_a(w.se_t, R, dm.dr + dm.d);
     if (!ok) return init_fail(h, RD_ERR_CUDA, "cuTensorMapEncodeTiled failed with %d for operand %p", failed_rc, failed_ptr);
   }
-  h->prefilled = false; h->batch = dm.B; h->ctx_bound = 0; h->launches = 0; h->err[0] = 0;
+  h->prefilled = false; h->batch = dm.B; h->ctx_bound = h->route_bound = 0; h->launches = 0; h->err[0] = 0;
   for (int i = 0; i < RD_ROUTE_COUNT; ++i) h->route[i] = 0;
   h->sampling = Sampling{0.0f, 0u, 0u};
   h->profiling = false;
@@ -976,7 +978,7 @@ int redrafter_prefill(rd_handle* h, const int32_t* tokens, const int32_t* prompt
       }
       CK(h, launch_prefill_rows(rows, w.row_tok, w.row_seq, w.row_pos, w.row_slot, w.row_ncache, w.row_local, w.last_row, w.seq_off, w.m_total, st));
     }
-    h->ctx_bound = longest;  // bound of the key extent for this pass
+    h->ctx_bound = h->route_bound = longest;  // bound of the key extent for this pass
     // Prompt passes keep the one-CTA projection for QKV, O and down: projection plus consumer take the same time with
     // either kernel (the fp32 intermediate bounds the pair), and the CTA pairs start later.
     if (!h->tc_pairs_prefill) h->tc_pairs = 0;
@@ -995,7 +997,7 @@ int redrafter_prefill(rd_handle* h, const int32_t* tokens, const int32_t* prompt
   // row b is sequence b's last prompt row: the root is the token at position prompt_len[b]
   CK(h, launch_argmax_rows(w.logits, g, dm.V, w.root, nullptr, w.one_b, batch, h->sampling, nullptr, w.ctx, 0, st));
   h->prefilled = true;
-  h->ctx_bound = longest;
+  h->ctx_bound = h->route_bound = longest;
   fb_invalidate(h);
   return RD_OK;
 }
@@ -1148,7 +1150,7 @@ int redrafter_set_state(rd_handle* h, void* stream, const int32_t* ctx, const in
 
 int redrafter_set_ctx_bound(rd_handle* h, int32_t max_ctx_now) {
   if (!h || max_ctx_now < 0) return RD_ERR_INVALID_ARG;
-  h->ctx_bound = max_ctx_now;
+  h->ctx_bound = h->route_bound = max_ctx_now;
   fb_invalidate(h);
   return RD_OK;
 }

@@ -160,3 +160,21 @@ def test_key_splits_do_not_depend_on_the_hosts_bound(heads, head_dim, batch):
         for a, b in zip(seen[0], other):
             assert torch.equal(a, b)
     eng.close()
+
+
+def test_the_feedback_of_context_lengths_changes_no_route():
+    """The first step's copy of the real lengths (a hundred tokens) has arrived when the second is enqueued and lowers the
+    host's bound: the second step takes the kernels that the calls alone decide on (here by the bound of 250)."""
+    cfg = dict(BASE, d_model=1024, n_heads=8, d_rnn=1024, max_batch=16, beam_width=16, max_ctx=400)
+    eng = ReDrafter(cfg, synth.make_weights(cfg, "cuda:0"))
+    rng = np.random.default_rng(26)
+    eng.set_state(dev(np.full(16, 100)), dev(rng.integers(0, cfg["vocab"], size=16)), torch.randn(16, 1024, device="cuda"), ctx_bound=250)
+    seen = []
+    for _ in range(2):
+        before = eng.route_counts()
+        eng.step(dev(rng.integers(0, cfg["vocab"], size=(16, 16, cfg["beam_length"]))))
+        eng.poll()
+        after = eng.route_counts()
+        seen.append({k: after[k] - before[k] for k in after})
+    assert seen[0]["att_rows128_tc5"] == cfg["n_layers"] and seen[0] == seen[1]
+    eng.close()
