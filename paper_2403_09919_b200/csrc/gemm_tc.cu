@@ -523,16 +523,19 @@ __device__ __forceinline__ void umma_commit_pair(uint32_t cluster_bar) {
 
 constexpr uint32_t SWAP_BYTES = 2 * 2 * 2 * 8 * 64 * 4;
 constexpr uint32_t ROW_INFO_BYTES = 2 * 256 * 8;
-// Row tiles of a launch of whole tiles: whole tiles run in waves of n_clusters, so the fewest waves times the cost of a tile win
-// (a tile's k-block costs its rows, and 64 rows' worth for its share of the weights).
-__host__ __device__ __forceinline__ GemmRows whole_row_tiles(int M, int mt, int n_wt, int n_clusters) {
+// Row tiles of a launch of whole tiles: whole tiles run in waves of n_clusters, so the fewest waves times the cost of a tile win.
+// A tile's k-block costs its rows, and WHOLE_WEIGHT_ROWS rows' worth for its share of the weights.  (64 instead of 128 cut 208 to
+// 340 rows into tiles too small: verification of 8 layers of the 7B shape, 256 rows 1.64 -> 1.55 ms, 336 rows 2.16 -> 1.99; 13B,
+// 6 layers, 568 rows 3.15 -> 3.00; 7B 1056 rows 4.67 -> 4.36; 96 and 192 lie between or level; nothing slower, 33B level.)
+constexpr int WHOLE_WEIGHT_ROWS = 128;
+__host__ __device__ __forceinline__ GemmRows whole_row_tiles(int M, int mt, int n_wt, int n_clusters, int weight_rows = WHOLE_WEIGHT_ROWS) {
   GemmRows best;
   int cost = 0x7fffffff;
   const int n0 = M > mt ? (M + mt - 1) / mt : 1;
   for (int n = n0; n < n0 + 4; ++n) {
     int rows = ((M + n - 1) / n + 15) & ~15;
     rows = rows < 16 ? 16 : rows > mt ? mt : rows;
-    const int c = (n_wt * n + n_clusters - 1) / n_clusters * (rows + 64);
+    const int c = (n_wt * n + n_clusters - 1) / n_clusters * (rows + weight_rows);
     if (c < cost) { cost = c; best = GemmRows(n, rows); }
   }
   return best;
@@ -1069,9 +1072,10 @@ static cudaError_t launch_gemm_tc2(const void* map_w, const void* const map_a[16
   return cudaGetLastError();
 }
 
-// What a launch of whole tiles over M rows leaves idle: tiles per cluster missing in the last wave, and rows of a tile.
+// What a launch of whole tiles over M rows leaves idle: tiles per cluster missing in the last wave, and rows of a tile.  (Tiles
+// chosen with weights as 64 rows: the constants of the rule that asks for it were fitted so.)
 void tc_whole_idle(int M, int m_max, int n_wt, int n_clusters, double* idle_tiles, double* tile_rows) {
-  const GemmRows g = whole_row_tiles(M, tc_pick_mt(m_max), n_wt, n_clusters);
+  const GemmRows g = whole_row_tiles(M, tc_pick_mt(m_max), n_wt, n_clusters, 64);
   const int tiles = n_wt * g.n, waves = (tiles + n_clusters - 1) / n_clusters;
   *idle_tiles = waves - (double)tiles / n_clusters;
   *tile_rows = g.rows;

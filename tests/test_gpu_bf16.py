@@ -399,7 +399,7 @@ def test_projection_on_cta_pairs_matches_the_one_cta_kernel(bw, batch, prompt):
 
 
 @pytest.mark.parametrize("bw,batch,prompt,d_ffn,heads", [(4, 1, 17, 64, 4), (8, 1, 129, 1376, 3), (16, 3, 300, 1440, 4), (32, 2, 700, 1040, 1),
-                                                         (8, 1, 1024, 9504, 5)])
+                                                         (8, 1, 1024, 9504, 5), (8, 2, 170, 9504, 1), (16, 3, 87, 11008, 1)])
 def test_projections_with_their_functions_match_the_separate_kernels(bw, batch, prompt, d_ffn, heads):
     """gate|up with SwiGLU and QKV with rotary embedding and cache write in their epilogues against projection and kernel:
     one tile, half tiles at the end (d_ffn / 64 odd or not whole; an odd number of heads), one row tile to several, more
