@@ -96,7 +96,7 @@ struct rd_handle {
   int tc_grid, tc_smem;
   const int32_t* att_seq_order = nullptr;   // sequences longest first for the pass being enqueued, or nullptr
   int tc_pairs;   // CTA pairs of the pair projection kernel that fit the device at once (0: not used)
-  int tc_pairs_avail, tc_pairs_min_rows;   // the pairs the device offers; row bound from which launches use them
+  int tc_pairs_avail, tc_pairs_min_rows;   // the pairs the device offers; row bound from which launches use them (0: the rules' own)
   bool tc_pairs_prefill;
   int qkv_min_rows;      // likewise for QKV and the rotary embedding
   int swiglu_min_rows;   // row bound from which gate|up takes SwiGLU along (0: use_fused_swiglu's own)
@@ -331,7 +331,7 @@ int gemm(rd_handle* h, const void* A, int lda, const void* W, int N, int K, cons
     // actual row count); made on first use
     const void* amaps[16];
     // (on CTA pairs each CTA loads half a row tile: heights 8..mt/2 in steps of 8)
-    const int pairs = tc_use_pairs(m_max, N, h->tc_grid, h->tc_pairs, h->tc_pairs_min_rows) ? h->tc_pairs : 0;
+    const int pairs = tc_use_pairs(m_max, N, h->tc_grid, h->tc_pairs, h->tc_pairs_min_rows > 0 ? h->tc_pairs_min_rows : 512) ? h->tc_pairs : 0;
     if (int rc = act_maps_of(h, A, K, mt, pairs ? 8 : 16, amaps)) return rc;
     int tr_slot = -1;
     unsigned long long* tr = gemm_trace_slot(h, (double)N * K * esize(h->dm.dtype), &tr_slot);
@@ -349,14 +349,26 @@ int gemm(rd_handle* h, const void* A, int lda, const void* W, int N, int K, cons
   return RD_OK;
 }
 
+int whole_clusters(const rd_handle* h) { return h->tc_pairs_avail < h->tc_grid / 2 ? h->tc_pairs_avail : h->tc_grid / 2; }
+
+// Whether a verification pass bounded by m_max rows runs on CTA pairs: from a bound of 640 rows, and from 512 where at half the
+// bound gate|up's whole tiles fill nine tenths of their waves.  8 layers, bounds of 528 and 574 rows with 0.25 / 0.4 / 0.5 / 0.75 of
+// them present, single CTAs -> pairs: 13B (fill 0.97) -5 / -8 / -5 to -13 / -15 %, 33B (0.95) -3 to -6 / -8 to -10 / -4 to -13 /
+// -11 to -13 %; 7B (0.77) +1 to +4 / +1 / -3 to +7 / -4 %, bound 633 +4 / +4 / +1 / -10 %; bound 656 -1 / -3 / -3 / -11 %.
+bool verify_on_pairs(const rd_handle* h, int m_max) {
+  if (h->tc_pairs_min_rows > 0) return m_max >= h->tc_pairs_min_rows;
+  if (m_max < 512 || m_max >= 640 || h->tc_pairs_avail <= 0) return m_max >= 640;
+  return tc_whole_fill(m_max / 2, m_max, (2 * h->dm.F + 255) / 256, whole_clusters(h)) >= 0.9;
+}
+
 // Whether a pass bounded by m_max rows takes the gate|up projection with SwiGLU in its epilogue.  Measured against the
 // two kernels: prompt passes, whose bound is their row count, win from about 350 rows (8 layers of the 7B shape: 264 rows
 // 1548 -> 1584 us, 320 1581 -> 1596, 400 1824 -> 1721, 500 2110 -> 1944; 13B 300 rows 1660 -> 1553); a verification pass
 // brings about half of its bound (7B: bound 328 6.77 -> 7.04 ms, 644 2958 -> 2939 us at 312 rows, 656 4190 -> 3782 at
 // 529; 33B, 644: 17.1 -> 16.2 ms; 7B batch 16, 1296: 19.1 -> 17.6 ms).
 bool use_fused_swiglu(const rd_handle* h, int m_max, bool exact) {
-  const int min_rows = h->swiglu_min_rows > 0 ? h->swiglu_min_rows : exact ? 352 : 512;
-  return m_max >= min_rows && h->dm.F % 2 == 0 && tc_use_pairs(m_max, 2 * h->dm.F, h->tc_grid, h->tc_pairs_avail, 0);
+  const bool many = h->swiglu_min_rows > 0 ? m_max >= h->swiglu_min_rows : exact ? m_max >= 352 : m_max >= 512 && verify_on_pairs(h, m_max);
+  return many && h->dm.F % 2 == 0 && tc_use_pairs(m_max, 2 * h->dm.F, h->tc_grid, h->tc_pairs_avail, 0);
 }
 
 // Whether such a pass takes the QKV projection with rotary embedding and cache write in its epilogue.  It has few tiles, so
@@ -370,9 +382,9 @@ bool use_fused_qkv(const rd_handle* h, int m_max, bool exact) {
   if (dm.hd != 128 || !tc_use_pairs(m_max, 3 * dm.d, h->tc_grid, h->tc_pairs_avail, 0)) return false;
   if (h->qkv_min_rows > 0) return m_max >= h->qkv_min_rows;
   if (exact) return m_max >= 352;
-  if (m_max < 512) return false;
+  if (m_max < 512 || !verify_on_pairs(h, m_max)) return false;
   double idle_tiles, tile_rows;
-  tc_whole_idle(m_max / 2, m_max, (3 * dm.H + 1) / 2, h->tc_pairs_avail < h->tc_grid / 2 ? h->tc_pairs_avail : h->tc_grid / 2, &idle_tiles, &tile_rows);
+  tc_whole_idle(m_max / 2, m_max, (3 * dm.H + 1) / 2, whole_clusters(h), &idle_tiles, &tile_rows);
   return idle_tiles * (dm.d / 64) * (tile_rows + 64) * 1.4e-3 < 8.0 + (double)(m_max / 2) * dm.d * 5.5e-6;
 }
 
@@ -386,7 +398,7 @@ int gemm_qkv(rd_handle* h, const void* A, int layer, const RowTables& rt, int m_
   if (int rc = act_maps_of(h, A, dm.d, tc_pick_mt(m_max), 8, amaps)) return rc;
   int tr_slot = -1;
   unsigned long long* tr = gemm_trace_slot(h, bytes, &tr_slot);
-  const int pairs = h->tc_pairs_avail < h->tc_grid / 2 ? h->tc_pairs_avail : h->tc_grid / 2;
+  const int pairs = whole_clusters(h);
   CK(h, launch_gemm_qkv(&iw->second, amaps, h->ws.qkv, kv_plane_ptr(h, layer, 0), kv_plane_ptr(h, layer, 1), h->ws.rope_tab, rt, dm, m_max,
                         h->ws.status, pairs, h->tc_smem, tr, chain, st));
   if (tr_slot >= 0) h->trace_prefetch[tr_slot] = tc_last_prefetch_bytes();
@@ -405,7 +417,7 @@ int gemm_swiglu(rd_handle* h, const void* A, const void* W, int m_max, void* act
   if (int rc = act_maps_of(h, A, dm.d, tc_pick_mt(m_max), 8, amaps)) return rc;
   int tr_slot = -1;
   unsigned long long* tr = gemm_trace_slot(h, bytes, &tr_slot);
-  const int pairs = h->tc_pairs_avail < h->tc_grid / 2 ? h->tc_pairs_avail : h->tc_grid / 2;
+  const int pairs = whole_clusters(h);
   CK(h, launch_gemm_swiglu(&iw->second, amaps, dm.F, dm.d, h->ws.m_total, m_max, act, h->ws.status, pairs, h->tc_smem, tr, chain, st));
   if (tr_slot >= 0) h->trace_prefetch[tr_slot] = tc_last_prefetch_bytes();
   h->route[RD_ROUTE_GEMM_PAIRS]++;
@@ -715,11 +727,12 @@ int do_verify(rd_handle* h, const rd_packed& pk, cudaStream_t st, int32_t* argma
   CKP(h, PROF_MISC, launch_build_rows_tree(pk, w.ctx, w.row_tok, w.row_seq, w.row_pos, w.row_slot, w.row_ncache, w.row_local,
                                w.row_out_index, w.seq_off, w.seq_order, argmax, w.m_total, dm, B, w.status, st));
   h->att_seq_order = B <= 1024 ? w.seq_order : nullptr;   // the row tables of this pass carry the sequences' order
+  if (!verify_on_pairs(h, m_max)) h->tc_pairs = 0;
   int rc = forward_layers(h, pk.mask, m_max, B, dm.NMAX, h->w.lm_head, st);
   h->att_seq_order = nullptr;
-  if (rc) return rc;
   GemmOut g;
-  rc = gemm(h, w.hidden_t, dm.d, h->w.lm_head, dm.V, dm.d, w.m_total, m_max, w.logits, dm.V, &g, nullptr, st, /*pair=*/1);
+  if (!rc) rc = gemm(h, w.hidden_t, dm.d, h->w.lm_head, dm.V, dm.d, w.m_total, m_max, w.logits, dm.V, &g, nullptr, st, /*pair=*/1);
+  h->tc_pairs = h->tc_pairs_avail;
   if (rc) return rc;
   CKP(h, PROF_MISC, launch_argmax_rows(w.logits, g, dm.V, argmax, w.row_out_index, w.m_total, m_max, h->sampling, w.row_seq, w.row_pos, 1, st));
   if (hidden) CKP(h, PROF_MISC, launch_scatter_rows(w.hidden_f, dm.d, hidden, w.row_out_index, w.m_total, m_max, st));
@@ -790,7 +803,7 @@ int redrafter_init(const rd_config* cfg, const rd_weights* wt, void* kv_cache, s
     if (ce == cudaSuccess) ce = drafter_prepare(dm.dtype);
     if (ce != cudaSuccess) return init_fail(h, RD_ERR_CUDA, "kernel set-up: %s", cudaGetErrorString(ce));
   }
-  h->tc_pairs = 0; h->tc_pairs_avail = 0; h->tc_pairs_min_rows = 512; h->tc_pairs_prefill = false;
+  h->tc_pairs = 0; h->tc_pairs_avail = 0; h->tc_pairs_min_rows = 0; h->tc_pairs_prefill = false;
   int sms = 0;
   {
     int dev = 0;
@@ -806,11 +819,10 @@ int redrafter_init(const rd_config* cfg, const rd_weights* wt, void* kv_cache, s
     if (ce == cudaSuccess) ce = attn_t5_prepare(dm.hd, dm.MW);
     if (ce != cudaSuccess)
       return init_fail(h, RD_ERR_CUDA, "tensor-core path set-up: %s", cudaGetErrorString(ce));
-    // CTA-pair projections (tuning toggles, read when the handle is made): from a bound of 512 rows in decode steps
-    // (8 layers of the 7B shape, one-CTA kernel against pairs: 312 rows 2939 / 2967 us, 435 3157 / 3088, 529 3782 / 3764,
-    // 674 4631 / 4468; 33B with 287 rows 16.2 / 15.8 ms; smaller bounds bring too few rows for the pairs' later start); RD_TC_CTA2=0 never, RD_TC_CTA2_MIN the row bound, RD_TC_CTA2_PREFILL=1 also in prompt passes.
+    // CTA-pair projections (tuning toggles, read when the handle is made): the drafter takes them from 512 rows, verification by
+    // its own rule; RD_TC_CTA2=0 never, RD_TC_CTA2_MIN the row bound for both, RD_TC_CTA2_PREFILL=1 also in prompt passes.
     if (getenv("RD_TC_CTA2") && atoi(getenv("RD_TC_CTA2")) == 0) h->tc_pairs_avail = 0;
-    h->tc_pairs_min_rows = getenv("RD_TC_CTA2_MIN") ? atoi(getenv("RD_TC_CTA2_MIN")) : 512;
+    h->tc_pairs_min_rows = getenv("RD_TC_CTA2_MIN") ? atoi(getenv("RD_TC_CTA2_MIN")) : 0;
     h->tc_pairs_prefill = getenv("RD_TC_CTA2_PREFILL") && atoi(getenv("RD_TC_CTA2_PREFILL")) != 0;
     h->qkv_min_rows = getenv("RD_QKV_MIN") ? atoi(getenv("RD_QKV_MIN")) : 0;
     h->swiglu_min_rows = getenv("RD_SWIGLU_MIN") ? atoi(getenv("RD_SWIGLU_MIN")) : 0;   // tuning toggle, as those above

@@ -1081,6 +1081,12 @@ void tc_whole_idle(int M, int m_max, int n_wt, int n_clusters, double* idle_tile
   *tile_rows = g.rows;
 }
 
+// Share of its waves that a launch of whole tiles over M rows fills.
+double tc_whole_fill(int M, int m_max, int n_wt, int n_clusters) {
+  const int tiles = n_wt * whole_row_tiles(M, tc_pick_mt(m_max), n_wt, n_clusters).n;
+  return (double)tiles / ((tiles + n_clusters - 1) / n_clusters * n_clusters);
+}
+
 // A projection of whole tiles on CTA pairs with the function behind it in the epilogue.
 template <int MODE>
 static cudaError_t launch_whole(TcParams p, const void* map_w, const void* const map_a[16], int m_max, int pairs, int smem_limit, Chain* chain,

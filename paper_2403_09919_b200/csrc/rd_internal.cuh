@@ -95,6 +95,7 @@ cudaError_t launch_gemm_tc(const void* map_w, const void* const map_a[16], int N
 cudaError_t launch_gemm_swiglu(const void* map_w, const void* const map_a[16], int F, int K, const int32_t* m_total, int m_max, void* act,
                                int32_t* status, int pairs, int smem_limit, unsigned long long* trace, Chain* chain, cudaStream_t st);
 
+double tc_whole_fill(int M, int m_max, int n_wt, int n_clusters);
 void tc_whole_idle(int M, int m_max, int n_wt, int n_clusters, double* idle_tiles, double* tile_rows);
 cudaError_t launch_gemm_qkv(const void* map_w, const void* const map_a[16], float* qkv, void* kcache, void* vcache, const float* table,
                             const RowTables& rt, const Dims& dm, int m_max, int32_t* status, int pairs, int smem_limit,
