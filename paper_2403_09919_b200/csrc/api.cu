@@ -558,14 +558,17 @@ int forward_layers(rd_handle* h, const uint32_t* mask, int m_max, int n_seq, int
     att_wide = wide_waves < 0 || (wide_waves > 0 && blocks > wide_waves * h->tc_grid);   // negative: always
     static const int t5_ok = getenv("RD_ATT_T5") ? atoi(getenv("RD_ATT_T5")) : 1;   // tuning toggle
     // (its 128-row tiles and 128-key chunks pay off when a sequence brings several hundred rows to the launch -- prompt
-    // processing -- or, in a verification pass, when a sequence fills at least half a tile and there are three chunks of
-    // keys: 8 layers of the 7B shape, 64-row kernel against this one, batch x context x beam width: 4 x 300 x 16 2363 ->
-    // 2298 us, 8 x 500 x 16 3368 -> 3216, 4 x 300 x 32 2981 -> 2945, 2 x 500 x 64 2995 -> 2864; 8 x 200 x 16 3136 -> 3147,
-    // 8 x 100 x 16 3062 -> 3107; the batched 7B step took 17.5 instead of 17.9 ms.  RD_ATT_T5=2 takes it whenever the
-    // 64-row kernel would run.)
+    // processing -- or, in a verification pass, when a sequence can fill at least half a tile and the context is long; from
+    // three chunks of keys on where a sequence can bring 96 rows or its tiles take a single wave.  4 layers, 64-row kernel ->
+    // this one, with 0.3 / 0.45 / 0.6 / 0.8 of the bound present: 7B 10 sequences of up to 106 rows, 400 tokens -1 / -3 / -3 /
+    // -2 %; 4 of 161, 400 tokens -1 / -3 / -4 / -6; 4 of 81 (128 tiles, one wave), 400 tokens -4 / -5 / -7 / -6; 13B 3 of 201,
+    // 260 tokens -5 / +2 / -5 / -6; but 16 of 81 (512 tiles) +4 / 0 / +3 / -4 at 260 tokens and +2 / +7 / +1 / -7 at 400, 33B
+    // 12 of 81 +4 / +2 / +2 / -2 and +7 / +4 / +2 / 0; the batched 7B step of 256 to 2048 tokens took 17.5 instead of 17.9 ms.
+    // RD_ATT_T5=2 takes it whenever the 64-row kernel would run.)
     static const int t5_rows = getenv("RD_ATT_T5_ROWS") ? atoi(getenv("RD_ATT_T5_ROWS")) : 64;   // tuning toggle
-    const bool t5_pays = rows_per_seq_max >= 512 ||
-                         (rows_per_seq_max >= t5_rows && h->route_bound + rows_per_seq_max >= (mask ? 320 : 1024));
+    const int t5_tiles = dm.H * n_seq * ((rows_per_seq_max + attn_t5_rows_per_block() - 1) / attn_t5_rows_per_block());
+    const int t5_keys = mask && (rows_per_seq_max >= 96 || t5_tiles <= h->tc_grid) ? 320 : 1024;
+    const bool t5_pays = rows_per_seq_max >= 512 || (rows_per_seq_max >= t5_rows && h->route_bound + rows_per_seq_max >= t5_keys);
     att_t5 = att_wide && !h->kv_maps.empty() && ((t5_ok == 1 && t5_pays) || t5_ok >= 2);
     if (att_t5) row_blocks = (rows_per_seq_max + attn_t5_rows_per_block() - 1) / attn_t5_rows_per_block();
     else if (att_wide) row_blocks = (rows_per_seq_max + attn_wide_rows_per_block() - 1) / attn_wide_rows_per_block();

@@ -113,6 +113,20 @@ def test_ragged_batch_long_contexts_take_the_tcgen05_kernel():
     assert route["att_rows128_tc5"] == cfg["n_layers"] and route["att_rows64"] == 0 and route["att_rows16"] == 0
 
 
+@pytest.mark.parametrize("heads,batch,bw,longest,tc5", [(8, 16, 16, 238, False), (8, 16, 16, 239, True),      # 128 tiles: one wave
+                                                       (16, 12, 20, 218, False), (16, 12, 20, 219, True),    # up to 101 rows
+                                                       (16, 16, 16, 942, False), (16, 16, 16, 943, True)])   # 81 rows, 256 tiles
+def test_verification_lines_of_the_tcgen05_kernel(heads, batch, bw, longest, tc5):
+    """Head dimension 128, either side of 320 keys (one wave of 128-row tiles, or 96 rows and more) and of 1024 keys (fewer
+    rows on several waves): contexts from 40 tokens, less than a chunk of keys of either kernel's tiles, to the longest."""
+    d = 128 * heads
+    cfg = dict(BASE, d_model=d, n_heads=heads, d_rnn=d, max_batch=batch, beam_width=bw, max_ctx=longest + 1 + 5 * bw + 16)
+    lens = [40 + (longest - 40) * b // (batch - 1) for b in range(batch)]
+    route, n_max, n_sum = verify_on_long_contexts(cfg, lens, follow=[0, batch - 1], rho=0.3, seed=27)
+    took, other = ("att_rows128_tc5", "att_rows64") if tc5 else ("att_rows64", "att_rows128_tc5")
+    assert route[took] == cfg["n_layers"] and route[other] == 0 and route["att_rows16"] == 0
+
+
 def test_long_context_few_heads_splits_the_keys():
     """The 33B workload's context length on few CTAs: 4096-token prompts, batch 2, 4 heads, beam width 8 (41 rows):
     16-row tiles whose keys are split over several CTAs and merged by the last one to arrive."""
@@ -165,14 +179,14 @@ def test_key_splits_do_not_depend_on_the_hosts_bound(heads, head_dim, batch):
 def test_the_feedback_of_context_lengths_changes_no_route():
     """The first step's copy of the real lengths (a hundred tokens) has arrived when the second is enqueued and lowers the
     host's bound: the second step takes the kernels that the calls alone decide on (here by the bound of 250)."""
-    cfg = dict(BASE, d_model=1024, n_heads=8, d_rnn=1024, max_batch=16, beam_width=16, max_ctx=400)
+    cfg = dict(BASE, d_model=1024, n_heads=8, d_rnn=1024, max_batch=16, beam_width=20, max_ctx=420)
     eng = ReDrafter(cfg, synth.make_weights(cfg, "cuda:0"))
     rng = np.random.default_rng(26)
     eng.set_state(dev(np.full(16, 100)), dev(rng.integers(0, cfg["vocab"], size=16)), torch.randn(16, 1024, device="cuda"), ctx_bound=250)
     seen = []
     for _ in range(2):
         before = eng.route_counts()
-        eng.step(dev(rng.integers(0, cfg["vocab"], size=(16, 16, cfg["beam_length"]))))
+        eng.step(dev(rng.integers(0, cfg["vocab"], size=(16, 20, cfg["beam_length"]))))
         eng.poll()
         after = eng.route_counts()
         seen.append({k: after[k] - before[k] for k in after})
