@@ -318,7 +318,9 @@ enum {
   RD_ROUTE_GEMM_PAIRS = 6,        /* projections on CTA pairs */
   RD_ROUTE_GEMM_ONE_CTA = 7,      /* projections on single CTAs (tensor cores) */
   RD_ROUTE_GEMM_SIMT = 8,         /* projections on CUDA cores */
-  RD_ROUTE_COUNT = 9
+  RD_ROUTE_GEMM_SWIGLU = 9,       /* of those on CTA pairs: gate|up with SwiGLU behind it */
+  RD_ROUTE_GEMM_QKV = 10,         /* of those on CTA pairs: QKV with rotary embedding and cache write behind it */
+  RD_ROUTE_COUNT = 11
 };
 RD_API int redrafter_route_counts(const rd_handle* h, int64_t* out, int32_t n);
 

@@ -403,6 +403,7 @@ int gemm_qkv(rd_handle* h, const void* A, int layer, const RowTables& rt, int m_
                         h->ws.status, pairs, h->tc_smem, tr, chain, st));
   if (tr_slot >= 0) h->trace_prefetch[tr_slot] = tc_last_prefetch_bytes();
   h->route[RD_ROUTE_GEMM_PAIRS]++;
+  h->route[RD_ROUTE_GEMM_QKV]++;
   return RD_OK;
 }
 
@@ -421,6 +422,7 @@ int gemm_swiglu(rd_handle* h, const void* A, const void* W, int m_max, void* act
   CK(h, launch_gemm_swiglu(&iw->second, amaps, dm.F, dm.d, h->ws.m_total, m_max, act, h->ws.status, pairs, h->tc_smem, tr, chain, st));
   if (tr_slot >= 0) h->trace_prefetch[tr_slot] = tc_last_prefetch_bytes();
   h->route[RD_ROUTE_GEMM_PAIRS]++;
+  h->route[RD_ROUTE_GEMM_SWIGLU]++;
   return RD_OK;
 }
 

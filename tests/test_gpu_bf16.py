@@ -398,12 +398,13 @@ def test_projection_on_cta_pairs_matches_the_one_cta_kernel(bw, batch, prompt):
     assert rel_err(outs[0][2], outs[1][2]) < 1e-2
 
 
-@pytest.mark.parametrize("bw,batch,prompt,d_ffn,heads", [(4, 1, 17, 64, 4), (8, 1, 129, 1376, 3), (16, 3, 300, 1440, 4), (32, 2, 700, 1040, 1),
+@pytest.mark.parametrize("bw,batch,prompt,d_ffn,heads", [(4, 1, 17, 64, 4), (4, 1, 17, 72, 4), (8, 1, 129, 1376, 3), (16, 3, 300, 1440, 4), (32, 2, 700, 1040, 1),
                                                          (8, 1, 1024, 9504, 5), (8, 2, 170, 9504, 1), (16, 3, 87, 11008, 1)])
 def test_projections_with_their_functions_match_the_separate_kernels(bw, batch, prompt, d_ffn, heads):
     """gate|up with SwiGLU and QKV with rotary embedding and cache write in their epilogues against projection and kernel:
-    one tile, half tiles at the end (d_ffn / 64 odd or not whole; an odd number of heads), one row tile to several, more
-    tiles than CTA pairs.  Sums differ in their grouping only (tolerance as between the projection kernels)."""
+    a gate|up of one tile, which keeps the separate kernels, and of one and an eighth; half tiles at the end (d_ffn / 64 odd or
+    not whole; an odd number of heads), one row tile to several, more tiles than CTA pairs.  Sums differ in their grouping
+    only (tolerance as between the projection kernels).  Prompt and verification each run the form that they are meant to."""
     d = 128 * heads
     cfg = dict(RAGGED, d_model=d, d_rnn=d, n_heads=heads, d_ffn=d_ffn, beam_width=bw, max_batch=batch, max_ctx=prompt + 200)
     outs, roots = [], None
@@ -415,8 +416,12 @@ def test_projections_with_their_functions_match_the_separate_kernels(bw, batch, 
             roots = r.eng.get_state()[1].clone()
         r.eng.set_state(None, roots, None)
         pk = r.eng.pack(dev(np.random.default_rng(1).integers(0, 3, size=(batch, bw, 5))))
+        prompt_route = r.eng.route_counts()
         am, hid, lg = r.eng.verify(pk, want_logits=True)
         r.eng.poll()
+        for before, after in ((dict.fromkeys(prompt_route, 0), prompt_route), (prompt_route, r.eng.route_counts())):
+            assert (after["gemm_qkv"] > before["gemm_qkv"]) == (not outs)
+            assert (after["gemm_swiglu"] > before["gemm_swiglu"]) == (not outs and 2 * d_ffn > 128)
         outs.append((pk.n.cpu().numpy(), lg.cpu().numpy(), r.eng.get_state()[2].cpu().numpy(), r.eng.kv_view().float().cpu().numpy()))
         r.eng.close()
     assert (outs[0][0] == outs[1][0]).all()

@@ -89,9 +89,9 @@ def test_wide_beam_long_context_takes_the_tcgen05_kernel():
     assert route["att_rows128_tc5"] == cfg["n_layers"] and route["att_rows64"] == 0 and route["att_rows16"] == 0
 
 
-def test_ragged_batch_takes_the_64_row_kernel_below_a_thousand_keys():
-    """Batch 16, beam width 16 (up to 81 rows per sequence), contexts from 256 to 900 tokens (4 to 15 chunks of keys):
-    tree-masked 64-row tiles, every sequence with its own context length and row count."""
+def test_ragged_batch_takes_the_64_row_kernel_at_head_dimension_64():
+    """Batch 16, beam width 16 (up to 81 rows per sequence), contexts from 256 to 900 tokens (4 to 15 chunks of keys), heads
+    too small for the tcgen05 kernel: tree-masked 64-row tiles, every sequence with its own context length and row count."""
     cfg = dict(BASE, d_model=512, n_heads=8, d_rnn=512, max_batch=16, beam_width=16, max_ctx=900 + 81 + 16)
     lens = [int(x) for x in np.random.default_rng(22).integers(256, 901, size=16)]
     lens[0], lens[5], lens[15] = 900, 256, 640
@@ -102,8 +102,8 @@ def test_ragged_batch_takes_the_64_row_kernel_below_a_thousand_keys():
 
 def test_ragged_batch_long_contexts_take_the_tcgen05_kernel():
     """The batched 7B workload's regime: batch 16, beam width 16 (up to 81 rows per sequence), contexts from 256 to 2048
-    tokens (2 to 17 chunks of 128 keys): from a thousand keys up, sequences that can fill half a 128-row tile go
-    through the tcgen05 kernel (head dimension 128), every sequence with its own context length and row count, most of
+    tokens (2 to 17 chunks of 128 keys): sequences that can fill half a 128-row tile go through the tcgen05 kernel (head
+    dimension 128) from a thousand keys up, and these, whose tiles take one wave, from 320; every sequence with its own context length and row count, most of
     every tile unused."""
     cfg = dict(BASE, d_model=1024, n_heads=8, d_rnn=1024, max_batch=16, beam_width=16, max_ctx=2048 + 81 + 16)
     lens = [int(x) for x in np.random.default_rng(22).integers(256, 2049, size=16)]
@@ -191,4 +191,29 @@ def test_the_feedback_of_context_lengths_changes_no_route():
         after = eng.route_counts()
         seen.append({k: after[k] - before[k] for k in after})
     assert seen[0]["att_rows128_tc5"] == cfg["n_layers"] and seen[0] == seen[1]
+    eng.close()
+
+
+@pytest.mark.parametrize("d_ffn,beam,verify_fused", [(9472, (102, 5), False), (9472, (73, 7), True),      # bounds of 511 and 512 rows
+                                                     (1376, (58, 11), False), (1376, (71, 9), True)])     # ... of 639 and 640
+def test_lines_of_the_projections_with_their_functions(d_ffn, beam, verify_fused):
+    """gate|up with SwiGLU and QKV with rotary embedding: prompt passes from 352 rows; verification passes from a bound of 512
+    rows where gate|up's tiles fill their waves (74 pairs of weight tiles at d_ffn = 9472), else from 640."""
+    cfg = dict(BASE, d_model=128, n_heads=1, d_rnn=128, d_ffn=d_ffn, beam_width=beam[0], beam_length=beam[1], max_ctx=1100)
+    eng = ReDrafter(cfg, synth.make_weights(cfg, "cuda:0"))
+    rng = np.random.default_rng(28)
+
+    def fused(call):
+        before = eng.route_counts()
+        call()
+        eng.poll()
+        after = eng.route_counts()
+        n = {after[k] - before[k] for k in ("gemm_swiglu", "gemm_qkv")}
+        assert n in ({0}, {cfg["n_layers"]})
+        return n != {0}
+
+    for rows in (351, 352):
+        assert fused(lambda: eng.prefill([rng.integers(0, cfg["vocab"], size=rows)])) == (rows == 352)
+    pk = eng.pack(dev(rng.integers(0, cfg["vocab"], size=(1, *beam))))
+    assert fused(lambda: eng.verify(pk)) == verify_fused
     eng.close()
