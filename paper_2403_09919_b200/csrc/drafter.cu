@@ -74,9 +74,7 @@ __device__ __forceinline__ void act_store4(__nv_bfloat16* p, float a, float b, f
   u.y = *reinterpret_cast<const uint32_t*>(&hi);
   *reinterpret_cast<uint2*>(p) = u;
 }
-template <typename T> __device__ __forceinline__ float4 act_bias4(const T* p);
-template <> __device__ __forceinline__ float4 act_bias4<float>(const float* p) { return *reinterpret_cast<const float4*>(p); }
-template <> __device__ __forceinline__ float4 act_bias4<__nv_bfloat16>(const __nv_bfloat16* p) {
+__device__ __forceinline__ float4 act_bias4(const __nv_bfloat16* p) {
   const uint2 g = *reinterpret_cast<const uint2*>(p);
   const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&g.x));
   const float2 b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&g.y));
@@ -86,9 +84,8 @@ template <> __device__ __forceinline__ float4 act_bias4<__nv_bfloat16>(const __n
 // One float4 of one row per thread, small CTAs spread over all SMs (what bounds the kernel is the rate at
 // which one SM pulls data out of the L2).  The bias is a weight and every address is a launch constant: both
 // are dealt with before the wait; after it the thread loads, adds and stores.
-template <typename T>
-__global__ void __maxnreg__(88) act_kernel(GemmOut proj, const T* __restrict__ bias, const float* resid, int ld_resid,
-                                           float* __restrict__ out_f, T* __restrict__ out_t, int ld_out, int N,
+__global__ void __maxnreg__(88) act_kernel(GemmOut proj, const __nv_bfloat16* __restrict__ bias, const float* resid, int ld_resid,
+                                           float* __restrict__ out_f, __nv_bfloat16* __restrict__ out_t, int ld_out, int N,
                                            const int32_t* __restrict__ m_total, ChainSync cs) {
   chain_begin(cs);
   const int m = blockIdx.y;
@@ -100,9 +97,9 @@ __global__ void __maxnreg__(88) act_kernel(GemmOut proj, const T* __restrict__ b
   float4 bv = make_float4(0.f, 0.f, 0.f, 0.f);
   const float* rp = resid ? resid + (size_t)m * ld_resid + n : nullptr;
   float* of = out_f + (size_t)m * ld_out + n;
-  T* ot = out_t + (size_t)m * ld_out + n;
+  __nv_bfloat16* ot = out_t + (size_t)m * ld_out + n;
   if (active) {
-    bv = act_bias4<T>(bias + n);
+    bv = act_bias4(bias + n);
     if (fast) { src = gemm_src(proj, 1, m, n); gemm_src_pin(src); }
     asm volatile("" : "+l"(rp), "+l"(of), "+l"(ot));
   }
@@ -135,7 +132,7 @@ cudaError_t launch_act(const GemmOut& proj, const void* bias, const float* resid
                        void* out_t, int ld_out, int N, const int32_t* m_total, int m_max, Chain* chain, cudaStream_t st) {
   dim3 grid((N / 4 + ACT_THREADS - 1) / ACT_THREADS, m_max);
   const ChainSync cs = chain ? chain->link(grid.x * grid.y, true) : ChainSync{nullptr, 0u, nullptr, nullptr, nullptr};
-  launch_pdl(act_kernel<__nv_bfloat16>, grid, ACT_THREADS, 0, st, proj, (const __nv_bfloat16*)bias, resid, ld_resid, out_f,
+  launch_pdl(act_kernel, grid, ACT_THREADS, 0, st, proj, (const __nv_bfloat16*)bias, resid, ld_resid, out_f,
              (__nv_bfloat16*)out_t, ld_out, N, m_total, cs);
   return cudaGetLastError();
 }

@@ -349,8 +349,7 @@ __device__ __forceinline__ void store2(__nv_bfloat16* p, float a, float b) {
   *reinterpret_cast<__nv_bfloat162*>(p) = __floats2bfloat162_rn(a, b);
 }
 
-template <typename T>
-__global__ void __maxnreg__(88) rope_kv_kernel(float* __restrict__ qkv, GemmOut proj, T* __restrict__ kc, T* __restrict__ vc,
+__global__ void __maxnreg__(88) rope_kv_kernel(float* __restrict__ qkv, GemmOut proj, __nv_bfloat16* __restrict__ kc, __nv_bfloat16* __restrict__ vc,
                                                const float2* __restrict__ table, RowTables rt, Dims dm, int* status,
                                                ChainSync cs) {
   chain_begin(cs);
@@ -452,9 +451,8 @@ __global__ void __maxnreg__(88) rope_kv_kernel(float* __restrict__ qkv, GemmOut 
 constexpr int ROPW_THREADS = 256;
 constexpr int ROPW_COLS = 1024;     // one item (two adjacent dimensions and their partners half a head on) per thread
 constexpr int ROPW_STAGES = 3;      // 3 x 3 x 4 KB per CTA (static shared memory)
-template <typename T>
 __global__ void __launch_bounds__(ROPW_THREADS, 4)
-    rope_kv_wide_kernel(float* __restrict__ qkv, GemmOut proj, T* __restrict__ kc, T* __restrict__ vc,
+    rope_kv_wide_kernel(float* __restrict__ qkv, GemmOut proj, __nv_bfloat16* __restrict__ kc, __nv_bfloat16* __restrict__ vc,
                         const float2* __restrict__ table, RowTables rt, Dims dm, int* status, ChainSync cs) {
   chain_begin(cs);
   __shared__ __align__(128) float ring[ROPW_STAGES][3][ROPW_COLS];   // 36 KB
@@ -568,12 +566,12 @@ cudaError_t launch_rope_kv(float* qkv, const GemmOut& proj, void* kcache, void* 
     const int gy = (4 * wide_sm_count() + (int)gw.x - 1) / (int)gw.x;
     gw.y = gy < m_max ? gy : m_max;
     const ChainSync cs = chain ? chain->link(gw.x * gw.y, true) : ChainSync{nullptr, 0u, nullptr, nullptr, nullptr};
-    launch_pdl(rope_kv_wide_kernel<__nv_bfloat16>, gw, ROPW_THREADS, 0, st, qkv, proj, (__nv_bfloat16*)kcache, (__nv_bfloat16*)vcache,
+    launch_pdl(rope_kv_wide_kernel, gw, ROPW_THREADS, 0, st, qkv, proj, (__nv_bfloat16*)kcache, (__nv_bfloat16*)vcache,
                reinterpret_cast<const float2*>(table), rt, dm, status, cs);
     return cudaGetLastError();
   }
   const ChainSync cs = chain ? chain->link(grid.x * grid.y, true) : ChainSync{nullptr, 0u, nullptr, nullptr, nullptr};
-  launch_pdl(rope_kv_kernel<__nv_bfloat16>, grid, ROPE_THREADS, 0, st, qkv, proj, (__nv_bfloat16*)kcache, (__nv_bfloat16*)vcache,
+  launch_pdl(rope_kv_kernel, grid, ROPE_THREADS, 0, st, qkv, proj, (__nv_bfloat16*)kcache, (__nv_bfloat16*)vcache,
              reinterpret_cast<const float2*>(table), rt, dm, status, cs);
   return cudaGetLastError();
 }
@@ -587,8 +585,7 @@ constexpr int SWIGLU_THREADS = 128;
 constexpr int SWIGLU_ITEMS = 2;
 constexpr int SWIGLU_FOLD = 2;  // a gate|up tile is cut between two CTAs at most once the stream is longer than a tile per CTA
 
-template <typename T>
-__global__ void __maxnreg__(88) swiglu_kernel(GemmOut proj, T* __restrict__ out, int F, const int32_t* __restrict__ m_total,
+__global__ void __maxnreg__(88) swiglu_kernel(GemmOut proj, __nv_bfloat16* __restrict__ out, int F, const int32_t* __restrict__ m_total,
                                               ChainSync cs) {
   chain_begin(cs);
 #ifdef RD_PROBE_EMPTY_BODIES   // ceiling probe (a build flag, never in the shipped library): keep the hand-off, drop the work
@@ -604,7 +601,7 @@ __global__ void __maxnreg__(88) swiglu_kernel(GemmOut proj, T* __restrict__ out,
   const bool single = proj.m_tiles_max == 1 || M <= proj.mt;   // rows that fit one row tile after all
   const bool fast = single;
   GemmSrc sg[SWIGLU_ITEMS], su[SWIGLU_ITEMS];
-  T* dst[SWIGLU_ITEMS];
+  __nv_bfloat16* dst[SWIGLU_ITEMS];
   bool act[SWIGLU_ITEMS];
 #pragma unroll
   for (int k = 0; k < SWIGLU_ITEMS; ++k) {
@@ -655,9 +652,8 @@ __global__ void __maxnreg__(88) swiglu_kernel(GemmOut proj, T* __restrict__ out,
 constexpr int SWS_THREADS = 256;
 constexpr int SWS_COLS = 2048;      // two float4 per thread
 constexpr int SWS_STAGES = 4;       // 4 x (8 + 8) KB per CTA
-template <typename T>
 __global__ void __launch_bounds__(SWS_THREADS, 3)
-    swiglu_wide_kernel(GemmOut proj, T* __restrict__ out, int F, const int32_t* __restrict__ m_total, int32_t* status,
+    swiglu_wide_kernel(GemmOut proj, __nv_bfloat16* __restrict__ out, int F, const int32_t* __restrict__ m_total, int32_t* status,
                        ChainSync cs) {
   chain_begin(cs);
   extern __shared__ __align__(128) uint8_t sws_smem[];
@@ -744,7 +740,7 @@ __global__ void __launch_bounds__(SWS_THREADS, 3)
 // Once per handle (and so per device): opt-in of the kernels that take more than 48 KB of dynamic shared memory.
 cudaError_t elementwise_prepare() {
   const int smem = SWS_STAGES * 2 * SWS_COLS * (int)sizeof(float);
-  return cudaFuncSetAttribute(swiglu_wide_kernel<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  return cudaFuncSetAttribute(swiglu_wide_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
 }
 
 // proj: the gate|up projection [M][2F]; out: [M][F].  F must be a multiple of 4.
@@ -758,11 +754,11 @@ cudaError_t launch_swiglu(const GemmOut& proj, void* out_t, int F, const int32_t
     const int gy = (3 * wide_sm_count() + (int)grid.x - 1) / (int)grid.x;
     grid.y = gy < m_max ? gy : m_max;
     const ChainSync cs = chain ? chain->link(grid.x * grid.y, true) : ChainSync{nullptr, 0u, nullptr, nullptr, nullptr};
-    launch_pdl(swiglu_wide_kernel<__nv_bfloat16>, grid, SWS_THREADS, smem, st, proj, (__nv_bfloat16*)out_t, F, m_total, status, cs);
+    launch_pdl(swiglu_wide_kernel, grid, SWS_THREADS, smem, st, proj, (__nv_bfloat16*)out_t, F, m_total, status, cs);
     return cudaGetLastError();
   }
   const ChainSync cs = chain ? chain->link(grid.x * grid.y, true) : ChainSync{nullptr, 0u, nullptr, nullptr, nullptr};
-  launch_pdl(swiglu_kernel<__nv_bfloat16>, grid, SWIGLU_THREADS, 0, st, proj, (__nv_bfloat16*)out_t, F, m_total, cs);
+  launch_pdl(swiglu_kernel, grid, SWIGLU_THREADS, 0, st, proj, (__nv_bfloat16*)out_t, F, m_total, cs);
   return cudaGetLastError();
 }
 
@@ -1049,8 +1045,9 @@ cudaError_t launch_ar_finish(const int32_t* argmax_c, const float* hidden_c, int
 }
 
 // Row tables of a prompt pass.  Tokens and runs come with the launch: copies from pageable host memory (nine per pass, and a
-// wait for them) kept the GPU idle between passes (64 tokens of the fp32
-// configuration 156 -> 139 us, of the small bf16 model 238 -> 211, 100 tokens of 8 layers of the 7B shape 1121 -> 1094).
+// wait for them) kept the GPU idle between passes (a call and the reads of state and logits that follow it, back to back
+// between two events: 64 tokens of the fp32 configuration 156 -> 139 us, of the small bf16 model 238 -> 211, 100 tokens of 8
+// layers of the 7B shape 1121 -> 1094).
 __global__ void __launch_bounds__(256) prefill_rows_kernel(const __grid_constant__ PrefillRows p, int32_t* row_tok, int32_t* row_seq, int32_t* row_pos, int32_t* row_slot,
                                     int32_t* row_ncache, int32_t* row_local, int32_t* last_row, int32_t* seq_off, int32_t* m_total) {
   pdl_enter();
