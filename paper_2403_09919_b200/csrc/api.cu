@@ -363,9 +363,9 @@ bool verify_on_pairs(const rd_handle* h, int m_max) {
 
 // Whether a pass bounded by m_max rows takes the gate|up projection with SwiGLU in its epilogue.  Measured against the
 // two kernels: prompt passes, whose bound is their row count, win from about 350 rows (8 layers of the 7B shape: 264 rows
-// 1548 -> 1584 us, 320 1581 -> 1596, 400 1824 -> 1721, 500 2110 -> 1944; 13B 300 rows 1660 -> 1553); a verification pass
-// brings about half of its bound (7B: bound 328 6.77 -> 7.04 ms, 644 2958 -> 2939 us at 312 rows, 656 4190 -> 3782 at
-// 529; 33B, 644: 17.1 -> 16.2 ms; 7B batch 16, 1296: 19.1 -> 17.6 ms).
+// 1548 -> 1584 us, 320 1581 -> 1596, 400 1824 -> 1721, 500 2110 -> 1944; 13B 300 rows 1660 -> 1553); verification passes
+// wherever they run on CTA pairs (bound 1296 with 96 / 176 / 256 / 336 / 416 / 576 / 1056 rows present: 7B +2 / +1 / 0 / +1 /
+// -1 / -7 / -13 %, 13B -1 / -1 / -4 / -4 / -6 / -8 / -8, 33B -3 / -5 / -6 / 0 / 0 / -6 / -8).
 bool use_fused_swiglu(const rd_handle* h, int m_max, bool exact) {
   const bool many = h->swiglu_min_rows > 0 ? m_max >= h->swiglu_min_rows : exact ? m_max >= 352 : m_max >= 512 && verify_on_pairs(h, m_max);
   return many && h->dm.F % 2 == 0 && tc_use_pairs(m_max, 2 * h->dm.F, h->tc_grid, h->tc_pairs_avail, 0);

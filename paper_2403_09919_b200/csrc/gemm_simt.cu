@@ -10,8 +10,9 @@
 // MT running sums, so a weight is read once per MT activation rows; these go through shared memory SIMT_CHUNK columns
 // at a time, once for the CTA's eight warps.  The first chunk's weights are requested before the wait.  What a row's
 // sums are does not depend on MT or on the other rows, so that verification and autoregressive steps agree bit for bit.
-// Measured on the fp32 configuration (d = 256, 2 layers): a step of 17 rows takes 172 us (259 with one kernel per
-// function and grid dependencies), a 64-token prompt 116 us (154), 16 prompts of 300 tokens 2.94 ms (3.18).
+// Measured on the fp32 configuration (d = 256, 2 layers), calls back to back between two events, against one kernel per
+// function and grid dependencies: a step of 14 rows 271 -> 177 us, a 64-token prompt 153 -> 88, 16 prompts of 300 tokens 3.19
+// -> 2.83 ms (the prompts with what their row tables no longer cost, see prefill_rows_kernel).
 #include "rd_internal.cuh"
 #include "pdl.cuh"
 
@@ -20,7 +21,9 @@ namespace rd {
 constexpr int SIMT_WARPS = 8;
 constexpr int SIMT_CHUNK = 512;   // columns of the activation rows in shared memory at a time
 // Launches bounded by more rows than this are bound by the CTAs an SM can hold and by the activations' way out of shared
-// memory: they request weights as they are needed (64 registers, four CTAs) and give a warp two weight rows always.
+// memory: they request weights as they are needed (64 registers, four CTAs, though 8 to 84 bytes a
+// thread spill: with three CTAs and no spills 16 prompts of 300 tokens take 3.77 ms instead of 2.83) and give a warp two
+// weight rows always.
 // Requesting ahead throughout: 16 prompts of 300 tokens 3.67 ms instead of 2.94; a line at 16 rows instead of 64: steps of
 // 17 to 41 rows 2 % slower.
 constexpr int SIMT_FEW_ROWS = 64;

@@ -547,12 +547,12 @@ __host__ __device__ __forceinline__ GemmRows whole_row_tiles(int M, int mt, int 
 // cluster c takes tiles c, c + C, ... of the (weight tile, row tile) list, row tile fastest, so the row tiles of a weight
 // tile run side by side; what whole tiles leave idle in the last wave is kept small by the choice of row tile
 // (whole_row_tiles).  The two-kernel form writes the sums as fp32 and reads them back (90 MB at 1024 rows of the 7B
-// shape, more than the L2 keeps, and the kernel between them): 133 + 4 + 34 us per layer there, now 140; a 512-token prompt
-// 9.21 -> 8.54 ms, 8192 tokens 153 -> 141 ms, the batch-16 step 19.1 -> 17.6 ms.
+// shape, more than the L2 keeps): 136 + 36 us per layer there, now 130 at 1.42 PFLOP/s (ncu, every launch alone with a cold L2);
+// in the running pass, between events, 8 layers 3568 -> 3256 us; a 512-token prompt 9.21 -> 8.54 ms, 8192 tokens 153 -> 141 ms.
 // QKV: likewise the QKV projection of a model with 128-dimensional heads, where a weight tile is one head of Q, K or V and lanes
 // i and i + 64 hold a rotary pair: rotated Q goes to the fp32 buffer that attention reads, rotated K and V to the cache.
-// QKV + rotary of a 1024-row prompt pass: 79 + 3 + 19 us per layer as two kernels; a 512-token prompt 8.32 -> 7.92 ms, 8192
-// tokens 137 -> 131 ms, the batch-16 step 17.1 -> 16.6 ms.
+// QKV + rotary of a 1024-row prompt pass: 80 + 27 us per layer as two kernels, now 81 (ncu, as above); between events 8 layers
+// 3256 -> 3054 us; a 512-token prompt 8.32 -> 7.92 ms, 8192 tokens 137 -> 131 ms, the batch-16 step 17.1 -> 16.6 ms.
 enum { TC2_PLAIN = 0, TC2_SWIGLU = 1, TC2_QKV = 2 };
 template <int EW, int MODE>
 __global__ void __launch_bounds__(tc_threads(EW), EW == 4 ? 4 : 2) gemm_tc2_kernel(const __grid_constant__ CUtensorMap map_w,
