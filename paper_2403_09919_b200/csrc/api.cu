@@ -548,7 +548,7 @@ int forward_layers(rd_handle* h, const uint32_t* mask, int m_max, int n_seq, int
                                       w.m_total, m_max, w.status, st));
   // attention launch geometry (tensor-core path): tiles of 16 rows per sequence; keys split over CTAs only
   // for long contexts with few tiles
-  int row_blocks = 1, n_splits = 1, split_chunks = 1;
+  int row_blocks = 1, n_splits = 1, split_chunks = 1, split_min = 1;
   bool att_wide = false, att_shallow = false, att_t5 = false;
   if (h->use_tc) {
     const int rpb = attn_tc_rows_per_block();
@@ -577,16 +577,22 @@ int forward_layers(rd_handle* h, const uint32_t* mask, int m_max, int n_seq, int
     // more 16-row CTAs than SMs (many sequences of a few rows): a two-chunk ring so that three CTAs share an SM
     static const int shallow_ok = getenv("RD_ATT_SHALLOW") ? atoi(getenv("RD_ATT_SHALLOW")) : 1;   // tuning toggle
     // Keys split over CTAs: with fewer tiles than half the SMs, one CTA per SM and at least three chunks each; with more, up
-    // to three CTAs per SM (short ring) of at least six chunks, which also evens out sequences of different lengths.  (8
-    // layers of the 7B shape, one split per SM and eight chunks before: autoregressive, 1 x 600 tokens 822 -> 807 us; 4 x
-    // 1100 940 -> 934; 2 x 800 tokens with 58 rows 1988 -> 1940.  Three per SM for few tiles too: 1 x 3000 877 -> 896; of
-    // three chunks: the 7B step at 512 tokens 8.35 -> 8.66 ms; two chunks each for few tiles: small steps 1.60 -> 1.64.)
+    // to three CTAs per SM (short ring) of at least six chunks, which also evens out sequences of different lengths -- but where
+    // the tiles alone leave no SM a second one, three splits or none.  (8 layers of the 7B shape, one split per SM and eight
+    // chunks before: autoregressive, 1 x 600 tokens 822 -> 807 us; 4 x 1100 940 -> 934; 3 x 2000 1026 -> 967; 2 x 800 tokens
+    // with 58 rows 1988 -> 1940.  Three per SM for few tiles too: 1 x 3000 877 -> 896; of three chunks: the 7B step at 512
+    // tokens 8.35 -> 8.66 ms; two chunks each for few tiles: small steps 1.60 -> 1.64; two splits of 96 tiles, whose 192 CTAs
+    // load the SMs unevenly and lose the long ring: a step at 1000 tokens 1841 instead of 1782 us, autoregressive, 3 x 800 907
+    // instead of 874.  Launches of fewer than 16 heads keep two splits: of the models here only the tests' have so few, and
+    // that a sequence of one chunk leaves a split empty is checked on them; without, 4 layers at 760 tokens 563 -> 534 us.)
     // The kernel takes the real lengths for it; the host's bound only limits the launch.
     const int max_chunks = (h->ctx_bound + rows_per_seq_max + 63) / 64;
     const bool few = 2 * blocks <= h->tc_grid;
     split_chunks = few ? 3 : 6;
+    split_min = !few && blocks <= h->tc_grid && dm.H >= 16 ? 3 : 1;
     n_splits = (few ? h->tc_grid : 3 * h->tc_grid) / blocks;
     if (n_splits > max_chunks / split_chunks) n_splits = max_chunks / split_chunks;
+    if (n_splits < split_min) n_splits = 1;
     if (n_splits > 16) n_splits = 16;
     if (n_splits < 1) n_splits = 1;
     while (n_splits > 1 && (long long)blocks * n_splits > ATT_MAX_SPLIT_BLOCKS) --n_splits;
@@ -631,7 +637,7 @@ int forward_layers(rd_handle* h, const uint32_t* mask, int m_max, int n_seq, int
                                     row_blocks, ch, st));
       else
         CK(h, launch_attention_tc(w.qkv, kv_plane_ptr(h, l, 0), kv_plane_ptr(h, l, 1), w.attn_t, rt, w.seq_off, dm, n_seq,
-                                  row_blocks, n_splits, split_chunks, w.att_scratch, w.att_counters,
+                                  row_blocks, n_splits, split_chunks, split_min, w.att_scratch, w.att_counters,
                                   (h->trace_next >= 0 && h->trace_next < TRACE_SLOTS) ? w.trace + (size_t)8 * h->trace_next++ : nullptr, ch,
                                   att_shallow ? 1 : 0, st));
     }

@@ -57,7 +57,7 @@ __global__ void __launch_bounds__(128) attention_tc_kernel(const float* __restri
                                                            const __nv_bfloat16* __restrict__ vc,
                                                            __nv_bfloat16* __restrict__ out, RowTables rt,
                                                            const int32_t* __restrict__ seq_off, Dims dm, int row_tiles,
-                                                           int split_chunks, float* __restrict__ scratch,
+                                                           int split_chunks, int split_min, float* __restrict__ scratch,
                                                            int32_t* __restrict__ counters, unsigned long long* dbg, ChainSync cs) {
   unsigned long long t_dbg[6] = {0, 0, 0, 0, 0, 0};
   RD_STAMP(0);
@@ -86,8 +86,9 @@ __global__ void __launch_bounds__(128) attention_tc_kernel(const float* __restri
   const int b = blockIdx.y / row_tiles, rb = blockIdx.y - b * row_tiles;
   const int z = blockIdx.z;
   const bool tree = rt.mask != nullptr;
-  // as many splits as leave each split_chunks chunks of the longest sequence
-  const int n_splits = gridDim.z == 1 ? 1 : min(max((min(rt.m_total[1], dm.max_ctx) + KEYS - 1) / KEYS / split_chunks, 1), (int)gridDim.z);
+  // as many splits as leave each split_chunks chunks of the longest sequence; none where that is fewer than split_min
+  int n_splits = min((min(rt.m_total[1], dm.max_ctx) + KEYS - 1) / KEYS / split_chunks, (int)gridDim.z);
+  if (n_splits < split_min) n_splits = 1;
   const int seq_row0 = seq_off[b], seq_rows = seq_off[b + 1] - seq_row0;
   const int row0 = seq_row0 + rb * ROWS;
   const int nrows = min(ROWS, seq_rows - rb * ROWS);
@@ -453,15 +454,15 @@ cudaError_t attn_tc_prepare(int hd, int MW) {
 }
 
 // grid (H, sequences * row_tiles, n_splits); n_splits: the most that the keys may be split, split_chunks: the fewest chunks of
-// the longest sequence that a split is worth; `shallow`: more CTAs than SMs, so several should share an SM
+// the longest sequence that a split is worth; split_min (>= 1): the fewest splits that are worth it; `shallow`: more CTAs than SMs, so several should share an SM
 cudaError_t launch_attention_tc(const float* qkv, const void* kcache, const void* vcache, void* out, const RowTables& rt,
                                 const int32_t* seq_off, const Dims& dm, int n_seq, int row_tiles, int n_splits,
-                                int split_chunks, float* scratch, int32_t* counters, unsigned long long* dbg, Chain* chain, int shallow, cudaStream_t st) {
+                                int split_chunks, int split_min, float* scratch, int32_t* counters, unsigned long long* dbg, Chain* chain, int shallow, cudaStream_t st) {
   dim3 grid(dm.H, n_seq * row_tiles, n_splits);
   const ChainSync cs = chain ? chain->link(grid.x * grid.y * grid.z) : ChainSync{nullptr, 0u, nullptr, nullptr, nullptr};
 #define RD_ATT_LAUNCH(HD, NST)                                                                                              \
   launch_pdl(attention_tc_kernel<HD, NST>, grid, 128, smem_bytes<HD, NST>(dm.MW), st, qkv, (const __nv_bfloat16*)kcache,    \
-             (const __nv_bfloat16*)vcache, (__nv_bfloat16*)out, rt, seq_off, dm, row_tiles, split_chunks, scratch, counters, dbg, cs)
+             (const __nv_bfloat16*)vcache, (__nv_bfloat16*)out, rt, seq_off, dm, row_tiles, split_chunks, split_min, scratch, counters, dbg, cs)
   if (dm.hd == 128) {
     if (shallow) RD_ATT_LAUNCH(128, NSTAGE_SHALLOW); else RD_ATT_LAUNCH(128, NSTAGE_DEEP);
   } else if (dm.hd == 64) {

@@ -127,7 +127,7 @@ int attn_tc_rows_per_block();
 cudaError_t attn_tc_prepare(int hd, int MW);
 cudaError_t launch_attention_tc(const float* qkv, const void* kcache, const void* vcache, void* out, const RowTables& rt,
                                 const int32_t* seq_off, const Dims& dm, int n_seq, int row_blocks, int n_splits,
-                                int split_chunks, float* scratch, int32_t* counters, unsigned long long* dbg, Chain* chain, int shallow, cudaStream_t st);
+                                int split_chunks, int split_min, float* scratch, int32_t* counters, unsigned long long* dbg, Chain* chain, int shallow, cudaStream_t st);
 cudaError_t elementwise_prepare();
 cudaError_t drafter_prepare(int dtype);
 cudaError_t launch_swiglu(const GemmOut& proj, void* out_t, int F, const int32_t* m_total, int m_max,

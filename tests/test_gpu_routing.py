@@ -176,6 +176,17 @@ def test_key_splits_do_not_depend_on_the_hosts_bound(heads, head_dim, batch):
     eng.close()
 
 
+@pytest.mark.parametrize("tokens,split", [(1007, False), (1008, True), (1100, True)])
+def test_tiles_of_one_wave_are_split_in_three_or_not_at_all(tokens, split):
+    """16 heads, one sequence of up to 81 rows: 96 tiles on 148 SMs.  Up to seventeen chunks of keys would make two splits and
+    stay whole.  From eighteen with all 81 rows (1008 tokens) the launch has three splits; the rows that are there leave
+    seventeen chunks at 1008 tokens, so the kernel keeps them whole, and eighteen at 1100.  Against the oracle each time."""
+    cfg = dict(BASE, d_model=2048, n_heads=16, d_rnn=2048, beam_width=16, max_ctx=1100 + 81 + 16)
+    route, n_max, n_sum = verify_on_long_contexts(cfg, [tokens], follow=[0], rho=0.3, seed=29)
+    assert 1008 + n_max <= 17 * 64
+    assert route["att_key_split"] == (cfg["n_layers"] if split else 0) and route["att_rows16"] + route["att_rows16_shallow"] == cfg["n_layers"]
+
+
 def test_the_feedback_of_context_lengths_changes_no_route():
     """The first step's copy of the real lengths (a hundred tokens) has arrived when the second is enqueued and lowers the
     host's bound: the second step takes the kernels that the calls alone decide on (here by the bound of 250)."""
