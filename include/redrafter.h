@@ -320,7 +320,8 @@ enum {
   RD_ROUTE_GEMM_SIMT = 8,         /* projections on CUDA cores */
   RD_ROUTE_GEMM_SWIGLU = 9,       /* of those on CTA pairs: gate|up with SwiGLU behind it */
   RD_ROUTE_GEMM_QKV = 10,         /* of those on CTA pairs: QKV with rotary embedding and cache write behind it */
-  RD_ROUTE_COUNT = 11
+  RD_ROUTE_ATT_KEYS_ON_LANES = 11,/* tiles of up to 96 rows on tcgen05, keys on the tensor-memory lanes */
+  RD_ROUTE_COUNT = 12
 };
 RD_API int redrafter_route_counts(const rd_handle* h, int64_t* out, int32_t n);
 

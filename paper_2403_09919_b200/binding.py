@@ -31,7 +31,7 @@ EXPORTS = ["redrafter_workspace_bytes", "redrafter_kv_bytes", "redrafter_init", 
            "redrafter_last_packed_rows"]
 
 ROUTES = ("att_rows16", "att_rows16_shallow", "att_rows64", "att_rows128_tc5", "att_key_split", "att_fp32", "gemm_pairs",
-          "gemm_one_cta", "gemm_simt", "gemm_swiglu", "gemm_qkv")
+          "gemm_one_cta", "gemm_simt", "gemm_swiglu", "gemm_qkv", "att_keys_on_lanes")
 
 
 class RdConfig(C.Structure):

@@ -56,6 +56,7 @@ struct Workspace {
   int32_t *att_counters, *sel_counters;
   unsigned int* chain_ctr;  // counters of the launch-to-launch hand-off
   float* att_scratch;
+  uint32_t* mask_t;   // [B][NMAX][MW] the pass's tree mask with rows and columns exchanged
   unsigned long long* trace;  // [TRACE_SLOTS][8] timestamps of traced projection launches
 };
 
@@ -98,9 +99,11 @@ struct rd_handle {
   int tc_pairs;   // CTA pairs of the pair projection kernel that fit the device at once (0: not used)
   int tc_pairs_avail, tc_pairs_min_rows;   // the pairs the device offers; row bound from which launches use them (0: the rules' own)
   bool tc_pairs_prefill;
+  int att_kl;            // attention with the keys on the lanes: 0 never, 1 by its rule, 2 wherever it can run
   int qkv_min_rows;      // likewise for QKV and the rotary embedding
   int swiglu_min_rows;   // row bound from which gate|up takes SwiGLU along (0: use_fused_swiglu's own)
   std::vector<TensorMapBox> kv_maps;   // [layer][K | V]: cache planes as [sequences * heads * max_ctx][head dim] matrices
+  std::vector<TensorMapBox> v_maps;    // [layer]: V planes of head dimension 128 as [2 halves][rows][64 dims]
   Chain chain;  // counter hand-off between the launches of a forward pass
   bool chain_allowed;   // RD_CHAIN=0: never hand over by counters
   bool chain_dirty;  // a launch failed after the chain had counted it: reset the counters before the next pass
@@ -237,6 +240,7 @@ void carve(Bump& bp, const Dims& dm, int m_cap, Workspace* w) {
   w->hist_b = bp.take<int32_t>((size_t)R * dm.L);
   w->tc_partial = bp.take<float>(dm.dtype == RD_DTYPE_BF16 ? tc_partial_floats(TC_MAX_GRID, tc_pick_mt(m_cap)) : 0);
   w->att_scratch = bp.take<float>(dm.dtype == RD_DTYPE_BF16 ? attn_tc_scratch_floats(ATT_MAX_SPLIT_BLOCKS, 1, dm.hd) : 0);
+  w->mask_t = bp.take<uint32_t>(dm.dtype == RD_DTYPE_BF16 ? (size_t)B * dm.NMAX * dm.MW : 0);
   w->trace = bp.take<unsigned long long>((size_t)TRACE_SLOTS * 8);
   bp.take<char>(256);
 }
@@ -537,6 +541,29 @@ int layers_simt(rd_handle* h, const RowTables& rt, int m_max, Chain* ch, cudaStr
   return RD_OK;
 }
 
+// Whether a pass takes the attention kernel with the keys on the lanes; `wide`: else it would take the 64- or 128-row kernel.
+// Measured per layer (4 layers, contexts of 60, 150-300, 500, 256-1024 and 2048 tokens, earlier kernel -> this one):
+// verification, 7B, 1 sequence of 30 / 82 rows -1 to -8 / -4 to -23 %; 4 of 32 -3 to -17; 8 of 30, 56, 85 -7 to 0, -8 to -1, -9 to 0;
+// 16 of 17, 30, 56 -12 to -5, -11 to -5, -9 to -3; 13B and 33B alike.  It loses
+// - where sequences of more than 64 rows leave every SM one wide tile, which the 64- and 128-row kernels walk as fast with less
+//   set-up (4 x 54 / 62 / 89 rows, 128 tiles: +1 to +5 / -1 to +9 / 0 to +9 %; 13B, 4 x 89, 160 tiles: +3 to -4), but where they
+//   can be cut into two tiles or more each, it is ahead again (152 rows, 32 tiles: -1 to -5);
+// - on several tiles per SM with less than a chunk of keys (60 tokens, 8 or 16 sequences: 0 to +3 %);
+// - in autoregressive steps of a single sequence, whose keys the 16-row kernel splits (7B +1 to +5 %, 33B -2 to +1), and of few
+//   keys (100 tokens: 0 to +3); 2 to 16 sequences of 500 to 2500 tokens -20 to 0, two points +1.5.
+// Models of fewer than 24 heads keep the earlier kernels, whose lines are held by tests; of the shapes here only the small models
+// of the tests have so few.
+bool use_keys_on_lanes(const rd_handle* h, bool tree, int n_seq, int rows_per_seq_max, bool wide) {
+  const Dims& dm = h->dm;
+  if (h->att_kl == 0 || h->kv_maps.empty() || !attn_kl_supported(dm.hd, dm.NMAX)) return false;
+  if (h->att_kl >= 2) return true;
+  const int tiles = dm.H * n_seq, G = h->tc_grid;
+  if (dm.H < 24) return false;
+  if (!tree) return rows_per_seq_max == 1 && tiles >= 64 && (h->route_bound >= 256 || tiles >= 3 * G);
+  if (wide && rows_per_seq_max > 64 && 2 * tiles > G && (tiles <= G || (rows_per_seq_max >= 96 && 4 * tiles <= 5 * G))) return false;
+  return tiles <= G || h->route_bound >= 128;
+}
+
 // Embedding -> n_layers x {attention block, FFN block} -> final norm.  Rows and masks come from the
 // row tables in the workspace; results: ws.hidden_f / ws.hidden_t (compact rows).
 int forward_layers(rd_handle* h, const uint32_t* mask, int m_max, int n_seq, int rows_per_seq_max, const void* after_w,
@@ -549,7 +576,7 @@ int forward_layers(rd_handle* h, const uint32_t* mask, int m_max, int n_seq, int
   // attention launch geometry (tensor-core path): tiles of 16 rows per sequence; keys split over CTAs only
   // for long contexts with few tiles
   int row_blocks = 1, n_splits = 1, split_chunks = 1, split_min = 1;
-  bool att_wide = false, att_shallow = false, att_t5 = false;
+  bool att_wide = false, att_shallow = false, att_t5 = false, att_kl = false;
   if (h->use_tc) {
     const int rpb = attn_tc_rows_per_block();
     row_blocks = (rows_per_seq_max + rpb - 1) / rpb;
@@ -597,6 +624,7 @@ int forward_layers(rd_handle* h, const uint32_t* mask, int m_max, int n_seq, int
     if (n_splits < 1) n_splits = 1;
     while (n_splits > 1 && (long long)blocks * n_splits > ATT_MAX_SPLIT_BLOCKS) --n_splits;
     att_shallow = shallow_ok && !att_wide && blocks * n_splits > h->tc_grid;
+    att_kl = t5_ok < 2 && wide_waves >= 0 && use_keys_on_lanes(h, mask != nullptr, n_seq, rows_per_seq_max, att_wide);
   }
   GemmOut g_qkv, g_o, g_gu, g_dn;
   // inside the layer loop every launch hands over to the next through a counter; the launches before
@@ -626,10 +654,13 @@ int forward_layers(rd_handle* h, const uint32_t* mask, int m_max, int n_seq, int
     }
     {
       ProfScope ps(h, 1, 0.0, st);
-      h->route[att_t5 ? RD_ROUTE_ATT_ROWS128_TC5 : att_wide ? RD_ROUTE_ATT_ROWS64
+      h->route[att_kl ? RD_ROUTE_ATT_KEYS_ON_LANES : att_t5 ? RD_ROUTE_ATT_ROWS128_TC5 : att_wide ? RD_ROUTE_ATT_ROWS64
                : att_shallow ? RD_ROUTE_ATT_ROWS16_SHALLOW : RD_ROUTE_ATT_ROWS16]++;
-      if (!att_t5 && !att_wide && n_splits > 1) h->route[RD_ROUTE_ATT_KEY_SPLIT]++;
-      if (att_t5)
+      if (!att_kl && !att_t5 && !att_wide && n_splits > 1) h->route[RD_ROUTE_ATT_KEY_SPLIT]++;
+      if (att_kl)
+        CK(h, launch_attention_kl(h->kv_maps[(size_t)l * 2].bytes, h->v_maps[l].bytes, w.qkv, w.attn_t, rt, w.seq_off, h->att_seq_order, w.mask_t, dm, n_seq,
+                                  attn_kl_row_tiles(rows_per_seq_max), h->tc_grid, w.status, ch, st));
+      else if (att_t5)
         CK(h, launch_attention_t5(h->kv_maps[(size_t)l * 2].bytes, h->kv_maps[(size_t)l * 2 + 1].bytes, w.qkv, w.attn_t, rt, w.seq_off, h->att_seq_order, dm, n_seq,
                                   row_blocks, w.status, ch, st));
       else if (att_wide)
@@ -736,7 +767,7 @@ int do_verify(rd_handle* h, const rd_packed& pk, cudaStream_t st, int32_t* argma
   const Dims& dm = h->dm;
   const int B = h->batch, m_max = B * dm.NMAX;
   CKP(h, PROF_MISC, launch_build_rows_tree(pk, w.ctx, w.row_tok, w.row_seq, w.row_pos, w.row_slot, w.row_ncache, w.row_local,
-                               w.row_out_index, w.seq_off, w.seq_order, argmax, w.m_total, dm, B, w.status, st));
+                               w.row_out_index, w.seq_off, w.seq_order, h->att_kl && attn_kl_supported(dm.hd, dm.NMAX) ? w.mask_t : nullptr, argmax, w.m_total, dm, B, w.status, st));
   h->att_seq_order = B <= 1024 ? w.seq_order : nullptr;   // the row tables of this pass carry the sequences' order
   if (!verify_on_pairs(h, m_max)) h->tc_pairs = 0;
   int rc = forward_layers(h, pk.mask, m_max, B, dm.NMAX, h->w.lm_head, st);
@@ -828,6 +859,7 @@ int redrafter_init(const rd_config* cfg, const rd_weights* wt, void* kv_cache, s
     if (ce == cudaSuccess) ce = attn_tc_prepare(dm.hd, dm.MW);
     if (ce == cudaSuccess) ce = attn_wide_prepare(dm.hd, dm.MW);
     if (ce == cudaSuccess) ce = attn_t5_prepare(dm.hd, dm.MW);
+    if (ce == cudaSuccess) ce = attn_kl_prepare(dm.hd);
     if (ce != cudaSuccess)
       return init_fail(h, RD_ERR_CUDA, "tensor-core path set-up: %s", cudaGetErrorString(ce));
     // CTA-pair projections (tuning toggles, read when the handle is made): the drafter takes them from 512 rows, verification by
@@ -835,6 +867,7 @@ int redrafter_init(const rd_config* cfg, const rd_weights* wt, void* kv_cache, s
     if (getenv("RD_TC_CTA2") && atoi(getenv("RD_TC_CTA2")) == 0) h->tc_pairs_avail = 0;
     h->tc_pairs_min_rows = getenv("RD_TC_CTA2_MIN") ? atoi(getenv("RD_TC_CTA2_MIN")) : 0;
     h->tc_pairs_prefill = getenv("RD_TC_CTA2_PREFILL") && atoi(getenv("RD_TC_CTA2_PREFILL")) != 0;
+    h->att_kl = getenv("RD_ATT_KL") ? atoi(getenv("RD_ATT_KL")) : 1;
     h->qkv_min_rows = getenv("RD_QKV_MIN") ? atoi(getenv("RD_QKV_MIN")) : 0;
     h->swiglu_min_rows = getenv("RD_SWIGLU_MIN") ? atoi(getenv("RD_SWIGLU_MIN")) : 0;   // tuning toggle, as those above
     h->tc_pairs = h->tc_pairs_avail;
@@ -843,9 +876,11 @@ int redrafter_init(const rd_config* cfg, const rd_weights* wt, void* kv_cache, s
       ce = cudaMemset(h->kv, 0, (size_t)dm.n_layers * 2 * h->kv_plane * esize(dm.dtype));
       if (ce != cudaSuccess) return init_fail(h, RD_ERR_CUDA, "clearing the KV cache: %s", cudaGetErrorString(ce));
       h->kv_maps.resize((size_t)dm.n_layers * 2);
+      h->v_maps.resize((size_t)dm.n_layers);
       for (int l = 0; l < dm.n_layers; ++l)
         for (int which = 0; which < 2; ++which)
-          if (tc_make_map(h->kv_maps[(size_t)l * 2 + which].bytes, kv_plane_ptr(h, l, which), (uint64_t)dm.B * dm.H * dm.max_ctx, dm.hd, 128) != 0)
+          if (tc_make_map(h->kv_maps[(size_t)l * 2 + which].bytes, kv_plane_ptr(h, l, which), (uint64_t)dm.B * dm.H * dm.max_ctx, dm.hd, 128) != 0 ||
+              (which && tc_make_map_halves(h->v_maps[l].bytes, kv_plane_ptr(h, l, which), (uint64_t)dm.B * dm.H * dm.max_ctx, 64) != 0))
             return init_fail(h, RD_ERR_CUDA, "tensor map of the KV cache (layer %d)", l);
     }
     if (dm.d % 8 || dm.F % 8 || dm.dh % 8) return init_fail(h, RD_ERR_SHAPE, "bf16 needs d_model, d_ffn multiples of 8");

@@ -918,7 +918,7 @@ cudaError_t launch_fill_i32(int32_t* p, int32_t v, int n, cudaStream_t st) {
 constexpr int ROWS_CTX = 1024;
 __global__ void __launch_bounds__(1024) build_rows_tree_kernel(rd_packed pk, const int32_t* __restrict__ ctx, int32_t* row_tok, int32_t* row_seq,
                                        int32_t* row_pos, int32_t* row_slot, int32_t* row_ncache, int32_t* row_local,
-                                       int32_t* row_out_index, int32_t* seq_off, int32_t* seq_order, int32_t* argmax, int32_t* m_total,
+                                       int32_t* row_out_index, int32_t* seq_off, int32_t* seq_order, uint32_t* mask_t, int32_t* argmax, int32_t* m_total,
                                        Dims dm, int B, int* status) {
   pdl_enter();
   extern __shared__ int32_t off[];  // [B+1], then the context lengths of a batch of up to ROWS_CTX sequences
@@ -977,15 +977,33 @@ __global__ void __launch_bounds__(1024) build_rows_tree_kernel(rd_packed pk, con
     row_local[m] = n;
     row_out_index[m] = idx;
   }
+  // The tree mask with rows and columns exchanged, 32 x 32 bits per warp and turn: lane i holds row r0 + i's word, the ballot of
+  // its bit k is the word of node 32 wd + k over those rows.
+  if (mask_t) {
+    const int tiles = dm.MW * dm.MW;
+    for (int t = w; t < B * tiles; t += (int)blockDim.x >> 5) {
+      const int b = t / tiles, rw = (t - b * tiles) / dm.MW, wd = t - b * tiles - rw * dm.MW;
+      const int n = off[b + 1] - off[b], r = rw * 32 + lane;
+      if (wd * 32 >= n) continue;   // (rows past n have no bits, but their words are read)
+      const uint32_t word = r < n ? pk.mask[((size_t)b * dm.NMAX + r) * dm.MW + wd] : 0u;
+      uint32_t mine = 0;
+#pragma unroll
+      for (int k = 0; k < 32; ++k) {
+        const uint32_t v = __ballot_sync(0xffffffffu, (word >> k) & 1u);
+        if (lane == k) mine = v;
+      }
+      if (wd * 32 + lane < n) mask_t[((size_t)b * dm.NMAX + wd * 32 + lane) * dm.MW + rw] = mine;
+    }
+  }
 }
 
 cudaError_t launch_build_rows_tree(const rd_packed& pk, const int32_t* ctx, int32_t* row_tok, int32_t* row_seq,
                                    int32_t* row_pos, int32_t* row_slot, int32_t* row_ncache, int32_t* row_local,
-                                   int32_t* row_out_index, int32_t* seq_off, int32_t* seq_order, int32_t* argmax, int32_t* m_total,
+                                   int32_t* row_out_index, int32_t* seq_off, int32_t* seq_order, uint32_t* mask_t, int32_t* argmax, int32_t* m_total,
                                    const Dims& dm, int B, int* status, cudaStream_t st) {
   launch_pdl(build_rows_tree_kernel, 1, 1024, ((size_t)B + 1 + (B <= ROWS_CTX ? B : 0)) * sizeof(int32_t), st, pk, ctx, row_tok, row_seq, row_pos, row_slot,
                                                                     row_ncache, row_local, row_out_index, seq_off,
-                                                                    B <= ROWS_CTX ? seq_order : nullptr, argmax, m_total, dm, B, status);
+                                                                    B <= ROWS_CTX ? seq_order : nullptr, mask_t, argmax, m_total, dm, B, status);
   return cudaGetLastError();
 }
 

@@ -944,6 +944,20 @@ int tc_make_map(void* out_map, const void* ptr, uint64_t rows, uint64_t cols, ui
   return (int)r;
 }
 
+// A matrix of 128 columns as [2 halves][rows][64 columns]: one box holds both halves of its rows, one behind the other.
+int tc_make_map_halves(void* out_map, const void* ptr, uint64_t rows, uint32_t box_rows) {
+  EncodeTiledFn fn = encode_fn();
+  if (!fn) return -1;
+  const cuuint64_t dims[3] = {64, rows, 2};
+  const cuuint64_t strides[2] = {256, 128};
+  const cuuint32_t box[3] = {64, box_rows, 2};
+  const cuuint32_t estr[3] = {1, 1, 1};
+  const CUresult r = fn((CUtensorMap*)out_map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(ptr), dims, strides, box,
+                        estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return (int)r;
+}
+
 int tc_weight_box_rows() { return TILE_N; }
 
 // Weight bytes the CTAs of the most recent launch (of this host thread) request BEFORE their dependency wait: the

@@ -82,6 +82,7 @@ cudaError_t launch_gemm_simt(int dtype, int epi, const SimtOperands& p, const Si
 
 // Tensor-core (tcgen05) projection, bf16 only.  Operands are passed as TMA descriptors.
 int tc_make_map(void* out_map, const void* ptr, uint64_t rows, uint64_t cols, uint32_t box_rows);
+int tc_make_map_halves(void* out_map, const void* ptr, uint64_t rows, uint32_t box_rows);
 int tc_weight_box_rows();
 int tc_pick_mt(int m_max);
 size_t tc_partial_floats(int grid, int mt);
@@ -119,6 +120,13 @@ cudaError_t attn_t5_prepare(int hd, int MW);
 cudaError_t launch_attention_t5(const void* map_k, const void* map_v, const float* qkv, void* out, const RowTables& rt,
                                 const int32_t* seq_off, const int32_t* seq_order, const Dims& dm, int n_seq, int row_tiles, int32_t* status, Chain* chain,
                                 cudaStream_t st);
+// head dimension 128, a few dozen rows per sequence: tcgen05 attention with the keys on the lanes
+int attn_kl_row_tiles(int rows);
+bool attn_kl_supported(int hd, int NMAX);
+cudaError_t attn_kl_prepare(int hd);
+cudaError_t launch_attention_kl(const void* map_k, const void* map_v, const float* qkv, void* out, const RowTables& rt,
+                                const int32_t* seq_off, const int32_t* seq_order, const uint32_t* mask_t, const Dims& dm, int n_seq, int row_tiles, int n_sms,
+                                int32_t* status, Chain* chain, cudaStream_t st);
 int attn_wide_rows_per_block();
 cudaError_t attn_wide_prepare(int hd, int MW);
 cudaError_t launch_attention_wide(const float* qkv, const void* kcache, const void* vcache, void* out, const RowTables& rt,
@@ -165,7 +173,7 @@ cudaError_t launch_pack(const int32_t* beams, const int32_t* root, const int32_t
                         const Dims& dm, int B, int no_tree, cudaStream_t st);
 cudaError_t launch_build_rows_tree(const rd_packed& pk, const int32_t* ctx, int32_t* row_tok, int32_t* row_seq,
                                    int32_t* row_pos, int32_t* row_slot, int32_t* row_ncache, int32_t* row_local,
-                                   int32_t* row_out_index, int32_t* seq_off, int32_t* seq_order, int32_t* argmax, int32_t* m_total,
+                                   int32_t* row_out_index, int32_t* seq_off, int32_t* seq_order, uint32_t* mask_t, int32_t* argmax, int32_t* m_total,
                                    const Dims& dm, int B, int* status, cudaStream_t st);
 cudaError_t launch_build_rows_ar(const int32_t* root, const int32_t* ctx, int32_t* row_tok, int32_t* row_seq,
                                  int32_t* row_pos, int32_t* row_slot, int32_t* row_ncache, int32_t* row_local,
