@@ -1,6 +1,7 @@
 // Small row-wise kernels of the verification forward (Section 3.4): embedding gather, RMSNorm,
 // rotary embedding + KV-cache write, SwiGLU, row argmax, row tables.  All are bandwidth-trivial
 // (activations of at most a few MB that stay in L2); they exist to feed the projections.
+#include <algorithm>
 #include <cstdlib>
 #include "rd_internal.cuh"
 #include "gemm_out.cuh"
@@ -187,9 +188,10 @@ static int wide_sm_count() {
   }
   return n;
 }
-// Partial slots loaded up front (a longer list takes the tail loop).  With more (tile pair, row tile) groups than CTAs a
+// Partial slots loaded up front, for all of a thread's columns before the first is used; a longer list takes further rounds of as many
+// (one load after the other took 10.4 us for the one row that a CTA of the 13B step has, 7.8 now: O's tiles lie between five CTAs).  With more (tile pair, row tile) groups than CTAs a
 // tile is cut at most once: gate|up always, QKV mostly; O and down have few tiles, cut among several CTAs each.
-constexpr int WIDE_FOLD_NORM = 2, WIDE_FOLD_ROPE = 2, WIDE_FOLD_SWIGLU = 1;
+constexpr int WIDE_FOLD_NORM = 2;
 
 template <typename T, int NORM_MAXV>
 __global__ void __launch_bounds__(NORM_THREADS, NORM_MAXV <= 2 ? 2 : 1)
@@ -197,34 +199,77 @@ __global__ void __launch_bounds__(NORM_THREADS, NORM_MAXV <= 2 ? 2 : 1)
                         float* __restrict__ out_f, int d, float eps, const int32_t* __restrict__ m_total, ChainSync cs) {
   chain_begin(cs);
   __shared__ float sh[32];
+  const int nvec = d >> 2;
+  const bool add = proj.raw != nullptr;   // x += the projection that ends the previous block (O or down)
   // inside a chain (but not as its first launch) the row count, written ahead of the chain, may be read before the wait
   const bool early = cs.signal_ptr != nullptr && cs.wait_ptr != nullptr;
   int M = early ? *m_total : 0;
+  Gain4<T> gn[NORM_MAXV];   // weights: requested before the wait
+#pragma unroll
+  for (int k = 0; k < NORM_MAXV; ++k) {
+    const int i = threadIdx.x + k * NORM_THREADS;
+    if (i < nvec) gn[k].load(gain + 4 * i);
+  }
   chain_wait_cta(cs);
   if (!early) M = *m_total;
-  const int nvec = d >> 2;
-  const bool add = proj.raw != nullptr;   // x += the projection that ends the previous block (O or down)
   const GemmRows m_tiles = add ? gemm_m_tiles(proj, M) : GemmRows();
+  const size_t slot = gemm_slot_stride(proj);
   for (int m = blockIdx.x; m < M; m += gridDim.x) {
     float4* xr = reinterpret_cast<float4*>(x + (size_t)m * d);
-    float4 v[NORM_MAXV];
-    GemmPending4<WIDE_FOLD_NORM> pd[NORM_MAXV];
+    float4 v[NORM_MAXV], raw[NORM_MAXV], t[NORM_MAXV][WIDE_FOLD_NORM];
 #pragma unroll
     for (int k = 0; k < NORM_MAXV; ++k) {
       const int i = threadIdx.x + k * NORM_THREADS;
       if (i < nvec) {
         v[k] = __ldcg(xr + i);
-        if (add) pd[k] = gemm_issue4<WIDE_FOLD_NORM>(proj, m_tiles, m, 4 * i);
+        if (add) raw[k] = __ldcg(reinterpret_cast<const float4*>(proj.raw + (size_t)m * proj.ld) + i);
+      }
+    }
+    // Where the columns' partial sums lie is worked out while the row is on its way (before the wait it would lengthen the wait:
+    // these CTAs start when the projection's leave): a place in the first extra contributor's slot, and how many there are.
+    uint32_t po[NORM_MAXV];
+    int pn[NORM_MAXV], more = 0;
+    const float* const part = proj.partial;
+    if (add) {
+#pragma unroll
+      for (int k = 0; k < NORM_MAXV; ++k) {
+        const int i = threadIdx.x + k * NORM_THREADS;
+        pn[k] = 0;
+        if (i < nvec) {
+          const GemmFold f = gemm_fold_or_none(proj, m_tiles, m, 4 * i);
+          po[k] = (uint32_t)((size_t)f.c_next * slot + f.off);
+          pn[k] = f.c_last - f.c_next + 1;
+          more = max(more, pn[k]);
+        }
+#pragma unroll
+        for (int c = 0; c < WIDE_FOLD_NORM; ++c)
+          t[k][c] = c < pn[k] ? __ldcg(reinterpret_cast<const float4*>(part + po[k] + c * slot)) : make_float4(0.f, 0.f, 0.f, 0.f);
       }
     }
     float ss = 0.f;
+    if (add) {
+      auto fold = [&]() {
+#pragma unroll
+        for (int k = 0; k < NORM_MAXV; ++k)
+#pragma unroll
+          for (int c = 0; c < WIDE_FOLD_NORM; ++c) { raw[k].x += t[k][c].x; raw[k].y += t[k][c].y; raw[k].z += t[k][c].z; raw[k].w += t[k][c].w; }
+      };
+      fold();
+      for (int c0 = WIDE_FOLD_NORM; c0 < more; c0 += WIDE_FOLD_NORM) {   // further contributors, again all loads before the first sum
+#pragma unroll
+        for (int k = 0; k < NORM_MAXV; ++k)
+#pragma unroll
+          for (int c = 0; c < WIDE_FOLD_NORM; ++c)
+            t[k][c] = c0 + c < pn[k] ? __ldcg(reinterpret_cast<const float4*>(part + po[k] + (c0 + c) * slot)) : make_float4(0.f, 0.f, 0.f, 0.f);
+        fold();
+      }
+    }
 #pragma unroll
     for (int k = 0; k < NORM_MAXV; ++k) {
       const int i = threadIdx.x + k * NORM_THREADS;
       if (i < nvec) {
         if (add) {
-          const float4 q = gemm_finish4(proj, m_tiles, pd[k]);
-          v[k].x += q.x; v[k].y += q.y; v[k].z += q.z; v[k].w += q.w;
+          v[k].x += raw[k].x; v[k].y += raw[k].y; v[k].z += raw[k].z; v[k].w += raw[k].w;
           xr[i] = v[k];
         }
         ss += v[k].x * v[k].x + v[k].y * v[k].y + v[k].z * v[k].z + v[k].w * v[k].w;
@@ -236,9 +281,7 @@ __global__ void __launch_bounds__(NORM_THREADS, NORM_MAXV <= 2 ? 2 : 1)
     for (int k = 0; k < NORM_MAXV; ++k) {
       const int i = threadIdx.x + k * NORM_THREADS;
       if (i < nvec) {
-        Gain4<T> gn;
-        gn.load(gain + 4 * i);
-        const float4 g = gn.get();
+        const float4 g = gn[k].get();
         const float y0 = v[k].x * r * g.x, y1 = v[k].y * r * g.y, y2 = v[k].z * r * g.z, y3 = v[k].w * r * g.w;
         const size_t o = (size_t)m * d + 4 * i;
         if (out_t) store4(out_t + o, y0, y1, y2, y3);
@@ -563,7 +606,7 @@ cudaError_t launch_rope_kv(float* qkv, const GemmOut& proj, void* kcache, void* 
     // several row tiles: four CTAs per SM (36 KB of stages each) walk the rows
     const int heads_per_cta = ROPW_COLS / dm.hd;
     dim3 gw((dm.H + heads_per_cta - 1) / heads_per_cta, 1);
-    const int gy = (4 * wide_sm_count() + (int)gw.x - 1) / (int)gw.x;
+    const int gy = std::max(1, 4 * wide_sm_count() / (int)gw.x);   // no CTA beyond one wave
     gw.y = gy < m_max ? gy : m_max;
     const ChainSync cs = chain ? chain->link(gw.x * gw.y, true) : ChainSync{nullptr, 0u, nullptr, nullptr, nullptr};
     launch_pdl(rope_kv_wide_kernel, gw, ROPW_THREADS, 0, st, qkv, proj, (__nv_bfloat16*)kcache, (__nv_bfloat16*)vcache,
@@ -648,7 +691,9 @@ __global__ void __maxnreg__(88) swiglu_kernel(GemmOut proj, __nv_bfloat16* __res
 // segment of a row (SWS_COLS x 4 bytes each, contiguous) come in through a ring of shared-memory stages filled by
 // thread 0 with bulk asynchronous copies, SWS_STAGES - 1 rows ahead of the row being worked on (stage.cuh), so what
 // the CTA has in flight does not depend on its registers.  Partial sums (with far more tiles than CTAs a tile is cut at
-// most once, and about one tile in five is) are added from global memory by the threads whose columns they concern.
+// most once, and about one tile in five is; at 150 to 250 rows nearly every tile) are requested by the threads whose columns they
+// concern before the row's stage is waited for: 240 rows of the 7B shape 13.5 -> 10 us, requested behind it before; 148 rows of
+// the 13B shape 16.8 -> 8.8, where the grid also had four CTAs more than fit at once.
 constexpr int SWS_THREADS = 256;
 constexpr int SWS_COLS = 2048;      // two float4 per thread
 constexpr int SWS_STAGES = 4;       // 4 x (8 + 8) KB per CTA
@@ -673,8 +718,7 @@ __global__ void __launch_bounds__(SWS_THREADS, 3)
   const int c0 = blockIdx.x * SWS_COLS;
   const int ncol = min(SWS_COLS, F - c0);
   const uint32_t seg_bytes = (uint32_t)ncol * 4u;
-  const int m_begin = gemm_rows_begin(M, gridDim.y, blockIdx.y), m_end = gemm_rows_begin(M, gridDim.y, blockIdx.y + 1);
-  const int n_rows = m_end - m_begin;
+  const int m_begin = gemm_rows_begin(M, gridDim.y, blockIdx.y), n_rows = gemm_rows_begin(M, gridDim.y, blockIdx.y + 1) - m_begin;
   auto issue = [&](int i) {   // thread 0: row m_begin + i into slot i % SWS_STAGES
     const int s = i % SWS_STAGES;
     const float* src = proj.raw + (size_t)(m_begin + i) * proj.ld + c0;
@@ -688,26 +732,35 @@ __global__ void __launch_bounds__(SWS_THREADS, 3)
   }
   const int j0 = threadIdx.x * 4, j1 = j0 + SWS_THREADS * 4;   // this thread's two float4 inside the segment
   const bool cut_any = proj.partial != nullptr;
-  int tile_end = 0, cur_tile = 0;
   const size_t slot = gemm_slot_stride(proj);
-  GemmFold fg[2], fu[2];   // the fold of a column changes only from one row tile to the next
-  bool cut[2] = {false, false};
+  // Where a column's partial sums lie changes only from one row tile to the next: the first extra contributor's sums of the
+  // tile's first row (gate, up), and how many contributors there are.
+  int tile0 = 0, tile_end = 0;
+  const float *pg[2], *pu[2];
+  int ng[2] = {0, 0}, nu[2] = {0, 0};
+  auto fold_at = [&](int row) {
+    tile0 = row / m_tiles.rows * m_tiles.rows;
+    tile_end = tile0 + m_tiles.rows;
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const int j = min(k ? j1 : j0, ncol - 4);
+      const GemmFold fg = gemm_fold(proj, m_tiles, tile0, c0 + j), fu = gemm_fold(proj, m_tiles, tile0, F + c0 + j);
+      pg[k] = proj.partial + (size_t)fg.c_next * slot + fg.off; ng[k] = fg.c_last - fg.c_next + 1;
+      pu[k] = proj.partial + (size_t)fu.c_next * slot + fu.off; nu[k] = fu.c_last - fu.c_next + 1;
+    }
+  };
   uint32_t s = 0, ph = 0;
   for (int i = 0; i < n_rows; ++i) {
     const int m = m_begin + i;
     if (threadIdx.x == 0 && i + SWS_STAGES - 1 < n_rows) issue(i + SWS_STAGES - 1);   // slot released by the last barrier
-    if (cut_any && m >= tile_end) {
-      cur_tile = m / m_tiles.rows;
-      tile_end = (cur_tile + 1) * m_tiles.rows;
+    if (cut_any && m >= tile_end) fold_at(m);
+    // the first extra contributor's sums are requested before the row's own are waited for (a tile rarely has a second)
+    const size_t doff = (size_t)(m - tile0) * 128;
+    float4 tg[2], tu[2];
 #pragma unroll
-      for (int k = 0; k < 2; ++k) {
-        const int j = k ? j1 : j0;
-        if (j < ncol) {
-          fg[k] = gemm_fold(proj, m_tiles, cur_tile * m_tiles.rows, c0 + j);
-          fu[k] = gemm_fold(proj, m_tiles, cur_tile * m_tiles.rows, F + c0 + j);
-          cut[k] = fg[k].c_next <= fg[k].c_last || fu[k].c_next <= fu[k].c_last;
-        }
-      }
+    for (int k = 0; k < 2; ++k) {
+      tg[k] = ng[k] > 0 ? __ldcg(reinterpret_cast<const float4*>(pg[k] + doff)) : make_float4(0.f, 0.f, 0.f, 0.f);
+      tu[k] = nu[k] > 0 ? __ldcg(reinterpret_cast<const float4*>(pu[k] + doff)) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
     stage_wait(bars_u + 8u * s, ph, status, DEV_ERR_TIMEOUT);
     const float* sg = ring + (size_t)(s * 2) * SWS_COLS;
@@ -717,16 +770,16 @@ __global__ void __launch_bounds__(SWS_THREADS, 3)
       const int j = k ? j1 : j0;
       if (j < ncol) {
         float4 g = *reinterpret_cast<const float4*>(sg + j), u = *reinterpret_cast<const float4*>(su + j);
-        if (cut[k]) {   // add the other contributors' sums in CTA order
-          const size_t doff = (size_t)(m - cur_tile * m_tiles.rows) * 128;
-          for (int c = fg[k].c_next; c <= fg[k].c_last; ++c) {
-            const float4 t = __ldcg(reinterpret_cast<const float4*>(proj.partial + (size_t)c * slot + fg[k].off + doff));
-            g.x += t.x; g.y += t.y; g.z += t.z; g.w += t.w;
-          }
-          for (int c = fu[k].c_next; c <= fu[k].c_last; ++c) {
-            const float4 t = __ldcg(reinterpret_cast<const float4*>(proj.partial + (size_t)c * slot + fu[k].off + doff));
-            u.x += t.x; u.y += t.y; u.z += t.z; u.w += t.w;
-          }
+        // the other contributors' sums in CTA order
+        g.x += tg[k].x; g.y += tg[k].y; g.z += tg[k].z; g.w += tg[k].w;
+        u.x += tu[k].x; u.y += tu[k].y; u.z += tu[k].z; u.w += tu[k].w;
+        for (int c = 1; c < ng[k]; ++c) {
+          const float4 t = __ldcg(reinterpret_cast<const float4*>(pg[k] + (size_t)c * slot + doff));
+          g.x += t.x; g.y += t.y; g.z += t.z; g.w += t.w;
+        }
+        for (int c = 1; c < nu[k]; ++c) {
+          const float4 t = __ldcg(reinterpret_cast<const float4*>(pu[k] + (size_t)c * slot + doff));
+          u.x += t.x; u.y += t.y; u.z += t.z; u.w += t.w;
         }
         store4(out + (size_t)m * F + c0 + j, silu_f(g.x) * u.x, silu_f(g.y) * u.y, silu_f(g.z) * u.z, silu_f(g.w) * u.w);
       }
@@ -751,7 +804,7 @@ cudaError_t launch_swiglu(const GemmOut& proj, void* out_t, int F, const int32_t
   if (m_max > WIDE_ROWS_MIN) {   // several row tiles: three CTAs per SM (64 KB of stages each) walk the rows
     const size_t smem = (size_t)SWS_STAGES * 2 * SWS_COLS * sizeof(float);   // opted in by elementwise_prepare
     grid.x = (F + SWS_COLS - 1) / SWS_COLS;
-    const int gy = (3 * wide_sm_count() + (int)grid.x - 1) / (int)grid.x;
+    const int gy = std::max(1, 3 * wide_sm_count() / (int)grid.x);   // no CTA beyond one wave
     grid.y = gy < m_max ? gy : m_max;
     const ChainSync cs = chain ? chain->link(grid.x * grid.y, true) : ChainSync{nullptr, 0u, nullptr, nullptr, nullptr};
     launch_pdl(swiglu_wide_kernel, grid, SWS_THREADS, smem, st, proj, (__nv_bfloat16*)out_t, F, m_total, status, cs);

@@ -310,40 +310,9 @@ __device__ __forceinline__ float4 gemm_value4(const GemmOut& g, GemmRows m_tiles
   return gemm_finish4(g, m_tiles, gemm_issue4<U>(g, m_tiles, m, n));
 }
 
-// Four consecutive columns with the fold worked out by the caller (a kernel that walks the rows of one row tile
-// computes it once per tile: only the offset inside the slot, doff, changes from row to row).
-template <int U>
-struct GemmPending4f {
-  float4 raw;
-  float4 q[U];
-};
-template <int U>
-__device__ __forceinline__ GemmPending4f<U> gemm_issue4f(const GemmOut& g, GemmRows m_tiles, const GemmFold& f, int m, int n, size_t doff) {
-  GemmPending4f<U> p;
-  p.raw = __ldcg(reinterpret_cast<const float4*>(g.raw + (size_t)m * g.ld + n));
-  const size_t slot = gemm_slot_stride(g);
-#pragma unroll
-  for (int j = 0; j < U; ++j) {
-    const int c = f.c_next + j;
-    p.q[j] = (c <= f.c_last)
-                 ? __ldcg(reinterpret_cast<const float4*>(g.partial + (size_t)c * slot + f.off + doff))
-                 : make_float4(0.f, 0.f, 0.f, 0.f);
-  }
-  return p;
-}
-template <int U>
-__device__ __forceinline__ float4 gemm_finish4f(const GemmOut& g, GemmRows m_tiles, const GemmFold& f, size_t doff, const GemmPending4f<U>& p) {
-  float4 v = p.raw;
-#pragma unroll
-  for (int j = 0; j < U; ++j) { v.x += p.q[j].x; v.y += p.q[j].y; v.z += p.q[j].z; v.w += p.q[j].w; }
-  const size_t slot = gemm_slot_stride(g);
-  for (int c = f.c_next + U; c <= f.c_last; ++c) {
-    const float4 t = __ldcg(reinterpret_cast<const float4*>(g.partial + (size_t)c * slot + f.off + doff));
-    v.x += t.x; v.y += t.y; v.z += t.z; v.w += t.w;
-  }
-  return v;
-}
 // Rows [begin, end) of a kernel that splits M rows evenly over `parts` CTAs, part `i`.
-__device__ __forceinline__ int gemm_rows_begin(int M, int parts, int i) { return (int)((long long)M * i / parts); }
+__device__ __forceinline__ int gemm_rows_begin(int M, int parts, int i) {
+  return M < (1 << 20) && parts < 2048 ? (int)((uint32_t)M * (uint32_t)i / (uint32_t)parts) : (int)((long long)M * i / parts);
+}
 
 }  // namespace rd
