@@ -188,9 +188,9 @@ static int wide_sm_count() {
   }
   return n;
 }
-// Partial slots loaded up front, for all of a thread's columns before the first is used; a longer list takes further rounds of as many
-// (one load after the other took 10.4 us for the one row that a CTA of the 13B step has, 7.8 now: O's tiles lie between five CTAs).  With more (tile pair, row tile) groups than CTAs a
-// tile is cut at most once: gate|up always, QKV mostly; O and down have few tiles, cut among several CTAs each.
+// Partial slots loaded up front, for all of a thread's columns before the first is used; a longer list takes further rounds of as
+// many.  (One load after the other, and the gain requested last, a row took 10.4 us in the 13B step, whose CTAs have one row each
+// and whose O tiles lie between five CTAs; 5.5 now.  240 rows of the 7B shape 7.3 -> 6.3 us a launch, 736 rows 15.8 -> 13.)
 constexpr int WIDE_FOLD_NORM = 2;
 
 template <typename T, int NORM_MAXV>
@@ -692,8 +692,8 @@ __global__ void __maxnreg__(88) swiglu_kernel(GemmOut proj, __nv_bfloat16* __res
 // thread 0 with bulk asynchronous copies, SWS_STAGES - 1 rows ahead of the row being worked on (stage.cuh), so what
 // the CTA has in flight does not depend on its registers.  Partial sums (with far more tiles than CTAs a tile is cut at
 // most once, and about one tile in five is; at 150 to 250 rows nearly every tile) are requested by the threads whose columns they
-// concern before the row's stage is waited for: 240 rows of the 7B shape 13.5 -> 10 us, requested behind it before; 148 rows of
-// the 13B shape 16.8 -> 8.8, where the grid also had four CTAs more than fit at once.
+// concern before the row's stage is waited for: 240 rows of the 7B shape 13.5 -> 10.5 us a launch, requested behind it before; 148
+// rows of the 13B shape 16.8 -> 9.0, where the grid also had four CTAs more than fit at once.
 constexpr int SWS_THREADS = 256;
 constexpr int SWS_COLS = 2048;      // two float4 per thread
 constexpr int SWS_STAGES = 4;       // 4 x (8 + 8) KB per CTA
