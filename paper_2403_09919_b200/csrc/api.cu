@@ -541,6 +541,13 @@ int layers_simt(rd_handle* h, const RowTables& rt, int m_max, Chain* ch, cudaStr
   return RD_OK;
 }
 
+// Whether this handle's verification and autoregressive passes can take the attention kernel with the keys on the lanes at all.
+// Models of fewer than 24 heads keep the earlier kernels, whose lines are held by tests; of the shapes here only the small models
+// of the tests have so few.
+bool keys_on_lanes_possible(const rd_handle* h) {
+  return h->att_kl != 0 && !h->kv_maps.empty() && attn_kl_supported(h->dm.hd, h->dm.NMAX) && (h->att_kl >= 2 || h->dm.H >= 24);
+}
+
 // Whether a pass takes the attention kernel with the keys on the lanes; `wide`: else it would take the 64- or 128-row kernel.
 // Measured per layer (4 layers, contexts of 60, 150-300, 500, 256-1024 and 2048 tokens, earlier kernel -> this one):
 // verification, 7B, 1 sequence of 30 / 82 rows -1 to -8 / -4 to -23 %; 4 of 32 -3 to -17; 8 of 30, 56, 85 -7 to 0, -8 to -1, -9 to 0;
@@ -549,18 +556,18 @@ int layers_simt(rd_handle* h, const RowTables& rt, int m_max, Chain* ch, cudaStr
 //   set-up (4 x 54 / 62 / 89 rows, 128 tiles: +1 to +5 / -1 to +9 / 0 to +9 %; 13B, 4 x 89, 160 tiles: +3 to -4), but where they
 //   can be cut into two tiles or more each, it is ahead again (152 rows, 32 tiles: -1 to -5);
 // - on several tiles per SM with less than a chunk of keys (60 tokens, 8 or 16 sequences: 0 to +3 %);
+// - on few tiles of up to 16 rows and a thousand keys, which the 16-row kernel splits (7B, 1 sequence of 11 rows, 2048 tokens +1.3 %,
+//   of 60 to 500 tokens -2; 13B, 3 rows, 1400 tokens +1.7);
 // - in autoregressive steps of a single sequence, whose keys the 16-row kernel splits (7B +1 to +5 %, 33B -2 to +1), and of few
 //   keys (100 tokens: 0 to +3); 2 to 16 sequences of 500 to 2500 tokens -20 to 0, two points +1.5.
-// Models of fewer than 24 heads keep the earlier kernels, whose lines are held by tests; of the shapes here only the small models
-// of the tests have so few.
 bool use_keys_on_lanes(const rd_handle* h, bool tree, int n_seq, int rows_per_seq_max, bool wide) {
   const Dims& dm = h->dm;
-  if (h->att_kl == 0 || h->kv_maps.empty() || !attn_kl_supported(dm.hd, dm.NMAX)) return false;
+  if (!keys_on_lanes_possible(h)) return false;
   if (h->att_kl >= 2) return true;
   const int tiles = dm.H * n_seq, G = h->tc_grid;
-  if (dm.H < 24) return false;
   if (!tree) return rows_per_seq_max == 1 && tiles >= 64 && (h->route_bound >= 256 || tiles >= 3 * G);
   if (wide && rows_per_seq_max > 64 && 2 * tiles > G && (tiles <= G || (rows_per_seq_max >= 96 && 4 * tiles <= 5 * G))) return false;
+  if (rows_per_seq_max <= 16 && tiles < 64 && h->route_bound >= 1024) return false;
   return tiles <= G || h->route_bound >= 128;
 }
 
@@ -767,7 +774,7 @@ int do_verify(rd_handle* h, const rd_packed& pk, cudaStream_t st, int32_t* argma
   const Dims& dm = h->dm;
   const int B = h->batch, m_max = B * dm.NMAX;
   CKP(h, PROF_MISC, launch_build_rows_tree(pk, w.ctx, w.row_tok, w.row_seq, w.row_pos, w.row_slot, w.row_ncache, w.row_local,
-                               w.row_out_index, w.seq_off, w.seq_order, h->att_kl && attn_kl_supported(dm.hd, dm.NMAX) ? w.mask_t : nullptr, argmax, w.m_total, dm, B, w.status, st));
+                               w.row_out_index, w.seq_off, w.seq_order, keys_on_lanes_possible(h) ? w.mask_t : nullptr, argmax, w.m_total, dm, B, w.status, st));
   h->att_seq_order = B <= 1024 ? w.seq_order : nullptr;   // the row tables of this pass carry the sequences' order
   if (!verify_on_pairs(h, m_max)) h->tc_pairs = 0;
   int rc = forward_layers(h, pk.mask, m_max, B, dm.NMAX, h->w.lm_head, st);

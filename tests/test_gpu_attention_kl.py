@@ -97,9 +97,10 @@ def test_ragged_batch_against_the_oracle(monkeypatch):
     (24, 8, 8, 127, False), (24, 8, 8, 128, True),     # more: from 128 tokens
     (24, 4, 26, 200, False), (24, 4, 12, 200, True),   # 96 wide tiles, where the 64- or 128-row kernel would run
     (24, 3, 26, 200, True),                            # 72: can be halved
+    (24, 2, 3, 1024, False), (24, 2, 3, 1023, True), (24, 2, 4, 1024, True), (24, 3, 3, 1024, True),   # 16 and 21 rows, 48 tiles and 72
     (23, 4, 8, 200, False)])
 def test_lines_of_verification(heads, batch, bw, tokens, taken):
-    cfg = config(heads, n_layers=1, max_batch=batch, beam_width=bw, max_ctx=400)
+    cfg = config(heads, n_layers=1, max_batch=batch, beam_width=bw, max_ctx=tokens + 200)
     eng = ReDrafter(cfg, synth.make_weights(cfg, "cuda:0"))
     rng = np.random.default_rng(8)
     eng.set_state(dev(np.full(batch, tokens)), dev(rng.integers(0, 1000, size=batch)), torch.randn(batch, cfg["d_model"], device="cuda"),
