@@ -339,7 +339,7 @@ __device__ __forceinline__ void kl_softmax(const KlParams& p, const KlCtx& t, co
         for (int i = 0; i < COLS; ++i) {
           const float down = sm->corr[col0 + i];
           sc[i] += down;
-          l[i] *= fast_exp2(down);
+          if (c > 0) l[i] *= fast_exp2(down);   // (the first chunk's reference may fall: its factor has no bound, and l is zero)
         }
         if (c > 0) {
           // O is complete through the chunk before this one and waits for this one's weights
@@ -418,7 +418,7 @@ __device__ __forceinline__ void kl_softmax(const KlParams& p, const KlCtx& t, co
       if (tip < COLS) {
         const int r = col0 + tip;
         const float sum = (sm->red[0][r] + sm->red[1][r]) + (sm->red[2][r] + sm->red[3][r]);
-        sm->corr[r] = sum > 0.f ? 1.f / sum : 0.f;
+        sm->corr[r] = sum == 0.f ? 0.f : 1.f / sum;   // a row without keys is zero, one of NaN stays so
       }
     }
     if (more) {   // Q -> bf16, K-major swizzled: 16-byte chunk i of row r lands at chunk i ^ (r & 7) of its 128-byte line

@@ -1,0 +1,137 @@
+"""Attention of verification passes and autoregressive steps against 64 bits, row by row and head by head (head dimension 128).
+
+One layer whose output is its attention: embeddings of +-1/16 that the norm turns into +-1, queries and new keys that depend on
+the first feature only (which is the same for every token), an output projection of 64 times the identity and no feed-forward
+part.  The hidden row is then the normalised sum of a small known vector and 64 times the attention output, and scores are
+whatever the cache is filled for."""
+import math
+
+import numpy as np
+import pytest
+import torch
+
+from helpers import dev
+from paper_2403_09919_b200 import synth
+from paper_2403_09919_b200.binding import ReDrafter
+
+pytestmark = pytest.mark.gpu
+
+HD = 128
+# A bf16 result is off by up to 2^-9 of each element; weights rounded to bf16 add as much at most.
+CLOSE = 2.0 ** -8
+LOG2E = 1 / math.log(2)
+
+
+class Attention:
+    """Verification passes and autoregressive steps of the model above.  `q`: the query of every row before its rotation,
+    [heads, 128]; `k_new`: likewise the keys of the new rows."""
+
+    def __init__(self, monkeypatch, heads, lens, beam, q, k_new, kl, max_ctx=None, seed=1):
+        d = heads * HD
+        self.heads, self.lens, self.d = heads, lens, d
+        self.cfg = dict(synth.CONFIGS["tiny"], dtype="bf16", n_layers=1, d_model=d, n_heads=heads, d_ffn=128, vocab=1000, d_rnn=d,
+                        max_batch=len(lens), beam_width=beam[0], beam_length=beam[1])
+        self.cfg["max_ctx"] = max_ctx or max(lens) + 1 + beam[0] * beam[1] + 8
+        gen = torch.Generator(device="cuda").manual_seed(seed)
+        w = synth.make_weights(self.cfg, "cuda:0")
+        emb = torch.where(torch.rand(1000, d, device="cuda", generator=gen) < 0.5, -1.0, 1.0) / 16
+        emb[:, 0] = 1 / 16
+        w["tok_emb"] = emb.to(torch.bfloat16)
+        qkv = w["wqkv.0"]
+        qkv[:2 * d] = 0
+        qkv[:d, 0], qkv[d:2 * d, 0] = q.reshape(-1).to(qkv), k_new.reshape(-1).to(qkv)
+        qkv[2 * d:] = torch.randn(d, d, device="cuda", generator=gen) / math.sqrt(d)
+        w["wo.0"] = (64 * torch.eye(d, device="cuda")).to(torch.bfloat16)
+        w["w_down.0"].zero_()
+        self.q, self.w = qkv[:d, 0].double().view(heads, HD), w
+        monkeypatch.setenv("RD_ATT_KL", str(kl))
+        self.eng = ReDrafter(self.cfg, w)
+        monkeypatch.delenv("RD_ATT_KL")
+        self.kv = self.eng.kv_view()[0]            # [2, batch, heads, max_ctx, 128]
+        self.kv[1].normal_(0.0, 1.0, generator=gen)
+        self.rng = np.random.default_rng(seed)
+        self.roots = dev(self.rng.integers(0, 1000, size=len(lens)))
+        self.h = torch.zeros(len(lens), d, device="cuda")
+        self.beams = dev(self.rng.integers(0, 1000, size=(len(lens), *beam)))
+
+    def start(self):
+        self.eng.set_state(dev(np.asarray(self.lens)), self.roots, self.h, batch=len(self.lens), ctx_bound=max(self.lens))
+
+    def verify(self, change=None):
+        """Hidden rows of a verification pass, sequence by sequence; `change` may alter the packed candidates."""
+        self.start()
+        self.pk = self.eng.pack(self.beams)
+        if change:
+            change(self.pk)
+        hidden = self.eng.verify(self.pk)[1]
+        self.eng.poll()
+        return [hidden[b, :int(n)] for b, n in enumerate(self.pk.n)]
+
+    def ar(self):
+        self.start()
+        self.eng.ar_step()
+        self.eng.poll()
+        return list(self.eng.get_state()[2][:, None])
+
+    def exact(self, b, tokens, pos, keys, see):
+        """64 bits: rows of `tokens` at `pos` over the first `keys` slots of sequence b's cache as it lies there; see: [rows, keys]."""
+        half = HD // 2
+        ang = pos.double()[:, None] * self.cfg["rope_theta"] ** (-torch.arange(half, dtype=torch.float64, device="cuda") / half)
+        c, s, q = ang.cos()[:, None], ang.sin()[:, None], self.q
+        q = torch.cat([q[:, :half] * c - q[:, half:] * s, q[:, half:] * c + q[:, :half] * s], -1).to(torch.bfloat16).double()
+        sc = torch.einsum("rhd,hkd->rhk", q, self.kv[0, b, :, :keys].double()) / math.sqrt(HD)
+        sc.masked_fill_(~see[:, None], -math.inf)
+        att = torch.einsum("rhk,hkd->rhd", sc.softmax(-1), self.kv[1, b, :, :keys].double())
+        x = self.w["tok_emb"][tokens.long()].double() + 64 * att.reshape(len(tokens), -1)
+        return x * torch.rsqrt(x.square().mean(-1, keepdim=True) + self.cfg["rms_eps"])
+
+    def exact_verify(self):
+        out = []
+        for b, n in enumerate(self.pk.n.tolist()):
+            c = self.lens[b]
+            words = self.pk.mask[b, :n].cpu().numpy().view(np.uint32)
+            bits = (words[:, :, None] >> np.arange(32, dtype=np.uint32)) & 1
+            see = torch.ones(n, c + n, dtype=torch.bool, device="cuda")
+            see[:, c:] = torch.from_numpy(bits.reshape(n, -1)[:, :n].astype(bool)).cuda()
+            out.append(self.exact(b, self.pk.tokens[b, :n], self.pk.pos[b, :n], c + n, see))
+        return out
+
+    def exact_ar(self):
+        return [self.exact(b, self.roots[b:b + 1], torch.tensor([c], device="cuda"), c + 1, torch.ones(1, c + 1, dtype=torch.bool, device="cuda"))
+                for b, c in enumerate(self.lens)]
+
+    def errors(self, got, ref):
+        """Relative error (2-norm) of every row and head."""
+        a, r = (torch.cat(t).double().view(-1, self.heads, HD) for t in (got, ref))
+        return (a - r).norm(dim=-1) / r.norm(dim=-1)
+
+    def route(self):
+        return {k: v for k, v in self.eng.route_counts().items() if k.startswith("att_") and v}
+
+
+def slow(heads, size):
+    """Vectors along the pair of dimensions that the rotary embedding turns least: the same at every position, nearly."""
+    v = torch.zeros(heads, HD, device="cuda")
+    v[:, HD // 2 - 1] = size
+    return v
+
+
+def fill_scores(a, b, scores):
+    """Cached keys of sequence b whose scores with `slow(heads, 8.0)` are `scores` (base 2) give or take a few."""
+    s = torch.as_tensor(scores, dtype=torch.float32, device="cuda") + torch.randn(a.heads, len(scores), device="cuda") * 1.5
+    a.kv[0, b, :, :len(scores)] = 0
+    a.kv[0, b, :, :len(scores), HD // 2 - 1] = (s / LOG2E * math.sqrt(HD) / 8.0).to(torch.bfloat16)
+
+
+@pytest.mark.parametrize("level", [-100.0, -126.0, -130.0, -1000.0])
+@pytest.mark.parametrize("lens,late", [([3, 5], 0.0), ([40, 150], 0.0), ([300, 420], 0.0), ([300, 700], 60.0), ([300, 700], -60.0),
+                                       ([300, 700], 900.0)])
+def test_first_chunk_of_low_scores(monkeypatch, level, lens, late):
+    """Every score of the first chunk of keys far below zero, so that the rows' reference falls; later chunks alike, or `late` above."""
+    torch.manual_seed(3)
+    a = Attention(monkeypatch, 4, lens, (5, 3), slow(4, 8.0), slow(4, (level + late) / LOG2E * math.sqrt(HD) / 8.0), 2)
+    for b, c in enumerate(lens):
+        fill_scores(a, b, [level] * min(c, 128) + [level + late] * max(c - 128, 0))
+    assert a.errors(a.verify(), a.exact_verify()).max() < CLOSE
+    assert a.errors(a.ar(), a.exact_ar()).max() < CLOSE
+    assert a.route() == {"att_keys_on_lanes": 2}
