@@ -276,8 +276,10 @@ __device__ __forceinline__ void kl_softmax(const KlParams& p, const KlCtx& t, co
 #pragma unroll
     for (int i = 0; i < COLS; ++i) l[i] = 0.f;
     // The rows' references start at zero, which serves any row with a score of at least -KL_LOW (one key whose scores all are
-    // settles it for its part), and move when a score exceeds one by KL_SLACK.
-    bool ok = true, moved = false;
+    // settles it for its part), and move when a score exceeds one by KL_SLACK.  A row that attends no key of the first chunks
+    // (`none`, of the row that this thread keeps the reference of) takes its reference from the first that it does attend: until
+    // then its part looks at every chunk's maxima (`hollow`).
+    bool ok = true, moved = false, none = true, hollow = false;
     for (int c = 0; c < n_chunks; ++c) {
       const int j = j0 + c;
       const uint32_t ph = (uint32_t)((j >> 1) & 1);
@@ -312,13 +314,14 @@ __device__ __forceinline__ void kl_softmax(const KlParams& p, const KlCtx& t, co
         for (int i = 1; i < COLS; ++i) mx = fmaxf(mx, sc[i]);
         far = mx > KL_SLACK;
       }
-      bool move = bar_any<128>(part_bar, far);
+      bool move = bar_any<128>(part_bar, far) || hollow;
       if (c == 0) {
         float low = sc[0];
 #pragma unroll
         for (int i = 1; i < COLS; ++i) low = fminf(low, sc[i]);
         // (where the first chunk is most of the keys, one of them often outweighs the rest: its weight is made one, and exact)
         move = !bar_any<128>(part_bar, ok && low >= -KL_LOW && n_chunks > 2) || move;
+        none = move;
       }
       if (move) {
         // references move: the maximum of every column over the chunk's keys
@@ -327,19 +330,20 @@ __device__ __forceinline__ void kl_softmax(const KlParams& p, const KlCtx& t, co
         bar_sync<128>(part_bar);
         if (tip < COLS) {
           const int r = col0 + tip;
-          // by how much row r's reference rises (in the first chunk it may also fall); a row without keys so far keeps its own
+          // by how much row r's reference rises (at its first keys it may also fall); a row without keys so far keeps its own
           const float m = fmaxf(fmaxf(sm->red[0][r], sm->red[1][r]), fmaxf(sm->red[2][r], sm->red[3][r]));
-          const float up = m == -INFINITY ? 0.f : c == 0 ? m : fmaxf(m, 0.f);
+          const float up = m == -INFINITY ? 0.f : none ? m : fmaxf(m, 0.f);
           sm->corr[r] = -up;
           sm->nref[r] -= up;
+          none = none && m == -INFINITY;
         }
         moved = true;
-        bar_sync<128>(part_bar);
+        hollow = bar_any<128>(part_bar, tip < COLS && none);
 #pragma unroll
         for (int i = 0; i < COLS; ++i) {
           const float down = sm->corr[col0 + i];
           sc[i] += down;
-          if (c > 0) l[i] *= fast_exp2(down);   // (the first chunk's reference may fall: its factor has no bound, and l is zero)
+          l[i] *= fast_exp2(fminf(down, 0.f));   // (where the reference falls, its factor has no bound, and the sums are zero)
         }
         if (c > 0) {
           // O is complete through the chunk before this one and waits for this one's weights
@@ -352,7 +356,7 @@ __device__ __forceinline__ void kl_softmax(const KlParams& p, const KlCtx& t, co
               tmem_ld4_nowait(o_addr + i, o);
               tmem_ld_wait();
 #pragma unroll
-              for (int n = 0; n < 4; ++n) o[n] *= fast_exp2(sm->corr[col0 + i + n]);
+              for (int n = 0; n < 4; ++n) o[n] *= fast_exp2(fminf(sm->corr[col0 + i + n], 0.f));
               tmem_st4(o_addr + i, o);
             }
             tmem_st_wait();

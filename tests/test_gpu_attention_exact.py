@@ -135,3 +135,22 @@ def test_first_chunk_of_low_scores(monkeypatch, level, lens, late):
     assert a.errors(a.verify(), a.exact_verify()).max() < CLOSE
     assert a.errors(a.ar(), a.exact_ar()).max() < CLOSE
     assert a.route() == {"att_keys_on_lanes": 2}
+
+
+def test_rows_whose_keys_all_lie_behind_the_first_chunk(monkeypatch):
+    """Candidates without a context, some of which attend nothing but themselves, as a mask of the caller's own may say: their
+    first key lies in the second chunk, far below zero."""
+    torch.manual_seed(3)
+    a = Attention(monkeypatch, 2, [0, 90], (32, 5), slow(2, 8.0), slow(2, -200 / LOG2E * math.sqrt(HD) / 8.0), 2)
+    fill_scores(a, 1, [-3.0] * 90)
+
+    def alone(pk):
+        pk.mask[0, 128:] = 0
+        for r in range(128, int(pk.n[0])):
+            bit = 1 << (r & 31)
+            pk.mask[0, r, r >> 5] = bit - (1 << 32) if bit >> 31 else bit
+
+    got = a.verify(alone)
+    assert int(a.pk.n[0]) > 130
+    assert a.errors(got, a.exact_verify()).max() < CLOSE
+    assert a.route() == {"att_keys_on_lanes": 1}
