@@ -20,8 +20,9 @@
 // dimensions of K, half of its keys of V) that the producer keeps filled across the tiles' ends, and the next tile's first
 // scores are formed while the one before is written out.
 // Roles: warp 0 = TMA producer, warps 1 and 2 = MMA issuers of the scores and of the output (the whole warp runs the loop, an
-// elected lane issues), warp 3 lays out the CTA's tiles, warps 4..19 = softmax and output.  Every wait is bounded (one second),
-// as in attention_t5.cu; a warp that gives up still takes part in the named barriers until all of its part have seen it.
+// elected lane issues), warp 3 lays out the CTA's tiles and clears the values behind their last keys, warps 4..19 = softmax and
+// output.  Every wait is bounded (one second), as in attention_t5.cu; a warp that gives up still takes part in the named barriers
+// until all of its part have seen it.
 //
 // What bounds it: the copies where every SM has tiles (7B, 16 sequences of 256 to 2048 tokens: 70 us a launch for 302 MB of keys and
 // values, launch and set-up included, 95 us before; 16 x 1024 tokens of one row each 57 against 69), else a chunk's chain of hand-overs
@@ -191,7 +192,7 @@ struct KlTile {
 };
 // Shared memory in front of the operands.
 struct KlShared {
-  unsigned long long bars[40];
+  unsigned long long bars[48];
   uint32_t tmem;
   volatile int abort_flag;
   int n_tiles, rows_max;
@@ -203,8 +204,8 @@ struct KlShared {
 };
 // S_* to PV_*: by chunk parity
 enum { KB_FULL = 0, KB_EMPTY = KL_MAX_SLOTS, KB_Q = 2 * KL_MAX_SLOTS, KB_S_FULL, KB_S_EMPTY = KB_S_FULL + 2, KB_P_FULL = KB_S_EMPTY + 2,
-       KB_PV_DONE = KB_P_FULL + 2, KB_COUNT = KB_PV_DONE + 2 };
-static_assert(KB_COUNT <= 40, "barriers");
+       KB_PV_DONE = KB_P_FULL + 2, KB_TAIL = KB_PV_DONE + 2, KB_COUNT = KB_TAIL + KL_MAX_SLOTS };
+static_assert(KB_COUNT <= 48, "barriers");
 
 // Chunks of a tile that some row may not attend whole: as many as the tree (or a causal tile) touches.
 __host__ __device__ constexpr int kl_vis_chunks(int nmax) { return ((nmax > KL_ROWS ? nmax : KL_ROWS) + KL_KEYS - 1) / KL_KEYS + 1; }
@@ -498,7 +499,7 @@ __global__ void __launch_bounds__(KL_THREADS, 1)
   if (warp == 0 && lane == 0) {
     asm volatile("prefetch.tensormap [%0];" ::"l"(&map_k) : "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(&map_v) : "memory");
-    for (int s = 0; s < KL_MAX_SLOTS; ++s) { mbar_init(bar(KB_FULL + s), 1); mbar_init(bar(KB_EMPTY + s), 1); }
+    for (int s = 0; s < KL_MAX_SLOTS; ++s) { mbar_init(bar(KB_FULL + s), 1); mbar_init(bar(KB_EMPTY + s), 1); mbar_init(bar(KB_TAIL + s), 1); }
     mbar_init(bar(KB_Q), KL_SOFT / 32);
     for (int s = 0; s < 2; ++s) {
       mbar_init(bar(KB_S_FULL + s), 1); mbar_init(bar(KB_S_EMPTY + s), KL_SOFT / 32);
@@ -630,7 +631,8 @@ __global__ void __launch_bounds__(KL_THREADS, 1)
           for (int kh = 0; kh < (both_halves(kext, c) ? 2 : 1); ++kh) {
             const int slot = k_slots + vs;
             if (!take(slot, v_ph, (c + 1) * KL_KEYS <= old_keys)) return;
-            const uint32_t fb = bar(KB_FULL + slot);
+            // (the values that the extent ends among are full when warp 3 has cleared the rest)
+            const uint32_t fb = bar((c * 2 + kh + 1) * 64 > kext ? KB_TAIL + slot : KB_FULL + slot);
             mbar_expect_tx(fb, KL_SLOT);
             load_box_3d(ring + (uint32_t)slot * KL_SLOT, &map_v, fb, 0, key_row0 + c * KL_KEYS + kh * 64, 0, pol);
             if (++vs == v_slots) { vs = 0; v_ph ^= 1u; }
@@ -733,6 +735,28 @@ __global__ void __launch_bounds__(KL_THREADS, 1)
         }
         j0 += n_chunks;
       }
+    }
+  } else if (warp == 3) {
+    // ===================== the end of every tile's values =====================
+    // Keys past the extent have weights of zero, but their slots may hold anything (and the box that crosses the last slot another
+    // head's or sequence's values), and zero times that has to be zero.  A warp of its own: the issuing one would do it between the
+    // weights of two chunks (which cost the 7B step 0.4 %, this 0.2).
+    int v_used = 0;       // V slots filled by the tiles before, in the ring's order
+    uint32_t tail_ph = 0;
+    bool ok = true;
+    for (int k = 0; k < n_tiles && ok; ++k) {
+      const int kext = sm->tiles[k].kext, rows = kext & 63;   // of the last half chunk
+      v_used += (kext + 63) >> 6;
+      if (rows == 0) continue;
+      const int slot = k_slots + (v_used - 1) % v_slots;
+      ok = __all_sync(0xffffffffu, mbar_wait(bar(KB_TAIL + slot), (tail_ph >> slot) & 1u, &sm->abort_flag, p.status)) != 0;
+      if (!ok) break;
+      tail_ph ^= 1u << slot;
+      uint4* const v = reinterpret_cast<uint4*>(gen + (ring - base) + (size_t)slot * KL_SLOT);   // [2 halves of the dimensions][64 keys][8]
+      for (int i = rows * 8 + lane; i < 64 * 8; i += 32) v[i] = v[64 * 8 + i] = make_uint4(0u, 0u, 0u, 0u);
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) mbar_arrive(bar(KB_FULL + slot));
     }
   } else if (warp >= 4) {
     // ===================== softmax and output =====================

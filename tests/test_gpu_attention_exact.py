@@ -154,3 +154,27 @@ def test_rows_whose_keys_all_lie_behind_the_first_chunk(monkeypatch):
     assert int(a.pk.n[0]) > 130
     assert a.errors(got, a.exact_verify()).max() < CLOSE
     assert a.route() == {"att_keys_on_lanes": 1}
+
+
+@pytest.mark.parametrize("beam,lens", [((1, 3), [77, 30, 250]), ((9, 5), [100, 30, 129]), ((3, 2), [249, 10, 63])])
+def test_nothing_behind_an_extent_reaches_the_output(monkeypatch, beam, lens):
+    """Slots behind a sequence's keys, and another sequence's cache, may hold anything: not-a-number and infinities there leave every
+    other row's bits alone, also where the last box of keys runs past the last slot into the next head's and sequence's."""
+    rows = 1 + beam[0] * beam[1]
+    q = torch.randn(3, HD, generator=torch.Generator().manual_seed(5)).cuda()
+    a = Attention(monkeypatch, 3, lens, beam, q, torch.ones(3, HD), 2, max_ctx=max(lens) + rows)
+    a.beams = dev(np.arange(len(lens) * rows)[:len(lens) * beam[0] * beam[1]].reshape(len(lens), *beam))
+    a.roots = dev(np.full(len(lens), 999))
+    a.kv[0].normal_()
+    clean = a.kv.clone()
+    for call in (a.verify, a.ar):
+        a.kv.copy_(clean)
+        want = [t.clone() for t in call()]
+        for bad in (math.nan, math.inf):
+            a.kv.copy_(clean)
+            for b, c in enumerate(lens):
+                a.kv[:, b, :, 0 if b == 1 else c:] = bad
+            got = call()
+            assert not torch.isfinite(got[1]).all()
+            assert torch.equal(got[0], want[0]) and torch.equal(got[2], want[2])
+    assert int(a.pk.n.min()) == rows and set(a.route()) == {"att_keys_on_lanes"}
