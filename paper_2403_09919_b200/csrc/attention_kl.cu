@@ -9,13 +9,15 @@
 //   softmax          sixteen warps, four per lane quarter with a quarter of the columns each: a thread has one key and those
 //                    rows.  A row's reference maximum is moved only when a score exceeds it by 2^32 (one vote per chunk): the
 //                    maximum over the keys lies across the lanes, and finding it for every chunk would cost more than the
-//                    exponentials.  Weights far from one have the same relative rounding; with the
-//                    maximum as reference the largest weight would be exactly one, so the sums (fp32) are those of the
-//                    rounded weights: what rounding does to a weight that outweighs the rest cancels in the quotient;
-//   O^T += V^T P^T   A = V chunk as it lies in the cache ([key][dim], MN-major), B = the weights, written to shared memory
-//                    as [16 rows][key] lines of 32 bytes (MN-major, 32-byte swizzle), D: lane = dimension, column = row.
+//                    exponentials.  With the maximum as reference the largest weight would be exactly one; here it is rounded
+//                    like the rest, which alone would make the output less exact than the other kernels' (2.3e-3 against
+//                    1.9 to 2.1e-3, scores of deviation 1.5).  So every weight goes in two parts, itself in bf16 and
+//                    what that rounding left, again in bf16 (to 2^-17 together; 1.65e-3, the rounding of the output);
+//   O^T += V^T P^T   A = V chunk as it lies in the cache ([key][dim], MN-major), B = the weights and behind them their
+//                    remainders as further columns, written to shared memory as [16 rows][key] lines of 32 bytes (MN-major,
+//                    32-byte swizzle), D: lane = dimension, column = row, and again for the remainders; the output adds the two.
 //
-// A tile is (head, sequence, up to 128 of its rows); a sequence with more rows is cut into equal tiles.  One CTA per SM takes
+// A tile is (head, sequence, up to 96 of its rows); a sequence with more rows is cut into equal tiles.  One CTA per SM takes
 // its tiles one after the other (longest sequences first): K and V come through two rings of 16 KB slots (half of a chunk's
 // dimensions of K, half of its keys of V) that the producer keeps filled across the tiles' ends, and the next tile's first
 // scores are formed while the one before is written out.
@@ -24,13 +26,15 @@
 // output.  Every wait is bounded (one second), as in attention_t5.cu; a warp that gives up still takes part in the named barriers
 // until all of its part have seen it.
 //
-// What bounds it: the copies where every SM has tiles (7B, 16 sequences of 256 to 2048 tokens: 70 us a launch for 302 MB of keys and
-// values, launch and set-up included, 95 us before; 16 x 1024 tokens of one row each 57 against 69), else a chunk's chain of hand-overs
+// What bounds it: the copies where every SM has tiles (7B, 16 sequences of 256 to 2048 tokens: 70 us a launch without the remainders
+// for 302 MB of keys and values, launch and set-up included, 95 us in the 64- and 128-row kernels), else a chunk's chain of hand-overs
 // (scores 0.25 us, weights 0.35 to 0.6 us by columns, the product; 0.8 to 1.5 us a chunk) and, in the first, the code's fetch.
-// In place, per layer of the 7B shape: 1 x 512 tokens 120 -> 117 us, 3 x 200 to 900 tokens of 39 rows 160 -> 143, 16 of
-// 56 rows 466 -> 444.  Tried: two smaller CTAs per SM (half the copies under way each: 2 to 5 % behind), the loop run once over
-// nothing before the wait (no gain), a common ring for K and V, copies that stay in the L2 (16 sequences 444 -> 450, 4 single rows
-// 120 -> 124).
+// The remainders take 0.3 % of a 7B step (30 rows, 512 tokens), 0.4 to 0.9 of the 7B calls, 1.5 of the batch-16 step and 2 of
+// 4 x 4096 tokens at 33B, most of it for forming and storing them (doubled columns alone: 0.3 %).  One buffer of weights
+// instead of two for tiles of 64 rows and more, which leaves the rings half as much again: 7B batch 16 33.4 -> 33.9 ms, 33B 32.2 -> 32.6.
+// Tried before: two smaller CTAs per SM (half the copies under way each: 2 to 5 % behind), the loop run once over nothing before
+// the wait (no gain), a common ring for K and V, copies that stay in the L2 (16 sequences 444 -> 450 us a layer, 4 single rows
+// 120 -> 124).  96 registers (640 threads), 68 bytes of them spilled in the widest tiles.
 #include "pdl.cuh"
 #include "rd_internal.cuh"
 #include "tcgen05.cuh"
@@ -47,7 +51,7 @@ constexpr int KL_SOFT = 128 * KL_PARTS;
 constexpr int KL_THREADS = 128 + KL_SOFT;
 constexpr uint32_t KL_SLOT = 16384;    // ring slot: 64 dimensions of 128 keys (K), 64 keys of 128 dimensions (V)
 constexpr int KL_MAX_SLOTS = 12;
-constexpr uint32_t KL_TMEM = 512;      // columns: two score buffers of 128, the output from 256
+constexpr uint32_t KL_TMEM = 512;      // columns: two score buffers of 128, the output from 256 (twice a tile's columns)
 constexpr int KL_MAX_TILES = 32;       // tiles of a CTA
 constexpr uint32_t KL_SMEM = 227 * 1024;
 constexpr float KL_SLACK = 32.0f;      // log2 by which a score may exceed its row's reference
@@ -148,6 +152,10 @@ __device__ __forceinline__ void mul2(float& x, float& y, float f) {   // both by
   asm("{\n\t.reg .b64 a, b;\n\tmov.b64 a, {%0, %1};\n\tmov.b64 b, {%2, %2};\n\tmul.rn.f32x2 a, a, b;\n\tmov.b64 {%0, %1}, a;\n\t}"
       : "+f"(x), "+f"(y) : "f"(f));
 }
+__device__ __forceinline__ void fma2(float& x, float& y, float f, float u, float v) {   // both times f, plus u and v
+  asm("{\n\t.reg .b64 a, b, c;\n\tmov.b64 a, {%0, %1};\n\tmov.b64 b, {%2, %2};\n\tmov.b64 c, {%3, %4};\n\tfma.rn.f32x2 a, a, b, c;\n\tmov.b64 {%0, %1}, a;\n\t}"
+      : "+f"(x), "+f"(y) : "f"(f), "f"(u), "f"(v));
+}
 __device__ __forceinline__ void add2(float& x, float& y, float u, float v) {
   asm("{\n\t.reg .b64 a, b;\n\tmov.b64 a, {%0, %1};\n\tmov.b64 b, {%2, %3};\n\tadd.rn.f32x2 a, a, b;\n\tmov.b64 {%0, %1}, a;\n\t}"
       : "+f"(x), "+f"(y) : "f"(u), "f"(v));
@@ -225,7 +233,7 @@ struct KlCtx {
 template <int COLS>
 __device__ __forceinline__ void kl_softmax(const KlParams& p, const KlCtx& t, const int n_tiles) {
   constexpr int N = KL_PARTS * COLS;
-  constexpr uint32_t TILE_BYTES = N * 256u;
+  constexpr uint32_t WEIGHT_BYTES = 2 * N * 256u;   // a chunk's weights and their remainders
   KlShared* sm = t.sm;
   const int st = (int)threadIdx.x - 128, tip = st & 127;   // thread of the softmax warps, of this part
   const int lane = threadIdx.x & 31, q4 = (st >> 5) & 3, part = st >> 7;
@@ -304,11 +312,16 @@ __device__ __forceinline__ void kl_softmax(const KlParams& p, const KlCtx& t, co
           for (int i = 0; i < COLS; ++i) sc[i] = ((seen >> i) & 1u) ? sc[i] : -INFINITY;
         }
         // to base 2: 1/sqrt(hd) * log2(e)
+        if (!moved) {
 #pragma unroll
-        for (int i = 0; i < COLS; i += 2) mul2(sc[i], sc[i + 1], scale2);
-        if (moved) {
+          for (int i = 0; i < COLS; i += 2) mul2(sc[i], sc[i + 1], scale2);
+        } else {
 #pragma unroll
-          for (int i = 0; i < COLS; ++i) sc[i] += sm->nref[col0 + i];
+          for (int i = 0; i < COLS; i += 4) {
+            const float4 n = *reinterpret_cast<const float4*>(&sm->nref[col0 + i]);
+            fma2(sc[i], sc[i + 1], scale2, n.x, n.y);
+            fma2(sc[i + 2], sc[i + 3], scale2, n.z, n.w);
+          }
         }
         float mx = sc[0];
 #pragma unroll
@@ -320,8 +333,7 @@ __device__ __forceinline__ void kl_softmax(const KlParams& p, const KlCtx& t, co
         float low = sc[0];
 #pragma unroll
         for (int i = 1; i < COLS; ++i) low = fminf(low, sc[i]);
-        // (where the first chunk is most of the keys, one of them often outweighs the rest: its weight is made one, and exact)
-        move = !bar_any<128>(part_bar, ok && low >= -KL_LOW && n_chunks > 2) || move;
+        move = !bar_any<128>(part_bar, ok && low >= -KL_LOW) || move;
         none = move;
       }
       if (move) {
@@ -353,12 +365,17 @@ __device__ __forceinline__ void kl_softmax(const KlParams& p, const KlCtx& t, co
             tc_fence_after();
 #pragma unroll 1
             for (int i = 0; i < COLS; i += 4) {
-              float o[4];
+              float o[4], r[4];
               tmem_ld4_nowait(o_addr + i, o);
+              tmem_ld4_nowait(o_addr + N + i, r);
               tmem_ld_wait();
 #pragma unroll
-              for (int n = 0; n < 4; ++n) o[n] *= fast_exp2(fminf(sm->corr[col0 + i + n], 0.f));
+              for (int n = 0; n < 4; ++n) {
+                const float f = fast_exp2(fminf(sm->corr[col0 + i + n], 0.f));
+                o[n] *= f; r[n] *= f;
+              }
               tmem_st4(o_addr + i, o);
+              tmem_st4(o_addr + N + i, r);
             }
             tmem_st_wait();
           }
@@ -367,26 +384,28 @@ __device__ __forceinline__ void kl_softmax(const KlParams& p, const KlCtx& t, co
       // this chunk's buffer of weights is free once the product of the chunk before last has read it
       if (ok && j >= 2) ok = wait_all(bar(KB_PV_DONE + (j & 1)), ph ^ 1u);
       if (ok) {
-        uint8_t* const line = p_line + (uint32_t)(j & 1) * TILE_BYTES;
-        uint32_t pk[COLS / 2];
+        // four weights at a time, and what their rounding left of them (exact in fp32) rounded again
+        uint8_t* const line = p_line + (uint32_t)(j & 1) * WEIGHT_BYTES;
+        uint32_t hi[4], lo[4];
 #pragma unroll
-        for (int i = 0; i < COLS; i += 2) {
-          pk[i / 2] = pack_bf16(fast_exp2(sc[i]), fast_exp2(sc[i + 1]));   // 2^(-inf) = 0
-          add2(l[i], l[i + 1], __uint_as_float(pk[i / 2] << 16), __uint_as_float(pk[i / 2] & 0xffff0000u));
-        }
-        if (COLS % 8 == 0) {
+        for (int i = 0; i < COLS; i += 4) {
+          const int col = col0 + i, at = COLS % 8 ? 0 : (i & 4) / 2;
 #pragma unroll
-          for (int i = 0; i < COLS; i += 8) {
-            const int col = col0 + i;
-            *reinterpret_cast<uint4*>(line + (col >> 4) * (KL_KEYS * 32) + ((((uint32_t)(col >> 3) & 1u) ^ p_swz) << 4)) =
-                make_uint4(pk[i / 2], pk[i / 2 + 1], pk[i / 2 + 2], pk[i / 2 + 3]);
+          for (int n = 0; n < 4; n += 2) {
+            const float x = fast_exp2(sc[i + n]), y = fast_exp2(sc[i + n + 1]);   // 2^(-inf) = 0
+            add2(l[i + n], l[i + n + 1], x, y);
+            const uint32_t h = pack_bf16(x, y);
+            float rx = __uint_as_float(h << 16), ry = __uint_as_float(h & 0xffff0000u);
+            fma2(rx, ry, -1.f, x, y);
+            hi[at + n / 2] = h; lo[at + n / 2] = pack_bf16(rx, ry);
           }
-        } else {
-#pragma unroll
-          for (int i = 0; i < COLS; i += 4) {
-            const int col = col0 + i;
-            *reinterpret_cast<uint2*>(line + (col >> 4) * (KL_KEYS * 32) + ((((uint32_t)(col >> 3) & 1u) ^ p_swz) << 4) + (col & 4) * 2) =
-                make_uint2(pk[i / 2], pk[i / 2 + 1]);
+          uint8_t* const to = line + (col >> 4) * (KL_KEYS * 32) + ((((uint32_t)(col >> 3) & 1u) ^ p_swz) << 4);
+          if (COLS % 8) {
+            *reinterpret_cast<uint2*>(to + (col & 4) * 2) = make_uint2(hi[0], hi[1]);
+            *reinterpret_cast<uint2*>(to + N * 256 + (col & 4) * 2) = make_uint2(lo[0], lo[1]);
+          } else if (i & 4) {
+            *reinterpret_cast<uint4*>(to) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+            *reinterpret_cast<uint4*>(to + N * 256) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
           }
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -450,16 +469,20 @@ __device__ __forceinline__ void kl_softmax(const KlParams& p, const KlCtx& t, co
       tc_fence_after();
       const int odd = lane & 1, nrows = tl.nrows;
       __nv_bfloat16* o = p.out + (size_t)(tl.row0 + col0 + odd) * p.dm.d + tl.head * KL_HD + q4 * 32 + (lane & ~1);
-      float ov[4];
+      float ov[4], rv[4];
       tmem_ld4_nowait(o_addr, ov);
+      tmem_ld4_nowait(o_addr + N, rv);
 #pragma unroll 1
       for (int i = 0; i < COLS; i += 4) {
         float v[4];
         tmem_ld_wait();
         if (col0 + i >= nrows) break;   // the same for the whole warp
 #pragma unroll
-        for (int n = 0; n < 4; ++n) v[n] = ov[n];
-        if (i + 4 < COLS) tmem_ld4_nowait(o_addr + i + 4, ov);
+        for (int n = 0; n < 4; ++n) v[n] = ov[n] + rv[n];
+        if (i + 4 < COLS) {
+          tmem_ld4_nowait(o_addr + i + 4, ov);
+          tmem_ld4_nowait(o_addr + N + i + 4, rv);
+        }
 #pragma unroll
         for (int n = 0; n < 4; n += 2) {
           const float2 inv = *reinterpret_cast<const float2*>(&sm->corr[col0 + i + n]);
@@ -586,14 +609,14 @@ __global__ void __launch_bounds__(KL_THREADS, 1)
   tc_fence_after();
   const uint32_t tmem = sm->tmem;
   const int n_tiles = sm->n_tiles;
-  // ---- operands behind KlShared, sized for the CTA's largest tile: its rows, two buffers of weights, and ring slots.  K and V
+  // ---- operands behind KlShared, sized for the CTA's largest tile: its rows, two buffers of weights and remainders, and ring slots.  K and V
   // have rings of their own because each is read by a warp of its own: in a common ring one reader could be a lap ahead of the
   // other, and a barrier's parity would mistake the laps.  V has a chunk's two slots more: the scores run two chunks ahead of
   // the output, so that K's slots come free as much earlier, and with the copies in turn, K a chunk ahead, both rings are full
   // of copies under way.
   const int N = max(16, (sm->rows_max + 15) & ~15);
   const uint32_t tile_bytes = (uint32_t)N * 256u;
-  const uint32_t sQ = base + kl_front_bytes(dm.NMAX), sP = sQ + tile_bytes, ring = sP + 2u * tile_bytes;
+  const uint32_t sQ = base + kl_front_bytes(dm.NMAX), sP = sQ + tile_bytes, ring = sP + 4u * tile_bytes;
   const int n_slots = min(KL_MAX_SLOTS, (int)((raw + KL_SMEM - ring) / KL_SLOT)), v_slots = n_slots / 2 + 1, k_slots = n_slots - v_slots;
   // second 64 keys of a chunk: multiplied only if some row attends one of them
   auto both_halves = [&](int kext, int c) { return kext - c * KL_KEYS > KL_KEYS / 2; };
@@ -677,7 +700,7 @@ __global__ void __launch_bounds__(KL_THREADS, 1)
       bool ok = true;
       int j0 = 0;   // chunks of the tiles before this one
       const uint32_t idesc_qk = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(KL_KEYS >> 4) << 24);
-      const uint32_t idesc_pv = idesc_qk | (1u << 15) | (1u << 16);   // both operands MN-major; M = 128 head dimensions
+      const uint32_t idesc_pv = idesc_qk + ((uint32_t)(N >> 3) << 17) | (1u << 15) | (1u << 16);   // N doubled (weights and remainders), both operands MN-major; M = 128 head dimensions
       const uint64_t q_desc = desc_kmajor(sQ);
       for (int k = 0; k < n_tiles && ok; ++k) {
         const KlTile& tl = sm->tiles[k];
@@ -714,7 +737,7 @@ __global__ void __launch_bounds__(KL_THREADS, 1)
             const bool live = c >= 0, on = live && leader;
             const int halves = both_halves(kext, c) ? 2 : 1;
             if (live) ok = wait_warp(bar(KB_P_FULL + (j & 1)), (uint32_t)((j >> 1) & 1));
-            const uint64_t p_desc = desc_mn32(sP + (uint32_t)(j & 1) * tile_bytes, KL_KEYS * 32);
+            const uint64_t p_desc = desc_mn32(sP + (uint32_t)(j & 1) * 2u * tile_bytes, KL_KEYS * 32);
 #pragma unroll 1
             for (int kh = 0; kh < halves && ok; ++kh) {
               if (live) {
@@ -787,9 +810,9 @@ __global__ void __launch_bounds__(KL_THREADS, 1)
 }  // namespace
 
 int attn_kl_row_tiles(int rows) { return (rows + KL_ROWS - 1) / KL_ROWS; }
-// Tiles of the most rows leave either ring a chunk.
+// Tiles of the most rows leave either ring a chunk (K two slots, V three).
 bool attn_kl_supported(int hd, int NMAX) {
-  return hd == KL_HD && 1024 + kl_front_bytes(NMAX) + 3u * KL_ROWS * 256u + 4u * KL_SLOT <= KL_SMEM;
+  return hd == KL_HD && 1024 + kl_front_bytes(NMAX) + 5u * KL_ROWS * 256u + 5u * KL_SLOT <= KL_SMEM;
 }
 
 cudaError_t attn_kl_prepare(int hd) {
