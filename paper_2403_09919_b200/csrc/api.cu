@@ -542,31 +542,39 @@ int layers_simt(rd_handle* h, const RowTables& rt, int m_max, Chain* ch, cudaStr
 }
 
 // Whether this handle's verification and autoregressive passes can take the attention kernel with the keys on the lanes at all.
-// Models of fewer than 24 heads keep the earlier kernels, whose lines are held by tests; of the shapes here only the small models
-// of the tests have so few.
+// Models of fewer than 24 heads keep the earlier kernels; that is where their lines are tested, not where they are faster.  Measured
+// per pass of 4 layers, contexts of 60 to 2000 tokens, models of 8, 12, 16 and 20 heads: with 4 sequences and more, of 31 or 81 rows,
+// -35 to +5 % (8 heads, 16 x 81 rows) with the keys on the lanes, autoregressive -15 to +8 %; with one sequence -5 to +6 % (31 rows), +1 to
+// +18 % (81 rows), autoregressive -3 to +15 %.
 bool keys_on_lanes_possible(const rd_handle* h) {
   return h->att_kl != 0 && !h->kv_maps.empty() && attn_kl_supported(h->dm.hd, h->dm.NMAX) && (h->att_kl >= 2 || h->dm.H >= 24);
 }
 
 // Whether a pass takes the attention kernel with the keys on the lanes; `wide`: else it would take the 64- or 128-row kernel.
-// Measured per layer (4 layers, contexts of 60, 150-300, 500, 256-1024 and 2048 tokens, earlier kernel -> this one):
-// verification, 7B, 1 sequence of 30 / 82 rows -1 to -8 / -4 to -23 %; 4 of 32 -3 to -17; 8 of 30, 56, 85 -7 to 0, -8 to -1, -9 to 0;
-// 16 of 17, 30, 56 -12 to -5, -11 to -5, -9 to -3; 13B and 33B alike.  It loses
-// - where sequences of more than 64 rows leave every SM one wide tile, which the 64- and 128-row kernels walk as fast with less
-//   set-up (4 x 54 / 62 / 89 rows, 128 tiles: +1 to +5 / -1 to +9 / 0 to +9 %; 13B, 4 x 89, 160 tiles: +3 to -4), but where they
-//   can be cut into two tiles or more each, it is ahead again (152 rows, 32 tiles: -1 to -5);
-// - on several tiles per SM with less than a chunk of keys (60 tokens, 8 or 16 sequences: 0 to +3 %);
-// - on few tiles of up to 16 rows and a thousand keys, which the 16-row kernel splits (7B, 1 sequence of 11 rows, 2048 tokens +1.3 %,
-//   of 60 to 500 tokens -2; 13B, 3 rows, 1400 tokens +1.7);
-// - in autoregressive steps of a single sequence, whose keys the 16-row kernel splits (7B +1 to +5 %, 33B -2 to +1), and of few
-//   keys (100 tokens: 0 to +3); 2 to 16 sequences of 500 to 2500 tokens -20 to 0, two points +1.5.
+// Measured per pass of 4 layers, earlier kernel -> this one (two in turn, 8 to 12 times; +-1 % where the power limit is reached):
+// - verification, 7B, 60 / 200 / 500 / 1000 / 2048 tokens: 1 sequence of 31 rows 0 / 0 / -2 / -3 / -4 %, of 81 +1 / 0 / -3 / -5 / -6; 8 of
+//   16 rows -2 to -9 (130 to 1000 tokens), of 51 +1 to -5, of 81 -6 to 0; 16 of 51 and 81 -4 to -10 and -9 to -3; 4 of 51 -6 to -30.
+// - Sequences of more than 64 rows that would take the 64- or 128-row kernel and leave every SM one wide tile stay there: 7B 4 x 81 rows
+//   -1 to +4 %, 13B 2 x 125 +3 to +12, 3 x 161 +1 to +2, 33B 2 x 81 +2 to +3.  13B 4 x 161 and 33B 3 x 161 (160 and 156 tiles) -1 to +1.
+// - Where the sequence can be cut into narrower tiles this kernel is ahead, as a tile of 48 or 64 rows takes less time per chunk: into two
+//   up to 192 rows (7B 1 x 151 -2 to -18), above into three, with rows as drafted beams pack them (45 to 70 % of the bound) at 300 / 1024 / 3000
+//   tokens: 7B bound of 321 rows 0 / -2 / -4 to +1 / 0 / -2 %, 13B 241 -1 / -2 / -4 to 0 / -2 / -3, 13B 321 0 / -1 / -2 to +1 / +1 / +2 (when
+//   all are different: 7B +5, 13B 241 +3, 13B 321 +4 / +6 / +10).  33B has room for two cuts only: 1 x 227 of 321 +5 / +7 / +15, 1 x 201 of
+//   201 +3 / +5 / +8, and stays with the 128-row kernel.
+// - On several tiles per SM it needs a chunk of keys (60 tokens, 8 or 16 sequences: -4 to +3 %); against the 128-row kernel there: 33B
+//   4 x 78 rows of 161, 1100 and 2500 tokens 0 and +1, 7B 16 x 52 rows of 81 -7, 16 x 81 -1.
+// - On few tiles of up to 16 rows and a thousand keys the 16-row kernel splits the keys (7B, 1 sequence of 11 and 16 rows, 2048 tokens 0;
+//   13B, 40 tiles, -2; 33B, 52 tiles, -4).
+// - Autoregressive steps: of a single sequence the 16-row kernel splits the keys (7B 750 and 1500 tokens +1 and +2 %, 33B -1 and -2); of 100
+//   to 130 tokens 0 to +3; 2 to 8 sequences of 260 tokens +1 to -2, of 600 -2 to -6.
 bool use_keys_on_lanes(const rd_handle* h, bool tree, int n_seq, int rows_per_seq_max, bool wide) {
   const Dims& dm = h->dm;
   if (!keys_on_lanes_possible(h)) return false;
   if (h->att_kl >= 2) return true;
   const int tiles = dm.H * n_seq, G = h->tc_grid;
   if (!tree) return rows_per_seq_max == 1 && tiles >= 64 && (h->route_bound >= 256 || tiles >= 3 * G);
-  if (wide && rows_per_seq_max > 64 && 2 * tiles > G && (tiles <= G || (rows_per_seq_max >= 96 && 4 * tiles <= 5 * G))) return false;
+  const int cuts = rows_per_seq_max > 192 ? 3 : 2;
+  if (wide && rows_per_seq_max > 64 && cuts * tiles > G && (tiles <= G || (rows_per_seq_max >= 96 && 4 * tiles <= 5 * G))) return false;
   if (rows_per_seq_max <= 16 && tiles < 64 && h->route_bound >= 1024) return false;
   return tiles <= G || h->route_bound >= 128;
 }

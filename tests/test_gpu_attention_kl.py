@@ -111,6 +111,21 @@ def test_lines_of_verification(heads, batch, bw, tokens, taken):
     eng.close()
 
 
+@pytest.mark.parametrize("heads,bw,taken", [
+    (49, 40, True), (50, 40, False), (50, 38, True), (40, 64, True),   # bounds of 201, 191 and 321 rows that the 64- or 128-row kernel would
+                                                                       # take: more than two tiles' need room for three on the SMs
+])
+def test_lines_of_single_sequences(heads, bw, taken):
+    cfg = config(heads, n_layers=1, beam_width=bw, max_ctx=700)
+    eng = ReDrafter(cfg, synth.make_weights(cfg, "cuda:0"))
+    rng = np.random.default_rng(8)
+    eng.set_state(dev(np.full(1, 300)), dev(rng.integers(0, 1000, size=1)), torch.randn(1, cfg["d_model"], device="cuda"), batch=1, ctx_bound=300)
+    eng.verify(eng.pack(dev(rng.integers(0, 1000, size=(1, bw, 5)))))
+    eng.poll()
+    assert eng.route_counts()["att_keys_on_lanes"] == (1 if taken else 0)
+    eng.close()
+
+
 @pytest.mark.parametrize("batch,tokens,taken", [(2, 300, False), (3, 255, False), (3, 256, True), (19, 40, True)])
 def test_lines_of_autoregressive_steps(batch, tokens, taken):
     cfg = config(24, n_layers=1, max_batch=batch, beam_width=2, max_ctx=400)
