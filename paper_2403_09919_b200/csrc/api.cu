@@ -561,6 +561,9 @@ bool keys_on_lanes_possible(const rd_handle* h) {
 //   tokens: 7B bound of 321 rows 0 / -2 / -4 to +1 / 0 / -2 %, 13B 241 -1 / -2 / -4 to 0 / -2 / -3, 13B 321 0 / -1 / -2 to +1 / +1 / +2 (when
 //   all are different: 7B +5, 13B 241 +3, 13B 321 +4 / +6 / +10).  33B has room for two cuts only: 1 x 227 of 321 +5 / +7 / +15, 1 x 201 of
 //   201 +3 / +5 / +8, and stays with the 128-row kernel.
+// - Sequences of more than 64 rows whose 16-row tiles fit one wave stay with the 16-row kernel, which has three to six times as many CTAs
+//   for them: 24 heads, 1 x 66 and 81 rows, 60 / 300 / 1000 / 2000 tokens +5 / +5 / +2 / 0 and +6 / +5 / +4 / +3 %, 28 heads 1 x 66 +4 / +3 / +1 /
+//   0; with 28 heads, 1 x 81 (168 tiles) +2 / 0 / -4 / -5.  (41 rows: 24 heads +2 / +1 / 0 / +1, 28 heads +1 / +1 / -4 / -5.)
 // - On several tiles per SM it needs a chunk of keys (60 tokens, 8 or 16 sequences: -4 to +3 %); against the 128-row kernel there: 33B
 //   4 x 78 rows of 161, 1100 and 2500 tokens 0 and +1, 7B 16 x 52 rows of 81 -7, 16 x 81 -1.
 // - On few tiles of up to 16 rows and a thousand keys the 16-row kernel splits the keys (7B, 1 sequence of 11 and 16 rows, 2048 tokens 0;
@@ -575,6 +578,7 @@ bool use_keys_on_lanes(const rd_handle* h, bool tree, int n_seq, int rows_per_se
   if (!tree) return rows_per_seq_max == 1 && tiles >= 64 && (h->route_bound >= 256 || tiles >= 3 * G);
   const int cuts = rows_per_seq_max > 192 ? 3 : 2;
   if (wide && rows_per_seq_max > 64 && cuts * tiles > G && (tiles <= G || (rows_per_seq_max >= 96 && 4 * tiles <= 5 * G))) return false;
+  if (rows_per_seq_max > 64 && tiles * ((rows_per_seq_max + 15) / 16) <= G) return false;
   if (rows_per_seq_max <= 16 && tiles < 64 && h->route_bound >= 1024) return false;
   return tiles <= G || h->route_bound >= 128;
 }

@@ -114,7 +114,7 @@ def test_lines_of_verification(heads, batch, bw, tokens, taken):
 @pytest.mark.parametrize("heads,bw,taken", [
     (49, 40, True), (50, 40, False), (50, 38, True), (40, 64, True),   # bounds of 201, 191 and 321 rows that the 64- or 128-row kernel would
                                                                        # take: more than two tiles' need room for three on the SMs
-])
+    (24, 16, False), (25, 16, True), (24, 12, True)])                  # 81 rows: 144 and 150 tiles of 16 rows; 61 rows
 def test_lines_of_single_sequences(heads, bw, taken):
     cfg = config(heads, n_layers=1, beam_width=bw, max_ctx=700)
     eng = ReDrafter(cfg, synth.make_weights(cfg, "cuda:0"))
