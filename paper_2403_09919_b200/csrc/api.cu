@@ -583,6 +583,67 @@ bool use_keys_on_lanes(const rd_handle* h, bool tree, int n_seq, int rows_per_se
   return tiles <= G || h->route_bound >= 128;
 }
 
+// How a pass's attention is launched.
+struct AttentionPlan {
+  // tiles of 16 rows per sequence (64, 128); keys split over CTAs only for long contexts with few tiles
+  int row_blocks = 1, n_splits = 1, split_chunks = 1, split_min = 1;
+  bool wide = false, shallow = false, t5 = false, kl = false;   // the 64-row kernel, the short ring, the 128-row kernel, the keys on the lanes
+};
+
+AttentionPlan plan_attention(const rd_handle* h, bool tree, int n_seq, int rows_per_seq_max) {
+  const Dims& dm = h->dm;
+  AttentionPlan p;
+  if (!h->use_tc) return p;
+  const int rpb = attn_tc_rows_per_block();
+  p.row_blocks = (rows_per_seq_max + rpb - 1) / rpb;
+  const int blocks = dm.H * n_seq * p.row_blocks;
+  // The 16-row kernel runs one CTA per SM; past a few waves of them the 64-row kernel (three CTAs per SM, each
+  // K/V chunk staged once for four times the rows) takes over.
+  static const int wide_waves = getenv("RD_ATT_WIDE") ? atoi(getenv("RD_ATT_WIDE")) : 4;   // tuning toggle
+  p.wide = wide_waves < 0 || (wide_waves > 0 && blocks > wide_waves * h->tc_grid);   // negative: always
+  static const int t5_ok = getenv("RD_ATT_T5") ? atoi(getenv("RD_ATT_T5")) : 1;   // tuning toggle
+  // (its 128-row tiles and 128-key chunks pay off when a sequence brings several hundred rows to the launch -- prompt
+  // processing -- or, in a verification pass, when a sequence can fill at least half a tile and the context is long; from
+  // three chunks of keys on where a sequence can bring 96 rows or its tiles take a single wave.  4 layers, 64-row kernel ->
+  // this one, with 0.3 / 0.45 / 0.6 / 0.8 of the bound present: 7B 10 sequences of up to 106 rows, 400 tokens -1 / -3 / -3 /
+  // -2 %; 4 of 161, 400 tokens -1 / -3 / -4 / -6; 4 of 81 (128 tiles, one wave), 400 tokens -4 / -5 / -7 / -6; 13B 3 of 201,
+  // 260 tokens -5 / +2 / -5 / -6; but 16 of 81 (512 tiles) +4 / 0 / +3 / -4 at 260 tokens and +2 / +7 / +1 / -7 at 400, 33B
+  // 12 of 81 +4 / +2 / +2 / -2 and +7 / +4 / +2 / 0; the batched 7B step of 256 to 2048 tokens took 17.5 instead of 17.9 ms.
+  // RD_ATT_T5=2 takes it whenever the 64-row kernel would run.)
+  static const int t5_rows = getenv("RD_ATT_T5_ROWS") ? atoi(getenv("RD_ATT_T5_ROWS")) : 64;   // tuning toggle
+  const int t5_tiles = dm.H * n_seq * ((rows_per_seq_max + attn_t5_rows_per_block() - 1) / attn_t5_rows_per_block());
+  const int t5_keys = tree && (rows_per_seq_max >= 96 || t5_tiles <= h->tc_grid) ? 320 : 1024;
+  const bool t5_pays = rows_per_seq_max >= 512 || (rows_per_seq_max >= t5_rows && h->route_bound + rows_per_seq_max >= t5_keys);
+  p.t5 = p.wide && !h->kv_maps.empty() && ((t5_ok == 1 && t5_pays) || t5_ok >= 2);
+  if (p.t5) p.row_blocks = (rows_per_seq_max + attn_t5_rows_per_block() - 1) / attn_t5_rows_per_block();
+  else if (p.wide) p.row_blocks = (rows_per_seq_max + attn_wide_rows_per_block() - 1) / attn_wide_rows_per_block();
+  // more 16-row CTAs than SMs (many sequences of a few rows): a two-chunk ring so that three CTAs share an SM
+  static const int shallow_ok = getenv("RD_ATT_SHALLOW") ? atoi(getenv("RD_ATT_SHALLOW")) : 1;   // tuning toggle
+  // Keys split over CTAs: with fewer tiles than half the SMs, one CTA per SM and at least three chunks each; with more, up
+  // to three CTAs per SM (short ring) of at least six chunks, which also evens out sequences of different lengths -- but where
+  // the tiles alone leave no SM a second one, three splits or none.  (8 layers of the 7B shape, one split per SM and eight
+  // chunks before: autoregressive, 1 x 600 tokens 822 -> 807 us; 4 x 1100 940 -> 934; 3 x 2000 1026 -> 967; 2 x 800 tokens
+  // with 58 rows 1988 -> 1940.  Three per SM for few tiles too: 1 x 3000 877 -> 896; of three chunks: the 7B step at 512
+  // tokens 8.35 -> 8.66 ms; two chunks each for few tiles: small steps 1.60 -> 1.64; two splits of 96 tiles, whose 192 CTAs
+  // load the SMs unevenly and lose the long ring: a step at 1000 tokens 1841 instead of 1782 us, autoregressive, 3 x 800 907
+  // instead of 874.  Launches of fewer than 16 heads keep two splits: of the models here only the tests' have so few, and
+  // that a sequence of one chunk leaves a split empty is checked on them; without, 4 layers at 760 tokens 563 -> 534 us.)
+  // The kernel takes the real lengths for it; the host's bound only limits the launch.
+  const int max_chunks = (h->ctx_bound + rows_per_seq_max + 63) / 64;
+  const bool few = 2 * blocks <= h->tc_grid;
+  p.split_chunks = few ? 3 : 6;
+  p.split_min = !few && blocks <= h->tc_grid && dm.H >= 16 ? 3 : 1;
+  p.n_splits = (few ? h->tc_grid : 3 * h->tc_grid) / blocks;
+  if (p.n_splits > max_chunks / p.split_chunks) p.n_splits = max_chunks / p.split_chunks;
+  if (p.n_splits < p.split_min) p.n_splits = 1;
+  if (p.n_splits > 16) p.n_splits = 16;
+  if (p.n_splits < 1) p.n_splits = 1;
+  while (p.n_splits > 1 && (long long)blocks * p.n_splits > ATT_MAX_SPLIT_BLOCKS) --p.n_splits;
+  p.shallow = shallow_ok && !p.wide && blocks * p.n_splits > h->tc_grid;
+  p.kl = t5_ok < 2 && wide_waves >= 0 && use_keys_on_lanes(h, tree, n_seq, rows_per_seq_max, p.wide);
+  return p;
+}
+
 // Embedding -> n_layers x {attention block, FFN block} -> final norm.  Rows and masks come from the
 // row tables in the workspace; results: ws.hidden_f / ws.hidden_t (compact rows).
 int forward_layers(rd_handle* h, const uint32_t* mask, int m_max, int n_seq, int rows_per_seq_max, const void* after_w,
@@ -592,59 +653,7 @@ int forward_layers(rd_handle* h, const uint32_t* mask, int m_max, int n_seq, int
   RowTables rt{w.row_tok, w.row_seq, w.row_pos, w.row_slot, w.row_ncache, w.row_local, mask, w.m_total};
   CKP(h, PROF_MISC, launch_embed_rope(dm.dtype, h->w.tok_emb, w.row_tok, w.row_pos, w.x, w.rope_tab, dm.d, dm.V, dm.hd, dm.theta,
                                       w.m_total, m_max, w.status, st));
-  // attention launch geometry (tensor-core path): tiles of 16 rows per sequence; keys split over CTAs only
-  // for long contexts with few tiles
-  int row_blocks = 1, n_splits = 1, split_chunks = 1, split_min = 1;
-  bool att_wide = false, att_shallow = false, att_t5 = false, att_kl = false;
-  if (h->use_tc) {
-    const int rpb = attn_tc_rows_per_block();
-    row_blocks = (rows_per_seq_max + rpb - 1) / rpb;
-    const int blocks = dm.H * n_seq * row_blocks;
-    // The 16-row kernel runs one CTA per SM; past a few waves of them the 64-row kernel (three CTAs per SM, each
-    // K/V chunk staged once for four times the rows) takes over.
-    static const int wide_waves = getenv("RD_ATT_WIDE") ? atoi(getenv("RD_ATT_WIDE")) : 4;   // tuning toggle
-    att_wide = wide_waves < 0 || (wide_waves > 0 && blocks > wide_waves * h->tc_grid);   // negative: always
-    static const int t5_ok = getenv("RD_ATT_T5") ? atoi(getenv("RD_ATT_T5")) : 1;   // tuning toggle
-    // (its 128-row tiles and 128-key chunks pay off when a sequence brings several hundred rows to the launch -- prompt
-    // processing -- or, in a verification pass, when a sequence can fill at least half a tile and the context is long; from
-    // three chunks of keys on where a sequence can bring 96 rows or its tiles take a single wave.  4 layers, 64-row kernel ->
-    // this one, with 0.3 / 0.45 / 0.6 / 0.8 of the bound present: 7B 10 sequences of up to 106 rows, 400 tokens -1 / -3 / -3 /
-    // -2 %; 4 of 161, 400 tokens -1 / -3 / -4 / -6; 4 of 81 (128 tiles, one wave), 400 tokens -4 / -5 / -7 / -6; 13B 3 of 201,
-    // 260 tokens -5 / +2 / -5 / -6; but 16 of 81 (512 tiles) +4 / 0 / +3 / -4 at 260 tokens and +2 / +7 / +1 / -7 at 400, 33B
-    // 12 of 81 +4 / +2 / +2 / -2 and +7 / +4 / +2 / 0; the batched 7B step of 256 to 2048 tokens took 17.5 instead of 17.9 ms.
-    // RD_ATT_T5=2 takes it whenever the 64-row kernel would run.)
-    static const int t5_rows = getenv("RD_ATT_T5_ROWS") ? atoi(getenv("RD_ATT_T5_ROWS")) : 64;   // tuning toggle
-    const int t5_tiles = dm.H * n_seq * ((rows_per_seq_max + attn_t5_rows_per_block() - 1) / attn_t5_rows_per_block());
-    const int t5_keys = mask && (rows_per_seq_max >= 96 || t5_tiles <= h->tc_grid) ? 320 : 1024;
-    const bool t5_pays = rows_per_seq_max >= 512 || (rows_per_seq_max >= t5_rows && h->route_bound + rows_per_seq_max >= t5_keys);
-    att_t5 = att_wide && !h->kv_maps.empty() && ((t5_ok == 1 && t5_pays) || t5_ok >= 2);
-    if (att_t5) row_blocks = (rows_per_seq_max + attn_t5_rows_per_block() - 1) / attn_t5_rows_per_block();
-    else if (att_wide) row_blocks = (rows_per_seq_max + attn_wide_rows_per_block() - 1) / attn_wide_rows_per_block();
-    // more 16-row CTAs than SMs (many sequences of a few rows): a two-chunk ring so that three CTAs share an SM
-    static const int shallow_ok = getenv("RD_ATT_SHALLOW") ? atoi(getenv("RD_ATT_SHALLOW")) : 1;   // tuning toggle
-    // Keys split over CTAs: with fewer tiles than half the SMs, one CTA per SM and at least three chunks each; with more, up
-    // to three CTAs per SM (short ring) of at least six chunks, which also evens out sequences of different lengths -- but where
-    // the tiles alone leave no SM a second one, three splits or none.  (8 layers of the 7B shape, one split per SM and eight
-    // chunks before: autoregressive, 1 x 600 tokens 822 -> 807 us; 4 x 1100 940 -> 934; 3 x 2000 1026 -> 967; 2 x 800 tokens
-    // with 58 rows 1988 -> 1940.  Three per SM for few tiles too: 1 x 3000 877 -> 896; of three chunks: the 7B step at 512
-    // tokens 8.35 -> 8.66 ms; two chunks each for few tiles: small steps 1.60 -> 1.64; two splits of 96 tiles, whose 192 CTAs
-    // load the SMs unevenly and lose the long ring: a step at 1000 tokens 1841 instead of 1782 us, autoregressive, 3 x 800 907
-    // instead of 874.  Launches of fewer than 16 heads keep two splits: of the models here only the tests' have so few, and
-    // that a sequence of one chunk leaves a split empty is checked on them; without, 4 layers at 760 tokens 563 -> 534 us.)
-    // The kernel takes the real lengths for it; the host's bound only limits the launch.
-    const int max_chunks = (h->ctx_bound + rows_per_seq_max + 63) / 64;
-    const bool few = 2 * blocks <= h->tc_grid;
-    split_chunks = few ? 3 : 6;
-    split_min = !few && blocks <= h->tc_grid && dm.H >= 16 ? 3 : 1;
-    n_splits = (few ? h->tc_grid : 3 * h->tc_grid) / blocks;
-    if (n_splits > max_chunks / split_chunks) n_splits = max_chunks / split_chunks;
-    if (n_splits < split_min) n_splits = 1;
-    if (n_splits > 16) n_splits = 16;
-    if (n_splits < 1) n_splits = 1;
-    while (n_splits > 1 && (long long)blocks * n_splits > ATT_MAX_SPLIT_BLOCKS) --n_splits;
-    att_shallow = shallow_ok && !att_wide && blocks * n_splits > h->tc_grid;
-    att_kl = t5_ok < 2 && wide_waves >= 0 && use_keys_on_lanes(h, mask != nullptr, n_seq, rows_per_seq_max, att_wide);
-  }
+  const AttentionPlan ap = plan_attention(h, mask != nullptr, n_seq, rows_per_seq_max);
   GemmOut g_qkv, g_o, g_gu, g_dn;
   // inside the layer loop every launch hands over to the next through a counter; the launches before
   // and after it use the grid dependency
@@ -673,23 +682,23 @@ int forward_layers(rd_handle* h, const uint32_t* mask, int m_max, int n_seq, int
     }
     {
       ProfScope ps(h, 1, 0.0, st);
-      h->route[att_kl ? RD_ROUTE_ATT_KEYS_ON_LANES : att_t5 ? RD_ROUTE_ATT_ROWS128_TC5 : att_wide ? RD_ROUTE_ATT_ROWS64
-               : att_shallow ? RD_ROUTE_ATT_ROWS16_SHALLOW : RD_ROUTE_ATT_ROWS16]++;
-      if (!att_kl && !att_t5 && !att_wide && n_splits > 1) h->route[RD_ROUTE_ATT_KEY_SPLIT]++;
-      if (att_kl)
+      h->route[ap.kl ? RD_ROUTE_ATT_KEYS_ON_LANES : ap.t5 ? RD_ROUTE_ATT_ROWS128_TC5 : ap.wide ? RD_ROUTE_ATT_ROWS64
+               : ap.shallow ? RD_ROUTE_ATT_ROWS16_SHALLOW : RD_ROUTE_ATT_ROWS16]++;
+      if (!ap.kl && !ap.t5 && !ap.wide && ap.n_splits > 1) h->route[RD_ROUTE_ATT_KEY_SPLIT]++;
+      if (ap.kl)
         CK(h, launch_attention_kl(h->kv_maps[(size_t)l * 2].bytes, h->v_maps[l].bytes, w.qkv, w.attn_t, rt, w.seq_off, h->att_seq_order, w.mask_t, dm, n_seq,
                                   attn_kl_row_tiles(rows_per_seq_max), h->tc_grid, w.status, ch, st));
-      else if (att_t5)
+      else if (ap.t5)
         CK(h, launch_attention_t5(h->kv_maps[(size_t)l * 2].bytes, h->kv_maps[(size_t)l * 2 + 1].bytes, w.qkv, w.attn_t, rt, w.seq_off, h->att_seq_order, dm, n_seq,
-                                  row_blocks, w.status, ch, st));
-      else if (att_wide)
+                                  ap.row_blocks, w.status, ch, st));
+      else if (ap.wide)
         CK(h, launch_attention_wide(w.qkv, kv_plane_ptr(h, l, 0), kv_plane_ptr(h, l, 1), w.attn_t, rt, w.seq_off, dm, n_seq,
-                                    row_blocks, ch, st));
+                                    ap.row_blocks, ch, st));
       else
         CK(h, launch_attention_tc(w.qkv, kv_plane_ptr(h, l, 0), kv_plane_ptr(h, l, 1), w.attn_t, rt, w.seq_off, dm, n_seq,
-                                  row_blocks, n_splits, split_chunks, split_min, w.att_scratch, w.att_counters,
+                                  ap.row_blocks, ap.n_splits, ap.split_chunks, ap.split_min, w.att_scratch, w.att_counters,
                                   (h->trace_next >= 0 && h->trace_next < TRACE_SLOTS) ? w.trace + (size_t)8 * h->trace_next++ : nullptr, ch,
-                                  att_shallow ? 1 : 0, st));
+                                  ap.shallow ? 1 : 0, st));
     }
     rc = gemm(h, w.attn_t, dm.d, h->wo[l], dm.d, dm.d, w.m_total, m_max, w.proj_d, dm.d, &g_o, ch, st, /*pair=*/1);
     if (rc) return rc;
@@ -786,7 +795,8 @@ int do_verify(rd_handle* h, const rd_packed& pk, cudaStream_t st, int32_t* argma
   const Dims& dm = h->dm;
   const int B = h->batch, m_max = B * dm.NMAX;
   CKP(h, PROF_MISC, launch_build_rows_tree(pk, w.ctx, w.row_tok, w.row_seq, w.row_pos, w.row_slot, w.row_ncache, w.row_local,
-                               w.row_out_index, w.seq_off, w.seq_order, keys_on_lanes_possible(h) ? w.mask_t : nullptr, argmax, w.m_total, dm, B, w.status, st));
+                               w.row_out_index, w.seq_off, w.seq_order, plan_attention(h, pk.mask != nullptr, B, dm.NMAX).kl ? w.mask_t : nullptr, argmax,
+                               w.m_total, dm, B, w.status, st));
   h->att_seq_order = B <= 1024 ? w.seq_order : nullptr;   // the row tables of this pass carry the sequences' order
   if (!verify_on_pairs(h, m_max)) h->tc_pairs = 0;
   int rc = forward_layers(h, pk.mask, m_max, B, dm.NMAX, h->w.lm_head, st);

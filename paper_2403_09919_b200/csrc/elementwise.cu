@@ -979,6 +979,25 @@ __global__ void __launch_bounds__(1024) build_rows_tree_kernel(rd_packed pk, con
   int32_t* s_ctx = off + B + 1;
   auto ctx_of = [&](int b) { return B <= ROWS_CTX ? s_ctx[b] : ctx[b]; };
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  if (blockIdx.x > 0) {
+    // The CTAs behind the first: the tree mask with rows and columns exchanged, 32 x 32 bits per warp and turn: lane i holds row
+    // r0 + i's word, the ballot of its bit k is the word of node 32 wd + k over those rows.
+    const int tiles = dm.MW * dm.MW;
+    for (int t = ((int)blockIdx.x - 1) * 32 + w; t < B * tiles; t += ((int)gridDim.x - 1) * 32) {
+      const int b = t / tiles, rw = (t - b * tiles) / dm.MW, wd = t - b * tiles - rw * dm.MW;
+      const int n = min(max(pk.n[b], 0), dm.NMAX), r = rw * 32 + lane;
+      if (wd * 32 >= n) continue;   // (rows past n have no bits, but their words are read)
+      const uint32_t word = r < n ? pk.mask[((size_t)b * dm.NMAX + r) * dm.MW + wd] : 0u;
+      uint32_t mine = 0;
+#pragma unroll
+      for (int k = 0; k < 32; ++k) {
+        const uint32_t v = __ballot_sync(0xffffffffu, (word >> k) & 1u);
+        if (lane == k) mine = v;
+      }
+      if (wd * 32 + lane < n) mask_t[((size_t)b * dm.NMAX + wd * 32 + lane) * dm.MW + rw] = mine;
+    }
+    return;
+  }
   // exclusive scan of the row counts, a block's worth of sequences at a time
   for (int b0 = 0, acc = 0; b0 < B; b0 += blockDim.x) {
     const int b = b0 + threadIdx.x;
@@ -1030,31 +1049,16 @@ __global__ void __launch_bounds__(1024) build_rows_tree_kernel(rd_packed pk, con
     row_local[m] = n;
     row_out_index[m] = idx;
   }
-  // The tree mask with rows and columns exchanged, 32 x 32 bits per warp and turn: lane i holds row r0 + i's word, the ballot of
-  // its bit k is the word of node 32 wd + k over those rows.
-  if (mask_t) {
-    const int tiles = dm.MW * dm.MW;
-    for (int t = w; t < B * tiles; t += (int)blockDim.x >> 5) {
-      const int b = t / tiles, rw = (t - b * tiles) / dm.MW, wd = t - b * tiles - rw * dm.MW;
-      const int n = off[b + 1] - off[b], r = rw * 32 + lane;
-      if (wd * 32 >= n) continue;   // (rows past n have no bits, but their words are read)
-      const uint32_t word = r < n ? pk.mask[((size_t)b * dm.NMAX + r) * dm.MW + wd] : 0u;
-      uint32_t mine = 0;
-#pragma unroll
-      for (int k = 0; k < 32; ++k) {
-        const uint32_t v = __ballot_sync(0xffffffffu, (word >> k) & 1u);
-        if (lane == k) mine = v;
-      }
-      if (wd * 32 + lane < n) mask_t[((size_t)b * dm.NMAX + wd * 32 + lane) * dm.MW + rw] = mine;
-    }
-  }
 }
 
 cudaError_t launch_build_rows_tree(const rd_packed& pk, const int32_t* ctx, int32_t* row_tok, int32_t* row_seq,
                                    int32_t* row_pos, int32_t* row_slot, int32_t* row_ncache, int32_t* row_local,
                                    int32_t* row_out_index, int32_t* seq_off, int32_t* seq_order, uint32_t* mask_t, int32_t* argmax, int32_t* m_total,
                                    const Dims& dm, int B, int* status, cudaStream_t st) {
-  launch_pdl(build_rows_tree_kernel, 1, 1024, ((size_t)B + 1 + (B <= ROWS_CTX ? B : 0)) * sizeof(int32_t), st, pk, ctx, row_tok, row_seq, row_pos, row_slot,
+  // With mask_t, a turn for every warp of up to 127 CTAs more.  (All turns in the one CTA: a pass of one layer of the 7B shape, 8 x 81 rows
+  // 353 -> 360 us, 4 x 300 560 -> 592, 16 x 161 1157 -> 1230, 16 x 300 2073 -> 2190.)
+  const int turns = mask_t ? (B * dm.MW * dm.MW + 31) / 32 : 0;
+  launch_pdl(build_rows_tree_kernel, 1 + (turns < 127 ? turns : 127), 1024, ((size_t)B + 1 + (B <= ROWS_CTX ? B : 0)) * sizeof(int32_t), st, pk, ctx, row_tok, row_seq, row_pos, row_slot,
                                                                     row_ncache, row_local, row_out_index, seq_off,
                                                                     B <= ROWS_CTX ? seq_order : nullptr, mask_t, argmax, m_total, dm, B, status);
   return cudaGetLastError();
