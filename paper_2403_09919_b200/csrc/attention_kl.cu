@@ -26,8 +26,9 @@
 // output.  Every wait is bounded (one second), as in attention_t5.cu; a warp that gives up still takes part in the named barriers
 // until all of its part have seen it.
 //
-// What bounds it: the copies where every SM has tiles (7B, 16 sequences of 256 to 2048 tokens: 70 us a launch without the remainders
-// for 302 MB of keys and values, launch and set-up included, 95 us in the 64- and 128-row kernels), else a chunk's chain of hand-overs
+// What bounds it: the copies where every SM has tiles (7B, 16 sequences of 1024 tokens and 52 rows: 69 us a launch for 309 MB, 4.5 TB/s
+// or 0.69 of the measured copy rate, tensor pipe 18 %; without the remainders 16 of 256 to 2048 tokens took 70 us, 95 in the 64- and
+// 128-row kernels), else a chunk's chain of hand-overs
 // (scores 0.25 us, weights 0.35 to 0.6 us by columns, the product; 0.8 to 1.5 us a chunk) and, in the first, the code's fetch.
 // The remainders take 0.3 % of a 7B step (30 rows, 512 tokens), 0.4 to 0.9 of the 7B calls, 1.5 of the batch-16 step and 2 of
 // 4 x 4096 tokens at 33B, most of it for forming and storing them (doubled columns alone: 0.3 %).  One buffer of weights
@@ -54,7 +55,7 @@ constexpr int KL_MAX_SLOTS = 12;
 constexpr uint32_t KL_TMEM = 512;      // columns: two score buffers of 128, the output from 256 (twice a tile's columns)
 constexpr int KL_MAX_TILES = 32;       // tiles of a CTA
 constexpr uint32_t KL_SMEM = 227 * 1024;
-constexpr float KL_SLACK = 32.0f;      // log2 by which a score may exceed its row's reference
+constexpr float KL_SLACK = 32.0f;      // log2 by which a score may exceed its row's reference (values beyond 2^80 could overflow the sums)
 constexpr float KL_LOW = 64.0f;        // ... and its largest may stay below it
 
 // K^T-major operands: see tcgen05.cuh for the K-major one.  MN-major, 128-byte swizzle: 64 elements per line, 8 keys 1024 bytes
@@ -543,7 +544,8 @@ __global__ void __launch_bounds__(KL_THREADS, 1)
       s_rows = p.seq_off[lane + 1] - s_row0;
       if (s_rows > 0) s_nc = p.rt.n_cache[s_row0];
     }
-    // rows that a tile may have: as few as leave every tile a CTA of its own (narrow tiles take less time per chunk), else the most
+    // rows that a tile may have: as few as leave every tile a CTA of its own (narrow tiles take less time per chunk), else the most.
+    // (The launch has as many CTAs as there are tiles of the most rows, so a sequence whose bound is one such tile is never cut.)
     int most = KL_ROWS, first = 0, count = 0;   // first, count: of this lane's sequence, when tiles are that narrow
     if (few)
       for (int m = 32; m < KL_ROWS && most == KL_ROWS; m += 16) {

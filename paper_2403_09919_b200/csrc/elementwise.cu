@@ -190,7 +190,8 @@ static int wide_sm_count() {
 }
 // Partial slots loaded up front, for all of a thread's columns before the first is used; a longer list takes further rounds of as
 // many.  (One load after the other, and the gain requested last, a row took 10.4 us in the 13B step, whose CTAs have one row each
-// and whose O tiles lie between five CTAs; 5.5 now.  240 rows of the 7B shape 7.3 -> 6.3 us a launch, 736 rows 15.8 -> 13.)
+// and whose O tiles lie between five CTAs; 5.5 now.  240 rows of the 7B shape 7.3 -> 6.3 us a launch, 736 rows 15.8 -> 13.  At 64 registers, two CTAs per SM, 4 bytes are spilled,
+// 16 in fp32.)
 constexpr int WIDE_FOLD_NORM = 2;
 
 template <typename T, int NORM_MAXV>

@@ -74,9 +74,9 @@ def test_matches_the_other_kernels(monkeypatch, heads, lens, beam, distinct):
 
 @pytest.mark.parametrize("kv_scale", [12.0, 60.0, 400.0])
 def test_scores_far_from_the_reference(monkeypatch, kv_scale):
-    """Scores of some tens, hundreds and thousands (base 2): rows whose largest lies above and below what a reference of zero
-    serves, in the first chunk and in later ones.  The softmax is then nearly a choice of one key, so that a lost or doubled
-    rescale shows in the first digit."""
+    """Scores of some tens, hundreds and thousands (base 2): rows whose largest lies above what a reference of zero serves, in the
+    first chunk and in later ones (below: test_gpu_attention_exact.py).  The softmax is then nearly a choice of one key, so that
+    a lost or doubled rescale shows in the first digit."""
     cfg = config(4, max_batch=3, beam_width=9, max_ctx=700)
     beams = np.random.default_rng(7).integers(0, 900, size=(3, 9, 5))
     ours = outputs(monkeypatch, cfg, [600, 130, 260], beams, kv_scale, RD_ATT_KL=2)

@@ -1,10 +1,10 @@
-"""Verification passes at the larger workloads' own context lengths, through the attention kernel each of them takes by
-default (Section 3.4: attention over the KV cache plus the tree mask).
+"""Verification passes at the larger workloads' own context lengths, through the attention kernels with the rows on the lanes
+(Section 3.4: attention over the KV cache plus the tree mask).
 
-The library picks among four bf16 attention kernels by row count, context length and the number of (head, sequence,
-row tile) CTAs.  The depth-reduced shape cases use prompts of about a hundred tokens and so never reach the kernels
-that the 13B (1024-token prompt, 321 rows), the batched 7B (contexts 256-2048, batch 16) and the 33B workload
-(4096-token prompts, batch 4) run on.  Each case here keeps what decides the routing -- head dimension, rows per
+The library picks among five bf16 attention kernels by the number of heads, row count, context length and the number of (head,
+sequence, row tile) CTAs.  Models of fewer than 24 heads, as here, take the four of this file; for the 7B, 13B and 33B shapes
+they are the ones beyond the lines of the fifth (test_gpu_attention_kl.py).  The depth-reduced shape cases use prompts of about a
+hundred tokens and so never reach the kernels of long contexts.  Each case here keeps what decides the routing -- head dimension, rows per
 sequence, context length, enough CTAs -- on a model small enough for the oracle (2 layers, d_model 512-2048), runs one
 planted-beam verification pass on top of a GPU-prefilled cache, checks it against the oracle element by element, and
 asserts through redrafter_route_counts that the intended kernel did the work.
